@@ -44,6 +44,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -58,6 +59,7 @@ constexpr int kStages = 4;                     // depth of the shared-memory rin
 constexpr int kTileBytes = kTile * 32;         // 16 bf16 per block
 constexpr size_t kWsFixedBytes = 2048;
 constexpr unsigned int kWaitLimit = 1u << 18;  // mbarrier polls before a wait gives up (a poll takes microseconds: about a second)
+constexpr unsigned int kGridWaitLimit = 1u << 21;  // polls of the grid's arrival counter before a CTA gives up (each most of a microsecond)
 constexpr unsigned int kProducerSleepNs = 32;  // the producer's pause between polls for a free stage
 constexpr int kBracketMinBeta = 2;             // the bracket needs two multipliers; a single one is modes 1-3
 
@@ -107,6 +109,7 @@ struct Params {
   unsigned int nblk;   // rows * cols/16
   unsigned int nbc;    // cols/16
   unsigned int ntiles;
+  unsigned int nbc_magic, nbc_shift;   // b / nbc == __umulhi(2 b, nbc_magic) >> nbc_shift for every b < 2^31
   int contiguous;      // ld == cols: a tile is one contiguous run of bytes
   int max_iters;
   float early_stop_rel;
@@ -267,31 +270,12 @@ struct __align__(128) Ring {
   int fail;
 };
 
-// The same ring with, per stage, the tile's 8-byte block states next to its weights.
-struct __align__(128) RingWithState {
-  unsigned char tile[kStages][kTileBytes];
-  unsigned char state[kStages][kTile * 8];
-  unsigned long long full[kStages];
-  unsigned long long empty[kStages];
-  int meta_tensor[kStages];
-  unsigned int meta_tile[kStages];
-  int fail;
-};
-
 // Producer: start the copies of tile `tile` of tensor `p` into stage `s` (one copy when rows
 // are contiguous, else one per row segment) and arm the stage's barrier with the byte count.
-template <typename R>
-__device__ __forceinline__ void ring_issue(R& ring, const Params& p, unsigned int tile, int s) {
+__device__ __forceinline__ void ring_issue(Ring& ring, const Params& p, unsigned int tile, int s) {
   const unsigned int b0 = tile * kTile;
   unsigned int nb = min(static_cast<unsigned int>(kTile), p.nblk - b0);
-  if constexpr (sizeof(R) == sizeof(RingWithState)) {
-    // the state array is padded to 256 bytes, so rounding the copy up to 16 stays inside it
-    const unsigned int sbytes = (nb * 8u + 15u) & ~15u;
-    mbar_expect_tx(&ring.full[s], nb * 32u + sbytes);
-    bulk_load(ring.state[s], p.state + b0, sbytes, &ring.full[s]);
-  } else {
-    mbar_expect_tx(&ring.full[s], nb * 32u);
-  }
+  mbar_expect_tx(&ring.full[s], nb * 32u);
   unsigned char* dst = ring.tile[s];
   if (p.contiguous) {
     bulk_load(dst, p.W + static_cast<size_t>(b0) * 16, nb * 32u, &ring.full[s]);
@@ -322,8 +306,7 @@ __device__ __forceinline__ int tensor_of(const Batch& bt, unsigned int g, unsign
 }
 
 // All threads: barriers ready before anyone uses them.
-template <typename R>
-__device__ __forceinline__ void ring_init(R& ring) {
+__device__ __forceinline__ void ring_init(Ring& ring) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&ring.full[s], 1);
@@ -349,8 +332,7 @@ __device__ __forceinline__ void record_failure(const Batch& bt) {
 // back.  After the last tile it posts an end marker.  A wait that gives up records the
 // failure, lets copies still in flight land (bounded) and ends the sequence; the consumers
 // then give up on their own.
-template <typename R>
-__device__ __forceinline__ void ring_produce(R& ring, const Batch& bt, int reverse, unsigned int run_mask) {
+__device__ __forceinline__ void ring_produce(Ring& ring, const Batch& bt, int reverse, unsigned int run_mask) {
   if (bt.idle_producer) return;   // test hook: nothing is fetched and nothing is in flight; the consumers give up
   unsigned int n = 0;
   bool ok = true;
@@ -382,12 +364,11 @@ __device__ __forceinline__ void ring_produce(R& ring, const Batch& bt, int rever
   }
 }
 
-// Consumer: the CTA's n-th stage.  Returns 0 with this thread's 32 bytes (and block state), the
+// Consumer: the CTA's n-th stage.  Returns 0 with this thread's 32 bytes, the
 // tile's tensor and its number, the stage handed back; 1 at the end marker; 2 when the wait
 // gave up.  On 1 and 2 the caller leaves its tile loop.
-template <typename R>
-__device__ __forceinline__ int ring_consume(R& ring, const Batch& bt, unsigned int n, uint4& v0, uint4& v1,
-                                            int& ti, unsigned int& tile, uint2* st = nullptr) {
+__device__ __forceinline__ int ring_consume(Ring& ring, const Batch& bt, unsigned int n, uint4& v0, uint4& v1,
+                                            int& ti, unsigned int& tile) {
   const int s = static_cast<int>(n % kStages);
   // the outcome is made the same for the whole warp
   if (!__all_sync(0xFFFFFFFFu, mbar_wait(&ring.full[s], (n / kStages) & 1u))) {
@@ -401,7 +382,6 @@ __device__ __forceinline__ int ring_consume(R& ring, const Batch& bt, unsigned i
   const uint4* src = reinterpret_cast<const uint4*>(ring.tile[s] + threadIdx.x * 32);
   v0 = src[0];
   v1 = src[1];
-  if constexpr (sizeof(R) == sizeof(RingWithState)) *st = reinterpret_cast<const uint2*>(ring.state[s])[threadIdx.x];
   mbar_arrive(&ring.empty[s]);
   return 0;
 }
@@ -491,30 +471,6 @@ __device__ __forceinline__ void code_sums(const Fixed& fx, unsigned int c0, unsi
   afix = __dp2a_hi(fx.pair[7], t3, a);
 }
 
-// The integer sums of the block's code vector under reciprocal scale r, from the magnitudes
-// alone: afix = sum fix_j * (2 m_j), b4 = sum (2 m_j)^2 with m_j = E2M1(fl(a_j * r)).  Without sign
-// bits the codes feed the byte permute as they are (the candidate loop only ranks; the signed
-// winner is re-made later).
-__device__ __forceinline__ void magnitude_sums(const float (&a)[16], const Fixed& fx, float r, unsigned int& afix,
-                                               unsigned int& b4) {
-  float x[16];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) mul2(a[2 * i], a[2 * i + 1], r, x[2 * i], x[2 * i + 1]);
-  const unsigned int c0 = e2m1x8(x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7]);
-  const unsigned int c1 = e2m1x8(x[8], x[9], x[10], x[11], x[12], x[13], x[14], x[15]);
-  const unsigned int t[4] = {twice_magnitude_x4(c0), twice_magnitude_x4(c0 >> 16), twice_magnitude_x4(c1),
-                             twice_magnitude_x4(c1 >> 16)};
-  unsigned int acc_a = 0, acc_b = 0;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    acc_b = __dp4a(t[q], t[q], acc_b);
-    acc_a = __dp2a_lo(fx.pair[2 * q], t[q], acc_a);
-    acc_a = __dp2a_hi(fx.pair[2 * q + 1], t[q], acc_a);
-  }
-  afix = acc_a;
-  b4 = acc_b;
-}
-
 // The same sums for a code vector whose scale lies far below the block maximum: binary64
 // accumulation in element order.
 __device__ __forceinline__ void code_sums_wide(const float (&w)[16], unsigned int c0, unsigned int c1, double& A,
@@ -591,51 +547,32 @@ __device__ __forceinline__ void load_weights(const float* h, unsigned int cb, do
 // tensor once (when the CTA's tile sequence leaves the tensor, or ends); the warp that arrives
 // last forwards the CTA's total to the tensor's global accumulators, one atomicAdd each.  No
 // CTA-wide barrier is involved.
-template <int N, bool kDet = false>
+template <int N>
 struct Slots {
   double acc[kMaxBatch][N];
-  // deterministic mode: each consumer warp's sums, added in warp order
-  double part[kMaxBatch][kDet ? kTile / 32 : 1][kDet ? N : 1];
   unsigned int count[kMaxBatch];
 };
 
 // All threads, before the tile loop (a __syncthreads follows in ring_init).
-template <int N, bool kDet>
-__device__ __forceinline__ void slots_clear(Slots<N, kDet>& sl) {
+template <int N>
+__device__ __forceinline__ void slots_clear(Slots<N>& sl) {
   for (int i = threadIdx.x; i < kMaxBatch * N; i += blockDim.x) (&sl.acc[0][0])[i] = 0.0;
   for (int i = threadIdx.x; i < kMaxBatch; i += blockDim.x) sl.count[i] = 0;
 }
 
-// Whole consumer warp: adds v[] for tensor `ti` and clears it.  With `ordered` the warps' sums are kept
-// apart and the last warp adds them in warp order and stores the CTA's total to dst (this CTA's own
-// slot) instead of adding it to a shared accumulator: the same bits on every run.
-template <int N, bool kDet>
-__device__ __forceinline__ void slots_add(Slots<N, kDet>& sl, int ti, double (&v)[N], double* const (&dst)[N]) {
-  constexpr bool ordered = kDet;
+// Whole consumer warp: adds v[] for tensor `ti` and clears it.
+template <int N>
+__device__ __forceinline__ void slots_add(Slots<N>& sl, int ti, double (&v)[N], double* const (&dst)[N]) {
 #pragma unroll
   for (int i = 0; i < N; ++i) v[i] = warp_sum(v[i]);
   if ((threadIdx.x & 31) == 0) {
-    if (ordered) {
 #pragma unroll
-      for (int i = 0; i < N; ++i) sl.part[ti][threadIdx.x >> 5][i] = v[i];
-    } else {
-#pragma unroll
-      for (int i = 0; i < N; ++i) atomicAdd(&sl.acc[ti][i], v[i]);
-    }
+    for (int i = 0; i < N; ++i) atomicAdd(&sl.acc[ti][i], v[i]);
     __threadfence_block();
     if (atomicAdd(&sl.count[ti], 1u) == kTile / 32 - 1) {
       __threadfence_block();
-      if (ordered) {
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-          double tot = 0.0;
-          for (int w = 0; w < kTile / 32; ++w) tot += *static_cast<volatile double*>(&sl.part[ti][w][i]);
-          *dst[i] = tot;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < N; ++i) atomicAdd(dst[i], atomicAdd(&sl.acc[ti][i], 0.0));
-      }
+      for (int i = 0; i < N; ++i) atomicAdd(dst[i], atomicAdd(&sl.acc[ti][i], 0.0));
     }
   }
 #pragma unroll
@@ -646,7 +583,7 @@ __device__ __forceinline__ void slots_add(Slots<N, kDet>& sl, int ti, double (&v
 // adds entries l, l + 32, ... in turn, then a fixed exchange tree); every lane gets the same bits.
 __device__ __forceinline__ double ordered_sum(const double* parts, int n) {
   double acc = 0.0;
-  for (int j = threadIdx.x & 31; j < n; j += 32) acc += parts[j];
+  for (int j = threadIdx.x & 31; j < n; j += 32) acc += __ldcg(parts + j);
   return warp_sum(acc);
 }
 
@@ -681,59 +618,6 @@ __device__ __forceinline__ void sumsq_block(const unsigned int (&u)[8], double& 
   }
 }
 
-// Eq. 1's tensor maximum, plus sum W^2 (binary64) for the error report.
-template <bool kDet>
-__global__ void __launch_bounds__(kThreads, 6) amax_kernel(const __grid_constant__ Batch bt, int reverse) {
-  __shared__ Ring ring;
-  __shared__ Slots<1, kDet> slots;
-  slots_clear(slots);
-  constexpr bool det = kDet;
-  if (det && threadIdx.x < bt.n) bt.t[threadIdx.x].det->sumsq[blockIdx.x] = 0.0;   // a CTA may never meet a tensor
-  ring_init(ring);
-  if (is_producer_warp()) {
-    if (threadIdx.x == kTile) ring_produce(ring, bt, reverse, 0xFFFFFFFFu);
-    return;
-  }
-  unsigned int mx = 0, nblk = 0;
-  double sq[2] = {0.0, 0.0};
-  int cur = -1;
-  for (unsigned int n = 0;; ++n) {
-    uint4 v0, v1;
-    int ti = -1;
-    unsigned int tile = 0;
-    const int rc = ring_consume(ring, bt, n, v0, v1, ti, tile);
-    if (rc != 0 || ti != cur) {
-      if (cur >= 0) {   // leaving tensor `cur`: hand over its maximum and sum
-        mx = max(mx & 0xFFFFu, mx >> 16);
-        mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-        if ((threadIdx.x & 31) == 0 && mx) atomicMax(&bt.t[cur].ws->amax_bits, mx);
-        double acc[1] = {sq[0] + sq[1]};
-        double* const dst[1] = {det ? &bt.t[cur].det->sumsq[blockIdx.x] : &bt.t[cur].ws->sumsq};
-        slots_add(slots, cur, acc, dst);
-        mx = 0;
-        sq[0] = sq[1] = 0.0;
-      }
-      if (rc != 0) break;
-      cur = ti;
-      nblk = bt.t[ti].nblk;
-    }
-    if (tile * kTile + threadIdx.x >= nblk) continue;
-    const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    // largest magnitude of the block with packed bf16 max (a NaN input comes out of the maximum
-    // as NaN, whose bits are above the infinity pattern)
-    unsigned int bmx = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      unsigned int m;
-      asm("abs.bf16x2 %0, %1;" : "=r"(m) : "r"(u[i]));
-      asm("max.NaN.bf16x2 %0, %0, %1;" : "+r"(bmx) : "r"(m));
-    }
-    bmx &= 0x7FFF7FFFu;
-    mx = __vmaxu2(mx, bmx);
-    sumsq_block(u, sq[0], sq[1]);
-  }
-}
-
 // Warp-level hand-over of two counters to a tensor's workspace.
 __device__ __forceinline__ void add_counters(Ws* ws, unsigned int& zeros, unsigned int& wide) {
   zeros = __reduce_add_sync(0xFFFFFFFFu, zeros);
@@ -743,103 +627,6 @@ __device__ __forceinline__ void add_counters(Ws* ws, unsigned int& zeros, unsign
     if (wide) atomicAdd(&ws->wide, static_cast<unsigned long long>(wide));
   }
   zeros = wide = 0;
-}
-
-// Algorithm 1 "Initialization" (Eq. 1): alpha0 = amax/(6*448), dd0 = E4M3(bmax/(6 alpha0)),
-// dq0 = dd0; first codes (Eq. 2); stage-0 sums for Eq. 5 and the starting error.  Codes and
-// scales are written here only when no iteration follows (final != 0).  Tensors with
-// non-finite or out-of-range input are skipped.
-template <bool kDet>
-__global__ void __launch_bounds__(kThreads) init_kernel(const __grid_constant__ Batch bt, int reverse, int final,
-                                                        int prev_grid) {
-  __shared__ Ring ring;
-  __shared__ Slots<3, kDet> slots;
-  slots_clear(slots);
-  constexpr bool det = kDet;
-  if (det) {
-    // this CTA's stage-0 slots start at zero; CTA 0 adds up the amax pass's per-CTA sums of squares in order
-    for (int i = threadIdx.x; i < bt.n * 3; i += kThreads) bt.t[i / 3].det->stage[0][i % 3][blockIdx.x] = 0.0;
-    if (blockIdx.x == 0)
-      for (int ti = threadIdx.x >> 5; ti < bt.n; ti += kThreads / 32) {
-        const double sq = ordered_sum(bt.t[ti].det->sumsq, prev_grid);
-        if ((threadIdx.x & 31) == 0) bt.t[ti].ws->sumsq = sq;
-      }
-  }
-  ring_init(ring);
-  if (is_producer_warp()) {
-    if (threadIdx.x == kTile) {
-      unsigned int run = 0;
-      for (int i = 0; i < bt.n; ++i)
-        if (!(status_from_amax(bt.t[i].ws->amax_bits) & (SOAR_STATUS_NONFINITE | SOAR_STATUS_RANGE))) run |= 1u << i;
-      ring_produce(ring, bt, reverse, run);
-    }
-    return;
-  }
-  float alpha = 1.0f, six_alpha = 6.0f;
-  double alpha_d = 1.0;
-  double acc[3] = {0.0, 0.0, 0.0};   // num, den, gsum
-  unsigned int zeros = 0, wide = 0;
-  int cur = -1;
-  Tensor p = {};   // the current tensor's pointers and size, kept in registers
-  for (unsigned int n = 0;; ++n) {
-    uint4 v0, v1;
-    int ti = -1;
-    unsigned int tile = 0;
-    const int rc = ring_consume(ring, bt, n, v0, v1, ti, tile);
-    if (rc != 0 || ti != cur) {
-      if (cur >= 0) {
-        Ws* ws = bt.t[cur].ws;
-        DetParts* dp = bt.t[cur].det;
-        double* const dst[3] = {det ? &dp->stage[0][0][blockIdx.x] : &ws->num[0],
-                                det ? &dp->stage[0][1][blockIdx.x] : &ws->den[0],
-                                det ? &dp->stage[0][2][blockIdx.x] : &ws->gsum[0]};
-        slots_add(slots, cur, acc, dst);
-        add_counters(ws, zeros, wide);
-      }
-      if (rc != 0) break;
-      cur = ti;
-      const unsigned int amax_bits = bt.t[ti].ws->amax_bits;
-      alpha = amax_bits == 0 ? 1.0f : __fdiv_rn(bits_to_mag(amax_bits), 2688.0f);
-      six_alpha = __fmul_rn(alpha, 6.0f);
-      alpha_d = static_cast<double>(alpha);
-      p = tensor_view(bt.t[ti]);
-    }
-    const unsigned int b = tile * kTile + threadIdx.x;
-    if (b >= p.nblk) continue;
-    Block blk;
-    unpack_block(v0, v1, blk);
-    uint2 codes;
-    if (blk.bmax == 0.0f) {
-      // all-zero block: codes carry the sign bits only, scale byte 0, left out of all sums
-      round_block(blk, 1.0f, codes.x, codes.y);
-      reinterpret_cast<uint2*>(p.packed)[b] = codes;
-      p.scales[b] = 0;
-      if (p.state != nullptr) p.state[b] = make_uint2(0u, 0u);
-      ++zeros;
-      continue;
-    }
-    int c = e4m3_encode(__fdiv_rn(blk.bmax, six_alpha));
-    c = max(c, 1);
-    const float v = e4m3_value(c);
-    const float r = recip_scale(alpha, v);
-    round_block(blk, r, codes.x, codes.y);
-    Fixed fx;
-    make_fixed(blk, fx);
-    double A, B;
-    block_sums(blk, fx, r, codes.x, codes.y, A, B, wide);
-    if (final) {
-      reinterpret_cast<uint2*>(p.packed)[b] = codes;
-      p.scales[b] = static_cast<uint8_t>(c);
-    }
-    if (p.state != nullptr)
-      p.state[b] = make_uint2(__float_as_uint(static_cast<float>(A)),
-                              static_cast<unsigned int>(B * 4.0) | (static_cast<unsigned int>(c) << 16));
-    const double vd = static_cast<double>(v);
-    const double sd = alpha_d * vd;
-    acc[0] = fma(A, vd, acc[0]);
-    acc[1] = fma(B * vd, vd, acc[1]);
-    acc[2] += sd * fma(sd, B, -2.0 * A);
-  }
 }
 
 // Error of stage s (Eq. 4) from the tensor sums.
@@ -876,36 +663,6 @@ __device__ __forceinline__ void iteration_head(const Params& p, int t, float& al
   run_out = run;
 }
 
-// Deterministic mode, head of the kernel that follows the pass which filled stage s (iteration s, or
-// the last kernel of the call): whole CTA.  For every tensor whose stage-s slots are current (the
-// filling pass worked on it), the slots of the `prev_grid` CTAs are added in index order into
-// latest[tensor][0..2]; CTA 0 also files the sums in the workspace header, where later kernels
-// read the stages before their own.  Every CTA computes the same bits.
-__device__ __forceinline__ void gather_stage(const Batch& bt, int s, int prev_grid, double (*latest)[3]) {
-  for (int ti = threadIdx.x >> 5; ti < bt.n; ti += blockDim.x >> 5) {
-    const Params& p = bt.t[ti];
-    int filled = 1;   // stage 0 comes from the init pass, which fills every tensor's slots
-    if (s > 0) {
-      float unused;
-      iteration_head(p, s - 1, unused, filled);
-    }
-    double v[3] = {0.0, 0.0, 0.0};
-    if (filled) {
-#pragma unroll
-      for (int i = 0; i < 3; ++i) v[i] = ordered_sum(p.det->stage[s & 1][i], prev_grid);
-    }
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-      for (int i = 0; i < 3; ++i) latest[ti][i] = v[i];
-      if (filled && blockIdx.x == 0) {
-        p.ws->num[s] = v[0];
-        p.ws->den[s] = v[1];
-        p.ws->gsum[s] = v[2];
-      }
-    }
-  }
-}
-
 // App. B.3's E4M3 codes around a block's analytic scale: d_lo .. d_hi before clipping (the
 // nearest code alone for n_dq == 1, else n_dq codes bracketing the scale).
 __device__ __forceinline__ void candidate_window(float center, int n_dq, int& d_lo, int& d_hi) {
@@ -917,18 +674,6 @@ __device__ __forceinline__ void candidate_window(float center, int n_dq, int& d_
     d_lo = cf - (n_dq / 2 - 1);
     d_hi = cf + n_dq / 2;
   }
-}
-
-// Eq. 6 with the new alpha from the previous winner's sums (all codes zero keeps the stored
-// scale), and the candidate codes around it.
-__device__ __forceinline__ float block_center(const uint2 st, float alpha, int n_dq, bool keep, int& d_lo,
-                                              int& d_hi) {
-  const int d_cur = static_cast<int>(st.y >> 16);
-  const float B0 = 0.25f * static_cast<float>(st.y & 0xFFFFu);
-  const float center = (B0 > 0.0f && !keep) ? __fdiv_rn(__uint_as_float(st.x), __fmul_rn(alpha, B0))
-                                             : e4m3_value(d_cur);
-  candidate_window(center, n_dq, d_lo, d_hi);
-  return center;
 }
 
 __device__ __forceinline__ int clip_code(int d) { return max(1, min(0x7E, d)); }
@@ -971,14 +716,18 @@ __device__ __forceinline__ void divisor_band(float alpha, float dv, float& lo, f
 
 // The range [ka, kb] of multipliers that can win for a code whose band is [lo, hi], for any start
 // index k: walks to the last multiplier with s_k <= lo, then on to the first with s_k >= hi.
-__device__ __forceinline__ void winning_range(const float* s_beta, int n_beta, float alpha, float center, float lo,
-                                           float hi, int k, int& ka, int& kb) {
+// s_beta: the multipliers, or pairs of neighbouring multipliers.
+__device__ __forceinline__ float multiplier(float b) { return b; }
+__device__ __forceinline__ float multiplier(float2 b) { return b.x; }
+template <typename B>
+__device__ __forceinline__ void winning_range(const B* s_beta, int n_beta, float alpha, float center, float lo, float hi,
+                                           int k, int& ka, int& kb) {
   k = max(0, min(n_beta - 1, k));
-  while (k >= 0 && grid_divisor(alpha, center, s_beta[k]) > lo) --k;
-  while (k + 1 < n_beta && grid_divisor(alpha, center, s_beta[k + 1]) <= lo) ++k;
+  while (k >= 0 && grid_divisor(alpha, center, multiplier(s_beta[k])) > lo) --k;
+  while (k + 1 < n_beta && grid_divisor(alpha, center, multiplier(s_beta[k + 1])) <= lo) ++k;
   ka = max(k, 0);
   kb = k + 1;
-  while (kb < n_beta && grid_divisor(alpha, center, s_beta[kb]) < hi) ++kb;
+  while (kb < n_beta && grid_divisor(alpha, center, multiplier(s_beta[kb])) < hi) ++kb;
   kb = min(kb, n_beta - 1);
 }
 
@@ -989,422 +738,7 @@ struct Winner {
   int d;
 };
 
-// One candidate of the search scored on the exact integer sums: codes (signs included), afix, 4B and
-// e = rho * 4B - afix, which orders candidates of one E4M3 code like their errors.
-struct Scored {
-  unsigned int c0, c1, afix, b4;
-  double e;
-};
-__device__ __forceinline__ void score_candidate(const Block& blk, const Fixed& fx, float s, double rho, Scored& o) {
-  round_block(blk, recip_fast(s), o.c0, o.c1);
-  code_sums(fx, o.c0, o.c1, o.afix, o.b4);
-  o.e = fma(rho, uint_to_double(o.b4), -uint_to_double(o.afix));
-}
-
-// One iteration t of Algorithm 1 for every block: Eq. 5 (from stage-t sums), Eq. 6,
-// App. B.3 candidate sets, Eq. 8 search, winner stored, stage-(t+1) sums accumulated.
-// Codes and scale bytes are written when `emit` is set (the state after this iteration may
-// be the one returned); the per-block sums are kept when `keep` is set (another iteration
-// may follow).  Modes 1 and 2 are the shapes with one quantization scale per E4M3 code and at most two
-// codes, whose passes are bound by HBM rather than by the candidate loop.  Mode 4 is the candidate
-// grid of App. B.3 searched through winning_range: per E4M3 code only the multipliers that can win
-// are rounded and scored, which gives the winner of the whole grid.
-template <int kMode, bool kDet>   // 0: candidate grid, every multiplier visited; 1: one candidate scale (beta = 1), at most two
-                       // codes; 2: the same with the coupled scale; 3: one candidate scale, any number of codes;
-                       // 4: candidate grid, only the multipliers that can win; 5: the same for grids so short that
-                       // a block's bracket often reaches past their first or last multiplier
-__global__ void __launch_bounds__(kThreads, (kMode == 1 || kMode == 3) ? 3 : 2)
-iterate_kernel(const __grid_constant__ Batch bt, int t, int reverse, int emit, int keep, int prev_grid) {
-  constexpr bool kSingle = kMode == 1 || kMode == 2 || kMode == 3;
-  __shared__ RingWithState ring;
-  __shared__ Slots<3, kDet> slots;
-  __shared__ float s_beta[kSingle ? 1 : SOAR_MAX_BETA];
-  __shared__ float s_alpha[kMaxBatch];
-  __shared__ double s_latest[kDet ? kMaxBatch : 1][3];
-  __shared__ unsigned int s_run;
-  constexpr bool det = kDet;
-  if (threadIdx.x == 0) s_run = 0;
-  if (det) {
-    // this CTA's slots of the stage it will fill start at zero; the stage the previous pass filled is added up
-    for (int i = threadIdx.x; i < bt.n * 3; i += kThreads) bt.t[i / 3].det->stage[(t + 1) & 1][i % 3][blockIdx.x] = 0.0;
-    gather_stage(bt, t, prev_grid, s_latest);
-  }
-  __syncthreads();
-  if (threadIdx.x < bt.n) {   // per tensor: still running?  its alpha for this iteration
-    float a;
-    int run;
-    iteration_head(bt.t[threadIdx.x], t, a, run, det ? s_latest[threadIdx.x] : nullptr);
-    s_alpha[threadIdx.x] = a;
-    if (run) atomicOr(&s_run, 1u << threadIdx.x);
-  }
-  const int n_dq = bt.t[0].n_dq, n_beta = bt.t[0].n_beta;
-  if (!kSingle) {
-    for (int k = threadIdx.x; k < n_beta; k += kThreads)
-      s_beta[k] = static_cast<float>((100.0 + static_cast<double>((k - n_beta / 2) * bt.t[0].beta_step_pct)) / 100.0);
-  }
-  slots_clear(slots);
-  __syncthreads();
-  if (s_run == 0) return;   // every tensor of the batch has stopped
-  ring_init(ring);
-  if (is_producer_warp()) {
-    if (threadIdx.x == kTile) ring_produce(ring, bt, reverse, s_run);
-    return;
-  }
-  float alpha = 1.0f;
-  double alpha_d = 1.0;
-  // mode 4: multiplier index of a scale ratio, k = (ratio - 1) * 100 / step + n_beta / 2
-  const float k_scale = 100.0f / static_cast<float>(max(bt.t[0].beta_step_pct, 1));
-  const float k_off = static_cast<float>(n_beta / 2) - k_scale;   // k = (dv / center) * k_scale + k_off
-
-  double acc[3] = {0.0, 0.0, 0.0};   // num, den, gsum of stage t+1
-  unsigned int wide = 0, unused_zeros = 0;
-  int cur = -1;
-  Tensor p = {};   // the current tensor's pointers and size, kept in registers
-  const int flags = bt.t[0].flags;
-  for (unsigned int n = 0;; ++n) {
-    uint4 v0, v1;
-    uint2 st;
-    int ti = -1;
-    unsigned int tile = 0;
-    const int rc = ring_consume(ring, bt, n, v0, v1, ti, tile, &st);
-    if (rc != 0 || ti != cur) {
-      if (cur >= 0) {
-        Ws* ws = bt.t[cur].ws;
-        DetParts* dp = bt.t[cur].det;
-        const int sb = (t + 1) & 1;
-        double* const dst[3] = {det ? &dp->stage[sb][0][blockIdx.x] : &ws->num[t + 1],
-                                det ? &dp->stage[sb][1][blockIdx.x] : &ws->den[t + 1],
-                                det ? &dp->stage[sb][2][blockIdx.x] : &ws->gsum[t + 1]};
-        slots_add(slots, cur, acc, dst);
-        add_counters(ws, unused_zeros, wide);
-      }
-      if (rc != 0) break;
-      cur = ti;
-      alpha = s_alpha[ti];
-      alpha_d = static_cast<double>(alpha);
-      if (kMode != 0) p = tensor_view(bt.t[ti]);
-    }
-    // the long candidate loop does better re-reading these from the parameter block per tile than
-    // carrying them in registers
-    if (kMode == 0) p = tensor_view(bt.t[ti]);
-    const unsigned int b = tile * kTile + threadIdx.x;
-    if (b >= p.nblk || (st.y >> 16) == 0) continue;   // past the end, or an all-zero block: nothing to optimise
-    Block blk;
-    unpack_block(v0, v1, blk);
-    int d_lo, d_hi;
-    const float center = block_center(st, alpha, n_dq, (flags & SOAR_FLAG_KEEP_BLOCK_SCALE) != 0, d_lo, d_hi);
-    const int dc0 = clip_code(d_lo), dc1 = clip_code(d_lo + 1);
-    const double sd0 = alpha_d * static_cast<double>(e4m3_value(dc0));
-    const double sd1 = alpha_d * static_cast<double>(e4m3_value(dc1));
-    Fixed fx;
-    make_fixed(blk, fx);
-    double best, bestA, bestB;
-    int best_d = dc0;
-    unsigned int best0, best1;
-    if (kMode == 2) {
-      // beta = 1 and the coupled scale of Sec. 3.2: each E4M3 candidate rounds the block with its
-      // own value and is scored with it
-      const float r0 = recip_scale(alpha, e4m3_value(dc0));
-      round_block(blk, r0, best0, best1);
-      block_sums(blk, fx, r0, best0, best1, bestA, bestB, wide);
-      best = sd0 * fma(sd0, bestB, -2.0 * bestA);
-      if (n_dq == 2) {
-        const float r1 = recip_scale(alpha, e4m3_value(dc1));
-        unsigned int c0, c1;
-        double A, B;
-        round_block(blk, r1, c0, c1);
-        block_sums(blk, fx, r1, c0, c1, A, B, wide);
-        const double g1 = sd1 * fma(sd1, B, -2.0 * A);
-        if (g1 < best) { best = g1; best_d = dc1; bestA = A; bestB = B; best0 = c0; best1 = c1; }
-      }
-    } else if (kSingle) {
-      // one quantization scale (beta = 1): the codes are fixed, only the E4M3 code is chosen
-      const float r = recip_scale(alpha, center);
-      round_block(blk, r, best0, best1);
-      block_sums(blk, fx, r, best0, best1, bestA, bestB, wide);
-      const double A2 = -2.0 * bestA;
-      best = sd0 * fma(sd0, bestB, A2);               // block error minus sum W^2
-      if (n_dq >= 2) {
-        const double g1 = sd1 * fma(sd1, bestB, A2);
-        if (g1 < best) { best = g1; best_d = dc1; }
-      }
-      if (kMode == 3) {
-        for (int d = d_lo + 2; d <= d_hi; ++d) {      // wider code windows (App. B.3 with more than two codes)
-          const int dc = clip_code(d);
-          const double sd = alpha_d * static_cast<double>(e4m3_value(dc));
-          const double g = sd * fma(sd, bestB, A2);
-          if (g < best) { best = g; best_d = dc; }
-        }
-      }
-    } else if (kMode == 4 || kMode == 5) {
-      const int nd = d_hi - d_lo + 1;
-      {
-        // Typical block: two E4M3 codes at most, each with exactly two multipliers that can win (the one
-        // just below value(code) / center and its successor), the exact integer sums valid and the
-        // fast reciprocal in range for the whole grid.  Those four candidates are scored in straight
-        // line; any other block takes the loops below.
-        const bool second = nd == 2 && dc1 != dc0;
-        const float per_center = __fdividef(k_scale, center);
-        const float dv0 = e4m3_value(dc0), dv1 = e4m3_value(dc1);
-        float lo0, hi0, lo1, hi1;
-        divisor_band(alpha, dv0, lo0, hi0);
-        divisor_band(alpha, dv1, lo1, hi1);
-        const int k0 = max(0, min(n_beta - 2, __float2int_rd(__fmaf_rn(dv0, per_center, k_off))));
-        const int k1 = max(0, min(n_beta - 2, __float2int_rd(__fmaf_rn(dv1, per_center, k_off))));
-        const float s00 = grid_divisor(alpha, center, s_beta[k0]), s01 = grid_divisor(alpha, center, s_beta[k0 + 1]);
-        const float s10 = grid_divisor(alpha, center, s_beta[k1]), s11 = grid_divisor(alpha, center, s_beta[k1 + 1]);
-        // the four divisors lie between s00 and s11 (or s01 without a second code): those two bound the range
-        // of the fast reciprocal, and the smallest one decides whether the exact integer sums hold
-        const float s_hi = second ? s11 : s01;
-        bool direct = nd <= 2 && fx.ok && recip_fast_ok(s00) && recip_fast_ok(s_hi) &&
-                      __fmul_rn(blk.bmax, recip_fast(s00)) <= 32.0f;
-        // Where the grid ends before the band does, one multiplier is all that can win: the first one when
-        // even its divisor lies beyond the band, the last one when even its divisor lies before it.  The
-        // pair then holds that multiplier twice.
-        // (Mode 5 only: a grid that spans 0.85 .. 1.15 holds the whole bracket of every regular block.)
-        const bool low0 = kMode == 5 && k0 == 0 && s00 >= hi0, high0 = kMode == 5 && k0 == n_beta - 2 && s01 <= lo0;
-        const bool low1 = kMode == 5 && k1 == 0 && s10 >= hi1, high1 = kMode == 5 && k1 == n_beta - 2 && s11 <= lo1;
-        direct = direct && ((s00 <= lo0 && s01 >= hi0) || low0 || high0);
-        if (second) direct = direct && ((s10 <= lo1 && s11 >= hi1) || low1 || high1);
-        if (direct) {
-          // error minus sum W^2 = 2 sd unit (rho * 4B - afix) with rho = sd / (8 unit): per code the two
-          // candidates are ranked on the exact integer sums, the codes' winners compared once
-          Scored a, c;
-          score_candidate(blk, fx, high0 ? s01 : s00, sd0 * fx.inv8, a);
-          {
-            Scored b2;
-            score_candidate(blk, fx, low0 ? s00 : s01, sd0 * fx.inv8, b2);
-            if (b2.e < a.e) a = b2;
-          }
-          double ga = 2.0 * sd0 * fx.unit * a.e;
-          best_d = dc0;
-          if (second) {
-            score_candidate(blk, fx, high1 ? s11 : s10, sd1 * fx.inv8, c);
-            Scored b2;
-            score_candidate(blk, fx, low1 ? s10 : s11, sd1 * fx.inv8, b2);
-            const bool later = b2.e < c.e;
-            if (later) c = b2;
-            const double gc = 2.0 * sd1 * fx.unit * c.e;
-            // equal errors: the earlier multiplier, as in grid order (k1 >= k0 always)
-            if (gc < ga) { ga = gc; a = c; best_d = dc1; }
-          }
-          best = ga;
-          best0 = a.c0;
-          best1 = a.c1;
-          bestA = uint_to_double(a.afix) * fx.unit;
-          bestB = uint_to_double(a.b4) * 0.25;
-        } else {
-          best = __longlong_as_double(0x7FF0000000000000ll);
-          bestA = bestB = 0.0;
-          best0 = best1 = 0u;
-          int best_k = 0, prev = -1;
-          for (int d = d_lo; d <= d_hi; ++d) {
-            const int dc = clip_code(d);
-            if (dc == prev) continue;   // clipping at the ends of the E4M3 range repeats a code
-            prev = dc;
-            const float dv = e4m3_value(dc);
-            const double sd = alpha_d * static_cast<double>(dv);
-            float lo, hi;
-            divisor_band(alpha, dv, lo, hi);
-            int ka, kb;
-            winning_range(s_beta, n_beta, alpha, center, lo, hi, __float2int_rd(__fmaf_rn(dv, per_center, k_off)), ka,
-                          kb);
-            for (int k = ka; k <= kb; ++k) {
-              const float sk = grid_divisor(alpha, center, s_beta[k]);
-              const float r = recip_fast_ok(sk) ? recip_fast(sk) : __frcp_rn(sk);
-              unsigned int c0, c1;
-              double A, B;
-              round_block(blk, r, c0, c1);
-              block_sums(blk, fx, r, c0, c1, A, B, wide);
-              const double g = sd * fma(sd, B, -2.0 * A);
-              // equal errors: the earlier multiplier, then the smaller code, as in grid order
-              if (g < best || (g == best && k < best_k)) {
-                best = g; bestA = A; bestB = B; best0 = c0; best1 = c1; best_d = dc; best_k = k;
-              }
-            }
-          }
-        }
-      }
-    } else {
-      // Eq. 8 over beta ascending, then scale code ascending; strict '<' keeps the first
-      // minimum.  Every candidate is scored in full, with no test for "same codes as the
-      // previous beta": under SIMT such a test only saves work when all 32 blocks of a warp
-      // pass it at once, and it costs instructions on every candidate.  The loop keeps just
-      // the best error and its (beta, code) index; the winner is re-made once at the end.
-      best = __longlong_as_double(0x7FF0000000000000ll);
-      int best_key = 0;
-      const int nd = d_hi - d_lo + 1;
-      // the reciprocal scale falls as beta grows, so the first candidate decides whether the
-      // exact integer sums hold for all of them
-      const bool coupled = (flags & SOAR_FLAG_COUPLED_SCALE) != 0;
-      const bool all_narrow = fx.ok && __fmul_rn(blk.bmax, recip_scale(alpha, __fmul_rn(center, s_beta[0]))) <= 32.0f;
-      // the products alpha * center * beta are monotone in beta: the end points bound them all
-      const bool fast_rcp = recip_fast_ok(__fmul_rn(alpha, __fmul_rn(center, s_beta[0]))) &&
-                            recip_fast_ok(__fmul_rn(alpha, __fmul_rn(center, s_beta[n_beta - 1])));
-      if (all_narrow && nd <= 2 && !coupled && fast_rcp) {
-        // error minus sum W^2 = sd^2 B - 2 sd A = q * (rho * (4B) - afix)  with  q = 2 sd unit > 0 and
-        // rho = sd / (8 unit): per E4M3 code the candidates are ranked by rho * 4B - afix alone (one fma),
-        // and the two codes' winners are compared once after the loop
-        const double rho0 = sd0 * fx.inv8, rho1 = sd1 * fx.inv8;
-        double h0 = best, h1 = best;
-        int k0 = 0, k1 = 0;
-        float mag[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) mag[j] = fabsf(blk.w[j]);
-        for (int k = 0; k < n_beta; ++k) {
-          const float r = recip_fast(__fmul_rn(alpha, __fmul_rn(center, s_beta[k])));
-          unsigned int afix, b4;
-          magnitude_sums(mag, fx, r, afix, b4);
-          const double ad = uint_to_double(afix), bd = uint_to_double(b4);
-          const double e0 = fma(rho0, bd, -ad);
-          if (e0 < h0) { h0 = e0; k0 = k; }
-          if (nd == 2) {
-            const double e1 = fma(rho1, bd, -ad);
-            if (e1 < h1) { h1 = e1; k1 = k; }
-          }
-        }
-        const double g0 = 2.0 * sd0 * fx.unit * h0;
-        const double g1 = (nd == 2) ? 2.0 * sd1 * fx.unit * h1 : best;
-        // first minimum in (beta, code) order
-        const bool second = g1 < g0 || (g1 == g0 && k1 < k0);
-        best = second ? g1 : g0;
-        best_key = second ? 2 * k1 + 1 : 2 * k0;
-      } else {
-        // general form: any number of E4M3 candidates, scales far below the block maximum, and the
-        // coupled arm of Sec. 3.2, where each E4M3 candidate rounds the block with its own value
-        for (int k = 0; k < n_beta; ++k) {
-          float r = recip_scale(alpha, __fmul_rn(center, s_beta[k]));
-          unsigned int c0, c1;
-          double A = 0.0, B = 0.0;
-          if (!coupled) {
-            round_block(blk, r, c0, c1);
-            block_sums(blk, fx, r, c0, c1, A, B, wide);
-          }
-          for (int d = 0; d < nd; ++d) {
-            const float dv = e4m3_value(clip_code(d_lo + d));
-            if (coupled) {
-              r = recip_scale(alpha, __fmul_rn(dv, s_beta[k]));
-              round_block(blk, r, c0, c1);
-              block_sums(blk, fx, r, c0, c1, A, B, wide);
-            }
-            const double sd = alpha_d * static_cast<double>(dv);
-            const double g = sd * fma(sd, B, -2.0 * A);
-            if (g < best) { best = g; best_key = (nd <= 2 ? 2 : nd) * k + d; }
-          }
-        }
-      }
-      // the winner, made again from its index
-      const int per = nd <= 2 ? 2 : nd;
-      const int bk = best_key / per;
-      best_d = clip_code(d_lo + (best_key - bk * per));
-      const float r = recip_scale(alpha, __fmul_rn(coupled ? e4m3_value(best_d) : center, s_beta[bk]));
-      round_block(blk, r, best0, best1);
-      unsigned int unused = 0;
-      block_sums(blk, fx, r, best0, best1, bestA, bestB, unused);
-    }
-    // The winner: codes and scale out, sums kept for the next iteration's Eq. 6.
-    if (emit) {
-      reinterpret_cast<uint2*>(p.packed)[b] = make_uint2(best0, best1);
-      p.scales[b] = static_cast<uint8_t>(best_d);
-    }
-    if (keep)
-      p.state[b] = make_uint2(__float_as_uint(static_cast<float>(bestA)),
-                              static_cast<unsigned int>(bestB * 4.0) | (static_cast<unsigned int>(best_d) << 16));
-    const double vd = static_cast<double>(e4m3_value(best_d));
-    acc[0] = fma(bestA, vd, acc[0]);
-    acc[1] = fma(bestB * vd, vd, acc[1]);
-    acc[2] += best;
-  }
-}
-
-// Where each tensor of a batch wants its alpha and its report (report may be null).
-struct Reports {
-  float* alpha[kMaxBatch];
-  soar_result* result[kMaxBatch];
-};
-
-// Replays the early-stop rule over the stage sums, writes alpha and the report; one CTA per tensor.
-__global__ void __launch_bounds__(128) finalize_kernel(const __grid_constant__ Batch bt,
-                                                       const __grid_constant__ Reports rp, int prev_grid) {
-  const Params& p = bt.t[blockIdx.x];
-  float* out_alpha = rp.alpha[blockIdx.x];
-  soar_result* res = rp.result[blockIdx.x];
-  __shared__ double s_num[SOAR_MAX_ITERS + 1], s_den[SOAR_MAX_ITERS + 1], s_sse[SOAR_MAX_ITERS + 1];
-  __shared__ double s_ta[SOAR_MAX_ITERS + 1];
-  __shared__ int s_iters;
-  if (p.det != nullptr) {
-    // deterministic mode: the stage the last pass filled is still in the per-CTA slots; this CTA (the
-    // only one working on this tensor) adds them up in order and files them in the header
-    if (threadIdx.x < 32) {
-      int filled = 1;
-      if (p.max_iters > 0) {
-        float unused;
-        iteration_head(p, p.max_iters - 1, unused, filled);
-      }
-      if (filled) {
-        double v[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) v[i] = ordered_sum(p.det->stage[p.max_iters & 1][i], prev_grid);
-        if (threadIdx.x == 0) {
-          p.ws->num[p.max_iters] = v[0];
-          p.ws->den[p.max_iters] = v[1];
-          p.ws->gsum[p.max_iters] = v[2];
-        }
-      }
-    }
-    __threadfence_block();
-    __syncthreads();
-  }
-  const Ws* ws = p.ws;
-  const unsigned int amax_bits = ws->amax_bits;
-  const int st = status_from_amax(amax_bits);
-  for (int i = threadIdx.x; i <= SOAR_MAX_ITERS; i += blockDim.x) {
-    const bool used = i <= p.max_iters;
-    s_num[i] = used ? ws->num[i] : 0.0;
-    s_den[i] = used ? ws->den[i] : 0.0;
-    s_sse[i] = (used && st == 0) ? stage_sse(ws, i) : 0.0;
-    s_ta[i] = 0.0;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float alpha = (st & SOAR_STATUS_ZERO_TENSOR) ? 1.0f : __fdiv_rn(bits_to_mag(amax_bits), 2688.0f);
-    int iters = 0;
-    s_ta[0] = static_cast<double>(alpha);
-    if (st == 0 && ws->error == 0) {
-      double prev = s_sse[0];
-      for (int i = 0; i < p.max_iters; ++i) {
-        if (s_den[i] > 0.0 && !(p.flags & SOAR_FLAG_KEEP_ALPHA)) alpha = static_cast<float>(s_num[i] / s_den[i]);
-        const double cur = s_sse[i + 1];
-        iters = i + 1;
-        s_ta[iters] = static_cast<double>(alpha);
-        if (stops_after(prev, cur, p.early_stop_rel)) break;
-        prev = cur;
-      }
-    }
-    s_iters = iters;
-    *out_alpha = alpha;
-    if (res != nullptr) {
-      res->status = st | ((ws->error & kErrWait) ? SOAR_STATUS_INTERNAL : 0) |
-                    ((ws->error & kErrWeight) ? SOAR_STATUS_BAD_WEIGHT : 0);
-      res->iters_run = iters;
-      res->alpha = alpha;
-      res->amax = bits_to_mag(amax_bits);
-      res->sse = s_sse[iters];
-      res->sse_init = s_sse[0];
-      res->sumsq = (st & SOAR_STATUS_ZERO_TENSOR) ? 0.0 : ws->sumsq;
-      res->zero_blocks = static_cast<int64_t>(ws->zero_blocks);
-      res->wide_candidates = static_cast<int64_t>(ws->wide);
-    }
-  }
-  __syncthreads();
-  if (res != nullptr) {
-    const int iters = s_iters;
-    for (int i = threadIdx.x; i <= SOAR_MAX_ITERS; i += blockDim.x) {
-      res->trace_alpha[i] = (i <= iters) ? s_ta[i] : 0.0;
-      res->trace_sse[i] = (i <= iters) ? s_sse[i] : 0.0;
-    }
-  }
-}
+#include "quantize_kernel.cuh"
 
 // Offset of scale (row, col) in the 128x4-tiled layout: tiles of 128 rows x 4 scale columns
 // (512 bytes), tile rows outermost; inside a tile row r and column c sit at
@@ -1413,22 +747,6 @@ __device__ __forceinline__ size_t swizzled_offset(unsigned int row, unsigned int
   const size_t tile = static_cast<size_t>(row >> 7) * col_tiles + (col >> 2);
   const unsigned int r = row & 127u;
   return tile * 512 + (r & 31u) * 16 + (r >> 5) * 4 + (col & 3u);
-}
-
-__global__ void __launch_bounds__(256) swizzle_kernel(const uint8_t* lin, uint8_t* sw, unsigned int rows,
-                                                      unsigned int nbc, unsigned int row_tiles,
-                                                      unsigned int col_tiles) {
-  const size_t total = static_cast<size_t>(row_tiles) * col_tiles * 512;
-  for (size_t o = static_cast<size_t>(blockIdx.x) * 256 + threadIdx.x; o < total;
-       o += static_cast<size_t>(gridDim.x) * 256) {
-    const size_t tile = o >> 9;
-    const unsigned int in = static_cast<unsigned int>(o & 511);
-    const unsigned int tr = static_cast<unsigned int>(tile / col_tiles);
-    const unsigned int tc = static_cast<unsigned int>(tile - static_cast<size_t>(tr) * col_tiles);
-    const unsigned int row = tr * 128 + ((in >> 2) & 3u) * 32 + (in >> 4);
-    const unsigned int col = tc * 4 + (in & 3u);
-    sw[o] = (row < rows && col < nbc) ? lin[static_cast<size_t>(row) * nbc + col] : 0;
-  }
 }
 
 // Eq. 3-4 on stored outputs: sum (w - q s)^2 and sum w^2, one binary64 fma per term, with the
@@ -2337,8 +1655,78 @@ size_t soar_batch_workspace_bytes(const soar_tensor_desc* tensors, int n, const 
 
 namespace {
 
-// Which launches a call makes: all of them (soar_quantize_batch), or one stage
-// (soar_quantize_stage; iterations t_lo <= t < t_hi for kStageIterate).
+// nbc's multiply-and-shift division, exact for every dividend below 2^31.
+void set_division(Params& p) {
+  unsigned int l = 0;
+  while ((1ull << l) < p.nbc) ++l;
+  p.nbc_shift = l;
+  p.nbc_magic = static_cast<unsigned int>(((1ull << (31 + l)) + p.nbc - 1) / p.nbc);
+}
+
+// CTAs of quantize_kernel<mode, det> an SM holds, asked of the runtime once per device.
+template <int kMode, bool kDet>
+int quantize_per_sm() {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
+  int n = known[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, quantize_kernel<kMode, kDet>, kQThreads, 0) != cudaSuccess || n <= 0)
+      n = 1;
+    known[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
+// Launches stages [lo, hi) of the quantizer for one group of matrices; more than one stage makes the launch
+// cooperative, so that its CTAs, which meet between stages, run at the same time.
+template <int kMode, bool kDet>
+cudaError_t launch_stages(const Batch& bt, const Reports& rp, unsigned int tiles, int lo, int hi, cudaStream_t st) {
+  unsigned int grid = static_cast<unsigned int>(sm_count() * quantize_per_sm<kMode, kDet>());
+  if (grid > static_cast<unsigned int>(kMaxGrid)) grid = kMaxGrid;   // the deterministic mode keeps one slot per CTA
+  const unsigned int want = (tiles + kQWarps - 1) / kQWarps;
+  if (want < grid) grid = want > 0 ? want : 1u;
+  if (hi - lo == 1) {
+    quantize_kernel<kMode, kDet><<<grid, kQThreads, 0, st>>>(bt, rp, lo, hi);
+    return cudaGetLastError();
+  }
+  void* args[] = {const_cast<Batch*>(&bt), const_cast<Reports*>(&rp), &lo, &hi};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&quantize_kernel<kMode, kDet>), dim3(grid), dim3(kQThreads),
+                                     args, 0, st);
+}
+
+cudaError_t launch_stages(int mode, bool det, const Batch& bt, const Reports& rp, unsigned int tiles, int lo, int hi,
+                          cudaStream_t st) {
+#define SOAR_STAGES(M) (det ? launch_stages<M, true>(bt, rp, tiles, lo, hi, st) : launch_stages<M, false>(bt, rp, tiles, lo, hi, st))
+  switch (mode) {
+    case 0: return SOAR_STAGES(0);
+    case 1: return SOAR_STAGES(1);
+    case 2: return SOAR_STAGES(2);
+    case 4: return SOAR_STAGES(4);
+    default: return SOAR_STAGES(5);
+  }
+#undef SOAR_STAGES
+}
+
+// kMode of quantize_kernel for a call's settings (see iterate_pass).
+int search_mode(const soar_cfg* cfg) {
+  const bool coupled = (cfg->flags & SOAR_FLAG_COUPLED_SCALE) != 0;
+  // one quantization scale per block: the codes are made once (any number of E4M3 codes scored on them; the coupled
+  // arm, where every code rounds the block anew, only with at most two)
+  if (cfg->n_beta == 1 && (cfg->n_dq <= 2 || !coupled)) return coupled ? 2 : 1;
+  // a grid of several multipliers with one quantization scale per multiplier: only those that can win are visited;
+  // the coupled arm with a grid, and multipliers that all coincide, visit them all
+  if (coupled || cfg->n_beta < kBracketMinBeta || cfg->beta_step_pct < 1) return 0;
+  // the brackets of two E4M3 codes around the Eq. 6 solution lie at multipliers 0.89 .. 1.13 (E4M3 values are at most
+  // an eighth apart): a grid from 0.85 to 1.15 or wider holds them whole, a shorter one needs the path that knows
+  // the grid's ends
+  const int half = cfg->n_beta / 2;
+  const bool spans = 100 - half * cfg->beta_step_pct <= 85 && 100 + (cfg->n_beta - 1 - half) * cfg->beta_step_pct >= 115;
+  return spans ? 4 : 5;
+}
+
+// Which part of a call is wanted: all of it (soar_quantize_batch), or one stage (soar_quantize_stage; iterations
+// t_lo <= t < t_hi for kStageIterate).
 enum : int { kStageAmax = 1, kStageInit = 2, kStageIterate = 4, kStageFinalize = 8, kStageAll = 15 };
 
 int run_batch(const soar_tensor_desc* tensors, int n, const soar_cfg* cfg, void* workspace, size_t workspace_bytes,
@@ -2372,10 +1760,7 @@ int run_batch(const soar_tensor_desc* tensors, int n, const soar_cfg* cfg, void*
       cudaMemsetAsync(headers, 0, static_cast<size_t>(n) * kWsFixedBytes, st) != cudaSuccess)
     return SOAR_ERR_CUDA;
 
-  // one quantization scale per block: the codes are made once (any number of E4M3 codes scored on them;
-  // the coupled arm, where every code rounds the block anew, only with at most two)
-  const bool single = cfg->n_beta == 1 && (cfg->n_dq <= 2 || !(cfg->flags & SOAR_FLAG_COUPLED_SCALE));
-  const bool may_stop = cfg->early_stop_rel > 0.0f;
+  const int mode = search_mode(cfg);
   for (int first = 0; first < n; first += kMaxBatch) {
     Batch bt;
     Reports rp;
@@ -2393,7 +1778,8 @@ int run_batch(const soar_tensor_desc* tensors, int n, const soar_cfg* cfg, void*
       p.ld = d.ld;
       p.nbc = static_cast<unsigned int>(d.cols / 16);
       p.nblk = static_cast<unsigned int>(d.rows * (d.cols / 16));
-      p.ntiles = (p.nblk + kTile - 1) / kTile;
+      p.ntiles = (p.nblk + 31) / 32;
+      set_division(p);
       p.contiguous = (d.ld == d.cols) ? 1 : 0;
       p.state = nullptr;
       if (cfg->max_iters > 0) {
@@ -2418,95 +1804,34 @@ int run_batch(const soar_tensor_desc* tensors, int n, const soar_cfg* cfg, void*
       p.beta_step_pct = cfg->beta_step_pct;
       p.flags = cfg->flags;
       tiles += p.ntiles;
-      bt.tile_end[j] = tiles;
       rp.alpha[j] = d.out_global_fp32;
       rp.result[j] = d.out_result;
+      rp.scales_sw[j] = want_sw ? static_cast<uint8_t*>(d.out_e4m3_scales_sw) : nullptr;
+      rp.rows[j] = static_cast<unsigned int>(d.rows);
     }
-    for (int j = bt.n; j < kMaxBatch; ++j) bt.tile_end[j] = 0xFFFFFFFFu;   // never reached by a tile index
-    bt.total_tiles = tiles;
 
-    // Passes alternate direction over the tiles (amax forward, init backward, iteration t forward
-    // for even t): each starts where the previous one ended, on data still in L2.
-    const unsigned int g_amax = det ? persistent_grid(amax_kernel<true>, tiles, kThreads)
-                                    : persistent_grid(amax_kernel<false>, tiles, kThreads);
-    const unsigned int g_init = det ? persistent_grid(init_kernel<true>, tiles, kThreads)
-                                    : persistent_grid(init_kernel<false>, tiles, kThreads);
-    unsigned int g_last = g_init;   // grid of the pass whose sums the next kernel's head reads
-    if (stages & kStageAmax) {
-      ScopedLaunch sl(K_AMAX, st);
-      if (det) amax_kernel<true><<<g_amax, kThreads, 0, st>>>(bt, 0);
-      else amax_kernel<false><<<g_amax, kThreads, 0, st>>>(bt, 0);
-    }
-    if (stages & kStageInit) {
-      ScopedLaunch sl(K_INIT, st);
-      const int final = cfg->max_iters == 0 ? 1 : 0;
-      if (det) init_kernel<true><<<g_init, kThreads, 0, st>>>(bt, 1, final, static_cast<int>(g_amax));
-      else init_kernel<false><<<g_init, kThreads, 0, st>>>(bt, 1, final, static_cast<int>(g_amax));
-    }
-    if (stages & kStageIterate) {
-      // a grid of several multipliers with one quantization scale per multiplier: only those that can win
-      // are visited (mode 4); the coupled arm and grids of a few multipliers visit them all (mode 0)
-      const bool bracketed = !(cfg->flags & SOAR_FLAG_COUPLED_SCALE) && cfg->n_beta >= kBracketMinBeta &&
-                             cfg->beta_step_pct >= 1;
-      // the brackets of two E4M3 codes around the Eq. 6 solution lie at multipliers 0.89 .. 1.13 (E4M3 values are
-      // at most an eighth apart): a grid from 0.85 to 1.15 or wider holds them whole (mode 4), a shorter one
-      // needs the straight-line path to know the grid's ends (mode 5)
-      const int half = cfg->n_beta / 2;
-      const bool spans = 100 - half * cfg->beta_step_pct <= 85 &&
-                         100 + (cfg->n_beta - 1 - half) * cfg->beta_step_pct >= 115;
-      const int mode = !single ? (bracketed ? (spans ? 4 : 5) : 0)
-                               : ((cfg->flags & SOAR_FLAG_COUPLED_SCALE) ? 2 : (cfg->n_dq <= 2 ? 1 : 3));
-      unsigned int g_it = 0;
-      for (int t = t_lo; t < t_hi; ++t) {
-        const int reverse = t & 1;
-        // with the early stop on, any iteration may turn out to be the last one
-        const int last = (t == cfg->max_iters - 1) ? 1 : 0;
-        const int emit = (may_stop || last) ? 1 : 0;
-        const int pg = static_cast<int>(g_last);
-        ScopedLaunch sl(K_ITERATE, st);
-#define SOAR_LAUNCH_ITERATE(M, D)                                                           \
-  do {                                                                                      \
-    if (g_it == 0) g_it = persistent_grid(iterate_kernel<M, D>, tiles, kThreads);           \
-    iterate_kernel<M, D><<<g_it, kThreads, 0, st>>>(bt, t, reverse, emit, !last, pg);       \
-  } while (0)
-        if (det) {
-          if (mode == 0) SOAR_LAUNCH_ITERATE(0, true);
-          else if (mode == 1) SOAR_LAUNCH_ITERATE(1, true);
-          else if (mode == 2) SOAR_LAUNCH_ITERATE(2, true);
-          else if (mode == 3) SOAR_LAUNCH_ITERATE(3, true);
-          else if (mode == 4) SOAR_LAUNCH_ITERATE(4, true);
-          else SOAR_LAUNCH_ITERATE(5, true);
-        } else {
-          if (mode == 0) SOAR_LAUNCH_ITERATE(0, false);
-          else if (mode == 1) SOAR_LAUNCH_ITERATE(1, false);
-          else if (mode == 2) SOAR_LAUNCH_ITERATE(2, false);
-          else if (mode == 3) SOAR_LAUNCH_ITERATE(3, false);
-          else if (mode == 4) SOAR_LAUNCH_ITERATE(4, false);
-          else SOAR_LAUNCH_ITERATE(5, false);
-        }
-#undef SOAR_LAUNCH_ITERATE
-        g_last = g_it;
+    const int report = kQStageIterate + cfg->max_iters, end = report + 1 + (want_sw ? 1 : 0);
+    cudaError_t err = cudaSuccess;
+    if (stages == kStageAll && !g_trace.on) {
+      // the whole call in one launch
+      err = launch_stages(mode, det, bt, rp, tiles, 0, end, st);
+    } else {
+      // stage by stage: a caller that combines the headers between stages, or a trace that times each of them
+      auto one = [&](int id, int s) {
+        if (err != cudaSuccess) return;
+        ScopedLaunch sl(id, st);
+        err = launch_stages(mode, det, bt, rp, tiles, s, s + 1, st);
+      };
+      if (stages & kStageAmax) one(K_AMAX, kQStageAmax);
+      if (stages & kStageInit) one(K_INIT, kQStageInit);
+      if (stages & kStageIterate)
+        for (int t = t_lo; t < t_hi; ++t) one(K_ITERATE, kQStageIterate + t);
+      if (stages & kStageFinalize) {
+        one(K_FINALIZE, report);
+        if (want_sw) one(K_SWIZZLE, report + 1);
       }
     }
-    if (!(stages & kStageFinalize)) continue;
-    {
-      ScopedLaunch sl(K_FINALIZE, st);
-      finalize_kernel<<<bt.n, 128, 0, st>>>(bt, rp, static_cast<int>(g_last));
-    }
-    if (want_sw) {
-      for (int j = 0; j < bt.n; ++j) {
-        const soar_tensor_desc& d = tensors[first + j];
-        const Params& p = bt.t[j];
-        const unsigned int rt = static_cast<unsigned int>((d.rows + 127) / 128);
-        const unsigned int ct = (p.nbc + 3) / 4;
-        const size_t total = static_cast<size_t>(rt) * ct * 512;
-        const size_t blocks = (total + 255) / 256;
-        const unsigned int grid = static_cast<unsigned int>(blocks < 65535u * 16u ? blocks : 65535u * 16u);
-        ScopedLaunch sl(K_SWIZZLE, st);
-        swizzle_kernel<<<grid, 256, 0, st>>>(p.scales, static_cast<uint8_t*>(d.out_e4m3_scales_sw),
-                                             static_cast<unsigned int>(d.rows), p.nbc, rt, ct);
-      }
-    }
+    if (err != cudaSuccess) return SOAR_ERR_CUDA;
   }
   return cudaGetLastError() == cudaSuccess ? SOAR_OK : SOAR_ERR_CUDA;
 }
@@ -2748,6 +2073,8 @@ int soar_quantize_weighted_batch(const soar_tensor_desc* tensors, const float* c
       bt.tile_end[j] = tiles;
       rp.alpha[j] = d.out_global_fp32;
       rp.result[j] = d.out_result;
+      rp.scales_sw[j] = want_sw ? static_cast<uint8_t*>(d.out_e4m3_scales_sw) : nullptr;
+      rp.rows[j] = static_cast<unsigned int>(d.rows);
     }
     for (int j = bt.n; j < kMaxBatch; ++j) bt.tile_end[j] = 0xFFFFFFFFu;   // never reached by a tile index
     bt.total_tiles = tiles;
@@ -2769,22 +2096,15 @@ int soar_quantize_weighted_batch(const soar_tensor_desc* tensors, const float* c
       ScopedLaunch sl(K_WEIGHTED_ITERATE, st);
       weighted_iterate_kernel<<<g_it, kThreads, 0, st>>>(bt, wb, t, reverse, (may_stop || last) ? 1 : 0, !last);
     }
+    const int report = kQStageIterate + cfg->max_iters;
     {
       ScopedLaunch sl(K_FINALIZE, st);
-      finalize_kernel<<<bt.n, 128, 0, st>>>(bt, rp, 0);
+      if (launch_stages(1, false, bt, rp, static_cast<unsigned int>(bt.n * kQWarps), report, report + 1, st) != cudaSuccess)
+        return SOAR_ERR_CUDA;
     }
     if (want_sw) {
-      for (int j = 0; j < bt.n; ++j) {
-        const soar_tensor_desc& d = tensors[first + j];
-        const Params& p = bt.t[j];
-        const unsigned int rt = static_cast<unsigned int>((d.rows + 127) / 128);
-        const unsigned int ct = (p.nbc + 3) / 4;
-        const size_t blocks = (static_cast<size_t>(rt) * ct * 512 + 255) / 256;
-        const unsigned int grid = static_cast<unsigned int>(blocks < 65535u * 16u ? blocks : 65535u * 16u);
-        ScopedLaunch sl(K_SWIZZLE, st);
-        swizzle_kernel<<<grid, 256, 0, st>>>(p.scales, static_cast<uint8_t*>(d.out_e4m3_scales_sw),
-                                             static_cast<unsigned int>(d.rows), p.nbc, rt, ct);
-      }
+      ScopedLaunch sl(K_SWIZZLE, st);
+      if (launch_stages(1, false, bt, rp, tiles * (kTile / 32), report + 1, report + 2, st) != cudaSuccess) return SOAR_ERR_CUDA;
     }
   }
   return cudaGetLastError() == cudaSuccess ? SOAR_OK : SOAR_ERR_CUDA;
