@@ -388,111 +388,122 @@ __device__ __forceinline__ void lay_out_pass(S& sh, const Batch& bt) {
   __syncthreads();
 }
 
-// One warp's walk over its share of the pass's tiles (positions first, first + step, ...; from the back of the
-// sequence for `reverse`: consecutive passes alternate so that a pass starts on what the previous one left in L2).
-// `enter(ti)` and `leave(ti)` bracket the tiles of one tensor; `body(b0, nb, v0, v1, st)` gets the tile's first block,
-// its number of blocks (lane's block valid when lane < nb), the lane's 32 bytes and, with kState, its block state.
+// One warp's run of tiles within one tensor: local tile numbers first, first + step, ... (`left` of them), where the
+// warp's positions in the pass's sequence fall into the tensor.  From the back of the sequence for `reverse`:
+// consecutive passes alternate so that a pass starts on what the previous one left in L2.
+struct Run {
+  int ti;
+  unsigned int left;
+  int tile, step;
+};
+
+// The run after `r` (r.ti = -1: the first one); left == 0 when the warp's share of the pass is over.
+template <typename S>
+__device__ __forceinline__ void next_run(const S& sh, int n, bool reverse, unsigned int warp, unsigned int warps, Run& r) {
+  r.left = 0;
+  int at = reverse ? n - 1 - r.ti : r.ti;
+  if (r.ti < 0) at = -1;
+  while (++at < n) {
+    const int ti = reverse ? n - 1 - at : at;
+    const unsigned int count = sh.count[ti], start = reverse ? sh.total - sh.start[ti] - count : sh.start[ti];
+    const unsigned int past = start % warps;
+    const unsigned int first = warp >= past ? warp - past : warp + warps - past;
+    if (first < count) {
+      r.ti = ti;
+      r.left = (count - 1 - first) / warps + 1;
+      r.tile = static_cast<int>(reverse ? count - 1 - first : first);
+      r.step = reverse ? -static_cast<int>(warps) : static_cast<int>(warps);
+      return;
+    }
+  }
+}
+
+// One warp's walk over its share of the pass's tiles.  `enter(ti)` and `leave(ti)` bracket the tiles of one tensor;
+// `body(b, v0, v1, st)` gets the lane's block number (past the tensor's end in the last tile: the body looks), its
+// 32 bytes and, with kState, its block state.  The warp number is broadcast so that the compiler sees the
+// bookkeeping as uniform; per tile it is a handful of instructions beside the copies.
 template <bool kState, typename S, typename Enter, typename Leave, typename Body>
 __device__ __forceinline__ void walk_tiles(S& sh, const Batch& bt, bool reverse, Enter enter, Leave leave, Body body) {
-  const unsigned int lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const unsigned int step = gridDim.x * kQWarps, first = blockIdx.x * kQWarps + warp, total = sh.total;
-  if (first >= total) return;
-  const unsigned int n = (total - first - 1) / step + 1;
+  const unsigned int lane = threadIdx.x & 31u, warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
+  const unsigned int warps = gridDim.x * kQWarps, me = blockIdx.x * kQWarps + warp;
   const unsigned int ring = smem_u32(sh.ring[warp]);
-  const unsigned int put = tile_chunk(lane) * 16, get = tile_chunk(2 * lane) * 16;
-  int g_step = static_cast<int>(step);
-  unsigned int g_in = first, g_out;
-  if (reverse) {
-    g_in = total - 1 - first;
-    g_step = -g_step;
-  }
-  g_out = g_in;
+  const unsigned int put = ring + tile_chunk(lane) * 16, get = ring + tile_chunk(2 * lane) * 16;
+  const unsigned int put_state = ring + kQStages * kQTileBytes + lane * 16, get_state = ring + kQStages * kQTileBytes + lane * 8;
 
-  // the feeding side's tensor
-  unsigned int f_start = 0, f_count = 0, f_nblk = 0;
-  const unsigned char* f_w = nullptr;
-  const unsigned char* f_state = nullptr;
-  bool f_contiguous = true;
-  int f_ti = 0;
-  auto feed = [&](unsigned int slot) {
-    unsigned int local = g_in - f_start;
-    if (local >= f_count) {
-      f_ti = 0;
-      while (g_in - sh.start[f_ti] >= sh.count[f_ti]) ++f_ti;
-      const Params& p = bt.t[f_ti];
-      f_start = sh.start[f_ti];
-      f_count = sh.count[f_ti];
-      f_nblk = p.nblk;
-      f_contiguous = p.contiguous != 0;
-      f_w = reinterpret_cast<const unsigned char*>(p.W) + (f_contiguous ? lane * 16 : 0);
-      if (kState) f_state = reinterpret_cast<const unsigned char*>(p.state) + lane * 16;
-      local = g_in - f_start;
+  Run f;          // the feeding side
+  f.ti = -1;
+  const unsigned char *f_w = nullptr, *f_state = nullptr;
+  long long f_w_step = 0, f_state_step = 0;
+  bool f_plain = true;   // contiguous, and every tile of the run whole
+  auto enter_feed = [&]() {
+    next_run(sh, bt.n, reverse, me, warps, f);
+    if (f.left == 0) return;
+    const Params& p = bt.t[f.ti];
+    // the ragged last tile is the last of a forward run, the first of a backward one
+    const int top = reverse ? f.tile : f.tile + static_cast<int>(f.left - 1) * f.step;
+    f_plain = p.contiguous && static_cast<unsigned int>(top) * 32 + 32 <= p.nblk;
+    f_w = reinterpret_cast<const unsigned char*>(p.W) + (f_plain ? static_cast<size_t>(f.tile) * kQTileBytes + lane * 16 : 0);
+    f_w_step = static_cast<long long>(f.step) * kQTileBytes;
+    if (kState) {
+      f_state = reinterpret_cast<const unsigned char*>(p.state) + static_cast<size_t>(f.tile) * kQStateBytes + lane * 16;
+      f_state_step = static_cast<long long>(f.step) * kQStateBytes;
     }
-    const unsigned int b0 = local * 32;
-    const unsigned int dst = slot + put;
-    const unsigned int nb = f_nblk - b0;
-    if (f_contiguous) {
-      const unsigned char* src = f_w + static_cast<size_t>(b0) * 32;
-      if (nb >= 32) {
-        copy16(dst, src);
-        copy16(dst + 512, src + 512);
-      } else {
-        if (lane < 2 * nb) copy16(dst, src);
-        if (lane + 32 < 2 * nb) copy16(dst + 512, src + 512);
-      }
+  };
+  auto feed = [&](unsigned int k) {
+    if (f.left == 0) return;
+    const unsigned int dst = put + k * kQTileBytes;
+    if (f_plain) {
+      copy16(dst, f_w);
+      copy16(dst + 512, f_w + 512);
+      f_w += f_w_step;
     } else {
-      const Params& p = bt.t[f_ti];
+      const Params& p = bt.t[f.ti];
+      const unsigned int b0 = static_cast<unsigned int>(f.tile) * 32;
 #pragma unroll
       for (unsigned int h = 0; h < 2; ++h) {
         const unsigned int b = b0 + h * 16 + (lane >> 1);
         const unsigned int row = __umulhi(2u * b, p.nbc_magic) >> p.nbc_shift;
         const unsigned char* src = f_w + (static_cast<long long>(row) * p.ld + (b - row * p.nbc) * 16) * 2 + (lane & 1u) * 16;
-        if (lane + 32 * h < 2 * nb) copy16(dst + 512 * h, src);
+        if (b < p.nblk) copy16(dst + 512 * h, src);
       }
+      f.tile += f.step;
     }
     if (kState) {
       // the state array is padded to 256 bytes, so whole tiles stay inside it
-      if (lane < 16) copy16(slot + kQTileBytes + lane * 16, f_state + static_cast<size_t>(b0) * 8);
+      if (lane < 16) copy16(put_state + k * kQStateBytes, f_state);
+      f_state += f_state_step;
     }
-    g_in += g_step;
+    if (--f.left == 0) enter_feed();
   };
 
-  unsigned int slot_in = 0, slot_out = 0;
+  enter_feed();
 #pragma unroll
   for (unsigned int k = 0; k < kQStages - 1; ++k) {
-    if (k < n) feed(ring + slot_in);
+    feed(k);
     copies_commit();
-    slot_in += kQSlotBytes;
   }
-  int ti = -1;
-  unsigned int t_start = 0, t_count = 0, t_nblk = 0;
-  for (unsigned int k = 0; k < n; ++k) {
-    copies_wait<kQStages - 2>();
-    __syncwarp();   // every lane's copies have landed, and every lane has read the slot that is filled next
-    if (k + kQStages - 1 < n) feed(ring + slot_in);
-    copies_commit();
-    slot_in = slot_in == (kQStages - 1) * kQSlotBytes ? 0u : slot_in + kQSlotBytes;
-    unsigned int local = g_out - t_start;
-    if (local >= t_count) {
-      if (ti >= 0) leave(ti);
-      ti = 0;
-      while (g_out - sh.start[ti] >= sh.count[ti]) ++ti;
-      t_start = sh.start[ti];
-      t_count = sh.count[ti];
-      t_nblk = bt.t[ti].nblk;
-      local = g_out - t_start;
-      enter(ti);
+  Run r;
+  r.ti = -1;
+  unsigned int k = 0;
+  for (next_run(sh, bt.n, reverse, me, warps, r); r.left != 0; next_run(sh, bt.n, reverse, me, warps, r)) {
+    enter(r.ti);
+    unsigned int b = static_cast<unsigned int>(r.tile) * 32 + lane;
+    const unsigned int b_step = static_cast<unsigned int>(r.step) * 32;
+    for (unsigned int left = r.left; left != 0; --left) {
+      copies_wait<kQStages - 2>();
+      __syncwarp();   // every lane's copies have landed, and every lane has read the slot that is filled next
+      feed((k + kQStages - 1) % kQStages);
+      copies_commit();
+      const unsigned int at = get + k * kQTileBytes;
+      const uint4 v0 = lds128(at), v1 = lds128(at ^ 16u);
+      uint2 st = make_uint2(0u, 0u);
+      if (kState) st = lds64(get_state + k * kQStateBytes);
+      k = (k + 1) % kQStages;
+      body(b, v0, v1, st);
+      b += b_step;
     }
-    const unsigned int at = ring + slot_out;
-    const uint4 v0 = lds128(at + get), v1 = lds128(at + (get ^ 16u));
-    uint2 st = make_uint2(0u, 0u);
-    if (kState) st = lds64(at + kQTileBytes + lane * 8);
-    slot_out = slot_out == (kQStages - 1) * kQSlotBytes ? 0u : slot_out + kQSlotBytes;
-    const unsigned int b0 = local * 32;
-    body(b0, t_nblk - b0, v0, v1, st);
-    g_out += g_step;
+    leave(r.ti);
   }
-  if (ti >= 0) leave(ti);
 }
 
 // A warp hands its sums for tensor ti to the CTA's.
@@ -580,8 +591,9 @@ __device__ __forceinline__ void amax_pass(QShared<kDet>& sh, const Batch& bt) {
   const unsigned int lane = threadIdx.x & 31u;
   unsigned int mx = 0;
   double sq[2] = {0.0, 0.0};
+  unsigned int nblk = 0;
   walk_tiles<false>(
-      sh, bt, false, [](int) {},
+      sh, bt, false, [&](int ti) { nblk = bt.t[ti].nblk; },
       [&](int ti) {
         mx = max(mx & 0xFFFFu, mx >> 16);
         mx = __reduce_max_sync(0xFFFFFFFFu, mx);
@@ -591,8 +603,8 @@ __device__ __forceinline__ void amax_pass(QShared<kDet>& sh, const Batch& bt) {
         mx = 0;
         sq[0] = sq[1] = 0.0;
       },
-      [&](unsigned int, unsigned int nb, const uint4& v0, const uint4& v1, const uint2&) {
-        if (lane >= nb) return;
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&) {
+        if (b >= nblk) return;
         const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
         // largest magnitude of the block with packed bf16 max (a NaN input comes out of the maximum
         // as NaN, whose bits are above the infinity pattern)
@@ -612,7 +624,6 @@ __device__ __forceinline__ void amax_pass(QShared<kDet>& sh, const Batch& bt) {
 // Eq. 5 and the starting error.  Codes and scales are written here only when no iteration follows (final).
 template <bool kDet>
 __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt, bool final) {
-  const unsigned int lane = threadIdx.x & 31u;
   float alpha = 1.0f, six_alpha = 6.0f, six_inv = 0.0f;
   double alpha_d = 1.0;
   bool tame = false;
@@ -633,9 +644,8 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt, bo
         hand_over(sh, ti, acc);
         hand_over_counters(sh, ti, zeros, wide);
       },
-      [&](unsigned int b0, unsigned int nb, const uint4& v0, const uint4& v1, const uint2&) {
-        if (lane >= nb) return;
-        const size_t b = static_cast<size_t>(b0) + lane;
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&) {
+        if (b >= p.nblk) return;
         PairBlock blk;
         unpack_pairs(v0, v1, blk);
         float bmax = 0.0f;
@@ -669,8 +679,13 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt, bo
           f.d = d;
           // A = afix / (2 S)
           f.A = __fmul_rn(__uint2float_rn(afix), __uint_as_float((__float_as_uint(s) & 0x7F800000u) - (11u << 23)));
-          const double sd = alpha_d * static_cast<double>(v);
-          f.g = sd * fma(sd * 0.25, uint_to_double(f.b4), -2.0 * static_cast<double>(f.A));
+          // error minus sum W^2 = alpha (h e) 4 / S^2 with h = v S / 4, e = alpha h 4B - afix (v may be subnormal in E4M3,
+          // never in binary32)
+          const unsigned int s_exp = __float_as_uint(s) & 0x7F800000u;
+          const double h = scaled_value(__float_as_uint(v), static_cast<int>(135u << 20) - static_cast<int>(s_exp >> 3));
+          const double e = fma(alpha_d * h, uint_to_double(f.b4), -uint_to_double(afix));
+          f.g = h * e * __hiloint2double(__double2hiint(alpha_d) + static_cast<int>(s_exp >> 2) - (272 << 20),
+                                         __double2loint(alpha_d));
         } else {
           f = start_general(v0, v1, alpha, &wide);
           v = e4m3_value(f.d);
@@ -698,7 +713,6 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt, bo
 //   kMode 5  the same for grids so short that a block's bracket often reaches past their first or last multiplier
 template <int kMode, bool kDet>
 __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt, bool reverse, bool emit, bool keep) {
-  const unsigned int lane = threadIdx.x & 31u;
   const int n_dq = bt.t[0].n_dq, n_beta = bt.t[0].n_beta, flags = bt.t[0].flags;
   const bool keep_scale = (flags & SOAR_FLAG_KEEP_BLOCK_SCALE) != 0;
   // multiplier index of a scale ratio: k = (ratio - 1) * 100 / step + n_beta / 2
@@ -722,170 +736,162 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
         hand_over(sh, ti, acc);
         hand_over_counters(sh, ti, zeros, wide);
       },
-      [&](unsigned int b0, unsigned int nb, const uint4& v0, const uint4& v1, const uint2& st) {
-        if (lane >= nb || st.y == 0u) return;   // past the end, or an all-zero block: nothing to optimise
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2& st) {
+        const bool active = b < p.nblk && st.y != 0u;   // past the end, or an all-zero block: nothing to optimise
         // Eq. 6, A / (alpha B): with 4B and alpha / 4 the powers of two cancel exactly
         const float b4_prev = __fsub_rn(__uint_as_float((st.y & 0xFFFu) | 0x4B000000u), 8388608.0f);
         const float stored = e4m3_value(static_cast<int>((st.y >> 12) & 0x7Fu));
         const float D = __fmul_rn(alpha_q, b4_prev);
         float center = quotient(__uint_as_float(st.x), D, recip_fast(D));
-        if (keep_scale && alpha_q > 0.0f) center = stored;
+        if (keep_scale) center = alpha_q > 0.0f ? stored : alpha_q;
         PairBlock blk;
         unpack_pairs(v0, v1, blk);
         // Regular block: the center inside the normal E4M3 range (which also rejects B = 0 and a NaN alpha_q), so the
-        // codes below and above it are its leading bits and the next.
+        // codes below and above it are its leading bits and the next.  The candidates are made and scored for every
+        // lane; what an irregular block gets from that is overwritten by the general search below.
         bool direct = __float_as_uint(center) - 0x3C800000u < 0x43E00000u - 0x3C800000u;
-        Candidate w;
-        unsigned int dv_bits = 0, s_exp = 0;
-        double g_scaled = 0.0;
-        if (direct) {
-          unsigned int dv0 = __float_as_uint(center) & 0xFFF00000u, dv1 = dv0 + 0x00100000u;
-          if (n_dq == 1) {   // the nearest code alone
-            dv0 = __float_as_uint(e4m3_value(e4m3_encode(center)));
-            dv1 = dv0;
-          }
-          const float v0f = __uint_as_float(dv0), v1f = __uint_as_float(dv1);
-          if (kMode == 4 || kMode == 5) {
-            float y;
-            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(center));
-            const float per_center = y * k_scale;
-            // floor by a round-down addition: the index sits in the low bits of the sum
-            const float t0 = __fadd_rd(__fmaf_rn(v0f, per_center, k_off), 12582912.0f);
-            const float t1 = __fadd_rd(__fmaf_rn(v1f, per_center, k_off), 12582912.0f);
-            int k0 = __float_as_int(t0) - 0x4B400000, k1 = __float_as_int(t1) - 0x4B400000;
-            if (kMode == 5) {
-              k0 = max(0, min(n_beta - 2, k0));
-              k1 = max(0, min(n_beta - 2, k1));
-            }
-            const uint2 q0 = lds64(pairs + 8u * static_cast<unsigned int>(k0));
-            const uint2 q1 = lds64(pairs + 8u * static_cast<unsigned int>(k1));
-            const pair_t cc = pair_of(center, center), aa = pair_of(alpha, alpha);
-            const pair_t m0 = pair_mul(cc, pair_of(__uint_as_float(q0.x), __uint_as_float(q0.y)));
-            const pair_t m1 = pair_mul(cc, pair_of(__uint_as_float(q1.x), __uint_as_float(q1.y)));
-            float a0, b0f, a1, b1;
-            halves(m0, a0, b0f);
-            halves(m1, a1, b1);
-            // The pair of multipliers must enclose the code's value with a margin that covers the three roundings
-            // from here to the scaled value (2^-24 each; see winning_range): 6 * 2^-24 does.  A block that misses it,
-            // one in several thousand, takes the exact walk.
-            constexpr float kUnder = 1.0f - 0x1.8p-22f, kOver = 1.0f + 0x1.8p-22f;
-            const bool below0 = a0 <= v0f * kUnder, above0 = b0f >= v0f * kOver;
-            const bool below1 = a1 <= v1f * kUnder, above1 = b1 >= v1f * kOver;
-            // Mode 5, where the grid ends before the band does: one multiplier is all that can win, the first one when
-            // even its divisor lies beyond the band, the last one when even its divisor lies before it.  The pair then
-            // holds that multiplier twice.
-            bool low0 = false, low1 = false, high0 = false, high1 = false;
-            if (kMode == 5) {
-              low0 = k0 == 0 && a0 >= v0f * kOver;
-              high0 = k0 == n_beta - 2 && b0f <= v0f * kUnder;
-              low1 = k1 == 0 && a1 >= v1f * kOver;
-              high1 = k1 == n_beta - 2 && b1 <= v1f * kUnder;
-            }
-            float s00, s01, s10, s11;
-            halves(pair_mul(aa, m0), s00, s01);
-            halves(pair_mul(aa, m1), s10, s11);
-            // the largest magnitude of the block below 32 times the smallest scale, from the exponents
-            direct = ((below0 && above0) || low0 || high0) && ((below1 && above1) || low1 || high1) &&
-                     st.y < (__float_as_uint(s00) & 0x7F800000u) + (5u << 23);
-            if (direct) {
-              if (kMode == 5) {
-                if (high0) s00 = s01;
-                if (low0) s01 = s00;
-                if (high1) s10 = s11;
-                if (low1) s11 = s10;
-              }
-              s_exp = __float_as_uint(s00) & 0x7F800000u;
-              FixedPairs fx;
-              make_fixed_pairs(blk, fixed_scale(s00), fx);
-              // h = dv S / 4; the exponent of S / 4 is 135 less s's biased one
-              const int k_field = static_cast<int>(135u << 20) - static_cast<int>(s_exp >> 3);
-              const double h0 = scaled_value(dv0, k_field), h1 = scaled_value(dv1, k_field);
-              const double rho0 = alpha_d * h0, rho1 = alpha_d * h1;
-              Candidate x, y2;
-              score_pairs(blk, fx, recip_fast(s00), rho0, w);
-              score_pairs(blk, fx, recip_fast(s01), rho0, x);
-              if (x.e < w.e) w = x;
-              score_pairs(blk, fx, recip_fast(s10), rho1, x);
-              score_pairs(blk, fx, recip_fast(s11), rho1, y2);
-              if (y2.e < x.e) x = y2;
-              // equal errors: the earlier multiplier, as in grid order (the second code's are never earlier)
-              const double g0 = h0 * w.e, g1 = h1 * x.e;
-              g_scaled = g0;
-              dv_bits = dv0;
-              if (g1 < g0) { w = x; g_scaled = g1; dv_bits = dv1; }
-            }
-          } else if (kMode == 1 || kMode == 2) {
-            const float s0 = __fmul_rn(alpha, kMode == 1 ? center : v0f), s1 = __fmul_rn(alpha, v1f);
-            direct = st.y < (__float_as_uint(s0) & 0x7F800000u) + (5u << 23);
-            if (direct) {
-              s_exp = __float_as_uint(s0) & 0x7F800000u;
-              FixedPairs fx;
-              make_fixed_pairs(blk, fixed_scale(s0), fx);
-              const int k_field = static_cast<int>(135u << 20) - static_cast<int>(s_exp >> 3);
-              const double h0 = scaled_value(dv0, k_field), h1 = scaled_value(dv1, k_field);
-              const double rho0 = alpha_d * h0, rho1 = alpha_d * h1;
-              score_pairs(blk, fx, recip_fast(s0), rho0, w);
-              g_scaled = h0 * w.e;
-              dv_bits = dv0;
-              if (kMode == 1 && n_dq > 2) {
-                // wider code windows: n_dq / 2 codes at or below the center, n_dq / 2 above, clipped
-                const int d_lo = static_cast<int>(dv0 >> 20) - 960 - (n_dq / 2 - 1);
-                g_scaled = __longlong_as_double(0x7FF0000000000000ll);
-                for (int i = 0; i < n_dq / 2 * 2; ++i) {
-                  const float dv = e4m3_value(clip_code(d_lo + i));
-                  const double h = static_cast<double>(dv) * __hiloint2double(k_field + (1023 << 20), 0);
-                  const double g = h * fma(alpha_d * h, uint_to_double(w.b4), -uint_to_double(w.afix));
-                  if (g < g_scaled) { g_scaled = g; dv_bits = __float_as_uint(dv); }
-                }
-              } else if (kMode == 1) {
-                const double g1 = h1 * fma(rho1, uint_to_double(w.b4), -uint_to_double(w.afix));
-                if (g1 < g_scaled) { g_scaled = g1; dv_bits = dv1; }
-              } else if (n_dq == 2) {
-                Candidate x;
-                score_pairs(blk, fx, recip_fast(s1), rho1, x);
-                const double g1 = h1 * x.e;
-                if (g1 < g_scaled) { w = x; g_scaled = g1; dv_bits = dv1; }
-              }
-            }
-          }
+        unsigned int dv0 = __float_as_uint(center) & 0xFFF00000u, dv1 = dv0 + 0x00100000u;
+        if (n_dq == 1) {   // the nearest code alone
+          dv0 = __float_as_uint(e4m3_value(e4m3_encode(center)));
+          dv1 = dv0;
         }
-        unsigned int c0, c1, b4, A_bits;
-        int d;
-        float v;
-        if (direct) {
-          c0 = w.c0;
-          c1 = w.c1;
-          b4 = w.b4;
-          v = __uint_as_float(dv_bits);
-          d = (kMode == 1 && n_dq > 2) ? e4m3_encode(v) : static_cast<int>(dv_bits >> 20) - 960;
-          // A = afix / (2 S); error minus sum W^2 = alpha (h e) 4 / S^2
-          A_bits = __float_as_uint(__fmul_rn(__uint2float_rn(w.afix), __uint_as_float(s_exp - (11u << 23))));
-          const double scale = __hiloint2double(__double2hiint(alpha_d) + static_cast<int>(s_exp >> 2) - (272 << 20),
-                                                __double2loint(alpha_d));
-          acc[1] = fma(g_scaled, scale, acc[1]);
+        const float v0f = __uint_as_float(dv0), v1f = __uint_as_float(dv1);
+        Candidate w;
+        unsigned int dv_bits = dv0, s_exp;
+        double g_scaled;
+        if (kMode == 4 || kMode == 5) {
+          float y;
+          asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(center));
+          const float per_center = y * k_scale;
+          // floor by a round-down addition: the index sits in the low bits of the sum
+          const float t0 = __fadd_rd(__fmaf_rn(v0f, per_center, k_off), 12582912.0f);
+          const float t1 = __fadd_rd(__fmaf_rn(v1f, per_center, k_off), 12582912.0f);
+          int k0 = static_cast<int>(__float_as_uint(t0) & (SOAR_MAX_BETA - 1)), k1 = static_cast<int>(__float_as_uint(t1) & (SOAR_MAX_BETA - 1));
+          if (kMode == 5) {
+            k0 = max(0, min(n_beta - 2, __float_as_int(t0) - 0x4B400000));
+            k1 = max(0, min(n_beta - 2, __float_as_int(t1) - 0x4B400000));
+          }
+          const uint2 q0 = lds64(pairs + 8u * static_cast<unsigned int>(k0));
+          const uint2 q1 = lds64(pairs + 8u * static_cast<unsigned int>(k1));
+          const pair_t cc = pair_of(center, center), aa = pair_of(alpha, alpha);
+          const pair_t m0 = pair_mul(cc, pair_of(__uint_as_float(q0.x), __uint_as_float(q0.y)));
+          const pair_t m1 = pair_mul(cc, pair_of(__uint_as_float(q1.x), __uint_as_float(q1.y)));
+          float a0, b0f, a1, b1;
+          halves(m0, a0, b0f);
+          halves(m1, a1, b1);
+          // The pair of multipliers must enclose the code's value with a margin that covers the three roundings
+          // from here to the scaled value (2^-24 each; see winning_range): 6 * 2^-24 does.  A block that misses it,
+          // one in several thousand, takes the exact walk.
+          constexpr float kUnder = 1.0f - 0x1.8p-22f, kOver = 1.0f + 0x1.8p-22f;
+          const bool below0 = a0 <= v0f * kUnder, above0 = b0f >= v0f * kOver;
+          const bool below1 = a1 <= v1f * kUnder, above1 = b1 >= v1f * kOver;
+          // Mode 5, where the grid ends before the band does: one multiplier is all that can win, the first one when
+          // even its divisor lies beyond the band, the last one when even its divisor lies before it.  The pair then
+          // holds that multiplier twice.
+          bool low0 = false, low1 = false, high0 = false, high1 = false;
+          if (kMode == 5) {
+            low0 = k0 == 0 && a0 >= v0f * kOver;
+            high0 = k0 == n_beta - 2 && b0f <= v0f * kUnder;
+            low1 = k1 == 0 && a1 >= v1f * kOver;
+            high1 = k1 == n_beta - 2 && b1 <= v1f * kUnder;
+          }
+          float s00, s01, s10, s11;
+          halves(pair_mul(aa, m0), s00, s01);
+          halves(pair_mul(aa, m1), s10, s11);
+          if (kMode == 5) {
+            if (high0) s00 = s01;
+            if (low0) s01 = s00;
+            if (high1) s10 = s11;
+            if (low1) s11 = s10;
+          }
+          s_exp = __float_as_uint(s00) & 0x7F800000u;
+          // the largest magnitude of the block below 32 times the smallest scale, from the exponents
+          direct = direct && ((below0 && above0) || low0 || high0) && ((below1 && above1) || low1 || high1) &&
+                   st.y < s_exp + (5u << 23);
+          FixedPairs fx;
+          make_fixed_pairs(blk, fixed_scale(s00), fx);
+          // h = dv S / 4; the exponent of S / 4 is 135 less s's biased one
+          const int k_field = static_cast<int>(135u << 20) - static_cast<int>(s_exp >> 3);
+          const double h0 = scaled_value(dv0, k_field), h1 = scaled_value(dv1, k_field);
+          const double rho0 = alpha_d * h0, rho1 = alpha_d * h1;
+          Candidate x, y2;
+          score_pairs(blk, fx, recip_fast(s00), rho0, w);
+          score_pairs(blk, fx, recip_fast(s01), rho0, x);
+          if (x.e < w.e) w = x;
+          score_pairs(blk, fx, recip_fast(s10), rho1, x);
+          score_pairs(blk, fx, recip_fast(s11), rho1, y2);
+          if (y2.e < x.e) x = y2;
+          // equal errors: the earlier multiplier, as in grid order (the second code's are never earlier)
+          const double g0 = h0 * w.e, g1 = h1 * x.e;
+          g_scaled = g0;
+          if (g1 < g0) { w = x; g_scaled = g1; dv_bits = dv1; }
+        } else if (kMode == 1 || kMode == 2) {
+          const float s0 = __fmul_rn(alpha, kMode == 1 ? center : v0f), s1 = __fmul_rn(alpha, v1f);
+          s_exp = __float_as_uint(s0) & 0x7F800000u;
+          direct = direct && st.y < s_exp + (5u << 23);
+          FixedPairs fx;
+          make_fixed_pairs(blk, fixed_scale(s0), fx);
+          const int k_field = static_cast<int>(135u << 20) - static_cast<int>(s_exp >> 3);
+          const double h0 = scaled_value(dv0, k_field), h1 = scaled_value(dv1, k_field);
+          const double rho0 = alpha_d * h0, rho1 = alpha_d * h1;
+          score_pairs(blk, fx, recip_fast(s0), rho0, w);
+          g_scaled = h0 * w.e;
+          if (kMode == 1 && n_dq > 2) {
+            // wider code windows: n_dq / 2 codes at or below the center, n_dq / 2 above, clipped
+            const int d_lo = static_cast<int>(dv0 >> 20) - 960 - (n_dq / 2 - 1);
+            g_scaled = __longlong_as_double(0x7FF0000000000000ll);
+            for (int i = 0; i < n_dq / 2 * 2; ++i) {
+              const float dv = e4m3_value(clip_code(d_lo + i));
+              const double h = static_cast<double>(dv) * __hiloint2double(k_field + (1023 << 20), 0);
+              const double g = h * fma(alpha_d * h, uint_to_double(w.b4), -uint_to_double(w.afix));
+              if (g < g_scaled) { g_scaled = g; dv_bits = __float_as_uint(dv); }
+            }
+          } else if (kMode == 1) {
+            const double g1 = h1 * fma(rho1, uint_to_double(w.b4), -uint_to_double(w.afix));
+            if (g1 < g_scaled) { g_scaled = g1; dv_bits = dv1; }
+          } else if (n_dq == 2) {
+            Candidate x;
+            score_pairs(blk, fx, recip_fast(s1), rho1, x);
+            const double g1 = h1 * x.e;
+            if (g1 < g_scaled) { w = x; g_scaled = g1; dv_bits = dv1; }
+          }
         } else {
+          s_exp = 0u;
+          g_scaled = 0.0;
+          w.c0 = w.c1 = w.afix = w.b4 = 0u;
+          direct = false;
+        }
+        // A = afix / (2 S); error minus sum W^2 = alpha (h e) 4 / S^2
+        float v = __uint_as_float(dv_bits), A = __fmul_rn(__uint2float_rn(w.afix), __uint_as_float(s_exp - (11u << 23)));
+        int d = (kMode == 1 && n_dq > 2) ? e4m3_encode(v) : static_cast<int>(dv_bits >> 20) - 960;
+        double g_scale = __hiloint2double(__double2hiint(alpha_d) + static_cast<int>(s_exp >> 2) - (272 << 20),
+                                          __double2loint(alpha_d));
+        if (active && !direct) {
           const float B0 = 0.25f * b4_prev;   // all codes zero keeps the stored scale
           center = (B0 > 0.0f && !keep_scale) ? __fdiv_rn(__uint_as_float(st.x), __fmul_rn(alpha, B0)) : stored;
           const Found f = kMode == 0 ? search_every(v0, v1, alpha, center, sh.beta, n_beta, n_dq,
                                                     (flags & SOAR_FLAG_COUPLED_SCALE) != 0, &wide)
                                      : search_general<kMode>(v0, v1, alpha, center, sh.beta, n_beta, n_dq, k_scale,
                                                              k_off, &wide);
-          c0 = f.c0;
-          c1 = f.c1;
-          b4 = f.b4;
+          w.c0 = f.c0;
+          w.c1 = f.c1;
+          w.b4 = f.b4;
           d = f.d;
           v = e4m3_value(d);
-          A_bits = __float_as_uint(f.A);
-          acc[1] += f.g;
+          A = f.A;
+          g_scaled = f.g;
+          g_scale = 1.0;
         }
-        const size_t b = static_cast<size_t>(b0) + lane;
-        if (emit) {
-          reinterpret_cast<uint2*>(p.packed)[b] = make_uint2(c0, c1);
-          p.scales[b] = static_cast<uint8_t>(d);
+        if (active) {
+          if (emit) {
+            reinterpret_cast<uint2*>(p.packed)[b] = make_uint2(w.c0, w.c1);
+            p.scales[b] = static_cast<uint8_t>(d);
+          }
+          if (keep) p.state[b] = make_uint2(__float_as_uint(A), pack_state(st.y & 0x7F800000u, d, w.b4));
+          // v^2 4B is exact in binary32: 8 + 12 significant bits
+          acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(v, v), __uint2float_rn(w.b4)));
+          acc[1] = fma(g_scaled, g_scale, acc[1]);
         }
-        if (keep) p.state[b] = make_uint2(A_bits, pack_state(st.y & 0x7F800000u, d, b4));
-        // v^2 4B is exact in binary32: 8 + 12 significant bits
-        acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(v, v), __uint2float_rn(b4)));
       });
 }
 
