@@ -2,12 +2,14 @@
 // tensor-wide sums of one pass combined before the next begins.  Included by soar.cu.
 //
 // Shape of the kernel.  Work is dealt in warp tiles of 32 blocks (1 KB of bf16, one 16-element block per lane):
-// warp w of the grid takes tiles w, w + warps, ... of the concatenated tiles of the tensors a pass works on.  A
-// warp feeds itself: its lanes start the 16-byte asynchronous copies of the tile kStages - 1 turns ahead and of its
-// block states into the warp's own slots of shared memory, so the tile loop has no block-wide barrier, no
-// producer to poll and no wait that could run out; one warp barrier per tile orders the slot's reuse.
-// Two CTAs of 256 threads per SM leave 128 registers a thread, which holds a block, the four candidates of the
-// search and their sums without spills.
+// warp w of the grid takes tiles w, w + warps, ... of the concatenated tiles of the tensors a pass works on.  A warp
+// feeds itself; there is no producer to poll, no block-wide barrier in the tile loop and no wait that could run out.
+//   Light passes (the maximum, the start, one candidate per block) are bound by HBM: the lanes start 16-byte
+//   asynchronous copies of the tile kStages - 1 turns ahead into the warp's own slots of shared memory.
+//   The search is bound by instruction issue: a lane loads its next block, 32 bytes with one 256-bit load, into
+//   registers one tile ahead, which costs 20 instructions a block less.
+// Two CTAs of 256 threads per SM leave 128 registers a thread, which holds a block, the next one, the four candidates
+// of the search and their sums without spills.
 //
 // Bytes 16 apart in a slot are exchanged between its two 128-byte halves (tile_chunk) so that the 32-byte reads
 // of neighbouring lanes meet no bank conflict.
@@ -19,7 +21,6 @@ constexpr int kQWarps = kQThreads / 32;
 constexpr int kQStages = 4;                        // slots of a warp's ring
 constexpr unsigned int kQTileBytes = 1024;         // 32 blocks of 16 bf16
 constexpr unsigned int kQStateBytes = 256;         // 32 block states of 8 bytes
-constexpr unsigned int kQSlotBytes = kQTileBytes + kQStateBytes;
 
 // Stages of a call, in order: amax, init, the iterations, the report.
 constexpr int kQStageAmax = 0, kQStageInit = 1, kQStageIterate = 2;
@@ -53,6 +54,26 @@ __device__ __forceinline__ uint4 lds128(unsigned int a) {
   asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
   return v;
 }
+// A block's 32 bytes, 32-byte aligned, read once per pass (not kept in L1).
+__device__ __forceinline__ void load_block32(const void* src, uint4& v0, uint4& v1) {
+  asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(v0.x), "=r"(v0.y), "=r"(v0.z), "=r"(v0.w), "=r"(v1.x), "=r"(v1.y), "=r"(v1.z), "=r"(v1.w)
+               : "l"(src));
+}
+// A block state: written by other SMs in the pass before, so from L2.
+__device__ __forceinline__ uint2 load_state(const void* src) {
+  uint2 v;
+  asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(src));
+  return v;
+}
+// Block b of a matrix wherever it lies: rows may be apart, 16-byte alignment is all that is given.
+__device__ __forceinline__ void load_block(const Params& p, unsigned int b, uint4& v0, uint4& v1) {
+  const unsigned int row = __umulhi(2u * b, p.nbc_magic) >> p.nbc_shift;
+  const uint4* src = reinterpret_cast<const uint4*>(p.W + static_cast<long long>(row) * p.ld +
+                                                    static_cast<long long>(b - row * p.nbc) * 16);
+  v0 = __ldg(src);
+  v1 = __ldg(src + 1);
+}
 __device__ __forceinline__ uint2 lds64(unsigned int a) {
   uint2 v;
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
@@ -74,6 +95,21 @@ __device__ __forceinline__ pair_t pair_mul(pair_t a, pair_t b) {
   pair_t d;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
+}
+
+__device__ __forceinline__ pair_t pair_fma(pair_t a, pair_t b, pair_t c) {
+  pair_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+// recip_fast of two divisors, given negated.
+__device__ __forceinline__ void pair_recip(pair_t neg, float& r_lo, float& r_hi) {
+  float lo, hi, y_lo, y_hi;
+  halves(neg, lo, hi);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y_lo) : "f"(-lo));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y_hi) : "f"(-hi));
+  const pair_t y = pair_of(y_lo, y_hi);
+  halves(pair_fma(y, pair_fma(neg, y, pair_of(1.0f, 1.0f)), y), r_lo, r_hi);
 }
 
 // fl(n / d) from y = fl(1 / d) (Markstein, "Computation of elementary functions on the IBM RISC System/6000
@@ -177,8 +213,10 @@ struct Found {
 // size, sums in binary64 where the integer ones do not hold, the coupled arm.  Out of line: the common blocks
 // never come here, and nothing of it weighs on their registers.  kMode as iterate_pass.
 template <int kMode>
-__device__ __noinline__ Found search_general(uint4 v0, uint4 v1, float alpha, float center, const float2* s_beta,
+__device__ __noinline__ Found search_general(const Params& p, unsigned int b, float alpha, float center, const float2* s_beta,
                                              int n_beta, int n_dq, float k_scale, float k_off, unsigned int* wide_out) {
+  uint4 v0, v1;
+  load_block(p, b, v0, v1);
   Block blk;
   unpack_block(v0, v1, blk);
   Fixed fx;
@@ -256,8 +294,10 @@ __device__ __noinline__ Found search_general(uint4 v0, uint4 v1, float alpha, fl
 
 // Every multiplier in turn, for the coupled arm with a grid and for grids whose multipliers all coincide: first
 // minimum in (beta, code) order.
-__device__ __noinline__ Found search_every(uint4 v0, uint4 v1, float alpha, float center, const float2* s_beta, int n_beta,
+__device__ __noinline__ Found search_every(const Params& p, unsigned int b, float alpha, float center, const float2* s_beta, int n_beta,
                                            int n_dq, bool coupled, unsigned int* wide_out) {
+  uint4 v0, v1;
+  load_block(p, b, v0, v1);
   Block blk;
   unpack_block(v0, v1, blk);
   Fixed fx;
@@ -305,7 +345,9 @@ __device__ __noinline__ Found search_every(uint4 v0, uint4 v1, float alpha, floa
 }
 
 // The max-based start of one block (Eq. 1-2) by the general rules, for an alpha outside tame_alpha.
-__device__ __noinline__ Found start_general(uint4 v0, uint4 v1, float alpha, unsigned int* wide_out) {
+__device__ __noinline__ Found start_general(const Params& p, unsigned int b, float alpha, unsigned int* wide_out) {
+  uint4 v0, v1;
+  load_block(p, b, v0, v1);
   Block blk;
   unpack_block(v0, v1, blk);
   Fixed fx;
@@ -328,9 +370,25 @@ __device__ __noinline__ Found start_general(uint4 v0, uint4 v1, float alpha, uns
 
 // ------------------------------------------------------------------ one CTA's shared state
 
+// Where a tensor's outputs go, kept in shared memory: two 16-byte reads per tile.  Left to itself the compiler re-reads
+// the parameter block at a computed address for every pointer and tile (18 instructions of 374), and held in registers
+// they would spill.
+struct __align__(16) View {
+  uint8_t* packed;
+  uint8_t* scales;
+  uint2* state;
+  unsigned long long pad;
+};
+__device__ __forceinline__ void load_view(unsigned int at, uint8_t*& packed, uint8_t*& scales, uint2*& state) {
+  asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(packed), "=l"(scales) : "r"(at));
+  asm volatile("ld.shared.u64 %0, [%1];" : "=l"(state) : "r"(at + 16));
+  __builtin_assume(__isGlobal(packed) && __isGlobal(scales) && __isGlobal(state));
+}
+
 template <bool kDet>
 struct __align__(128) QShared {
-  unsigned char ring[kQWarps][kQStages * kQSlotBytes];
+  unsigned char ring[kQWarps][kQStages * (kQTileBytes + kQStateBytes)];   // also write_report's scratch
+  View view[kMaxBatch];
   float2 beta[SOAR_MAX_BETA];              // {multiplier k, multiplier k + 1}
   // sums of the stage in hand, per tensor: {sum W^2, -} in the amax pass, {4 den, gsum} later
   double acc[kMaxBatch][2];
@@ -419,10 +477,11 @@ __device__ __forceinline__ void next_run(const S& sh, int n, bool reverse, unsig
 }
 
 // One warp's walk over its share of the pass's tiles.  `enter(ti)` and `leave(ti)` bracket the tiles of one tensor;
-// `body(b, v0, v1, st)` gets the lane's block number (past the tensor's end in the last tile: the body looks), its
-// 32 bytes and, with kState, its block state.  The warp number is broadcast so that the compiler sees the
-// bookkeeping as uniform; per tile it is a handful of instructions beside the copies.
-template <bool kState, typename S, typename Enter, typename Leave, typename Body>
+// `body(b, v0, v1, st, next)` gets the lane's block number (past the tensor's end in the last tile: the body looks), its
+// 32 bytes and, with kState, its block state, and calls next() once it is done with these registers.  kRing: tiles
+// come through the warp's slots in shared memory, three ahead; else through registers, one ahead.  The warp
+// number is broadcast so that the compiler sees the bookkeeping as uniform.
+template <bool kRing, bool kState, typename S, typename Enter, typename Leave, typename Body>
 __device__ __forceinline__ void walk_tiles(S& sh, const Batch& bt, bool reverse, Enter enter, Leave leave, Body body) {
   const unsigned int lane = threadIdx.x & 31u, warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
   const unsigned int warps = gridDim.x * kQWarps, me = blockIdx.x * kQWarps + warp;
@@ -432,24 +491,31 @@ __device__ __forceinline__ void walk_tiles(S& sh, const Batch& bt, bool reverse,
 
   Run f;          // the feeding side
   f.ti = -1;
+  f.left = 0;
   const unsigned char *f_w = nullptr, *f_state = nullptr;
+  unsigned int f_b = 0, f_step = 0;      // the lane's block (registers)
   long long f_w_step = 0, f_state_step = 0;
-  bool f_plain = true;   // contiguous, and every tile of the run whole
+  bool f_plain = true;   // contiguous, every tile of the run whole, and 32-byte aligned where that matters
   auto enter_feed = [&]() {
     next_run(sh, bt.n, reverse, me, warps, f);
     if (f.left == 0) return;
     const Params& p = bt.t[f.ti];
     // the ragged last tile is the last of a forward run, the first of a backward one
     const int top = reverse ? f.tile : f.tile + static_cast<int>(f.left - 1) * f.step;
-    f_plain = p.contiguous && static_cast<unsigned int>(top) * 32 + 32 <= p.nblk;
-    f_w = reinterpret_cast<const unsigned char*>(p.W) + (f_plain ? static_cast<size_t>(f.tile) * kQTileBytes + lane * 16 : 0);
-    f_w_step = static_cast<long long>(f.step) * kQTileBytes;
-    if (kState) {
-      f_state = reinterpret_cast<const unsigned char*>(p.state) + static_cast<size_t>(f.tile) * kQStateBytes + lane * 16;
+    f_w = reinterpret_cast<const unsigned char*>(p.W);
+    f_state = reinterpret_cast<const unsigned char*>(p.state);
+    f_plain = p.contiguous && static_cast<unsigned int>(top) * 32 + 32 <= p.nblk &&
+              (kRing || (reinterpret_cast<uintptr_t>(f_w) & 31u) == 0);
+    f_b = static_cast<unsigned int>(f.tile) * 32 + lane;
+    f_step = static_cast<unsigned int>(f.step) * 32;
+    if (kRing) {
+      if (f_plain) f_w += static_cast<size_t>(f.tile) * kQTileBytes + lane * 16;
+      f_w_step = static_cast<long long>(f.step) * kQTileBytes;
+      f_state += static_cast<size_t>(f.tile) * kQStateBytes + lane * 16;
       f_state_step = static_cast<long long>(f.step) * kQStateBytes;
     }
   };
-  auto feed = [&](unsigned int k) {
+  auto feed_ring = [&](unsigned int k) {
     if (f.left == 0) return;
     const unsigned int dst = put + k * kQTileBytes;
     if (f_plain) {
@@ -458,7 +524,7 @@ __device__ __forceinline__ void walk_tiles(S& sh, const Batch& bt, bool reverse,
       f_w += f_w_step;
     } else {
       const Params& p = bt.t[f.ti];
-      const unsigned int b0 = static_cast<unsigned int>(f.tile) * 32;
+      const unsigned int b0 = f_b - lane;
 #pragma unroll
       for (unsigned int h = 0; h < 2; ++h) {
         const unsigned int b = b0 + h * 16 + (lane >> 1);
@@ -466,7 +532,7 @@ __device__ __forceinline__ void walk_tiles(S& sh, const Batch& bt, bool reverse,
         const unsigned char* src = f_w + (static_cast<long long>(row) * p.ld + (b - row * p.nbc) * 16) * 2 + (lane & 1u) * 16;
         if (b < p.nblk) copy16(dst + 512 * h, src);
       }
-      f.tile += f.step;
+      f_b += f_step;
     }
     if (kState) {
       // the state array is padded to 256 bytes, so whole tiles stay inside it
@@ -475,31 +541,56 @@ __device__ __forceinline__ void walk_tiles(S& sh, const Batch& bt, bool reverse,
     }
     if (--f.left == 0) enter_feed();
   };
+  auto feed_registers = [&](uint4& v0, uint4& v1, uint2& st) {
+    if (f.left == 0) return;
+    if (f_plain) {
+      load_block32(f_w + static_cast<size_t>(f_b) * 32, v0, v1);
+      if (kState) st = load_state(f_state + static_cast<size_t>(f_b) * 8);
+    } else {
+      const Params& p = bt.t[f.ti];
+      if (f_b < p.nblk) {
+        load_block(p, f_b, v0, v1);
+        if (kState) st = load_state(f_state + static_cast<size_t>(f_b) * 8);
+      }
+    }
+    f_b += f_step;
+    if (--f.left == 0) enter_feed();
+  };
 
+  uint4 v0 = make_uint4(0u, 0u, 0u, 0u), v1 = v0;
+  uint2 st = make_uint2(0u, 0u);
+  unsigned int slot = 0;
   enter_feed();
+  if (kRing) {
 #pragma unroll
-  for (unsigned int k = 0; k < kQStages - 1; ++k) {
-    feed(k);
-    copies_commit();
+    for (unsigned int k = 0; k < kQStages - 1; ++k) {
+      feed_ring(k);
+      copies_commit();
+    }
+  } else {
+    feed_registers(v0, v1, st);
   }
   Run r;
   r.ti = -1;
-  unsigned int k = 0;
   for (next_run(sh, bt.n, reverse, me, warps, r); r.left != 0; next_run(sh, bt.n, reverse, me, warps, r)) {
     enter(r.ti);
     unsigned int b = static_cast<unsigned int>(r.tile) * 32 + lane;
     const unsigned int b_step = static_cast<unsigned int>(r.step) * 32;
     for (unsigned int left = r.left; left != 0; --left) {
-      copies_wait<kQStages - 2>();
-      __syncwarp();   // every lane's copies have landed, and every lane has read the slot that is filled next
-      feed((k + kQStages - 1) % kQStages);
-      copies_commit();
-      const unsigned int at = get + k * kQTileBytes;
-      const uint4 v0 = lds128(at), v1 = lds128(at ^ 16u);
-      uint2 st = make_uint2(0u, 0u);
-      if (kState) st = lds64(get_state + k * kQStateBytes);
-      k = (k + 1) % kQStages;
-      body(b, v0, v1, st);
+      if (kRing) {
+        copies_wait<kQStages - 2>();
+        __syncwarp();   // every lane's copies have landed, and every lane has read the slot that is filled next
+        feed_ring((slot + kQStages - 1) % kQStages);
+        copies_commit();
+        const unsigned int at = get + slot * kQTileBytes;
+        v0 = lds128(at);
+        v1 = lds128(at ^ 16u);
+        if (kState) st = lds64(get_state + slot * kQStateBytes);
+        slot = (slot + 1) % kQStages;
+        body(b, v0, v1, st, []() {});
+      } else {
+        body(b, v0, v1, st, [&]() { feed_registers(v0, v1, st); });
+      }
       b += b_step;
     }
     leave(r.ti);
@@ -592,7 +683,7 @@ __device__ __forceinline__ void amax_pass(QShared<kDet>& sh, const Batch& bt) {
   unsigned int mx = 0;
   double sq[2] = {0.0, 0.0};
   unsigned int nblk = 0;
-  walk_tiles<false>(
+  walk_tiles<true, false>(
       sh, bt, false, [&](int ti) { nblk = bt.t[ti].nblk; },
       [&](int ti) {
         mx = max(mx & 0xFFFFu, mx >> 16);
@@ -603,8 +694,8 @@ __device__ __forceinline__ void amax_pass(QShared<kDet>& sh, const Batch& bt) {
         mx = 0;
         sq[0] = sq[1] = 0.0;
       },
-      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&) {
-        if (b >= nblk) return;
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next) {
+        const bool here = b < nblk;
         const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
         // largest magnitude of the block with packed bf16 max (a NaN input comes out of the maximum
         // as NaN, whose bits are above the infinity pattern)
@@ -615,22 +706,28 @@ __device__ __forceinline__ void amax_pass(QShared<kDet>& sh, const Batch& bt) {
           asm("abs.bf16x2 %0, %1;" : "=r"(m) : "r"(u[i]));
           asm("max.NaN.bf16x2 %0, %0, %1;" : "+r"(bmx) : "r"(m));
         }
-        mx = __vmaxu2(mx, bmx & 0x7FFF7FFFu);
-        sumsq_block(u, sq[0], sq[1]);
+        if (here) {
+          mx = __vmaxu2(mx, bmx & 0x7FFF7FFFu);
+          sumsq_block(u, sq[0], sq[1]);
+        }
+        next();
       });
 }
 
 // Algorithm 1 "Initialization" (Eq. 1): dd0 = E4M3(bmax/(6 alpha0)), dq0 = dd0; first codes (Eq. 2); stage-0 sums for
-// Eq. 5 and the starting error.  Codes and scales are written here only when no iteration follows (final).
+// Eq. 5 and the starting error.  Codes and scales are written here only when no iteration follows, the block states only when one does.
 template <bool kDet>
-__device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt, bool final) {
+__device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt) {
   float alpha = 1.0f, six_alpha = 6.0f, six_inv = 0.0f;
   double alpha_d = 1.0;
   bool tame = false;
   double acc[2] = {0.0, 0.0};   // 4 den, gsum
   unsigned int zeros = 0, wide = 0;
-  Tensor p = {};
-  walk_tiles<false>(
+  int tensor = 0;
+  unsigned int nblk = 0, view = 0;
+  unsigned int keep = bt.t[0].max_iters > 0;
+  asm volatile("" : "+r"(keep));
+  walk_tiles<true, false>(
       sh, bt, true,
       [&](int ti) {
         alpha = sh.alpha[ti];
@@ -638,16 +735,22 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt, bo
         tame = tame_alpha(alpha);
         six_inv = __frcp_rn(six_alpha);
         alpha_d = static_cast<double>(alpha);
-        p = tensor_view(bt.t[ti]);
+        nblk = bt.t[ti].nblk;
+        view = smem_u32(&sh.view[ti]);
+        tensor = ti;
       },
       [&](int ti) {
         hand_over(sh, ti, acc);
         hand_over_counters(sh, ti, zeros, wide);
       },
-      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&) {
-        if (b >= p.nblk) return;
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next) {
         PairBlock blk;
         unpack_pairs(v0, v1, blk);
+        next();
+        if (b >= nblk) return;
+        uint8_t *packed, *scales;
+        uint2* state;
+        load_view(view, packed, scales, state);
         float bmax = 0.0f;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
@@ -659,9 +762,9 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt, bo
           // all-zero block: codes carry the sign bits only, scale byte 0, left out of all sums
           unsigned int c0, c1;
           round_pairs(blk, 1.0f, c0, c1);
-          reinterpret_cast<uint2*>(p.packed)[b] = make_uint2(c0, c1);
-          p.scales[b] = 0;
-          if (p.state != nullptr) p.state[b] = make_uint2(0u, 0u);
+          reinterpret_cast<uint2*>(packed)[b] = make_uint2(c0, c1);
+          scales[b] = 0;
+          if (keep) state[b] = make_uint2(0u, 0u);
           ++zeros;
           return;
         }
@@ -687,15 +790,14 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt, bo
           f.g = h * e * __hiloint2double(__double2hiint(alpha_d) + static_cast<int>(s_exp >> 2) - (272 << 20),
                                          __double2loint(alpha_d));
         } else {
-          f = start_general(v0, v1, alpha, &wide);
+          f = start_general(bt.t[tensor], b, alpha, &wide);
           v = e4m3_value(f.d);
         }
-        if (final) {
-          reinterpret_cast<uint2*>(p.packed)[b] = make_uint2(f.c0, f.c1);
-          p.scales[b] = static_cast<uint8_t>(f.d);
-        }
-        if (p.state != nullptr)
-          p.state[b] = make_uint2(__float_as_uint(f.A), pack_state(__float_as_uint(bmax) & 0x7F800000u, f.d, f.b4));
+        if (!keep) {
+          reinterpret_cast<uint2*>(packed)[b] = make_uint2(f.c0, f.c1);
+          scales[b] = static_cast<uint8_t>(f.d);
+        } else
+          state[b] = make_uint2(__float_as_uint(f.A), pack_state(__float_as_uint(bmax) & 0x7F800000u, f.d, f.b4));
         // v^2 4B is exact in binary32: 8 + 12 significant bits
         acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(v, v), __uint2float_rn(f.b4)));
         acc[1] += f.g;
@@ -709,12 +811,15 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt, bo
 //   kMode 0  every multiplier in turn (the coupled arm with a grid)
 //   kMode 1  one quantization scale per block (beta = 1): the codes are made once, only the E4M3 code is chosen
 //   kMode 2  beta = 1 with the coupled scale: each E4M3 code rounds the block with its own value
-//   kMode 4  the grid of App. B.3, only the multipliers that can win
-//   kMode 5  the same for grids so short that a block's bracket often reaches past their first or last multiplier
+//   kMode 3  the grid of App. B.3 around the stored scale (Sec. 3.3 alone), only the multipliers that can win
+//   kMode 4  the grid of App. B.3 around the Eq. 6 solution with two E4M3 codes, only the multipliers that can win
+//   kMode 5  the same for any number of codes, and for grids so short that a block's bracket often reaches past their
+//            first or last multiplier
 template <int kMode, bool kDet>
-__device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt, bool reverse, bool emit, bool keep) {
+__device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt, bool reverse, unsigned int emit, unsigned int keep) {
+  asm volatile("" : "+r"(emit), "+r"(keep));   // in registers, not worked out again per tile
   const int n_dq = bt.t[0].n_dq, n_beta = bt.t[0].n_beta, flags = bt.t[0].flags;
-  const bool keep_scale = (flags & SOAR_FLAG_KEEP_BLOCK_SCALE) != 0;
+  const bool keep_scale = kMode == 3 || (kMode != 4 && (flags & SOAR_FLAG_KEEP_BLOCK_SCALE) != 0);
   // multiplier index of a scale ratio: k = (ratio - 1) * 100 / step + n_beta / 2
   const float k_scale = 100.0f / static_cast<float>(max(bt.t[0].beta_step_pct, 1));
   const float k_off = static_cast<float>(n_beta / 2) - k_scale;
@@ -723,35 +828,40 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
   double alpha_d = 1.0;
   double acc[2] = {0.0, 0.0};           // 4 den, gsum
   unsigned int wide = 0, zeros = 0;
-  Tensor p = {};
-  walk_tiles<true>(
+  int tensor = 0;
+  unsigned int nblk = 0, view = 0;
+  walk_tiles<kMode == 1, true>(
       sh, bt, reverse,
       [&](int ti) {
         alpha = sh.alpha[ti];
         alpha_q = (kMode != 0 && (n_dq <= 2 || kMode == 1) && tame_alpha(alpha)) ? 0.25f * alpha : __uint_as_float(0x7FC00000u);
         alpha_d = static_cast<double>(alpha);
-        p = tensor_view(bt.t[ti]);
+        nblk = bt.t[ti].nblk;
+        view = smem_u32(&sh.view[ti]);
+        tensor = ti;
       },
       [&](int ti) {
         hand_over(sh, ti, acc);
         hand_over_counters(sh, ti, zeros, wide);
       },
-      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2& st) {
-        const bool active = b < p.nblk && st.y != 0u;   // past the end, or an all-zero block: nothing to optimise
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2& state, auto next) {
+        PairBlock blk;
+        unpack_pairs(v0, v1, blk);
+        const uint2 st = state;
+        next();
+        const bool active = b < nblk && st.y != 0u;   // past the end, or an all-zero block: nothing to optimise
         // Eq. 6, A / (alpha B): with 4B and alpha / 4 the powers of two cancel exactly
         const float b4_prev = __fsub_rn(__uint_as_float((st.y & 0xFFFu) | 0x4B000000u), 8388608.0f);
         const float stored = e4m3_value(static_cast<int>((st.y >> 12) & 0x7Fu));
         const float D = __fmul_rn(alpha_q, b4_prev);
         float center = quotient(__uint_as_float(st.x), D, recip_fast(D));
         if (keep_scale) center = alpha_q > 0.0f ? stored : alpha_q;
-        PairBlock blk;
-        unpack_pairs(v0, v1, blk);
         // Regular block: the center inside the normal E4M3 range (which also rejects B = 0 and a NaN alpha_q), so the
         // codes below and above it are its leading bits and the next.  The candidates are made and scored for every
         // lane; what an irregular block gets from that is overwritten by the general search below.
         bool direct = __float_as_uint(center) - 0x3C800000u < 0x43E00000u - 0x3C800000u;
         unsigned int dv0 = __float_as_uint(center) & 0xFFF00000u, dv1 = dv0 + 0x00100000u;
-        if (n_dq == 1) {   // the nearest code alone
+        if (kMode != 3 && kMode != 4 && n_dq == 1) {   // the nearest code alone
           dv0 = __float_as_uint(e4m3_value(e4m3_encode(center)));
           dv1 = dv0;
         }
@@ -759,13 +869,16 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
         Candidate w;
         unsigned int dv_bits = dv0, s_exp;
         double g_scaled;
-        if (kMode == 4 || kMode == 5) {
+        if (kMode >= 3) {
           float y;
           asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(center));
           const float per_center = y * k_scale;
-          // floor by a round-down addition: the index sits in the low bits of the sum
-          const float t0 = __fadd_rd(__fmaf_rn(v0f, per_center, k_off), 12582912.0f);
-          const float t1 = __fadd_rd(__fmaf_rn(v1f, per_center, k_off), 12582912.0f);
+          // floor by a round-down addition: the index sits in the low bits of the sum.  Mode 3, where the center is an
+          // E4M3 value and a multiplier often falls on a code exactly, takes the multiplier before the nearest one, and
+          // three candidates.
+          const float k_low = kMode == 3 ? k_off - 0.5f : k_off;
+          const float t0 = __fadd_rd(__fmaf_rn(v0f, per_center, k_low), 12582912.0f);
+          const float t1 = __fadd_rd(__fmaf_rn(v1f, per_center, k_low), 12582912.0f);
           int k0 = static_cast<int>(__float_as_uint(t0) & (SOAR_MAX_BETA - 1)), k1 = static_cast<int>(__float_as_uint(t1) & (SOAR_MAX_BETA - 1));
           if (kMode == 5) {
             k0 = max(0, min(n_beta - 2, __float_as_int(t0) - 0x4B400000));
@@ -773,12 +886,18 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
           }
           const uint2 q0 = lds64(pairs + 8u * static_cast<unsigned int>(k0));
           const uint2 q1 = lds64(pairs + 8u * static_cast<unsigned int>(k1));
-          const pair_t cc = pair_of(center, center), aa = pair_of(alpha, alpha);
+          const pair_t cc = pair_of(center, center), aa = pair_of(-alpha, -alpha);
           const pair_t m0 = pair_mul(cc, pair_of(__uint_as_float(q0.x), __uint_as_float(q0.y)));
           const pair_t m1 = pair_mul(cc, pair_of(__uint_as_float(q1.x), __uint_as_float(q1.y)));
           float a0, b0f, a1, b1;
           halves(m0, a0, b0f);
           halves(m1, a1, b1);
+          pair_t m2 = m0;
+          if (kMode == 3) {   // {second multiplier above code 0's pair, the same for code 1}
+            m2 = pair_mul(cc, pair_of(__uint_as_float(lds64(pairs + 8u * static_cast<unsigned int>(k0 + 1)).y),
+                                      __uint_as_float(lds64(pairs + 8u * static_cast<unsigned int>(k1 + 1)).y)));
+            halves(m2, b0f, b1);
+          }
           // The pair of multipliers must enclose the code's value with a margin that covers the three roundings
           // from here to the scaled value (2^-24 each; see winning_range): 6 * 2^-24 does.  A block that misses it,
           // one in several thousand, takes the exact walk.
@@ -795,32 +914,45 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
             low1 = k1 == 0 && a1 >= v1f * kOver;
             high1 = k1 == n_beta - 2 && b1 <= v1f * kUnder;
           }
-          float s00, s01, s10, s11;
-          halves(pair_mul(aa, m0), s00, s01);
-          halves(pair_mul(aa, m1), s10, s11);
+          // divisors, negated as pair_recip wants them
+          pair_t n0 = pair_mul(aa, m0), n1 = pair_mul(aa, m1);
           if (kMode == 5) {
-            if (high0) s00 = s01;
-            if (low0) s01 = s00;
-            if (high1) s10 = s11;
-            if (low1) s11 = s10;
+            float lo, hi;
+            halves(n0, lo, hi);
+            n0 = pair_of(high0 ? hi : lo, low0 ? lo : hi);
+            halves(n1, lo, hi);
+            n1 = pair_of(high1 ? hi : lo, low1 ? lo : hi);
           }
+          float s00, s01;
+          halves(n0, s00, s01);
           s_exp = __float_as_uint(s00) & 0x7F800000u;
           // the largest magnitude of the block below 32 times the smallest scale, from the exponents
           direct = direct && ((below0 && above0) || low0 || high0) && ((below1 && above1) || low1 || high1) &&
                    st.y < s_exp + (5u << 23);
           FixedPairs fx;
-          make_fixed_pairs(blk, fixed_scale(s00), fx);
+          make_fixed_pairs(blk, __uint_as_float((264u << 23) - s_exp), fx);
           // h = dv S / 4; the exponent of S / 4 is 135 less s's biased one
           const int k_field = static_cast<int>(135u << 20) - static_cast<int>(s_exp >> 3);
           const double h0 = scaled_value(dv0, k_field), h1 = scaled_value(dv1, k_field);
           const double rho0 = alpha_d * h0, rho1 = alpha_d * h1;
           Candidate x, y2;
-          score_pairs(blk, fx, recip_fast(s00), rho0, w);
-          score_pairs(blk, fx, recip_fast(s01), rho0, x);
+          float r00, r01, r10, r11;
+          pair_recip(n0, r00, r01);
+          pair_recip(n1, r10, r11);
+          score_pairs(blk, fx, r00, rho0, w);
+          score_pairs(blk, fx, r01, rho0, x);
           if (x.e < w.e) w = x;
-          score_pairs(blk, fx, recip_fast(s10), rho1, x);
-          score_pairs(blk, fx, recip_fast(s11), rho1, y2);
+          score_pairs(blk, fx, r10, rho1, x);
+          score_pairs(blk, fx, r11, rho1, y2);
           if (y2.e < x.e) x = y2;
+          if (kMode == 3) {
+            float r02, r12;
+            pair_recip(pair_mul(aa, m2), r02, r12);
+            score_pairs(blk, fx, r02, rho0, y2);
+            if (y2.e < w.e) w = y2;
+            score_pairs(blk, fx, r12, rho1, y2);
+            if (y2.e < x.e) x = y2;
+          }
           // equal errors: the earlier multiplier, as in grid order (the second code's are never earlier)
           const double g0 = h0 * w.e, g1 = h1 * x.e;
           g_scaled = g0;
@@ -864,14 +996,14 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
         // A = afix / (2 S); error minus sum W^2 = alpha (h e) 4 / S^2
         float v = __uint_as_float(dv_bits), A = __fmul_rn(__uint2float_rn(w.afix), __uint_as_float(s_exp - (11u << 23)));
         int d = (kMode == 1 && n_dq > 2) ? e4m3_encode(v) : static_cast<int>(dv_bits >> 20) - 960;
-        double g_scale = __hiloint2double(__double2hiint(alpha_d) + static_cast<int>(s_exp >> 2) - (272 << 20),
+        const double g_scale = __hiloint2double(__double2hiint(alpha_d) + static_cast<int>(s_exp >> 2) - (272 << 20),
                                           __double2loint(alpha_d));
         if (active && !direct) {
           const float B0 = 0.25f * b4_prev;   // all codes zero keeps the stored scale
           center = (B0 > 0.0f && !keep_scale) ? __fdiv_rn(__uint_as_float(st.x), __fmul_rn(alpha, B0)) : stored;
-          const Found f = kMode == 0 ? search_every(v0, v1, alpha, center, sh.beta, n_beta, n_dq,
+          const Found f = kMode == 0 ? search_every(bt.t[tensor], b, alpha, center, sh.beta, n_beta, n_dq,
                                                     (flags & SOAR_FLAG_COUPLED_SCALE) != 0, &wide)
-                                     : search_general<kMode>(v0, v1, alpha, center, sh.beta, n_beta, n_dq, k_scale,
+                                     : search_general<kMode>(bt.t[tensor], b, alpha, center, sh.beta, n_beta, n_dq, k_scale,
                                                              k_off, &wide);
           w.c0 = f.c0;
           w.c1 = f.c1;
@@ -879,15 +1011,18 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
           d = f.d;
           v = e4m3_value(d);
           A = f.A;
-          g_scaled = f.g;
-          g_scale = 1.0;
+          g_scaled = 0.0;
+          acc[1] += f.g;
         }
+        uint8_t *packed, *scales;
+        uint2* states;
+        load_view(view, packed, scales, states);
         if (active) {
           if (emit) {
-            reinterpret_cast<uint2*>(p.packed)[b] = make_uint2(w.c0, w.c1);
-            p.scales[b] = static_cast<uint8_t>(d);
+            reinterpret_cast<uint2*>(packed)[b] = make_uint2(w.c0, w.c1);
+            scales[b] = static_cast<uint8_t>(d);
           }
-          if (keep) p.state[b] = make_uint2(__float_as_uint(A), pack_state(st.y & 0x7F800000u, d, w.b4));
+          if (keep) states[b] = make_uint2(__float_as_uint(A), pack_state(st.y & 0x7F800000u, d, w.b4));
           // v^2 4B is exact in binary32: 8 + 12 significant bits
           acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(v, v), __uint2float_rn(w.b4)));
           acc[1] = fma(g_scaled, g_scale, acc[1]);
@@ -1029,6 +1164,11 @@ quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Report
   __shared__ double s_latest[kDet ? kMaxBatch : 1][3];
   const int tid = threadIdx.x;
   const int T = bt.t[0].max_iters, report = kQStageIterate + T, flags = bt.t[0].flags;
+  if (tid < bt.n) {
+    sh.view[tid].packed = bt.t[tid].packed;
+    sh.view[tid].scales = bt.t[tid].scales;
+    sh.view[tid].state = bt.t[tid].state;
+  }
   if (tid < kMaxBatch) {
     sh.acc[tid][0] = sh.acc[tid][1] = 0.0;
     sh.amax[tid] = sh.zeros[tid] = sh.wide[tid] = 0u;
@@ -1040,7 +1180,7 @@ quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Report
     sh.failed = 0;
     sh.run = (1u << bt.n) - 1u;
   }
-  if (kMode == 0 || kMode >= 4) {
+  if (kMode == 0 || kMode >= 3) {
     const int n_beta = bt.t[0].n_beta, step = bt.t[0].beta_step_pct;
     for (int k = tid; k < n_beta; k += kQThreads) {
       const float lo = static_cast<float>((100.0 + static_cast<double>((k - n_beta / 2) * step)) / 100.0);
@@ -1112,7 +1252,7 @@ quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Report
       amax_pass(sh, bt);
       file_sums(sh, bt, -1);
     } else if (s == kQStageInit) {
-      init_pass(sh, bt, T == 0);
+      init_pass(sh, bt);
       file_sums(sh, bt, 0);
     } else {
       const int t = s - kQStageIterate;

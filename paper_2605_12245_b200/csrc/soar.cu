@@ -1702,6 +1702,7 @@ cudaError_t launch_stages(int mode, bool det, const Batch& bt, const Reports& rp
     case 0: return SOAR_STAGES(0);
     case 1: return SOAR_STAGES(1);
     case 2: return SOAR_STAGES(2);
+    case 3: return SOAR_STAGES(3);
     case 4: return SOAR_STAGES(4);
     default: return SOAR_STAGES(5);
   }
@@ -1718,11 +1719,12 @@ int search_mode(const soar_cfg* cfg) {
   // the coupled arm with a grid, and multipliers that all coincide, visit them all
   if (coupled || cfg->n_beta < kBracketMinBeta || cfg->beta_step_pct < 1) return 0;
   // the brackets of two E4M3 codes around the Eq. 6 solution lie at multipliers 0.89 .. 1.13 (E4M3 values are at most
-  // an eighth apart): a grid from 0.85 to 1.15 or wider holds them whole, a shorter one needs the path that knows
-  // the grid's ends
+  // an eighth apart): a grid from 0.85 to 1.15 or wider holds them whole, a shorter one (and another number of codes)
+  // needs the path that knows the grid's ends
   const int half = cfg->n_beta / 2;
   const bool spans = 100 - half * cfg->beta_step_pct <= 85 && 100 + (cfg->n_beta - 1 - half) * cfg->beta_step_pct >= 115;
-  return spans ? 4 : 5;
+  if (!spans || cfg->n_dq != 2) return 5;
+  return (cfg->flags & SOAR_FLAG_KEEP_BLOCK_SCALE) ? 3 : 4;
 }
 
 // Which part of a call is wanted: all of it (soar_quantize_batch), or one stage (soar_quantize_stage; iterations
