@@ -430,7 +430,7 @@ int soar_mx_quantize(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld,
  *     workspaces.
  */
 #define SOAR_STATIC_MAX_ELEMENTS (1ll << 24)                 /* e.g. one 4096 x 4096 matrix */
-#define SOAR_STATIC_SCRATCH_BYTES (2048 + 9 * (1 << 20))    /* 8 B of state + 1 scale byte per block */
+#define SOAR_STATIC_SCRATCH_BYTES (2048 + 9 * (1 << 20) + 7936)   /* 8 B of state + 1 scale byte per block */
 int soar_quantize_static(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld,
                          const soar_cfg* cfg, void* out_fp4_packed, void* out_e4m3_scales,
                          void* out_e4m3_scales_sw, float* out_global_fp32,

@@ -377,7 +377,7 @@ struct __align__(16) View {
   uint8_t* packed;
   uint8_t* scales;
   uint2* state;
-  unsigned long long pad;
+  uint8_t* tiled;   // tiled scales written by the start pass itself; null for none
 };
 __device__ __forceinline__ void load_view(unsigned int at, uint8_t*& packed, uint8_t*& scales, uint2*& state) {
   asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(packed), "=l"(scales) : "r"(at));
@@ -387,6 +387,7 @@ __device__ __forceinline__ void load_view(unsigned int at, uint8_t*& packed, uin
 
 template <bool kDet>
 struct __align__(128) QShared {
+  static constexpr bool kOrdered = kDet, kSolo = false, kResident = false;
   unsigned char ring[kQWarps][kQStages * (kQTileBytes + kQStateBytes)];   // also write_report's scratch
   View view[kMaxBatch];
   float2 beta[SOAR_MAX_BETA];              // {multiplier k, multiplier k + 1}
@@ -446,9 +447,10 @@ __device__ __forceinline__ void lay_out_pass(S& sh, const Batch& bt) {
   __syncthreads();
 }
 
-// One warp's run of tiles within one tensor: local tile numbers first, first + step, ... (`left` of them), where the
-// warp's positions in the pass's sequence fall into the tensor.  From the back of the sequence for `reverse`:
-// consecutive passes alternate so that a pass starts on what the previous one left in L2.
+// One warp's run of tiles within one tensor: local tile numbers tile, tile + step, ... (`left` of them), those whose
+// positions in the pass's sequence are the warp's own number modulo the number of warps.  For `reverse` the same
+// tiles from the last to the first: consecutive passes alternate so that a pass starts on what the previous one
+// left in L2.
 struct Run {
   int ti;
   unsigned int left;
@@ -463,29 +465,109 @@ __device__ __forceinline__ void next_run(const S& sh, int n, bool reverse, unsig
   if (r.ti < 0) at = -1;
   while (++at < n) {
     const int ti = reverse ? n - 1 - at : at;
-    const unsigned int count = sh.count[ti], start = reverse ? sh.total - sh.start[ti] - count : sh.start[ti];
-    const unsigned int past = start % warps;
-    const unsigned int first = warp >= past ? warp - past : warp + warps - past;
+    const unsigned int count = sh.count[ti];
+    unsigned int first = warp;
+    if constexpr (!S::kSolo) {
+      const unsigned int past = sh.start[ti] % warps;
+      first = warp >= past ? warp - past : warp + warps - past;
+    }
     if (first < count) {
       r.ti = ti;
       r.left = (count - 1 - first) / warps + 1;
-      r.tile = static_cast<int>(reverse ? count - 1 - first : first);
+      r.tile = static_cast<int>(reverse ? first + (r.left - 1) * warps : first);
       r.step = reverse ? -static_cast<int>(warps) : static_cast<int>(warps);
       return;
     }
   }
 }
 
+// Warps of a CTA, and the shared address of a warp's tile slots.
+template <typename S>
+__device__ __forceinline__ unsigned int cta_warps() {
+  if constexpr (S::kSolo) return blockDim.x >> 5;
+  else return kQWarps;
+}
+template <typename S>
+__device__ __forceinline__ unsigned int slots_of(S& sh, unsigned int warp) {
+  if constexpr (S::kSolo) return sh.slots + warp * sh.per_warp * (kQTileBytes + kQStateBytes);
+  else return smem_u32(sh.ring[warp]);
+}
+
+// Waits until at most n of the lane's copy groups are in flight.
+__device__ __forceinline__ void copies_wait_upto(unsigned int n) {
+  switch (n) {
+    case 0: copies_wait<0>(); break;
+    case 1: copies_wait<1>(); break;
+    case 2: copies_wait<2>(); break;
+    case 3: copies_wait<3>(); break;
+    default: copies_wait<4>(); break;
+  }
+}
+
+// The walk over tiles that stay in shared memory for the whole call: the warp's own slots, filled once by load_resident
+// (one copy group per tile), the block states beside them.
+template <bool kState, typename S, typename B, typename Enter, typename Leave, typename Body>
+__device__ __forceinline__ void walk_resident(S& sh, const B& bt, Enter enter, Leave leave, Body body) {
+  const unsigned int lane = threadIdx.x & 31u, warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
+  const unsigned int warps = gridDim.x * cta_warps<S>(), me = blockIdx.x * cta_warps<S>() + warp, tiles = bt.t[0].ntiles;
+  if (me >= tiles) return;
+  const unsigned int n = (tiles - 1 - me) / warps + 1;
+  unsigned int at = slots_of(sh, warp);
+  unsigned int b = me * 32 + lane;
+  const unsigned int get = tile_chunk(2 * lane) * 16;
+  enter(0);
+  for (unsigned int k = 0; k < n; ++k) {
+    if (!kState) {   // (the passes that read states come later)
+      copies_wait_upto(n - 1 - k);
+      __syncwarp();
+    }
+    const uint4 v0 = lds128(at + get), v1 = lds128((at + get) ^ 16u);
+    const unsigned int state_at = at + kQTileBytes + lane * 8;
+    uint2 st = make_uint2(0u, 0u);
+    if (kState) st = lds64(state_at);
+    body(b, v0, v1, st, []() {}, state_at);
+    at += kQTileBytes + kQStateBytes;
+    b += warps * 32;
+  }
+  leave(0);
+}
+
+// Starts the copies of every tile of the warp into its slots.
+template <typename S, typename B>
+__device__ __forceinline__ void load_resident(S& sh, const B& bt) {
+  const Params& p = bt.t[0];
+  const unsigned int lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = gridDim.x * cta_warps<S>();
+  unsigned int at = slots_of(sh, warp) + tile_chunk(lane) * 16;
+  const unsigned char* const w = reinterpret_cast<const unsigned char*>(p.W);
+  for (unsigned int tile = blockIdx.x * cta_warps<S>() + warp; tile < p.ntiles; tile += warps) {
+#pragma unroll
+    for (unsigned int h = 0; h < 2; ++h) {
+      const unsigned int b = tile * 32 + h * 16 + (lane >> 1);
+      const unsigned int row = p.contiguous ? 0u : __umulhi(2u * b, p.nbc_magic) >> p.nbc_shift;
+      const unsigned char* src = w + (static_cast<long long>(row) * (p.ld - static_cast<long long>(p.nbc) * 16) +
+                                      static_cast<long long>(b) * 16) * 2 + (lane & 1u) * 16;
+      if (b < p.nblk) copy16(at + 512 * h, src);
+    }
+    copies_commit();
+    at += kQTileBytes + kQStateBytes;
+  }
+}
+
 // One warp's walk over its share of the pass's tiles.  `enter(ti)` and `leave(ti)` bracket the tiles of one tensor;
-// `body(b, v0, v1, st, next)` gets the lane's block number (past the tensor's end in the last tile: the body looks), its
-// 32 bytes and, with kState, its block state, and calls next() once it is done with these registers.  kRing: tiles
+// `body(b, v0, v1, st, next, state_at)` gets the lane's block number (past the tensor's end in the last tile: the body
+// looks), its 32 bytes and, with kState, its block state, and calls next() once it is done with these registers;
+// state_at is where a resident block keeps its state in shared memory.  kRing: tiles
 // come through the warp's slots in shared memory, three ahead; else through registers, one ahead.  The warp
 // number is broadcast so that the compiler sees the bookkeeping as uniform.
-template <bool kRing, bool kState, typename S, typename Enter, typename Leave, typename Body>
-__device__ __forceinline__ void walk_tiles(S& sh, const Batch& bt, bool reverse, Enter enter, Leave leave, Body body) {
+template <bool kRing, bool kState, typename S, typename B, typename Enter, typename Leave, typename Body>
+__device__ __forceinline__ void walk_tiles(S& sh, const B& bt, bool reverse, Enter enter, Leave leave, Body body) {
+  if constexpr (S::kResident) {
+    walk_resident<kState>(sh, bt, enter, leave, body);
+    return;
+  } else {
   const unsigned int lane = threadIdx.x & 31u, warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
-  const unsigned int warps = gridDim.x * kQWarps, me = blockIdx.x * kQWarps + warp;
-  const unsigned int ring = smem_u32(sh.ring[warp]);
+  const unsigned int warps = gridDim.x * cta_warps<S>(), me = blockIdx.x * cta_warps<S>() + warp;
+  const unsigned int ring = slots_of(sh, warp);
   const unsigned int put = ring + tile_chunk(lane) * 16, get = ring + tile_chunk(2 * lane) * 16;
   const unsigned int put_state = ring + kQStages * kQTileBytes + lane * 16, get_state = ring + kQStages * kQTileBytes + lane * 8;
 
@@ -500,7 +582,7 @@ __device__ __forceinline__ void walk_tiles(S& sh, const Batch& bt, bool reverse,
     next_run(sh, bt.n, reverse, me, warps, f);
     if (f.left == 0) return;
     const Params& p = bt.t[f.ti];
-    // the ragged last tile is the last of a forward run, the first of a backward one
+    // the ragged last tile of a tensor is the last of a forward run, the first of a backward one
     const int top = reverse ? f.tile : f.tile + static_cast<int>(f.left - 1) * f.step;
     f_w = reinterpret_cast<const unsigned char*>(p.W);
     f_state = reinterpret_cast<const unsigned char*>(p.state);
@@ -587,36 +669,41 @@ __device__ __forceinline__ void walk_tiles(S& sh, const Batch& bt, bool reverse,
         v1 = lds128(at ^ 16u);
         if (kState) st = lds64(get_state + slot * kQStateBytes);
         slot = (slot + 1) % kQStages;
-        body(b, v0, v1, st, []() {});
+        body(b, v0, v1, st, []() {}, 0u);
       } else {
-        body(b, v0, v1, st, [&]() { feed_registers(v0, v1, st); });
+        body(b, v0, v1, st, [&]() { feed_registers(v0, v1, st); }, 0u);
       }
       b += b_step;
     }
     leave(r.ti);
   }
+  }
 }
 
 // A warp hands its sums for tensor ti to the CTA's.
-template <bool kDet>
-__device__ __forceinline__ void hand_over(QShared<kDet>& sh, int ti, double (&v)[2]) {
+template <typename S>
+__device__ __forceinline__ void hand_over(S& sh, int ti, double (&v)[2]) {
   v[0] = warp_sum(v[0]);
   v[1] = warp_sum(v[1]);
   if ((threadIdx.x & 31) == 0) {
-    if (kDet) {
+    if constexpr (S::kSolo) {
+      sh.part[threadIdx.x >> 5][0] = v[0];
+      sh.part[threadIdx.x >> 5][1] = v[1];
+    } else if constexpr (S::kOrdered) {
       sh.part[ti][threadIdx.x >> 5][0] += v[0];
       sh.part[ti][threadIdx.x >> 5][1] += v[1];
+      atomicOr(&sh.visited, 1u << ti);
     } else {
       atomicAdd(&sh.acc[ti][0], v[0]);
       atomicAdd(&sh.acc[ti][1], v[1]);
+      atomicOr(&sh.visited, 1u << ti);
     }
-    atomicOr(&sh.visited, 1u << ti);
   }
   v[0] = v[1] = 0.0;
 }
 
-template <bool kDet>
-__device__ __forceinline__ void hand_over_counters(QShared<kDet>& sh, int ti, unsigned int& zeros, unsigned int& wide) {
+template <typename S>
+__device__ __forceinline__ void hand_over_counters(S& sh, int ti, unsigned int& zeros, unsigned int& wide) {
   zeros = __reduce_add_sync(0xFFFFFFFFu, zeros);
   wide = __reduce_add_sync(0xFFFFFFFFu, wide);
   if ((threadIdx.x & 31) == 0) {
@@ -676,9 +763,30 @@ __device__ __forceinline__ void file_sums(QShared<kDet>& sh, const Batch& bt, in
 
 // ------------------------------------------------------------------ passes
 
+// A block's carried state goes to the workspace, or stays in shared memory with a resident block.
+template <typename S>
+__device__ __forceinline__ void put_state(uint2* state, unsigned int b, unsigned int state_at, uint2 v) {
+  if constexpr (S::kResident) asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(state_at), "r"(v.x), "r"(v.y) : "memory");
+  else state[b] = v;
+}
+
+// A scale byte of the start pass when it is the last one: row-major, tiled, or both.
+template <typename S>
+__device__ __forceinline__ void put_scale(const S& sh, const Params& p, uint8_t* scales, unsigned int b, int d) {
+  if constexpr (S::kSolo) {
+    uint8_t* const tiled = sh.view[0].tiled;
+    if (tiled != nullptr) {
+      const unsigned int row = __umulhi(2u * b, p.nbc_magic) >> p.nbc_shift;
+      tiled[swizzled_offset(row, b - row * p.nbc, (p.nbc + 3) / 4)] = static_cast<uint8_t>(d);
+      if (sh.tiled_only) return;
+    }
+  }
+  scales[b] = static_cast<uint8_t>(d);
+}
+
 // Eq. 1's tensor maximum, plus sum W^2 (binary64) for the error report.
-template <bool kDet>
-__device__ __forceinline__ void amax_pass(QShared<kDet>& sh, const Batch& bt) {
+template <typename S, typename B>
+__device__ __forceinline__ void amax_pass(S& sh, const B& bt) {
   const unsigned int lane = threadIdx.x & 31u;
   unsigned int mx = 0;
   double sq[2] = {0.0, 0.0};
@@ -694,7 +802,7 @@ __device__ __forceinline__ void amax_pass(QShared<kDet>& sh, const Batch& bt) {
         mx = 0;
         sq[0] = sq[1] = 0.0;
       },
-      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next) {
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next, unsigned int) {
         const bool here = b < nblk;
         const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
         // largest magnitude of the block with packed bf16 max (a NaN input comes out of the maximum
@@ -715,9 +823,10 @@ __device__ __forceinline__ void amax_pass(QShared<kDet>& sh, const Batch& bt) {
 }
 
 // Algorithm 1 "Initialization" (Eq. 1): dd0 = E4M3(bmax/(6 alpha0)), dq0 = dd0; first codes (Eq. 2); stage-0 sums for
-// Eq. 5 and the starting error.  Codes and scales are written here only when no iteration follows, the block states only when one does.
-template <bool kDet>
-__device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt) {
+// Eq. 5 and the starting error.  Codes and scales are written here only when no iteration follows, the block states only when
+// one does.
+template <typename S, typename B>
+__device__ __forceinline__ void init_pass(S& sh, const B& bt) {
   float alpha = 1.0f, six_alpha = 6.0f, six_inv = 0.0f;
   double alpha_d = 1.0;
   bool tame = false;
@@ -743,7 +852,7 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt) {
         hand_over(sh, ti, acc);
         hand_over_counters(sh, ti, zeros, wide);
       },
-      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next) {
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next, unsigned int state_at) {
         PairBlock blk;
         unpack_pairs(v0, v1, blk);
         next();
@@ -763,8 +872,8 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt) {
           unsigned int c0, c1;
           round_pairs(blk, 1.0f, c0, c1);
           reinterpret_cast<uint2*>(packed)[b] = make_uint2(c0, c1);
-          scales[b] = 0;
-          if (keep) state[b] = make_uint2(0u, 0u);
+          put_scale(sh, bt.t[tensor], scales, b, 0);
+          if (keep) put_state<S>(state, b, state_at, make_uint2(0u, 0u));
           ++zeros;
           return;
         }
@@ -795,9 +904,11 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt) {
         }
         if (!keep) {
           reinterpret_cast<uint2*>(packed)[b] = make_uint2(f.c0, f.c1);
-          scales[b] = static_cast<uint8_t>(f.d);
-        } else
-          state[b] = make_uint2(__float_as_uint(f.A), pack_state(__float_as_uint(bmax) & 0x7F800000u, f.d, f.b4));
+          put_scale(sh, bt.t[tensor], scales, b, f.d);
+        } else {
+          put_state<S>(state, b, state_at,
+                       make_uint2(__float_as_uint(f.A), pack_state(__float_as_uint(bmax) & 0x7F800000u, f.d, f.b4)));
+        }
         // v^2 4B is exact in binary32: 8 + 12 significant bits
         acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(v, v), __uint2float_rn(f.b4)));
         acc[1] += f.g;
@@ -815,8 +926,8 @@ __device__ __forceinline__ void init_pass(QShared<kDet>& sh, const Batch& bt) {
 //   kMode 4  the grid of App. B.3 around the Eq. 6 solution with two E4M3 codes, only the multipliers that can win
 //   kMode 5  the same for any number of codes, and for grids so short that a block's bracket often reaches past their
 //            first or last multiplier
-template <int kMode, bool kDet>
-__device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt, bool reverse, unsigned int emit, unsigned int keep) {
+template <int kMode, typename S, typename B>
+__device__ __forceinline__ void iterate_pass(S& sh, const B& bt, bool reverse, unsigned int emit, unsigned int keep) {
   asm volatile("" : "+r"(emit), "+r"(keep));   // in registers, not worked out again per tile
   const int n_dq = bt.t[0].n_dq, n_beta = bt.t[0].n_beta, flags = bt.t[0].flags;
   const bool keep_scale = kMode == 3 || (kMode != 4 && (flags & SOAR_FLAG_KEEP_BLOCK_SCALE) != 0);
@@ -844,7 +955,7 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
         hand_over(sh, ti, acc);
         hand_over_counters(sh, ti, zeros, wide);
       },
-      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2& state, auto next) {
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2& state, auto next, unsigned int state_at) {
         PairBlock blk;
         unpack_pairs(v0, v1, blk);
         const uint2 st = state;
@@ -899,8 +1010,8 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
             halves(m2, b0f, b1);
           }
           // The pair of multipliers must enclose the code's value with a margin that covers the three roundings
-          // from here to the scaled value (2^-24 each; see winning_range): 6 * 2^-24 does.  A block that misses it,
-          // one in several thousand, takes the exact walk.
+          // from here to the scaled value (2^-24 each; see winning_range): 6 * 2^-24 does.  Where one of the two lies
+          // inside the band, in one block of seven thousand, its neighbour on the other side can win too.
           constexpr float kUnder = 1.0f - 0x1.8p-22f, kOver = 1.0f + 0x1.8p-22f;
           const bool below0 = a0 <= v0f * kUnder, above0 = b0f >= v0f * kOver;
           const bool below1 = a1 <= v1f * kUnder, above1 = b1 >= v1f * kOver;
@@ -927,8 +1038,10 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
           halves(n0, s00, s01);
           s_exp = __float_as_uint(s00) & 0x7F800000u;
           // the largest magnitude of the block below 32 times the smallest scale, from the exponents
-          direct = direct && ((below0 && above0) || low0 || high0) && ((below1 && above1) || low1 || high1) &&
-                   st.y < s_exp + (5u << 23);
+          const bool enclosed = below0 && above0 && below1 && above1;
+          direct = direct && st.y < s_exp + (5u << 23);
+          if (kMode == 5) direct = direct && ((below0 && above0) || low0 || high0) && ((below1 && above1) || low1 || high1);
+          if (kMode == 3) direct = direct && enclosed;
           FixedPairs fx;
           make_fixed_pairs(blk, __uint_as_float((264u << 23) - s_exp), fx);
           // h = dv S / 4; the exponent of S / 4 is 135 less s's biased one
@@ -952,6 +1065,22 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
             if (y2.e < w.e) w = y2;
             score_pairs(blk, fx, r12, rho1, y2);
             if (y2.e < x.e) x = y2;
+          }
+          if (kMode == 4 && !enclosed) {
+            // the third multiplier: before the pair when the first of it is not below the band, after it when the second
+            // is not above; equal errors go to the earlier one
+            if (!below0 || !above0) {
+              const uint2 q = lds64(pairs + 8u * static_cast<unsigned int>(below0 ? k0 + 1 : max(k0 - 1, 0)));
+              const float m = __uint_as_float(below0 ? q.y : q.x);
+              score_pairs(blk, fx, recip_fast(grid_divisor(alpha, center, m)), rho0, y2);
+              if (y2.e < w.e || (!below0 && y2.e == w.e)) w = y2;
+            }
+            if (!below1 || !above1) {
+              const uint2 q = lds64(pairs + 8u * static_cast<unsigned int>(below1 ? k1 + 1 : max(k1 - 1, 0)));
+              const float m = __uint_as_float(below1 ? q.y : q.x);
+              score_pairs(blk, fx, recip_fast(grid_divisor(alpha, center, m)), rho1, y2);
+              if (y2.e < x.e || (!below1 && y2.e == x.e)) x = y2;
+            }
           }
           // equal errors: the earlier multiplier, as in grid order (the second code's are never earlier)
           const double g0 = h0 * w.e, g1 = h1 * x.e;
@@ -1022,7 +1151,8 @@ __device__ __forceinline__ void iterate_pass(QShared<kDet>& sh, const Batch& bt,
             reinterpret_cast<uint2*>(packed)[b] = make_uint2(w.c0, w.c1);
             scales[b] = static_cast<uint8_t>(d);
           }
-          if (keep) states[b] = make_uint2(__float_as_uint(A), pack_state(st.y & 0x7F800000u, d, w.b4));
+          if (keep)
+            put_state<S>(states, b, state_at, make_uint2(__float_as_uint(A), pack_state(st.y & 0x7F800000u, d, w.b4)));
           // v^2 4B is exact in binary32: 8 + 12 significant bits
           acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(v, v), __uint2float_rn(w.b4)));
           acc[1] = fma(g_scaled, g_scale, acc[1]);
@@ -1101,7 +1231,8 @@ __device__ __forceinline__ void tile_scales(const Params& p, unsigned int rows, 
   const bool words = nbc % 4 == 0 && reinterpret_cast<uintptr_t>(p.scales) % 4 == 0;
   const bool out16 = reinterpret_cast<uintptr_t>(sw) % 16 == 0;
   const unsigned int lane = threadIdx.x & 31u;
-  for (unsigned int tile = blockIdx.x * kQWarps + (threadIdx.x >> 5); tile < tiles; tile += gridDim.x * kQWarps) {
+  const unsigned int warps = blockDim.x >> 5;
+  for (unsigned int tile = blockIdx.x * warps + (threadIdx.x >> 5); tile < tiles; tile += gridDim.x * warps) {
     const unsigned int tr = tile / col_tiles, col = (tile - tr * col_tiles) * 4;
     unsigned int w[4];
 #pragma unroll
@@ -1168,6 +1299,7 @@ quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Report
     sh.view[tid].packed = bt.t[tid].packed;
     sh.view[tid].scales = bt.t[tid].scales;
     sh.view[tid].state = bt.t[tid].state;
+    sh.view[tid].tiled = nullptr;
   }
   if (tid < kMaxBatch) {
     sh.acc[tid][0] = sh.acc[tid][1] = 0.0;
@@ -1257,7 +1389,7 @@ quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Report
     } else {
       const int t = s - kQStageIterate;
       const bool last = t == T - 1;
-      iterate_pass<kMode, kDet>(sh, bt, (t & 1) != 0, bt.t[0].early_stop_rel > 0.0f || last, !last);
+      iterate_pass<kMode>(sh, bt, (t & 1) != 0, bt.t[0].early_stop_rel > 0.0f || last, !last);
       file_sums(sh, bt, t + 1);
     }
     ++s;

@@ -47,6 +47,7 @@
 #include <atomic>
 #include <mutex>
 #include <new>
+#include <random>
 #include <vector>
 
 #include "soar.h"
@@ -128,6 +129,11 @@ struct Batch {
   unsigned int total_tiles;
   unsigned int tile_end[kMaxBatch];   // running sum of the tensors' tile counts
   Params t[kMaxBatch];
+};
+// The same for one tensor (a smaller parameter block makes a cheaper launch).
+struct Single {
+  static constexpr int n = 1;
+  Params t[1];
 };
 static_assert(sizeof(Batch) <= 3072, "kernel parameter block too large");
 
@@ -738,8 +744,6 @@ struct Winner {
   int d;
 };
 
-#include "quantize_kernel.cuh"
-
 // Offset of scale (row, col) in the 128x4-tiled layout: tiles of 128 rows x 4 scale columns
 // (512 bytes), tile rows outermost; inside a tile row r and column c sit at
 // (r % 32) * 16 + (r / 32) * 4 + c.
@@ -748,6 +752,9 @@ __device__ __forceinline__ size_t swizzled_offset(unsigned int row, unsigned int
   const unsigned int r = row & 127u;
   return tile * 512 + (r & 31u) * 16 + (r >> 5) * 4 + (col & 3u);
 }
+
+#include "quantize_kernel.cuh"
+#include "solo_kernel.cuh"
 
 // Eq. 3-4 on stored outputs: sum (w - q s)^2 and sum w^2, one binary64 fma per term, with the
 // bf16 values widened by the conversion instruction (which runs beside the integer and
@@ -1625,7 +1632,7 @@ size_t soar_workspace_bytes(int64_t rows, int64_t cols, const soar_cfg* cfg) {
   if (cfg->max_iters > 0) n += round256(nblk * sizeof(uint2));
   if (!(cfg->scale_layout & SOAR_SCALES_LINEAR)) n += round256(nblk);
   if (cfg->flags & SOAR_FLAG_DETERMINISTIC) n += round256(sizeof(DetParts));
-  return n;
+  return n + exchange_bytes(static_cast<unsigned int>((nblk + 31) / 32));
 }
 
 size_t soar_swizzled_scale_bytes(int64_t rows, int64_t cols) {
@@ -1727,6 +1734,105 @@ int search_mode(const soar_cfg* cfg) {
   return (cfg->flags & SOAR_FLAG_KEEP_BLOCK_SCALE) ? 3 : 4;
 }
 
+// A number no earlier call of this process used, and that memory left by another is not likely to hold: a counter
+// from a random start through a 64-bit mixing function (the finalizer of SplitMix64; Steele, Lea and Flood, "Fast
+// splittable pseudorandom number generators", OOPSLA 2014).
+unsigned long long call_nonce() {
+  static const unsigned long long seed = [] {
+    std::random_device rd;
+    return (static_cast<unsigned long long>(rd()) << 32) ^ rd();
+  }();
+  static std::atomic<unsigned long long> calls;
+  unsigned long long z = seed + 0x9E3779B97F4A7C15ull * (calls.fetch_add(1, std::memory_order_relaxed) + 1);
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+  return z ^ (z >> 31);
+}
+
+// One matrix in one launch (see solo_grid); the tiles stay in shared memory when every warp's fit its slots.
+template <int kMode, bool kRes>
+cudaError_t launch_solo(const SoloArgs& a, unsigned int grid, unsigned int warps, cudaStream_t st) {
+  const unsigned int slots = warps * (kRes ? a.per_warp : static_cast<unsigned int>(kQStages));
+  const size_t dynamic = static_cast<size_t>(slots) * (kQTileBytes + kQStateBytes);
+  {
+    static std::atomic<bool> raised[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!raised[dev].load(std::memory_order_acquire)) {
+      const unsigned int most = kSoloWarps * (kRes ? kResidentTiles : static_cast<unsigned int>(kQStages));
+      const cudaError_t err = cudaFuncSetAttribute(solo_kernel<kMode, kRes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>(most * (kQTileBytes + kQStateBytes)));
+      if (err != cudaSuccess) return err;
+      raised[dev].store(true, std::memory_order_release);
+    }
+  }
+  if (grid == 1) {
+    solo_kernel<kMode, kRes><<<1, warps * 32, dynamic, st>>>(a);
+    return cudaGetLastError();
+  }
+  void* args[] = {const_cast<SoloArgs*>(&a)};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&solo_kernel<kMode, kRes>), dim3(grid), dim3(warps * 32), args,
+                                     dynamic, st);
+}
+
+int run_solo(const soar_tensor_desc& d, const soar_cfg* cfg, uint8_t* workspace, int mode, cudaStream_t st) {
+  const bool want_lin = (cfg->scale_layout & SOAR_SCALES_LINEAR) != 0;
+  const bool want_sw = (cfg->scale_layout & SOAR_SCALES_SWIZZLED) != 0;
+  SoloArgs a;
+  memset(&a, 0, sizeof(a));
+  Params& p = a.m.t[0];
+  uint8_t* next = workspace + kWsFixedBytes;
+  p.W = static_cast<const uint16_t*>(d.W_bf16);
+  p.packed = static_cast<uint8_t*>(d.out_fp4_packed);
+  p.ws = reinterpret_cast<Ws*>(workspace);
+  p.ld = d.ld;
+  p.nbc = static_cast<unsigned int>(d.cols / 16);
+  p.nblk = static_cast<unsigned int>(d.rows * (d.cols / 16));
+  p.ntiles = (p.nblk + 31) / 32;
+  set_division(p);
+  p.contiguous = (d.ld == d.cols) ? 1 : 0;
+  if (cfg->max_iters > 0) {
+    p.state = reinterpret_cast<uint2*>(next);
+    next += round256(static_cast<size_t>(p.nblk) * sizeof(uint2));
+  }
+  if (want_lin) {
+    p.scales = static_cast<uint8_t*>(d.out_e4m3_scales);
+  } else {
+    p.scales = next;
+    next += round256(p.nblk);
+  }
+  p.max_iters = cfg->max_iters;
+  p.early_stop_rel = cfg->early_stop_rel;
+  p.n_dq = cfg->n_dq;
+  p.n_beta = cfg->n_beta;
+  p.beta_step_pct = cfg->beta_step_pct;
+  p.flags = cfg->flags;
+  a.alpha = d.out_global_fp32;
+  a.result = d.out_result;
+  a.tiled = want_sw ? static_cast<uint8_t*>(d.out_e4m3_scales_sw) : nullptr;
+  a.exchange = next;
+  a.nonce = call_nonce();
+  a.rows = static_cast<unsigned int>(d.rows);
+  a.tiled_only = want_lin ? 0 : 1;
+  a.idle = g_idle_producer;
+  const unsigned int sms = static_cast<unsigned int>(sm_count()), warps = solo_warps(p.ntiles);
+  const unsigned int grid = solo_grid(p.ntiles, sms < kSoloMaxGrid ? sms : kSoloMaxGrid);
+  a.per_warp = (p.ntiles + grid * warps - 1) / (grid * warps);
+  const bool resident = a.per_warp <= kResidentTiles;
+  cudaError_t err;
+#define SOAR_SOLO(M) err = resident ? launch_solo<M, true>(a, grid, warps, st) : launch_solo<M, false>(a, grid, warps, st)
+  switch (mode) {
+    case 0: SOAR_SOLO(0); break;
+    case 1: SOAR_SOLO(1); break;
+    case 2: SOAR_SOLO(2); break;
+    case 3: SOAR_SOLO(3); break;
+    case 4: SOAR_SOLO(4); break;
+    default: SOAR_SOLO(5); break;
+  }
+#undef SOAR_SOLO
+  return err == cudaSuccess ? SOAR_OK : SOAR_ERR_CUDA;
+}
+
 // Which part of a call is wanted: all of it (soar_quantize_batch), or one stage (soar_quantize_stage; iterations
 // t_lo <= t < t_hi for kStageIterate).
 enum : int { kStageAmax = 1, kStageInit = 2, kStageIterate = 4, kStageFinalize = 8, kStageAll = 15 };
@@ -1758,11 +1864,12 @@ int run_batch(const soar_tensor_desc* tensors, int n, const soar_cfg* cfg, void*
   // workspace: the n headers first (one memset clears them all), then each tensor's arrays
   uint8_t* const headers = static_cast<uint8_t*>(workspace);
   uint8_t* next = headers + static_cast<size_t>(n) * kWsFixedBytes;
+  const int mode = search_mode(cfg);
+  if (n == 1 && stages == kStageAll && !g_trace.on) return run_solo(tensors[0], cfg, headers, mode, st);
   if ((stages & kStageAmax) &&
       cudaMemsetAsync(headers, 0, static_cast<size_t>(n) * kWsFixedBytes, st) != cudaSuccess)
     return SOAR_ERR_CUDA;
 
-  const int mode = search_mode(cfg);
   for (int first = 0; first < n; first += kMaxBatch) {
     Batch bt;
     Reports rp;
@@ -1799,6 +1906,7 @@ int run_batch(const soar_tensor_desc* tensors, int n, const soar_cfg* cfg, void*
         p.det = reinterpret_cast<DetParts*>(next);
         next += round256(sizeof(DetParts));
       }
+      next += exchange_bytes(p.ntiles);   // used by calls on one matrix
       p.max_iters = cfg->max_iters;
       p.early_stop_rel = cfg->early_stop_rel;
       p.n_dq = cfg->n_dq;
@@ -1881,8 +1989,10 @@ int soar_quantize(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld, co
 // Built-in scratch of soar_quantize_static.  In host code the symbol below is only a handle:
 // the device address comes from cudaGetSymbolAddress, looked up once per device.
 static __device__ __align__(256) unsigned char g_static_scratch[SOAR_STATIC_SCRATCH_BYTES];
-// the largest accepted matrix needs exactly this much: the header, 8 bytes of state and one scale byte per block
-static_assert(kWsFixedBytes + (SOAR_STATIC_MAX_ELEMENTS / 16) * (sizeof(uint2) + 1) == SOAR_STATIC_SCRATCH_BYTES,
+// the largest accepted matrix needs exactly this much: the header, 8 bytes of state and one scale byte per block, and the
+// packets its CTAs exchange
+static_assert(kWsFixedBytes + (SOAR_STATIC_MAX_ELEMENTS / 16) * (sizeof(uint2) + 1) + exchange_bytes(SOAR_STATIC_MAX_ELEMENTS / 512) ==
+                  SOAR_STATIC_SCRATCH_BYTES,
               "SOAR_STATIC_SCRATCH_BYTES does not match the workspace of SOAR_STATIC_MAX_ELEMENTS");
 
 namespace {

@@ -1,0 +1,312 @@
+// One matrix, one launch.  The passes are quantize_kernel's; what differs is how they meet and where the weights stay.
+// Included by soar.cu after quantize_kernel.cuh.
+//
+// Small matrices are bound by latency: what counts is the chain from the last block of one pass to the first of the
+// next.  With the sums added by atomics in memory zeroed by a memset, that chain took 3.5 of the 5 microseconds of an
+// iteration at any size.  Here every CTA stores its sums in a slot of its own, arrives at a counter and, when all
+// have, reads everybody's slots and adds them in the same order on every run: 1.6 us from the last arrival on, for 2 to
+// 148 CTAs.  (Polling tagged slots instead, with no counter, is 0.7 us when all CTAs come at the same moment but 3 us
+// when some wait for others, as they do.)  The grid is one CTA of 16 warps per SM rather than two of 8: 296 CTAs need
+// 0.7 us more.
+//
+// Matrices whose tiles fit the shared memory of the grid (12 million weights) are read from HBM once and stay
+// there, and so do their block states (kResident); larger ones stream through the passes like a batch.
+//
+// Nothing has to be zero before the launch, so no memset goes ahead of it: CTA 0 clears the counter while the first
+// pass runs and says so in a flag, whose value is nonce + epoch.  The nonce is new for every call the host makes; the
+// epoch is a word of the workspace that CTA 0 advances at the end of a call, after every CTA has read it, so that
+// the replay of a captured call does not take the flag of the replay before for its own.  Whatever the workspace
+// held before a call, it would have to hold the 64-bit flag of a call not made yet to be taken for open.
+
+#pragma once
+
+constexpr int kSoloWarps = 16;                     // most warps of a CTA (8 in small grids)
+constexpr unsigned int kSoloMaxGrid = 160;
+constexpr unsigned int kResidentTiles = 10;        // slots a warp can have: 200 KB a CTA
+constexpr size_t kSlotBytes = 24;                  // three numbers of one CTA and pass
+
+// One warp per tile while 32 CTAs of 8 warps suffice (fewer warps an SM make a tile's latency shorter), then CTAs of 16
+// warps, one an SM.
+constexpr unsigned int solo_warps(unsigned int tiles) { return tiles <= 256 ? 8 : kSoloWarps; }
+constexpr unsigned int solo_grid(unsigned int tiles, unsigned int most) {
+  const unsigned int want = (tiles + solo_warps(tiles) - 1) / solo_warps(tiles);
+  return want < most ? want : most;
+}
+// Workspace of the exchange: epoch, flag and counter, then the slots of even and of odd passes; none for one CTA.
+constexpr size_t exchange_bytes(unsigned int tiles) {
+  const size_t grid = solo_grid(tiles, kSoloMaxGrid);
+  return grid > 1 ? (256 + 2 * grid * kSlotBytes + 255) / 256 * 256 : 0;
+}
+
+struct SoloArgs {
+  Single m;
+  float* alpha;
+  soar_result* result;     // or null
+  uint8_t* tiled;          // tiled scales, or null
+  unsigned char* exchange;
+  unsigned long long nonce;
+  unsigned int rows;
+  unsigned int per_warp;   // resident: slots of a warp
+  int tiled_only;          // the caller wants no row-major scales
+  int idle;                // test hook: nobody arrives, every wait runs out
+};
+
+template <bool kRes>
+struct __align__(128) SoloShared {
+  static constexpr bool kOrdered = true, kSolo = true, kResident = kRes;
+  View view[1];
+  float2 beta[SOAR_MAX_BETA];
+  double part[kSoloWarps][2];        // each warp's sums of the pass
+  unsigned long long red[2][kSoloMaxGrid / 32][3];   // the grid's numbers, by the warp that read them
+  double trace_alpha[SOAR_MAX_ITERS + 1], trace_sse[SOAR_MAX_ITERS + 1];
+  float alpha[1];
+  unsigned int amax[1], zeros[1], wide[1];
+  unsigned int start[1], count[1], total;
+  unsigned int slots;                // shared address of the warps' tile slots
+  unsigned int per_warp;
+  int tiled_only;
+  int failed;
+};
+
+// Sums of the grid, the same bits in every thread.
+struct Totals {
+  double a, g;                       // sum W^2 and nothing (kMax), else 4 den and gsum
+  unsigned int amax;                 // kMax: the maximum's bits
+  unsigned long long counts;         // zero blocks in the low half, wide candidates in the high one (CTA 0 only)
+};
+
+// Before the first exchange (one thread): CTA 0 clears the counter and opens the flag, the others wait for it.
+__device__ __forceinline__ void open_counter(const SoloArgs& a, unsigned long long tag, int& failed) {
+  unsigned long long* const flag = reinterpret_cast<unsigned long long*>(a.exchange + 8);
+  if (blockIdx.x == 0) {
+    *reinterpret_cast<volatile unsigned int*>(a.exchange + 64) = 0u;
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(flag), "l"(tag) : "memory");
+  } else {
+    unsigned long long seen = 0;
+    unsigned int polls = 0;
+    do {
+      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(flag) : "memory");
+    } while (seen != tag && ++polls < kGridWaitLimit);
+    if (seen != tag) failed = 1;
+  }
+}
+
+// After a pass, all threads of all CTAs: exchanges the CTAs' sums.  `pass` counts from 1.  What the CTAs wrote to global
+// memory before is visible to all after.  With `last` only CTA 0 waits for the sums.  False when a wait ran out.
+template <bool kMax, typename S>
+__device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned int pass, bool last, Totals& out) {
+  __syncthreads();
+  const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
+  unsigned long long* const slots = reinterpret_cast<unsigned long long*>(a.exchange + 256 + turn * (grid * kSlotBytes));
+  if (tid < 32) {
+    double x = 0.0, g = 0.0;
+    if (lane < blockDim.x / 32) {
+      x = sh.part[lane][0];
+      g = sh.part[lane][1];
+    }
+    x = warp_sum(x);
+    g = warp_sum(g);
+    const unsigned long long second = kMax ? sh.amax[0] : static_cast<unsigned long long>(__double_as_longlong(g));
+    const unsigned long long counts = sh.zeros[0] | (static_cast<unsigned long long>(sh.wide[0]) << 32);
+    __syncwarp();
+    if (lane == 0) sh.zeros[0] = sh.wide[0] = 0u;
+    if (grid == 1) {
+      if (lane == 0) {
+        sh.red[turn][0][0] = static_cast<unsigned long long>(__double_as_longlong(x));
+        sh.red[turn][0][1] = second;
+        sh.red[turn][0][2] = counts;
+      }
+    } else {
+      if (lane < 3)
+        __stcg(slots + lane * grid + blockIdx.x,
+               lane == 0 ? static_cast<unsigned long long>(__double_as_longlong(x)) : lane == 1 ? second : counts);
+      __syncwarp();
+      if (lane == 0) {
+        unsigned int* const arrived = reinterpret_cast<unsigned int*>(a.exchange + 64);
+        if (!a.idle) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
+        if (!last || blockIdx.x == 0) {
+          unsigned int seen = 0, polls = 0;
+          do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(arrived) : "memory");
+          } while (seen < pass * grid && ++polls < kGridWaitLimit);
+          if (seen < pass * grid) sh.failed = 1;
+        }
+      }
+    }
+  }
+  if (last && blockIdx.x != 0) return true;
+  __syncthreads();
+  const unsigned int warps = (grid + 31) / 32;
+  if (grid > 1) {
+    if (tid < warps * 32) {
+      double x = 0.0, g = 0.0;
+      unsigned int mx = 0;
+      unsigned long long counts = 0;
+      if (tid < grid) {
+        x = __longlong_as_double(static_cast<long long>(__ldcg(slots + tid)));
+        const unsigned long long second = __ldcg(slots + grid + tid);
+        if (kMax) mx = static_cast<unsigned int>(second);
+        else g = __longlong_as_double(static_cast<long long>(second));
+        if (blockIdx.x == 0) counts = __ldcg(slots + 2 * grid + tid);
+      }
+      x = warp_sum(x);
+      if (kMax) mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+      else g = warp_sum(g);
+      if (blockIdx.x == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) counts += __shfl_xor_sync(0xFFFFFFFFu, counts, o);
+      }
+      if (lane == 0) {
+        sh.red[turn][tid >> 5][0] = static_cast<unsigned long long>(__double_as_longlong(x));
+        sh.red[turn][tid >> 5][1] = kMax ? mx : static_cast<unsigned long long>(__double_as_longlong(g));
+        sh.red[turn][tid >> 5][2] = counts;   // zero blocks do not overflow the low half: a matrix has at most 2^31 blocks
+      }
+    }
+    __syncthreads();
+  }
+  out.a = out.g = 0.0;
+  out.amax = 0;
+  out.counts = 0;
+  for (unsigned int w = 0; w < warps; ++w) {
+    out.a += __longlong_as_double(static_cast<long long>(sh.red[turn][w][0]));
+    if (kMax) out.amax = max(out.amax, static_cast<unsigned int>(sh.red[turn][w][1]));
+    else out.g += __longlong_as_double(static_cast<long long>(sh.red[turn][w][1]));
+    out.counts += sh.red[turn][w][2];
+  }
+  return sh.failed == 0;
+}
+
+// Zeroes of the tiled layout: rows up to a multiple of 128, scale columns up to a multiple of 4.
+__device__ __forceinline__ void clear_tile_padding(const Params& p, unsigned int rows, uint8_t* tiled) {
+  const unsigned int nbc = p.nbc, ct = (nbc + 3) / 4, padded = (rows + 127) / 128 * 128;
+  const unsigned int me = blockIdx.x * blockDim.x + threadIdx.x, all = gridDim.x * blockDim.x;
+  for (unsigned int i = me; i < (padded - rows) * ct * 4; i += all) {
+    const unsigned int r = i / (ct * 4), c = i - r * (ct * 4);
+    tiled[swizzled_offset(rows + r, c, ct)] = 0;
+  }
+  if (nbc % 4 != 0)
+    for (unsigned int r = me; r < rows; r += all)
+      for (unsigned int c = nbc; c < ct * 4; ++c) tiled[swizzled_offset(r, c, ct)] = 0;
+}
+
+template <int kMode, bool kRes>
+__global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_constant__ SoloArgs a) {
+  extern __shared__ __align__(128) unsigned char tile_slots[];
+  __shared__ SoloShared<kRes> sh;
+  const int tid = threadIdx.x;
+  const Params& p = a.m.t[0];
+  const int T = p.max_iters, flags = p.flags;
+  if (tid == 0) {
+    sh.view[0].packed = p.packed;
+    sh.view[0].scales = p.scales;
+    sh.view[0].state = p.state;
+    sh.view[0].tiled = T == 0 ? a.tiled : nullptr;
+    sh.amax[0] = sh.zeros[0] = sh.wide[0] = 0u;
+    sh.start[0] = 0u;
+    sh.count[0] = sh.total = p.ntiles;
+    sh.slots = smem_u32(tile_slots);
+    sh.per_warp = kRes ? a.per_warp : kQStages;
+    sh.tiled_only = a.tiled_only;
+    sh.failed = 0;
+  }
+  if (tid < kSoloWarps) sh.part[tid][0] = sh.part[tid][1] = 0.0;
+  unsigned long long epoch = 0;
+  if (gridDim.x > 1) epoch = __ldcg(reinterpret_cast<const unsigned long long*>(a.exchange));
+  if (kMode == 0 || kMode >= 3) {
+    const int n_beta = p.n_beta, step = p.beta_step_pct;
+    for (int k = tid; k < n_beta; k += static_cast<int>(blockDim.x)) {
+      const float lo = static_cast<float>((100.0 + static_cast<double>((k - n_beta / 2) * step)) / 100.0);
+      const float hi = static_cast<float>((100.0 + static_cast<double>((k + 1 - n_beta / 2) * step)) / 100.0);
+      sh.beta[k] = make_float2(lo, hi);
+    }
+  }
+  __syncthreads();
+  if (kRes) load_resident(sh, a.m);
+  if (T == 0 && a.tiled != nullptr) clear_tile_padding(p, a.rows, a.tiled);
+  if (gridDim.x > 1 && tid == 0) open_counter(a, a.nonce + epoch, sh.failed);
+  unsigned int pass = 0;
+  Totals tot;
+  bool ok;
+  amax_pass(sh, a.m);
+  ok = exchange<true>(sh, a, ++pass, false, tot);
+  const double sumsq = tot.a;
+  const unsigned int amax_bits = tot.amax;
+  const int st = status_from_amax(amax_bits);
+  const float alpha0 = amax_bits == 0 ? 1.0f : __fdiv_rn(bits_to_mag(amax_bits), 2688.0f);
+  float alpha = alpha0;
+  int iters = 0;
+  unsigned long long zero_blocks = 0, wide = 0;
+  double sse = 0.0;
+  // every thread keeps the call's scalars itself, and writes the same alpha for the passes to read
+  sh.alpha[0] = alpha;
+  if (ok && !(st & (SOAR_STATUS_NONFINITE | SOAR_STATUS_RANGE))) {
+    const bool tile_after = T > 0 && a.tiled != nullptr;
+    init_pass(sh, a.m);
+    ok = exchange<false>(sh, a, ++pass, T == 0, tot);
+    if (T == 0 && blockIdx.x != 0) return;   // nothing left to do but CTA 0's report
+    if (st == 0) sse = fmax(sumsq + tot.g, 0.0);
+    zero_blocks = tot.counts & 0xFFFFFFFFull;
+    wide = tot.counts >> 32;
+    if (tid == 0) {
+      sh.trace_alpha[0] = static_cast<double>(alpha0);
+      sh.trace_sse[0] = sse;
+    }
+    const bool may_stop = p.early_stop_rel > 0.0f;
+    for (int t = 0; st == 0 && ok && t < T; ++t) {
+      // Eq. 5; the numerator follows from the two sums carried (see file_sums)
+      const double ad = static_cast<double>(alpha), den = 0.25 * tot.a;
+      if (den > 0.0 && !(flags & SOAR_FLAG_KEEP_ALPHA)) alpha = static_cast<float>((ad * ad * den - tot.g) / (2.0 * ad * den));
+      sh.alpha[0] = alpha;
+      iterate_pass<kMode>(sh, a.m, (t & 1) != 0, may_stop || t == T - 1, t != T - 1);
+      const bool last = t == T - 1 && !tile_after;
+      ok = exchange<false>(sh, a, ++pass, last, tot);
+      if (last && blockIdx.x != 0) return;
+      const double cur = fmax(sumsq + tot.g, 0.0);
+      wide += tot.counts >> 32;
+      iters = t + 1;
+      if (tid == 0) {
+        sh.trace_alpha[iters] = static_cast<double>(alpha);
+        sh.trace_sse[iters] = cur;
+      }
+      const bool stop = stops_after(sse, cur, p.early_stop_rel);
+      sse = cur;
+      if (stop) break;
+    }
+    if (ok && tile_after) tile_scales(p, a.rows, a.tiled);
+  }
+  if (!ok) {
+    // a wait ran out: say so in the report and leave
+    if (tid == 0) {
+      if (gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange) = epoch + 1;
+      if (a.result != nullptr) {
+        a.result->status = SOAR_STATUS_INTERNAL;
+        a.result->iters_run = 0;
+      }
+    }
+    return;
+  }
+  if (blockIdx.x != 0) return;
+  if (tid == 0) {
+    if (gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange) = epoch + 1;
+    *a.alpha = alpha;
+    if (a.result != nullptr) {
+      soar_result* const res = a.result;
+      res->status = st;
+      res->iters_run = iters;
+      res->alpha = alpha;
+      res->amax = bits_to_mag(amax_bits);
+      res->sse = sse;
+      res->sse_init = st == 0 ? sh.trace_sse[0] : 0.0;
+      res->sumsq = (st & SOAR_STATUS_ZERO_TENSOR) ? 0.0 : sumsq;
+      res->zero_blocks = static_cast<int64_t>(zero_blocks);
+      res->wide_candidates = static_cast<int64_t>(wide);
+    }
+  }
+  if (a.result != nullptr) {
+    __syncthreads();
+    for (int i = tid; i <= SOAR_MAX_ITERS; i += static_cast<int>(blockDim.x)) {
+      a.result->trace_alpha[i] = i == 0 ? static_cast<double>(alpha0) : i <= iters ? sh.trace_alpha[i] : 0.0;
+      a.result->trace_sse[i] = (i <= iters && st == 0) ? sh.trace_sse[i] : 0.0;
+    }
+  }
+}
