@@ -198,29 +198,43 @@ def soar_quantize_launches(cfg: SoarCfg) -> int:
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream_ptr(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    if s.device.index != torch.cuda.current_device():
-        raise SoarError(f"stream belongs to cuda:{s.device.index} but the current device is "
+    if stream is None:
+        # the handle itself: building a torch.cuda.Stream around it takes longer than the launch
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if stream.device.index != torch.cuda.current_device():
+        raise SoarError(f"stream belongs to cuda:{stream.device.index} but the current device is "
                         f"cuda:{torch.cuda.current_device()}")
-    return C.c_void_p(s.cuda_stream)
+    return stream.cuda_stream
 
 
 def _require_cuda(*tensors):
     """Every tensor must live on the current CUDA device: the library launches there, on a stream of that
     device, and a pointer into another GPU's memory would reach kernels that cannot address it."""
-    cur = torch.cuda.current_device() if torch.cuda.is_available() else None
+    first = next((t for t in tensors if t is not None), None)
+    cur = None
+    if first is not None and first.get_device() >= 0:       # (-1: not a CUDA tensor)
+        cur = torch.cuda.current_device()
     for t in tensors:
-        if t is None:
+        if t is None or t.get_device() == cur:
             continue
         if not t.is_cuda:
             raise SoarError("device pointers required: tensor is not on a CUDA device")
-        if t.device.index != cur:
+        if t.device.index != torch.cuda.current_device():
             raise SoarError(f"tensor lives on cuda:{t.device.index} but the current device is cuda:{cur}: "
                             "make the tensor's device current (torch.cuda.device) before the call")
+
+
+def _matrix(W):
+    """Rows and columns of a bf16 CUDA matrix with unit column stride."""
+    if W.get_device() < 0:
+        _require_cuda(W)
+    if W.dtype is not torch.bfloat16 or W.dim() != 2 or W.stride(1) != 1:
+        raise SoarError("W must be a 2-D bf16 tensor with unit column stride")
+    return W.shape
 
 
 @dataclass
@@ -264,19 +278,17 @@ def alloc_buffers(rows: int, cols: int, cfg: SoarCfg, device="cuda", weighted: b
 def soar_quantize(W: torch.Tensor, cfg: SoarCfg, out: QuantBuffers | None = None, stream=None,
                   ld: int | None = None) -> QuantBuffers:
     """Enqueue ``soar_quantize`` for a bf16 CUDA matrix (2-D, unit column stride)."""
-    _require_cuda(W)
-    if W.dtype != torch.bfloat16 or W.dim() != 2 or W.stride(1) != 1:
-        raise SoarError("W must be a 2-D bf16 tensor with unit column stride")
-    rows, cols = W.shape
-    ld = W.stride(0) if ld is None else ld
+    rows, cols = _matrix(W)
     if out is None:
         out = alloc_buffers(rows, cols, cfg, W.device)
-    _require_cuda(out.packed, out.scales, out.scales_sw, out.alpha, out.result, out.workspace)
-    rc = lib().soar_quantize(
-        _ptr(W), rows, cols, ld, C.byref(cfg), _ptr(out.packed), _ptr(out.scales),
-        _ptr(out.scales_sw), _ptr(out.alpha), _ptr(out.workspace), out.workspace.numel(),
-        _ptr(out.result), _stream_ptr(stream))
-    _check(rc, "soar_quantize")
+    packed, scales, scales_sw, alpha, result, ws = (out.packed, out.scales, out.scales_sw, out.alpha, out.result,
+                                                    out.workspace)
+    _require_cuda(W, packed, scales, scales_sw, alpha, result, ws)
+    rc = (_lib or lib()).soar_quantize(
+        W.data_ptr(), rows, cols, W.stride(0) if ld is None else ld, C.byref(cfg), _ptr(packed), _ptr(scales),
+        _ptr(scales_sw), _ptr(alpha), _ptr(ws), ws.numel(), _ptr(result), _stream_ptr(stream))
+    if rc:
+        _check(rc, "soar_quantize")
     return out
 
 
@@ -284,9 +296,7 @@ def soar_quantize_weighted(W: torch.Tensor, col_weight: torch.Tensor, cfg: SoarC
                            out: QuantBuffers | None = None, stream=None) -> QuantBuffers:
     """Enqueue ``soar_quantize_weighted``: ``col_weight`` is a float32 CUDA vector of W.shape[1] entries."""
     _require_cuda(W, col_weight)
-    if W.dtype != torch.bfloat16 or W.dim() != 2 or W.stride(1) != 1:
-        raise SoarError("W must be a 2-D bf16 tensor with unit column stride")
-    rows, cols = W.shape
+    rows, cols = _matrix(W)
     if col_weight.dtype != torch.float32 or col_weight.shape != (cols,) or not col_weight.is_contiguous():
         raise SoarError("col_weight must be a contiguous float32 vector with one entry per column")
     if out is None:
@@ -303,12 +313,10 @@ def soar_quantize_weighted(W: torch.Tensor, col_weight: torch.Tensor, cfg: SoarC
 def _descs(Ws, outs):
     d = (SoarTensorDesc * len(Ws))()
     for i, (W, o) in enumerate(zip(Ws, outs)):
+        rows, cols = _matrix(W)
         _require_cuda(W, o.packed, o.scales, o.scales_sw, o.alpha, o.result)
-        if W.dtype != torch.bfloat16 or W.dim() != 2 or W.stride(1) != 1:
-            raise SoarError("W must be a 2-D bf16 tensor with unit column stride")
-        nul = lambda t: None if t is None else t.data_ptr()  # noqa: E731
-        d[i] = SoarTensorDesc(W.data_ptr(), W.shape[0], W.shape[1], W.stride(0), o.packed.data_ptr(),
-                              nul(o.scales), nul(o.scales_sw), o.alpha.data_ptr(), nul(o.result))
+        d[i] = SoarTensorDesc(W.data_ptr(), rows, cols, W.stride(0), o.packed.data_ptr(), _ptr(o.scales),
+                              _ptr(o.scales_sw), o.alpha.data_ptr(), _ptr(o.result))
     return d
 
 
@@ -388,10 +396,8 @@ def soar_quantize_static(W: torch.Tensor, cfg: SoarCfg, out: QuantBuffers, strea
     """Enqueue ``soar_quantize_static``: the quantizer for callers that cannot allocate device
     memory.  ``out`` supplies the output tensors only; its ``workspace`` is not passed on (the
     library uses its built-in scratch), and matrices above ``STATIC_MAX_ELEMENTS`` are refused."""
+    rows, cols = _matrix(W)
     _require_cuda(W, out.packed, out.scales, out.scales_sw, out.alpha, out.result)
-    if W.dtype != torch.bfloat16 or W.dim() != 2 or W.stride(1) != 1:
-        raise SoarError("W must be a 2-D bf16 tensor with unit column stride")
-    rows, cols = W.shape
     rc = lib().soar_quantize_static(
         _ptr(W), rows, cols, W.stride(0), C.byref(cfg), _ptr(out.packed), _ptr(out.scales),
         _ptr(out.scales_sw), _ptr(out.alpha), _ptr(out.result), _stream_ptr(stream))
@@ -414,15 +420,12 @@ class MxBuffers:
 def soar_mx_quantize(W: torch.Tensor, n_dq: int = 2, n_beta: int = 101, beta_step_pct: int = 1,
                      out: MxBuffers | None = None, stream=None) -> MxBuffers:
     """Enqueue ``soar_mx_quantize`` (MXFP4, blocks of 32; ``n_beta == 0``: the format's plain rule)."""
-    _require_cuda(W)
-    if W.dtype != torch.bfloat16 or W.dim() != 2 or W.stride(1) != 1:
-        raise SoarError("W must be a 2-D bf16 tensor with unit column stride")
-    rows, cols = W.shape
+    rows, cols = _matrix(W)
     if out is None:
         u8 = dict(dtype=torch.uint8, device=W.device)
         out = MxBuffers(torch.empty((rows, cols // 2), **u8), torch.empty((rows, max(cols // 32, 1)), **u8),
                         torch.empty(C.sizeof(SoarMxResult), **u8))
-    _require_cuda(out.packed, out.scales, out.result)
+    _require_cuda(W, out.packed, out.scales, out.result)
     rc = lib().soar_mx_quantize(_ptr(W), rows, cols, W.stride(0), n_dq, n_beta, beta_step_pct, _ptr(out.packed),
                                 _ptr(out.scales), _ptr(out.result), _stream_ptr(stream))
     _check(rc, "soar_mx_quantize")
@@ -439,7 +442,7 @@ def soar_dequant_error(W: torch.Tensor, packed: torch.Tensor, scales: torch.Tens
         out = torch.empty(2, dtype=torch.float64, device=W.device)
     rc = lib().soar_dequant_error(
         _ptr(W), rows, cols, W.stride(0), _ptr(packed), _ptr(scales), scale_layout, _ptr(alpha),
-        C.c_void_p(out.data_ptr()), C.c_void_p(out.data_ptr() + 8), _stream_ptr(stream))
+        out.data_ptr(), out.data_ptr() + 8, _stream_ptr(stream))
     _check(rc, "soar_dequant_error")
     return out
 
@@ -454,7 +457,7 @@ def soar_dequant_error_weighted(W: torch.Tensor, col_weight: torch.Tensor, packe
         out = torch.empty(2, dtype=torch.float64, device=W.device)
     rc = lib().soar_dequant_error_weighted(
         _ptr(W), rows, cols, W.stride(0), _ptr(col_weight), _ptr(packed), _ptr(scales), scale_layout,
-        _ptr(alpha), C.c_void_p(out.data_ptr()), C.c_void_p(out.data_ptr() + 8), _stream_ptr(stream))
+        _ptr(alpha), out.data_ptr(), out.data_ptr() + 8, _stream_ptr(stream))
     _check(rc, "soar_dequant_error_weighted")
     return out
 
