@@ -1288,11 +1288,9 @@ __device__ __forceinline__ void gather_sums(const Batch& bt, int s, double (*lat
 
 // Stages [stage_lo, stage_hi) of a call: amax, init, max_iters iterations, the report, the tiled scales.  A launch
 // over more than one stage is cooperative: its CTAs meet between stages.
-template <int kMode, bool kDet>
-__global__ void __launch_bounds__(kQThreads, 2)
-quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Reports rp, int stage_lo, int stage_hi) {
-  __shared__ QShared<kDet> sh;
-  __shared__ double s_latest[kDet ? kMaxBatch : 1][3];
+template <bool kDet, typename S, typename Passes>
+__device__ __forceinline__ void run_stages(S& sh, double (*s_latest)[3], const Batch& bt, const Reports& rp, int stage_lo,
+                                           int stage_hi, const Passes& passes) {
   const int tid = threadIdx.x;
   const int T = bt.t[0].max_iters, report = kQStageIterate + T, flags = bt.t[0].flags;
   if (tid < bt.n) {
@@ -1312,7 +1310,7 @@ quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Report
     sh.failed = 0;
     sh.run = (1u << bt.n) - 1u;
   }
-  if (kMode == 0 || kMode >= 3) {
+  if (Passes::kGrid) {
     const int n_beta = bt.t[0].n_beta, step = bt.t[0].beta_step_pct;
     for (int k = tid; k < n_beta; k += kQThreads) {
       const float lo = static_cast<float>((100.0 + static_cast<double>((k - n_beta / 2) * step)) / 100.0);
@@ -1340,7 +1338,8 @@ quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Report
         if (tid < bt.n) {
           const unsigned int amax_bits = __ldcg(&bt.t[tid].ws->amax_bits);
           sh.alpha[tid] = amax_bits == 0 ? 1.0f : __fdiv_rn(bits_to_mag(amax_bits), 2688.0f);
-          go = !(status_from_amax(amax_bits) & (SOAR_STATUS_NONFINITE | SOAR_STATUS_RANGE));
+          go = !(status_from_amax(amax_bits) & (SOAR_STATUS_NONFINITE | SOAR_STATUS_RANGE)) &&
+               __ldcg(&bt.t[tid].ws->error) == 0u;
         }
         const unsigned int run = __ballot_sync(0xFFFFFFFFu, go);
         if (tid == 0) sh.run = run;
@@ -1381,15 +1380,15 @@ quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Report
     }
     lay_out_pass(sh, bt);
     if (s == kQStageAmax) {
-      amax_pass(sh, bt);
+      passes.amax(sh, bt);
       file_sums(sh, bt, -1);
     } else if (s == kQStageInit) {
-      init_pass(sh, bt);
+      passes.init(sh, bt);
       file_sums(sh, bt, 0);
     } else {
       const int t = s - kQStageIterate;
       const bool last = t == T - 1;
-      iterate_pass<kMode>(sh, bt, (t & 1) != 0, bt.t[0].early_stop_rel > 0.0f || last, !last);
+      passes.iterate(sh, bt, (t & 1) != 0, bt.t[0].early_stop_rel > 0.0f || last, !last);
       file_sums(sh, bt, t + 1);
     }
     ++s;
@@ -1427,4 +1426,25 @@ quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Report
   if (any_tiled && stage_hi > report + 1)
     for (int ti = 0; ti < bt.n; ++ti)
       if (rp.scales_sw[ti] != nullptr) tile_scales(bt.t[ti], rp.rows[ti], rp.scales_sw[ti]);
+}
+
+template <int kMode>
+struct SearchPasses {
+  static constexpr bool kGrid = kMode == 0 || kMode >= 3;
+  template <typename S>
+  __device__ __forceinline__ void amax(S& sh, const Batch& bt) const { amax_pass(sh, bt); }
+  template <typename S>
+  __device__ __forceinline__ void init(S& sh, const Batch& bt) const { init_pass(sh, bt); }
+  template <typename S>
+  __device__ __forceinline__ void iterate(S& sh, const Batch& bt, bool reverse, bool emit, bool keep) const {
+    iterate_pass<kMode>(sh, bt, reverse, emit, keep);
+  }
+};
+
+template <int kMode, bool kDet>
+__global__ void __launch_bounds__(kQThreads, 2)
+quantize_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Reports rp, int stage_lo, int stage_hi) {
+  __shared__ QShared<kDet> sh;
+  __shared__ double s_latest[kDet ? kMaxBatch : 1][3];
+  run_stages<kDet>(sh, s_latest, bt, rp, stage_lo, stage_hi, SearchPasses<kMode>{});
 }

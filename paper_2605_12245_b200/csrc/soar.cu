@@ -137,22 +137,6 @@ struct Single {
 };
 static_assert(sizeof(Batch) <= 3072, "kernel parameter block too large");
 
-// What a consumer needs of its current tensor, copied out of the parameter block once per tensor.
-struct Tensor {
-  uint8_t* packed;
-  uint8_t* scales;
-  uint2* state;
-  unsigned int nblk;
-};
-__device__ __forceinline__ Tensor tensor_view(const Params& p) {
-  Tensor v;
-  v.packed = p.packed;
-  v.scales = p.scales;
-  v.state = p.state;
-  v.nblk = p.nblk;
-  return v;
-}
-
 // ------------------------------------------------------------------ number formats
 
 __device__ __forceinline__ float bits_to_mag(unsigned int bf16_bits) {
@@ -211,12 +195,6 @@ __device__ __forceinline__ float e2m1_code_value(unsigned int code3) {
 // patterns instead costs two register moves and a binary64 add on pipes that are busy
 // (38.5 against 39.4 ms per Llama-3-70B-shaped layer in the candidate loop).
 __device__ __forceinline__ double uint_to_double(unsigned int v) { return __uint2double_rn(v); }
-
-// The same from bit patterns (2^52 + v, minus 2^52), for the places that convert sixteen values
-// per block at once: there the conversion pipe would be the busy one.
-__device__ __forceinline__ double uint_to_double_bits(unsigned int v) {
-  return __hiloint2double(0x43300000, static_cast<int>(v)) - 4503599627370496.0;
-}
 
 // ------------------------------------------------------------------ shared-memory tile ring
 
@@ -624,17 +602,6 @@ __device__ __forceinline__ void sumsq_block(const unsigned int (&u)[8], double& 
   }
 }
 
-// Warp-level hand-over of two counters to a tensor's workspace.
-__device__ __forceinline__ void add_counters(Ws* ws, unsigned int& zeros, unsigned int& wide) {
-  zeros = __reduce_add_sync(0xFFFFFFFFu, zeros);
-  wide = __reduce_add_sync(0xFFFFFFFFu, wide);
-  if ((threadIdx.x & 31) == 0) {
-    if (zeros) atomicAdd(&ws->zero_blocks, static_cast<unsigned long long>(zeros));
-    if (wide) atomicAdd(&ws->wide, static_cast<unsigned long long>(wide));
-  }
-  zeros = wide = 0;
-}
-
 // Error of stage s (Eq. 4) from the tensor sums.
 __device__ __forceinline__ double stage_sse(const Ws* ws, int s) {
   return fmax(ws->sumsq + ws->gsum[s], 0.0);
@@ -737,13 +704,6 @@ __device__ __forceinline__ void winning_range(const B* s_beta, int n_beta, float
   kb = min(kb, n_beta - 1);
 }
 
-// A block's winner of Eq. 8: error minus sum W^2, its sums, codes (signs included) and E4M3 code.
-struct Winner {
-  double g, A, B;
-  unsigned int c0, c1;
-  int d;
-};
-
 // Offset of scale (row, col) in the 128x4-tiled layout: tiles of 128 rows x 4 scale columns
 // (512 bytes), tile rows outermost; inside a tile row r and column c sit at
 // (r % 32) * 16 + (r / 32) * 4 + c.
@@ -755,6 +715,7 @@ __device__ __forceinline__ size_t swizzled_offset(unsigned int row, unsigned int
 
 #include "quantize_kernel.cuh"
 #include "solo_kernel.cuh"
+#include "weighted_kernel.cuh"
 
 // Eq. 3-4 on stored outputs: sum (w - q s)^2 and sum w^2, one binary64 fma per term, with the
 // bf16 values widened by the conversion instruction (which runs beside the integer and
@@ -829,460 +790,6 @@ __global__ void __launch_bounds__(kThreads) dequant_error_kernel(const __grid_co
   if (failed) acc[0] = acc[1] = __longlong_as_double(0x7FF8000000000000ll);
   double* const dst[2] = {out_sse, out_sumsq};
   slots_add(slots, 0, acc, dst);
-}
-
-// ------------------------------------------------------------------ column-weighted objective
-//
-// Sec. 5 proposes to minimise the output distortion ||(W - What) X||^2 in CJSO and DSS; its
-// diagonal form is sum_ij h_j (W_ij - What_ij)^2 with h_j the second moment of input channel j.
-// Algorithm 1 is unchanged except that the block sums carry the weights,
-//   A = sum h_j |w_j| m_j,   B = sum h_j m_j^2,
-// in Eq. 5, Eq. 6 and the error of Eq. 8.  The weights are arbitrary binary32 numbers, so the
-// integer dot products of the unweighted kernels do not apply: the sums are binary64, taken in
-// element order (each product is exact: 24 + 8 + 2 and 24 + 4 significant bits), and the state
-// kept between iterations is {A, B} in binary64 plus the scale code.
-
-struct Weighted {
-  const float* h;    // cols weights
-  double2* sums;     // per block {A, B} of the current codes; null when T == 0
-  uint8_t* code;     // per block stored scale code (0: all-zero block); null when T == 0
-};
-// One launch works on up to kMaxBatch matrices (see Batch): entry i belongs to bt.t[i].
-struct WeightedBatch {
-  Weighted t[kMaxBatch];
-};
-
-// A and B of a code vector (sign bits ignored) for hw[j] = h_j |w_j| and hd[j] = h_j.
-__device__ __forceinline__ void weighted_sums(const double (&hw)[16], const double (&hd)[16], unsigned int c0,
-                                              unsigned int c1, double& A, double& B) {
-  const unsigned int m0 = c0 & 0x77777777u, m1 = c1 & 0x77777777u;
-  const unsigned int t[4] = {twice_magnitude_x4(m0), twice_magnitude_x4(m0 >> 16), twice_magnitude_x4(m1),
-                             twice_magnitude_x4(m1 >> 16)};
-  double a = 0.0, b = 0.0;
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const double dm = uint_to_double_bits((t[j >> 2] >> (8 * (j & 3))) & 0xFFu);   // 2 m_j
-    a = fma(hw[j], dm, a);
-    b = fma(hd[j], dm * dm, b);
-  }
-  // halving every term halves every partial sum exactly
-  A = 0.5 * a;
-  B = 0.25 * b;
-}
-
-// The same sums for ranking candidates: two interleaved partial chains per sum instead of one
-// sixteen-long chain of dependent additions.  The result may differ from weighted_sums in the
-// last bit, which only a tie between candidates could feel.
-__device__ __forceinline__ void weighted_sums_split(const double (&hw)[16], const double (&hd)[16], unsigned int c0,
-                                                    unsigned int c1, double& A, double& B) {
-  const unsigned int t[4] = {twice_magnitude_x4(c0), twice_magnitude_x4(c0 >> 16), twice_magnitude_x4(c1),
-                             twice_magnitude_x4(c1 >> 16)};
-  double a[2] = {0.0, 0.0}, b[2] = {0.0, 0.0};
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const double dm = uint_to_double_bits((t[j >> 2] >> (8 * (j & 3))) & 0xFFu);
-    a[j & 1] = fma(hw[j], dm, a[j & 1]);
-    b[j & 1] = fma(hd[j], dm * dm, b[j & 1]);
-  }
-  A = 0.5 * (a[0] + a[1]);
-  B = 0.25 * (b[0] + b[1]);
-}
-
-// A and B of a code vector (sign bits ignored) from the block's sixteen column weights and signed
-// elements, in element order like weighted_sums and with the same roundings, but widening each
-// weight and magnitude where it is used, so that only a few binary64 values are live at a time.
-__device__ __forceinline__ void weighted_sums_streamed(const float (&h)[16], const float (&w)[16], unsigned int c0,
-                                                       unsigned int c1, double& A, double& B) {
-  const unsigned int m0 = c0 & 0x77777777u, m1 = c1 & 0x77777777u;
-  const unsigned int t[4] = {twice_magnitude_x4(m0), twice_magnitude_x4(m0 >> 16), twice_magnitude_x4(m1),
-                             twice_magnitude_x4(m1 >> 16)};
-  double a = 0.0, b = 0.0;
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const double dm = uint_to_double_bits((t[j >> 2] >> (8 * (j & 3))) & 0xFFu);   // 2 m_j
-    const double hd = static_cast<double>(h[j]);
-    a = fma(hd * static_cast<double>(fabsf(w[j])), dm, a);
-    b = fma(hd, dm * dm, b);
-  }
-  A = 0.5 * a;
-  B = 0.25 * b;
-}
-
-// hd[j] = h_j and hw[j] = h_j |w_j| of a block, binary64 (both exact).
-__device__ __forceinline__ void block_weights(const float* h, unsigned int cb, const Block& mags, double (&hd)[16],
-                                              double (&hw)[16]) {
-  load_weights(h, cb, hd);
-#pragma unroll
-  for (int j = 0; j < 16; ++j) hw[j] = hd[j] * static_cast<double>(mags.w[j]);
-}
-
-__device__ __forceinline__ bool weight_ok(float h) {
-  return h == 0.0f || (h >= 0x1p-20f && h <= 0x1p20f);
-}
-
-// Eq. 1's tensor maximum, sum h_j W^2 for the error report, and the check of the weights.
-__global__ void __launch_bounds__(kThreads, 2)
-weighted_amax_kernel(const __grid_constant__ Batch bt, const __grid_constant__ WeightedBatch wb) {
-  __shared__ Ring ring;
-  __shared__ Slots<1> slots;
-  slots_clear(slots);
-  ring_init(ring);
-  if (is_producer_warp()) {
-    if (threadIdx.x == kTile) ring_produce(ring, bt, 0, 0xFFFFFFFFu);
-    return;
-  }
-  unsigned int mx = 0, nblk = 0, nbc = 1;
-  const float* h = nullptr;
-  bool bad = false;
-  double sq[1] = {0.0};
-  int cur = -1;
-  for (unsigned int n = 0;; ++n) {
-    uint4 v0, v1;
-    int ti = -1;
-    unsigned int tile = 0;
-    const int rc = ring_consume(ring, bt, n, v0, v1, ti, tile);
-    if (rc != 0 || ti != cur) {
-      if (cur >= 0) {   // leaving tensor `cur`: hand over its maximum, its sum and the outcome of the weight check
-        mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-        const bool any_bad = __any_sync(0xFFFFFFFFu, bad);
-        if ((threadIdx.x & 31) == 0) {
-          if (mx) atomicMax(&bt.t[cur].ws->amax_bits, mx);
-          if (any_bad) atomicOr(&bt.t[cur].ws->error, kErrWeight);
-        }
-        double* const dst[1] = {&bt.t[cur].ws->sumsq};
-        slots_add(slots, cur, sq, dst);
-        mx = 0;
-        bad = false;
-      }
-      if (rc != 0) break;
-      cur = ti;
-      nblk = bt.t[ti].nblk;
-      nbc = bt.t[ti].nbc;
-      h = wb.t[ti].h;
-    }
-    const unsigned int b = tile * kTile + threadIdx.x;
-    if (b >= nblk) continue;
-    const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    double hd[16];
-    load_weights(h, b % nbc, hd);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      // magnitude bit patterns order like the magnitudes; NaN patterns lie above infinity's
-      mx = max(mx, max(u[i] & 0x7FFFu, (u[i] >> 16) & 0x7FFFu));
-      const double wl = static_cast<double>(__uint_as_float(u[i] << 16));
-      const double wh = static_cast<double>(__uint_as_float(u[i] & 0xFFFF0000u));
-      sq[0] = fma(hd[2 * i], wl * wl, sq[0]);
-      sq[0] = fma(hd[2 * i + 1], wh * wh, sq[0]);
-      bad = bad || !weight_ok(static_cast<float>(hd[2 * i])) || !weight_ok(static_cast<float>(hd[2 * i + 1]));
-    }
-  }
-}
-
-// Algorithm 1 "Initialization" (Eq. 1; the weights play no part in it), the first codes, and
-// the weighted stage-0 sums of Eq. 5 and of the starting error.
-__global__ void __launch_bounds__(kThreads, 2)
-weighted_init_kernel(const __grid_constant__ Batch bt, const __grid_constant__ WeightedBatch wb, int reverse,
-                     int final) {
-  __shared__ Ring ring;
-  __shared__ Slots<3> slots;
-  slots_clear(slots);
-  ring_init(ring);
-  if (is_producer_warp()) {
-    if (threadIdx.x == kTile) {
-      unsigned int run = 0;
-      for (int i = 0; i < bt.n; ++i)
-        if (!(status_from_amax(bt.t[i].ws->amax_bits) & (SOAR_STATUS_NONFINITE | SOAR_STATUS_RANGE)) &&
-            bt.t[i].ws->error == 0)
-          run |= 1u << i;
-      ring_produce(ring, bt, reverse, run);
-    }
-    return;
-  }
-  float alpha = 1.0f, six_alpha = 6.0f;
-  double alpha_d = 1.0;
-  double acc[3] = {0.0, 0.0, 0.0};   // num, den, gsum
-  unsigned int zeros = 0, unused_wide = 0;
-  int cur = -1;
-  Tensor p = {};
-  Weighted wq = {};
-  unsigned int nbc = 1;
-  for (unsigned int n = 0;; ++n) {
-    uint4 v0, v1;
-    int ti = -1;
-    unsigned int tile = 0;
-    const int rc = ring_consume(ring, bt, n, v0, v1, ti, tile);
-    if (rc != 0 || ti != cur) {
-      if (cur >= 0) {
-        Ws* ws = bt.t[cur].ws;
-        double* const dst[3] = {&ws->num[0], &ws->den[0], &ws->gsum[0]};
-        slots_add(slots, cur, acc, dst);
-        add_counters(ws, zeros, unused_wide);
-      }
-      if (rc != 0) break;
-      cur = ti;
-      const unsigned int amax_bits = bt.t[ti].ws->amax_bits;
-      alpha = amax_bits == 0 ? 1.0f : __fdiv_rn(bits_to_mag(amax_bits), 2688.0f);
-      six_alpha = __fmul_rn(alpha, 6.0f);
-      alpha_d = static_cast<double>(alpha);
-      p = tensor_view(bt.t[ti]);
-      nbc = bt.t[ti].nbc;
-      wq = wb.t[ti];
-    }
-    const unsigned int b = tile * kTile + threadIdx.x;
-    if (b >= p.nblk) continue;
-    Block blk;
-    unpack_block(v0, v1, blk);
-    uint2 codes;
-    if (blk.bmax == 0.0f) {
-      round_block(blk, 1.0f, codes.x, codes.y);
-      reinterpret_cast<uint2*>(p.packed)[b] = codes;
-      p.scales[b] = 0;
-      if (wq.code != nullptr) wq.code[b] = 0;
-      ++zeros;
-      continue;
-    }
-    int c = e4m3_encode(__fdiv_rn(blk.bmax, six_alpha));
-    c = max(c, 1);
-    const float v = e4m3_value(c);
-    round_block(blk, recip_scale(alpha, v), codes.x, codes.y);
-    double hd[16], hw[16];
-    load_weights(wq.h, b % nbc, hd);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) hw[j] = hd[j] * static_cast<double>(fabsf(blk.w[j]));
-    double A, B;
-    weighted_sums(hw, hd, codes.x, codes.y, A, B);
-    if (final) {
-      reinterpret_cast<uint2*>(p.packed)[b] = codes;
-      p.scales[b] = static_cast<uint8_t>(c);
-    }
-    if (wq.sums != nullptr) {
-      wq.sums[b] = make_double2(A, B);
-      wq.code[b] = static_cast<uint8_t>(c);
-    }
-    const double vd = static_cast<double>(v);
-    const double sd = alpha_d * vd;
-    acc[0] = fma(A, vd, acc[0]);
-    acc[1] = fma(B * vd, vd, acc[1]);
-    acc[2] += sd * fma(sd, B, -2.0 * A);
-  }
-}
-
-// Eq. 8 for one block over the whole grid with binary64 sums for every candidate, first minimum in
-// (beta, code) order; the winner is then made again with its signs and its sums in element order.
-// Serves the coupled arm and the blocks whose candidates can cost exactly the same (see
-// weighted_iterate_kernel).  Out of line and fed from memory (sixteen bf16 values at w16, the weights
-// at h), so that nothing of it weighs on the registers of the common path.
-__device__ __noinline__ void weighted_whole_grid_search(const float* h, unsigned int cb, const uint16_t* w16,
-                                                        float alpha, float center, const float* s_beta, int n_beta,
-                                                        int d_lo, int nd, bool coupled, bool fast_rcp, Winner* out) {
-  Block blk, mags;
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(w16);
-    unpack_block(__ldg(src), __ldg(src + 1), blk);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) mags.w[j] = fabsf(blk.w[j]);
-  }
-  const double alpha_d = static_cast<double>(alpha);
-  double best = __longlong_as_double(0x7FF0000000000000ll);
-  int best_key = 0;
-  {
-    double hd[16], hw[16];
-    block_weights(h, cb, mags, hd, hw);
-    for (int k = 0; k < n_beta; ++k) {
-      unsigned int c0, c1;
-      double A = 0.0, B = 0.0;
-      if (!coupled) {
-        const float s = __fmul_rn(alpha, __fmul_rn(center, s_beta[k]));
-        round_block(mags, fast_rcp ? recip_fast(s) : __frcp_rn(s), c0, c1);
-        weighted_sums_split(hw, hd, c0, c1, A, B);
-      }
-      for (int d = 0; d < nd; ++d) {
-        const float dv = e4m3_value(clip_code(d_lo + d));
-        if (coupled) {
-          round_block(mags, recip_scale(alpha, __fmul_rn(dv, s_beta[k])), c0, c1);
-          weighted_sums_split(hw, hd, c0, c1, A, B);
-        }
-        const double sd = alpha_d * static_cast<double>(dv);
-        const double g = sd * fma(sd, B, -2.0 * A);
-        if (g < best) { best = g; best_key = nd * k + d; }
-      }
-    }
-  }
-  Winner w;
-  const int bk = best_key / nd;
-  w.d = clip_code(d_lo + (best_key - bk * nd));
-  round_block(blk, recip_scale(alpha, __fmul_rn(coupled ? e4m3_value(w.d) : center, s_beta[bk])), w.c0, w.c1);
-  float hf[16];
-  {
-    const float4* src = reinterpret_cast<const float4*>(h) + static_cast<size_t>(cb) * 4;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float4 v = __ldg(src + q);
-      hf[4 * q] = v.x; hf[4 * q + 1] = v.y; hf[4 * q + 2] = v.z; hf[4 * q + 3] = v.w;
-    }
-  }
-  weighted_sums_streamed(hf, blk.w, w.c0, w.c1, w.A, w.B);
-  w.g = best;
-  *out = w;
-}
-
-// One iteration t of Algorithm 1 under the weighted objective: Eq. 5 from the stage-t sums,
-// Eq. 6 per block from its stored {A, B}, App. B.3's candidates, Eq. 8 with the weighted
-// error written as  sum h w^2 + sd^2 B - 2 sd A  (sd = alpha * candidate scale value), first
-// minimum in (beta, code) order.  All of cfg's shapes and arms run through this one kernel, on up
-// to kMaxBatch matrices per launch like the unweighted kernels.
-__global__ void __launch_bounds__(kThreads, 2)
-weighted_iterate_kernel(const __grid_constant__ Batch bt, const __grid_constant__ WeightedBatch wb, int t,
-                        int reverse, int emit, int keep) {
-  __shared__ Ring ring;
-  __shared__ Slots<3> slots;
-  __shared__ float s_beta[SOAR_MAX_BETA];
-  __shared__ float s_alpha[kMaxBatch];
-  __shared__ unsigned int s_run;
-  if (threadIdx.x == 0) s_run = 0;
-  __syncthreads();
-  if (threadIdx.x < bt.n) {   // per tensor: still running?  its alpha for this iteration
-    float a;
-    int run;
-    iteration_head(bt.t[threadIdx.x], t, a, run);
-    s_alpha[threadIdx.x] = a;
-    if (run) atomicOr(&s_run, 1u << threadIdx.x);
-  }
-  const Params& p0 = bt.t[0];
-  const int n_dq = p0.n_dq, n_beta = p0.n_beta;
-  for (int k = threadIdx.x; k < n_beta; k += kThreads)
-    s_beta[k] = static_cast<float>((100.0 + static_cast<double>((k - n_beta / 2) * p0.beta_step_pct)) / 100.0);
-  slots_clear(slots);
-  __syncthreads();
-  if (s_run == 0) return;   // every tensor of the batch has stopped (Sec. 4.1), or was rejected
-  ring_init(ring);
-  if (is_producer_warp()) {
-    if (threadIdx.x == kTile) ring_produce(ring, bt, reverse, s_run);
-    return;
-  }
-  float alpha = 1.0f;
-  double alpha_d = 1.0;
-  const bool coupled = (p0.flags & SOAR_FLAG_COUPLED_SCALE) != 0;
-  const bool keep_scale = (p0.flags & SOAR_FLAG_KEEP_BLOCK_SCALE) != 0;
-  // multiplier index of a scale ratio: k = (ratio - 1) * 100 / step + n_beta / 2
-  const bool bracketed = p0.beta_step_pct >= 1 && n_beta >= 2;
-  const float k_scale = 100.0f / static_cast<float>(max(p0.beta_step_pct, 1));
-  const float k_off = static_cast<float>(n_beta / 2) - k_scale;
-  double acc[3] = {0.0, 0.0, 0.0};   // num, den, gsum of stage t+1
-  unsigned int exact_blocks = 0, unused_zeros = 0;
-  int cur = -1;
-  for (unsigned int n = 0;; ++n) {
-    uint4 v0, v1;
-    int ti = -1;
-    unsigned int tile = 0;
-    const int rc = ring_consume(ring, bt, n, v0, v1, ti, tile);
-    if (rc != 0 || ti != cur) {
-      if (cur >= 0) {
-        Ws* ws = bt.t[cur].ws;
-        double* const dst[3] = {&ws->num[t + 1], &ws->den[t + 1], &ws->gsum[t + 1]};
-        slots_add(slots, cur, acc, dst);
-        add_counters(ws, unused_zeros, exact_blocks);   // reported as soar_result.wide_candidates
-      }
-      if (rc != 0) break;
-      cur = ti;
-      alpha = s_alpha[ti];
-      alpha_d = static_cast<double>(alpha);
-    }
-    // pointers and sizes of the current tensor are re-read from the parameter block per tile rather than
-    // carried in registers across the scoring of the block
-    const Params& p = bt.t[ti];
-    const Weighted& wq = wb.t[ti];
-    const unsigned int b = tile * kTile + threadIdx.x;
-    if (b >= p.nblk) continue;
-    const int d_cur = wq.code[b];
-    if (d_cur == 0) continue;   // all-zero block
-    const double2 ab = wq.sums[b];
-    Block blk;
-    unpack_block(v0, v1, blk);
-    const unsigned int row = b / p.nbc, cb = b - row * p.nbc;
-    // Eq. 6 (binary32 steps); a block whose weighted codes are all zero keeps its stored scale
-    const float center = (ab.y > 0.0 && !keep_scale)
-                             ? __fdiv_rn(static_cast<float>(ab.x), __fmul_rn(alpha, static_cast<float>(ab.y)))
-                             : e4m3_value(d_cur);
-    int d_lo, d_hi;
-    candidate_window(center, n_dq, d_lo, d_hi);
-    const int nd = d_hi - d_lo + 1;
-    // the products alpha * center * beta are monotone in beta: the end points bound them all
-    const bool fast_rcp = !coupled && recip_fast_ok(__fmul_rn(alpha, __fmul_rn(center, s_beta[0]))) &&
-                          recip_fast_ok(__fmul_rn(alpha, __fmul_rn(center, s_beta[n_beta - 1])));
-    float hf[16];
-    {
-      const float4* src = reinterpret_cast<const float4*>(wq.h) + static_cast<size_t>(cb) * 4;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float4 v = __ldg(src + q);
-        hf[4 * q] = v.x; hf[4 * q + 1] = v.y; hf[4 * q + 2] = v.z; hf[4 * q + 3] = v.w;
-      }
-    }
-    // The weighted error of element j, h_j (a_j - m sd)^2, is convex in m like the unweighted one, so per
-    // E4M3 code only the multipliers of winning_range can win (see there).  When a column's weight is zero,
-    // its code costs nothing whatever it is, and equal errors of different codes occur all along the grid:
-    // such blocks, and the coupled arm, walk the whole grid.
-    bool zero_weight = false;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) zero_weight = zero_weight || hf[j] == 0.0f;
-    unsigned int best0 = 0, best1 = 0;
-    double bestA = 0.0, bestB = 0.0;
-    int best_d = clip_code(d_lo);
-    if (!coupled && bracketed && !zero_weight) {
-      double best = __longlong_as_double(0x7FF0000000000000ll);
-      int best_k = 0, prev = -1;
-      const float per_center = __fdividef(k_scale, center);
-      for (int d = d_lo; d <= d_hi; ++d) {
-        const int dc = clip_code(d);
-        if (dc == prev) continue;   // clipping at the ends of the E4M3 range repeats a code
-        prev = dc;
-        const float dv = e4m3_value(dc);
-        const double sd = alpha_d * static_cast<double>(dv);
-        float lo, hi;
-        divisor_band(alpha, dv, lo, hi);
-        int ka = max(0, min(n_beta - 2, __float2int_rd(__fmaf_rn(dv, per_center, k_off))));
-        int kb = ka + 1;
-        if (!(grid_divisor(alpha, center, s_beta[ka]) <= lo && grid_divisor(alpha, center, s_beta[kb]) >= hi))
-          winning_range(s_beta, n_beta, alpha, center, lo, hi, ka, ka, kb);
-        for (int k = ka; k <= kb; ++k) {
-          const float sk = grid_divisor(alpha, center, s_beta[k]);
-          unsigned int c0, c1;
-          round_block(blk, fast_rcp ? recip_fast(sk) : __frcp_rn(sk), c0, c1);
-          double A, B;
-          weighted_sums_streamed(hf, blk.w, c0, c1, A, B);
-          const double g = sd * fma(sd, B, -2.0 * A);
-          // equal errors: the earlier multiplier, then the smaller code, as in grid order
-          if (g < best || (g == best && k < best_k)) {
-            best = g; bestA = A; bestB = B; best0 = c0; best1 = c1; best_d = dc; best_k = k;
-          }
-        }
-      }
-    } else {
-      Winner w;
-      weighted_whole_grid_search(wq.h, cb, p.W + static_cast<long long>(row) * p.ld + static_cast<long long>(cb) * 16,
-                                 alpha, center, s_beta, n_beta, d_lo, nd, coupled, fast_rcp, &w);
-      ++exact_blocks;
-      best0 = w.c0;
-      best1 = w.c1;
-      bestA = w.A;
-      bestB = w.B;
-      best_d = w.d;
-    }
-    if (emit) {
-      reinterpret_cast<uint2*>(p.packed)[b] = make_uint2(best0, best1);
-      p.scales[b] = static_cast<uint8_t>(best_d);
-    }
-    if (keep) {
-      wq.sums[b] = make_double2(bestA, bestB);
-      wq.code[b] = static_cast<uint8_t>(best_d);
-    }
-    const double vd = static_cast<double>(e4m3_value(best_d));
-    const double sd = alpha_d * vd;
-    acc[0] = fma(bestA, vd, acc[0]);
-    acc[1] = fma(bestB * vd, vd, acc[1]);
-    acc[2] += sd * fma(sd, bestB, -2.0 * bestA);
-  }
 }
 
 // ------------------------------------------------------------------ MXFP4 (Sec. 4.3, "DSS on MXFP4")
@@ -1670,29 +1177,30 @@ void set_division(Params& p) {
   p.nbc_magic = static_cast<unsigned int>(((1ull << (31 + l)) + p.nbc - 1) / p.nbc);
 }
 
-// CTAs of quantize_kernel<mode, det> an SM holds, asked of the runtime once per device.
-template <int kMode, bool kDet>
-int quantize_per_sm() {
-  static std::atomic<int> known[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
-  int n = known[dev].load(std::memory_order_relaxed);
-  if (n == 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, quantize_kernel<kMode, kDet>, kQThreads, 0) != cudaSuccess || n <= 0)
-      n = 1;
-    known[dev].store(n, std::memory_order_relaxed);
+// Grid of a stage machine's launch: every SM filled to the kernel's occupancy (asked of the runtime once per device),
+// never more CTAs than eight tiles each give work.
+template <typename K>
+unsigned int stage_grid(K kernel, std::atomic<int> (&known)[64], unsigned int tiles) {
+  int dev = 0, n = 1;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
+    n = known[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kQThreads, 0) != cudaSuccess || n <= 0) n = 1;
+      known[dev].store(n, std::memory_order_relaxed);
+    }
   }
-  return n;
+  unsigned int grid = static_cast<unsigned int>(sm_count() * n);
+  if (grid > static_cast<unsigned int>(kMaxGrid)) grid = kMaxGrid;   // the deterministic mode keeps one slot per CTA
+  const unsigned int want = (tiles + kQWarps - 1) / kQWarps;
+  return want < grid ? (want > 0 ? want : 1u) : grid;
 }
 
 // Launches stages [lo, hi) of the quantizer for one group of matrices; more than one stage makes the launch
 // cooperative, so that its CTAs, which meet between stages, run at the same time.
 template <int kMode, bool kDet>
 cudaError_t launch_stages(const Batch& bt, const Reports& rp, unsigned int tiles, int lo, int hi, cudaStream_t st) {
-  unsigned int grid = static_cast<unsigned int>(sm_count() * quantize_per_sm<kMode, kDet>());
-  if (grid > static_cast<unsigned int>(kMaxGrid)) grid = kMaxGrid;   // the deterministic mode keeps one slot per CTA
-  const unsigned int want = (tiles + kQWarps - 1) / kQWarps;
-  if (want < grid) grid = want > 0 ? want : 1u;
+  static std::atomic<int> known[64];
+  const unsigned int grid = stage_grid(quantize_kernel<kMode, kDet>, known, tiles);
   if (hi - lo == 1) {
     quantize_kernel<kMode, kDet><<<grid, kQThreads, 0, st>>>(bt, rp, lo, hi);
     return cudaGetLastError();
@@ -1714,6 +1222,25 @@ cudaError_t launch_stages(int mode, bool det, const Batch& bt, const Reports& rp
     default: return SOAR_STAGES(5);
   }
 #undef SOAR_STAGES
+}
+
+// The same for the weighted kernel.
+template <bool kFast>
+cudaError_t launch_weighted(const Batch& bt, const Weighted& wt, const Reports& rp, unsigned int tiles, int lo, int hi,
+                            cudaStream_t st) {
+  static std::atomic<int> known[64];
+  const unsigned int grid = stage_grid(weighted_kernel<kFast>, known, tiles);
+  if (hi - lo == 1) {
+    weighted_kernel<kFast><<<grid, kQThreads, 0, st>>>(bt, wt, rp, lo, hi);
+    return cudaGetLastError();
+  }
+  void* args[] = {const_cast<Batch*>(&bt), const_cast<Weighted*>(&wt), const_cast<Reports*>(&rp), &lo, &hi};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&weighted_kernel<kFast>), dim3(grid), dim3(kQThreads), args, 0,
+                                     st);
+}
+cudaError_t launch_weighted(bool fast, const Batch& bt, const Weighted& wt, const Reports& rp, unsigned int tiles, int lo, int hi,
+                            cudaStream_t st) {
+  return fast ? launch_weighted<true>(bt, wt, rp, tiles, lo, hi, st) : launch_weighted<false>(bt, wt, rp, tiles, lo, hi, st);
 }
 
 // kMode of quantize_kernel for a call's settings (see iterate_pass).
@@ -2139,13 +1666,13 @@ int soar_quantize_weighted_batch(const soar_tensor_desc* tensors, const float* c
   uint8_t* const headers = static_cast<uint8_t*>(workspace);
   uint8_t* next = headers + static_cast<size_t>(n) * kWsFixedBytes;
   if (cudaMemsetAsync(headers, 0, static_cast<size_t>(n) * kWsFixedBytes, st) != cudaSuccess) return SOAR_ERR_CUDA;
-  const bool may_stop = cfg->early_stop_rel > 0.0f;
+  const bool fast = search_mode(cfg) == 4;
   for (int first = 0; first < n; first += kMaxBatch) {
     Batch bt;
-    WeightedBatch wb;
+    Weighted wt;
     Reports rp;
     memset(&bt, 0, sizeof(bt));
-    memset(&wb, 0, sizeof(wb));
+    memset(&wt, 0, sizeof(wt));
     memset(&rp, 0, sizeof(rp));
     bt.n = (n - first < kMaxBatch) ? n - first : kMaxBatch;
     bt.idle_producer = g_idle_producer;
@@ -2153,21 +1680,19 @@ int soar_quantize_weighted_batch(const soar_tensor_desc* tensors, const float* c
     for (int j = 0; j < bt.n; ++j) {
       const soar_tensor_desc& d = tensors[first + j];
       Params& p = bt.t[j];
-      Weighted& wq = wb.t[j];
       p.W = static_cast<const uint16_t*>(d.W_bf16);
       p.packed = static_cast<uint8_t*>(d.out_fp4_packed);
       p.ws = reinterpret_cast<Ws*>(headers + static_cast<size_t>(first + j) * kWsFixedBytes);
       p.ld = d.ld;
       p.nbc = static_cast<unsigned int>(d.cols / 16);
       p.nblk = static_cast<unsigned int>(d.rows * (d.cols / 16));
-      p.ntiles = (p.nblk + kTile - 1) / kTile;
+      p.ntiles = (p.nblk + 31) / 32;
+      set_division(p);
       p.contiguous = (d.ld == d.cols) ? 1 : 0;
-      wq.h = col_weights[first + j];
+      wt.h[j] = col_weights[first + j];
       if (cfg->max_iters > 0) {
-        wq.sums = reinterpret_cast<double2*>(next);
-        next += round256(static_cast<size_t>(p.nblk) * sizeof(double2));
-        wq.code = next;
-        next += round256(p.nblk);
+        p.state = reinterpret_cast<uint2*>(next);
+        next += round256(static_cast<size_t>(p.nblk) * sizeof(double2)) + round256(p.nblk);
       }
       if (want_lin) {
         p.scales = static_cast<uint8_t*>(d.out_e4m3_scales);
@@ -2182,44 +1707,25 @@ int soar_quantize_weighted_batch(const soar_tensor_desc* tensors, const float* c
       p.beta_step_pct = cfg->beta_step_pct;
       p.flags = cfg->flags;
       tiles += p.ntiles;
-      bt.tile_end[j] = tiles;
       rp.alpha[j] = d.out_global_fp32;
       rp.result[j] = d.out_result;
       rp.scales_sw[j] = want_sw ? static_cast<uint8_t*>(d.out_e4m3_scales_sw) : nullptr;
       rp.rows[j] = static_cast<unsigned int>(d.rows);
     }
-    for (int j = bt.n; j < kMaxBatch; ++j) bt.tile_end[j] = 0xFFFFFFFFu;   // never reached by a tile index
-    bt.total_tiles = tiles;
-
-    int reverse = 1;   // the first pass runs forward; each later one starts where the last ended
-    {
-      ScopedLaunch sl(K_WEIGHTED_AMAX, st);
-      weighted_amax_kernel<<<persistent_grid(weighted_amax_kernel, tiles, kThreads), kThreads, 0, st>>>(bt, wb);
+    const int report = kQStageIterate + cfg->max_iters, end = report + 1 + (want_sw ? 1 : 0);
+    cudaError_t err = cudaSuccess;
+    if (!g_trace.on) {
+      err = launch_weighted(fast, bt, wt, rp, tiles, 0, end, st);
+    } else {   // stage by stage, each of them timed
+      for (int s = 0; s < end && err == cudaSuccess; ++s) {
+        ScopedLaunch sl(s == kQStageAmax ? K_WEIGHTED_AMAX : s == kQStageInit ? K_WEIGHTED_INIT
+                        : s < report ? K_WEIGHTED_ITERATE : s == report ? K_FINALIZE : K_SWIZZLE, st);
+        err = launch_weighted(fast, bt, wt, rp, tiles, s, s + 1, st);
+      }
     }
-    {
-      ScopedLaunch sl(K_WEIGHTED_INIT, st);
-      weighted_init_kernel<<<persistent_grid(weighted_init_kernel, tiles, kThreads), kThreads, 0, st>>>(
-          bt, wb, reverse, cfg->max_iters == 0 ? 1 : 0);
-    }
-    const unsigned int g_it = persistent_grid(weighted_iterate_kernel, tiles, kThreads);
-    for (int t = 0; t < cfg->max_iters; ++t) {
-      reverse ^= 1;
-      const int last = (t == cfg->max_iters - 1) ? 1 : 0;
-      ScopedLaunch sl(K_WEIGHTED_ITERATE, st);
-      weighted_iterate_kernel<<<g_it, kThreads, 0, st>>>(bt, wb, t, reverse, (may_stop || last) ? 1 : 0, !last);
-    }
-    const int report = kQStageIterate + cfg->max_iters;
-    {
-      ScopedLaunch sl(K_FINALIZE, st);
-      if (launch_stages(1, false, bt, rp, static_cast<unsigned int>(bt.n * kQWarps), report, report + 1, st) != cudaSuccess)
-        return SOAR_ERR_CUDA;
-    }
-    if (want_sw) {
-      ScopedLaunch sl(K_SWIZZLE, st);
-      if (launch_stages(1, false, bt, rp, tiles * (kTile / 32), report + 1, report + 2, st) != cudaSuccess) return SOAR_ERR_CUDA;
-    }
+    if (err != cudaSuccess) return SOAR_ERR_CUDA;
   }
-  return cudaGetLastError() == cudaSuccess ? SOAR_OK : SOAR_ERR_CUDA;
+  return SOAR_OK;
 }
 
 int soar_quantize_weighted(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld, const float* col_weight,
