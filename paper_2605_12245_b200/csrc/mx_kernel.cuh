@@ -1,0 +1,367 @@
+// MXFP4 (Sec. 4.3, "DSS on MXFP4").  Included by soar.cu after quantize_kernel.cuh, whose tile walk it uses.
+//
+// The other microscaling format: E2M1 elements in blocks of 32 with one shared power-of-two scale (an E8M0 byte, value
+// 2^(code - 127)) and no tensor-wide scale.  The paper reports results and no procedure; the reading built here (the
+// oracle's) is Sec. 3.3 (i)-(ii) with alpha = 1:
+//   plain rule  shared exponent floor(log2 bmax) - 2, elements rounded to nearest even, saturated;
+//   search      high-precision scale D* = fl(bmax / 6) (Eq. 1); dequantization candidates the n_dq E8M0 values around
+//               D* (App. B.3's rule on powers of two; for two candidates the plain exponent is always one of them);
+//               quantization candidates D* * beta_k on App. B.3's grid; Eq. 8 over all pairs, first minimum in
+//               (beta, code) order.
+// One pass over W, no workspace.  Two neighbouring lanes share a block of 32, sixteen elements each.
+//
+// With a power-of-two scale everything Eq. 8 compares is an integer: with magnitudes in units of 2^(cf - 11), the error
+// minus sum W^2 under the scale 2^cf is (4B << 9) - A' in those units, and under 2^(cf + 1) twice (4B << 10) - A'.  So a
+// candidate costs two lanes one exchange of one integer and no binary64 operation, and exactly equal errors compare
+// equal.  They are common (bf16 inputs sit exactly on midpoints in a fifth of all blocks): inside the bracket the grid's
+// order decides, outside it every code change changes the error strictly (see winning_range).
+//
+// Bound by instruction issue: see mx_kernel for what it measures.
+
+#pragma once
+
+struct MxArgs {
+  Single m;
+  uint8_t* scales;
+  soar_mx_result* res;
+  unsigned long long tag;   // opens the result for sums (see mx_kernel)
+  int n_dq, n_beta, step_pct;
+  int idle;                 // test hook: the result is never opened, every wait runs out
+};
+
+struct __align__(128) MxShared {
+  static constexpr bool kOrdered = true, kSolo = true, kResident = false;
+  unsigned char ring[kQWarps][kQStages * (kQTileBytes + kQStateBytes)];
+  float2 beta[SOAR_MAX_BETA];
+  double part[kQWarps][2];
+  unsigned int count[1], start[1], total;
+  unsigned int slots, per_warp;
+  unsigned int amax, zeros, wide;
+  int failed;
+};
+
+__device__ __forceinline__ double pair_sum(unsigned int pair_mask, double v) {
+  return v + __shfl_xor_sync(pair_mask, v, 1);
+}
+
+struct MxFound {
+  double g;
+  float r;
+  int code;
+};
+
+// The search by the general rules, out of line, both lanes of a block together: any number of codes, any grid, any
+// magnitude.
+__device__ __noinline__ MxFound mx_search_general(const Params& p, unsigned int b, float bmax, const float2* s_beta, int n_dq,
+                                                  int n_beta, int step_pct, unsigned int* wide_out) {
+  const unsigned int pair_mask = 3u << (threadIdx.x & 30u);
+  uint4 v0, v1;
+  load_block(p, b, v0, v1);
+  Block blk;
+  unpack_block(v0, v1, blk);
+  Fixed fx;
+  make_fixed(blk, fx);
+  unsigned int wide = 0;
+  const float center = __fdiv_rn(bmax, 6.0f);
+  const int cf = static_cast<int>(__float_as_uint(center) >> 23);      // biased: value 2^(cf - 127) <= center
+  int d_lo, d_hi;
+  if (n_dq <= 1) {
+    const float mid = __uint_as_float((static_cast<unsigned int>(cf) << 23) | 0x400000u);   // 1.5 * 2^(cf - 127)
+    d_lo = d_hi = center > mid ? cf + 1 : cf;
+  } else {
+    d_lo = cf - (n_dq / 2 - 1);
+    d_hi = cf + n_dq / 2;
+  }
+  MxFound f;
+  f.g = __longlong_as_double(0x7FF0000000000000ll);
+  f.r = 1.0f;
+  f.code = 0;
+  const bool bracketed = n_beta >= kBracketMinBeta && step_pct >= 1;
+  const float k_scale = 100.0f / static_cast<float>(max(step_pct, 1));
+  const float k_off = static_cast<float>(n_beta / 2) - k_scale;
+  const float per_center = __fdividef(k_scale, center);
+  int best_k = 0;
+  // bracketed: per code the multipliers of winning_range; otherwise every multiplier, all codes scored on it
+  for (int d0 = d_lo, prev = -1; d0 <= (bracketed ? d_hi : d_lo); ++d0) {
+    int ka = 0, kb = n_beta - 1;
+    if (bracketed) {
+      const int dc = max(0, min(254, d0));
+      if (dc == prev) continue;   // clipping at the ends of the E8M0 range repeats a code
+      prev = dc;
+      const float sdf = static_cast<float>(__hiloint2double((dc + 896) << 20, 0));   // exact (2^-127 is a binary32 subnormal)
+      winning_range(s_beta, n_beta, 1.0f, center, __fmul_rn(sdf, 1.0f - 0x1p-21f), __fmul_rn(sdf, 1.0f + 0x1p-21f),
+                    __float2int_rd(__fmaf_rn(sdf, per_center, k_off)), ka, kb);
+    }
+    for (int k = ka; k <= kb; ++k) {
+      const float r = recip_scale(1.0f, __fmul_rn(center, s_beta[k].x));
+      unsigned int c0, c1;
+      double A, B;
+      round_block(blk, r, c0, c1);
+      block_sums(blk, fx, r, c0, c1, A, B, wide);
+      A = pair_sum(pair_mask, A);
+      B = pair_sum(pair_mask, B);
+      for (int d = d0; d <= (bracketed ? d0 : d_hi); ++d) {
+        const int dc = max(0, min(254, d));
+        if (!bracketed && d > d0 && dc == max(0, min(254, d - 1))) continue;
+        const double sd = __hiloint2double((dc + 896) << 20, 0);
+        const double g = sd * fma(sd, B, -2.0 * A);
+        // equal errors: the earlier multiplier, then the smaller code, as in grid order
+        if (g < f.g || (bracketed && g == f.g && k < best_k)) {
+          f.g = g;
+          f.r = r;
+          f.code = dc;
+          best_k = k;
+        }
+      }
+    }
+  }
+  *wide_out += wide;
+  return f;
+}
+
+// One lane's half of a candidate: codes, and (4B << shift) - A' of both halves.
+__device__ __forceinline__ int mx_score(const PairBlock& b, const FixedPairs& fx, float r, int shift, unsigned int mask,
+                                        unsigned int& c0, unsigned int& c1) {
+  unsigned int afix, b4;
+  round_pairs(b, r, c0, c1);
+  pair_code_sums(fx, c0, c1, afix, b4);
+  const int e = static_cast<int>(b4 << shift) - static_cast<int>(afix);
+  return e + __shfl_xor_sync(mask, e, 1);
+}
+
+// kSearch 0: the plain rule; 1: the search by the general rules; 2: the search with two codes on a grid that starts at
+// half the center or below and has steps of a quarter or less (the paper's: 0.50 .. 1.50 in hundredths), where a block
+// has two multipliers per code to try, or three when one falls on the code exactly, which with eight significant bits
+// in bmax is one block in seventeen.
+//
+// The result is also where the sums meet: CTA 0 clears it while the tiles are on their way and opens it by writing the
+// call's tag to `reserved`, the other CTAs add when they have seen the tag, and the one that comes last turns the sums
+// into the report (and `reserved` into what it documents, so that the replay of a captured call does not find the tag).
+// No memset before, no kernel after.
+template <int kSearch>
+__global__ void __launch_bounds__(kQThreads, kSearch == 0 ? 3 : 2) mx_kernel(const __grid_constant__ MxArgs a) {
+  __shared__ MxShared sh;
+  const Params& p = a.m.t[0];
+  const unsigned int tid = threadIdx.x, lane = tid & 31u;
+  soar_mx_result* const res = a.res;
+  if (tid == 0) {
+    sh.start[0] = 0u;
+    sh.count[0] = sh.total = p.ntiles;
+    sh.slots = smem_u32(sh.ring);
+    sh.per_warp = kQStages;
+    sh.amax = sh.zeros = sh.wide = 0u;
+    sh.failed = 0;
+  }
+  if (tid < kQWarps) sh.part[tid][0] = sh.part[tid][1] = 0.0;
+  if (kSearch)
+    for (int k = static_cast<int>(tid); k < a.n_beta; k += kQThreads) {
+      const float lo = static_cast<float>((100.0 + static_cast<double>((k - a.n_beta / 2) * a.step_pct)) / 100.0);
+      const float hi = static_cast<float>((100.0 + static_cast<double>((k + 1 - a.n_beta / 2) * a.step_pct)) / 100.0);
+      sh.beta[k] = make_float2(lo, hi);
+    }
+  if (blockIdx.x == 0 && tid == 32) {
+    res->status = 0;
+    res->amax_bits = 0u;
+    res->amax = 0.0f;
+    res->pad_ = 0;             // arrivals
+    res->sse = 0.0;            // sum of the blocks' errors minus sum W^2
+    res->sumsq = 0.0;
+    res->zero_blocks = 0;
+    res->wide_candidates = 0;
+    if (!a.idle) asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&res->reserved), "l"(a.tag) : "memory");
+  }
+  __syncthreads();
+  const unsigned int pair_mask = 3u << (lane & 30u);
+  const bool first_of_pair = (lane & 1u) == 0u;
+  const float sixth = __frcp_rn(6.0f);
+  const int n_beta = a.n_beta;
+  const float k_scale = 100.0f / static_cast<float>(max(a.step_pct, 1));
+  const float k_off = static_cast<float>(n_beta / 2) - k_scale;
+  const unsigned int pairs = smem_u32(sh.beta);
+  double acc = 0.0, sq[2] = {0.0, 0.0};
+  unsigned int zeros = 0, wide = 0, mx = 0;
+  uint8_t* packed = p.packed;
+  uint8_t* scales = a.scales;
+  unsigned int nblk = p.nblk;
+  asm volatile("" : "+l"(packed), "+l"(scales), "+r"(nblk));
+  __builtin_assume(__isGlobal(packed) && __isGlobal(scales));
+  walk_tiles<true, false>(
+      sh, a.m, false, [](int) {},
+      [&](int) {
+        double v[2] = {acc, sq[0] + sq[1]};
+        hand_over(sh, 0, v);
+      },
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next, unsigned int) {
+        const bool here = b < nblk;   // pairs go together: nblk is even
+        const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+        unsigned int m2 = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          unsigned int m;
+          asm("abs.bf16x2 %0, %1;" : "=r"(m) : "r"(u[i]));
+          asm("max.NaN.bf16x2 %0, %0, %1;" : "+r"(m2) : "r"(m));
+        }
+        m2 &= 0x7FFF7FFFu;
+        if (here) {
+          mx = __vmaxu2(mx, m2);
+          sumsq_block(u, sq[0], sq[1]);
+        }
+        m2 = max(m2 & 0xFFFFu, m2 >> 16);
+        m2 = max(m2, __shfl_xor_sync(0xFFFFFFFFu, m2, 1));
+        const float bmax = __uint_as_float(m2 << 16);
+        PairBlock blk;
+        unpack_pairs(v0, v1, blk);
+        next();
+        unsigned int c0, c1;
+        int code;
+        double g;
+        bool direct = bmax >= 0x1p-60f && bmax <= 0x1p60f;
+        if (kSearch == 0) {
+          // scale 2^X with X = floor(log2 bmax) - 2, and bmax / 2^X below 8
+          const unsigned int sd_bits = (__float_as_uint(bmax) & 0x7F800000u) - (2u << 23);
+          code = static_cast<int>(sd_bits >> 23);
+          FixedPairs fx;
+          make_fixed_pairs(blk, fixed_scale(__uint_as_float(sd_bits)), fx);
+          // S = 2^(10 - X): error minus sum W^2 = sd (sd B - 2 A) = 2^(2X - 10) ((4B << 8) - A')
+          const int e = mx_score(blk, fx, __uint_as_float((254u << 23) - sd_bits), 8, 0xFFFFFFFFu, c0, c1);
+          g = static_cast<double>(e) * __hiloint2double((2 * (code - 127) - 10 + 1023) << 20, 0);
+        } else if (kSearch == 2) {
+          const float center = quotient(bmax, 6.0f, sixth);
+          const unsigned int dv0 = __float_as_uint(center) & 0x7F800000u, dv1 = dv0 + 0x00800000u;
+          const float v0f = __uint_as_float(dv0), v1f = __uint_as_float(dv1);
+          float y;
+          asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(center));
+          const float per_center = y * k_scale;
+          const float t0 = __fadd_rd(__fmaf_rn(v0f, per_center, k_off), 12582912.0f);
+          const float t1 = __fadd_rd(__fmaf_rn(v1f, per_center, k_off), 12582912.0f);
+          const int k0 = max(0, min(n_beta - 2, __float_as_int(t0) - 0x4B400000));
+          const int k1 = max(0, min(n_beta - 2, __float_as_int(t1) - 0x4B400000));
+          const uint2 q0 = lds64(pairs + 8u * static_cast<unsigned int>(k0));
+          const uint2 q1 = lds64(pairs + 8u * static_cast<unsigned int>(k1));
+          const pair_t cc = pair_of(-center, -center);
+          const pair_t n0 = pair_mul(cc, pair_of(__uint_as_float(q0.x), __uint_as_float(q0.y)));
+          pair_t n1 = pair_mul(cc, pair_of(__uint_as_float(q1.x), __uint_as_float(q1.y)));
+          float a0, b0f, a1, b1;
+          halves(n0, a0, b0f);
+          halves(n1, a1, b1);
+          constexpr float kUnder = 1.0f - 0x1.8p-22f, kOver = 1.0f + 0x1.8p-22f;   // as in iterate_pass
+          const bool below0 = -a0 <= v0f * kUnder, above0 = -b0f >= v0f * kOver;
+          const bool below1 = -a1 <= v1f * kUnder, above1 = -b1 >= v1f * kOver;
+          // even the last multiplier's divisor lies before the upper code: it alone can win
+          const bool high1 = k1 == n_beta - 2 && -b1 <= v1f * kUnder;
+          if (high1) n1 = pair_of(b1, b1);
+          FixedPairs fx;
+          make_fixed_pairs(blk, __uint_as_float((265u << 23) - dv0), fx);   // S = 2^(11 - cf)
+          float r00, r01, r10, r11;
+          pair_recip(n0, r00, r01);
+          pair_recip(n1, r10, r11);
+          unsigned int d0, d1, e0, e1;
+          int s0 = mx_score(blk, fx, r00, 9, 0xFFFFFFFFu, c0, c1);
+          const int s1 = mx_score(blk, fx, r01, 9, 0xFFFFFFFFu, d0, d1);
+          if (s1 < s0) { s0 = s1; c0 = d0; c1 = d1; }
+          int s2 = mx_score(blk, fx, r10, 10, 0xFFFFFFFFu, d0, d1);
+          const int s3 = mx_score(blk, fx, r11, 10, 0xFFFFFFFFu, e0, e1);
+          if (s3 < s2) { s2 = s3; d0 = e0; d1 = e1; }
+          if (!(below0 && above0 && below1 && (above1 || high1))) {
+            // a multiplier inside a code's band: its neighbour on the other side can win too (equal errors: the earlier)
+            const int t0k = !below0 ? k0 - 1 : !above0 ? k0 + 2 : -1, t1k = !below1 ? k1 - 1 : !above1 && !high1 ? k1 + 2 : -1;
+            if (t0k >= 0 && t0k < n_beta) {
+              const int s = mx_score(blk, fx, recip_fast(__fmul_rn(center, sh.beta[t0k].x)), 9, pair_mask, e0, e1);
+              if (s < s0 || (!below0 && s == s0)) { s0 = s; c0 = e0; c1 = e1; }
+            }
+            if (t1k >= 0 && t1k < n_beta) {
+              const int s = mx_score(blk, fx, recip_fast(__fmul_rn(center, sh.beta[t1k].x)), 10, pair_mask, e0, e1);
+              if (s < s2 || (!below1 && s == s2)) { s2 = s; d0 = e0; d1 = e1; }
+            }
+          }
+          code = static_cast<int>(dv0 >> 23);
+          if (2 * s2 < s0) { s0 = 2 * s2; c0 = d0; c1 = d1; ++code; }
+          // error minus sum W^2 = 2^(2 cf - 11) s0
+          g = static_cast<double>(s0) * __hiloint2double((2 * (static_cast<int>(dv0 >> 23) - 127) - 11 + 1023) << 20, 0);
+        } else {
+          direct = false;
+        }
+        if (here && !direct) {
+          g = 0.0;
+          code = 0;
+          if (!(bmax >= 0x1p-120f)) {
+            // zero (or vanishing) block: scale code 0, zero codes with the inputs' sign bits
+            round_pairs(blk, 0.0f, c0, c1);
+            if (first_of_pair) ++zeros;
+          } else if (kSearch == 0) {
+            Block full;
+            uint4 w0, w1;
+            load_block(p, b, w0, w1);
+            unpack_block(w0, w1, full);
+            Fixed fx;
+            make_fixed(full, fx);
+            const int X = static_cast<int>(__float_as_uint(bmax) >> 23) - 129;
+            code = X + 127;
+            const float r = __uint_as_float(static_cast<unsigned int>(127 - X) << 23);   // 2^-X
+            double A, B;
+            round_block(full, r, c0, c1);
+            block_sums(full, fx, r, c0, c1, A, B, wide);
+            A = pair_sum(pair_mask, A);
+            B = pair_sum(pair_mask, B);
+            const double sd = __hiloint2double((code + 896) << 20, 0);   // 2^(code - 127)
+            g = sd * fma(sd, B, -2.0 * A);
+          } else {
+            const MxFound f = mx_search_general(p, b, bmax, sh.beta, a.n_dq, n_beta, a.step_pct, &wide);
+            round_pairs(blk, f.r, c0, c1);
+            g = f.g;
+            code = f.code;
+          }
+        }
+        if (here) {
+          reinterpret_cast<uint2*>(packed)[b] = make_uint2(c0, c1);
+          if (first_of_pair) {
+            scales[b >> 1] = static_cast<uint8_t>(code);
+            acc += g;
+          }
+        }
+      });
+  mx = max(mx & 0xFFFFu, mx >> 16);
+  mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+  zeros = __reduce_add_sync(0xFFFFFFFFu, zeros);
+  wide = __reduce_add_sync(0xFFFFFFFFu, wide);
+  if (lane == 0) {
+    if (mx) atomicMax(&sh.amax, mx);
+    if (zeros) atomicAdd(&sh.zeros, zeros);
+    if (wide) atomicAdd(&sh.wide, wide);
+  }
+  __syncthreads();
+  if (tid != 0) return;
+  unsigned long long seen = 0;
+  unsigned int polls = 0;
+  do {
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(&res->reserved) : "memory");
+  } while (seen != a.tag && ++polls < kGridWaitLimit);
+  if (seen != a.tag) {
+    res->status = SOAR_STATUS_INTERNAL;
+    return;
+  }
+  double err = 0.0, ss = 0.0;
+  for (int w = 0; w < kQWarps; ++w) {
+    err += sh.part[w][0];
+    ss += sh.part[w][1];
+  }
+  atomicAdd(&res->sse, err);
+  atomicAdd(&res->sumsq, ss);
+  if (sh.amax) atomicMax(&res->amax_bits, sh.amax);
+  if (sh.zeros) atomicAdd(reinterpret_cast<unsigned long long*>(&res->zero_blocks), static_cast<unsigned long long>(sh.zeros));
+  if (sh.wide) atomicAdd(reinterpret_cast<unsigned long long*>(&res->wide_candidates), static_cast<unsigned long long>(sh.wide));
+  __threadfence();
+  if (atomicAdd(&res->pad_, 1) != static_cast<int>(gridDim.x) - 1) return;
+  // the last CTA: the report from the sums
+  __threadfence();
+  const unsigned int amax_bits = __ldcg(&res->amax_bits);
+  const double gsum = __ldcg(&res->sse), sumsq = __ldcg(&res->sumsq);
+  int st = 0;
+  if (amax_bits >= 0x7F80u) st |= SOAR_STATUS_NONFINITE;
+  if (amax_bits == 0) st |= SOAR_STATUS_ZERO_TENSOR;
+  res->status = st;
+  res->amax = bits_to_mag(amax_bits);
+  res->pad_ = 0;
+  res->sse = fmax(sumsq + gsum, 0.0);
+  res->reserved = gsum;
+}
