@@ -14,7 +14,7 @@ ROOT = os.path.dirname(HERE)
 SOURCES = [os.path.join(HERE, "csrc", "soar.cu")]
 HEADERS = [os.path.join(ROOT, "include", "soar.h")] + [
     os.path.join(HERE, "csrc", f) for f in ("quantize_kernel.cuh", "solo_kernel.cuh", "weighted_kernel.cuh",
-                                             "mx_kernel.cuh")]
+                                             "mx_kernel.cuh", "error_kernel.cuh")]
 LIB = os.path.join(HERE, "libsoar.so")
 
 NVCC_FLAGS = [

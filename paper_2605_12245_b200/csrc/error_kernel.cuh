@@ -1,0 +1,113 @@
+// Eq. 3-4 on stored outputs: sum (w - q s)^2 and sum w^2.  Included by soar.cu after quantize_kernel.cuh, whose tile walk
+// it uses.
+//
+// Stored codes and scales need not belong to each other (this is a checker of arbitrary triples), so every term is taken
+// as it stands: one binary64 fused multiply-add for the difference and one for each square.  What bounds the pass is
+// instruction issue, so the rest is kept short: the signed code values come from byte permutes over the high words of
+// their binary64 forms instead of a table in shared memory (sixteen reads a block), a block's weights, codes and scale
+// byte are fetched one tile ahead into registers, and the four sums are carried over all tiles.  kWeighted multiplies
+// every term by its column's weight h_j, and takes its tiles through the ring: with its 2 CTAs an SM one tile ahead in
+// registers is too little (218 against 178 us).
+// 28672 x 8192: 138 -> 124 us unweighted (602 MB: 4.9 TB/s); weighted 178 us.
+
+#pragma once
+
+struct ErrorArgs {
+  Single m;
+  const uint8_t* scales;
+  const float* alpha;
+  const float* h;
+  double* sse;
+  double* sumsq;
+  int tiled;                // scales lie in the 128x4-tiled layout
+  int idle;                 // test hook: the sums are reported as failed
+};
+
+// kRing: tiles come through the warps' slots (walk_tiles).
+template <bool kRing>
+struct __align__(128) ErrorShared {
+  static constexpr bool kOrdered = true, kSolo = true, kResident = false;
+  unsigned char ring[kRing ? kQWarps : 1][kRing ? kQStages * (kQTileBytes + kQStateBytes) : 128];
+  double part[kQWarps][2];
+  unsigned int count[1], start[1], total;
+  unsigned int slots, per_warp;
+};
+
+template <bool kWeighted>
+__global__ void __launch_bounds__(kQThreads, kWeighted ? 2 : 4) dequant_error_kernel(const __grid_constant__ ErrorArgs a) {
+  using Shared = ErrorShared<kWeighted>;
+  __shared__ Shared sh;
+  const Params& p = a.m.t[0];
+  const unsigned int tid = threadIdx.x;
+  if (tid == 0) {
+    sh.start[0] = 0u;
+    sh.count[0] = sh.total = p.ntiles;
+    sh.slots = smem_u32(sh.ring);
+    sh.per_warp = kQStages;
+  }
+  if (tid < kQWarps) sh.part[tid][0] = sh.part[tid][1] = 0.0;
+  __syncthreads();
+  const double quarter_alpha = 0.25 * static_cast<double>(__ldg(a.alpha));
+  const unsigned int nblk = p.nblk, step = gridDim.x * kQThreads;
+  const uint2* const codes = reinterpret_cast<const uint2*>(p.packed);
+  // a block's codes and scale byte, one tile ahead
+  uint2 cw = make_uint2(0u, 0u);
+  unsigned int sc = 0;
+  auto fetch = [&](unsigned int b) {
+    if (b < nblk) {
+      cw = __ldg(codes + b);
+      size_t at = b;
+      if (a.tiled) {
+        const unsigned int row = __umulhi(2u * b, p.nbc_magic) >> p.nbc_shift;
+        at = swizzled_offset(row, b - row * p.nbc, (p.nbc + 3) / 4);
+      }
+      sc = __ldg(a.scales + at);
+    }
+  };
+  fetch(first_block<Shared>());
+  double e[2] = {0.0, 0.0}, q[2] = {0.0, 0.0};
+  walk_tiles<kWeighted, false>(
+      sh, a.m, false, [](int) {},
+      [&](int) {
+        double v[2] = {e[0] + e[1], q[0] + q[1]};
+        hand_over(sh, 0, v);
+      },
+      [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next, unsigned int) {
+        const uint2 c = cw;
+        const double s = quarter_alpha * static_cast<double>(e4m3_value(static_cast<int>(sc & 0x7Fu)));
+        fetch(b + step);
+        const bool here = b < nblk;
+        const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+        if (here) {
+          [[maybe_unused]] float hv[16];
+          if constexpr (kWeighted) weights_of(a.h, b - (__umulhi(2u * b, p.nbc_magic) >> p.nbc_shift) * p.nbc, hv);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            unsigned int hi[4];
+            code_words<true>((i < 2 ? c.x : c.y) >> (16 * (i & 1)), hi);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const unsigned int word = u[2 * i + (k >> 1)];
+              const double w = (k & 1) ? widen_high(word) : widen_low(word);
+              const double d = fma(-__hiloint2double(static_cast<int>(hi[k]), 0), s, w);
+              if constexpr (kWeighted) {
+                const double h = static_cast<double>(hv[4 * i + k]);
+                e[k & 1] = fma(h, d * d, e[k & 1]);
+                q[k & 1] = fma(h, w * w, q[k & 1]);
+              } else {
+                e[k & 1] = fma(d, d, e[k & 1]);
+                q[k & 1] = fma(w, w, q[k & 1]);
+              }
+            }
+          }
+        }
+        next();
+      });
+  __syncthreads();
+  if (tid < 2) {
+    double v = 0.0;
+    for (int w = 0; w < kQWarps; ++w) v += sh.part[w][tid];
+    if (a.idle) v = __longlong_as_double(0x7FF8000000000000ll);
+    atomicAdd(tid == 0 ? a.sse : a.sumsq, v);
+  }
+}

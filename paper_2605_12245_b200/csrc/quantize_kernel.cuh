@@ -80,6 +80,28 @@ __device__ __forceinline__ uint2 lds64(unsigned int a) {
   return v;
 }
 
+// High words of the binary64 forms of 4m for the four codes in the low half of `codes` (the low words are zero), negative
+// where kSigned and the code is.  Scaled by four the eight values 0, 2, 4, 6, 8, 12, 16, 24 have high words 0, 4000,
+// 4010, 4018, 4020, 4028, 4030, 4038 over sixteen zero bits: two lookups per four codes give the two bytes, and one
+// permute per element places them; its two zero bytes are the second byte's sign bit, which is always clear, replicated.
+template <bool kSigned>
+__device__ __forceinline__ void code_words(unsigned int codes, unsigned int (&hi)[4]) {
+  const unsigned int m = codes & 0x77777777u;
+  unsigned int b3 = __byte_perm(0x40404000u, 0x40404040u, m);
+  const unsigned int b2 = __byte_perm(0x18100000u, 0x38302820u, m);
+  if (kSigned) {
+    // a set sign bit in a selector replicates the top bit of the byte: 0xFF where negative, 0xC0 where not (the instruction
+    // itself: the intrinsic drops that bit)
+    unsigned int neg;
+    asm("prmt.b32 %0, %1, %1, %2;" : "=r"(neg) : "r"(0xC0C0C0C0u), "r"(codes));
+    b3 |= (neg << 2) & 0x80808080u;
+  }
+  asm("prmt.b32 %0, %1, %2, 0x4088;" : "=r"(hi[0]) : "r"(b2), "r"(b3));
+  asm("prmt.b32 %0, %1, %2, 0x5199;" : "=r"(hi[1]) : "r"(b2), "r"(b3));
+  asm("prmt.b32 %0, %1, %2, 0x62AA;" : "=r"(hi[2]) : "r"(b2), "r"(b3));
+  asm("prmt.b32 %0, %1, %2, 0x73BB;" : "=r"(hi[3]) : "r"(b2), "r"(b3));
+}
+
 // Two binary32 values in one register pair, and the packed operations on them (each half rounds to nearest like
 // the scalar operation).
 typedef unsigned long long pair_t;
@@ -491,6 +513,12 @@ template <typename S>
 __device__ __forceinline__ unsigned int slots_of(S& sh, unsigned int warp) {
   if constexpr (S::kSolo) return sh.slots + warp * sh.per_warp * (kQTileBytes + kQStateBytes);
   else return smem_u32(sh.ring[warp]);
+}
+
+// The first block of a lane's first tile of a forward pass over one tensor.
+template <typename S>
+__device__ __forceinline__ unsigned int first_block() {
+  return (blockIdx.x * cta_warps<S>() + (threadIdx.x >> 5)) * 32 + (threadIdx.x & 31u);
 }
 
 // Waits until at most n of the lane's copy groups are in flight.

@@ -54,14 +54,8 @@
 
 namespace {
 
-constexpr int kTile = 256;                     // blocks per tile = consumer threads per CTA
-constexpr int kThreads = kTile + 32;           // plus one producer warp that issues the copies
-constexpr int kStages = 4;                     // depth of the shared-memory ring
-constexpr int kTileBytes = kTile * 32;         // 16 bf16 per block
 constexpr size_t kWsFixedBytes = 2048;
-constexpr unsigned int kWaitLimit = 1u << 18;  // mbarrier polls before a wait gives up (a poll takes microseconds: about a second)
 constexpr unsigned int kGridWaitLimit = 1u << 21;  // polls of the grid's arrival counter before a CTA gives up (each most of a microsecond)
-constexpr unsigned int kProducerSleepNs = 32;  // the producer's pause between polls for a free stage
 constexpr int kBracketMinBeta = 2;             // the bracket needs two multipliers; a single one is modes 1-3
 
 struct Ws {
@@ -125,9 +119,7 @@ struct Params {
 constexpr int kMaxBatch = 16;
 struct Batch {
   int n;
-  int idle_producer;          // test hook: the producer fetches nothing, so every consumer wait runs out
-  unsigned int total_tiles;
-  unsigned int tile_end[kMaxBatch];   // running sum of the tensors' tile counts
+  int idle_producer;          // test hook: no CTA arrives anywhere, so every wait runs out
   Params t[kMaxBatch];
 };
 // The same for one tensor (a smaller parameter block makes a cheaper launch).
@@ -196,178 +188,13 @@ __device__ __forceinline__ float e2m1_code_value(unsigned int code3) {
 // (38.5 against 39.4 ms per Llama-3-70B-shaped layer in the candidate loop).
 __device__ __forceinline__ double uint_to_double(unsigned int v) { return __uint2double_rn(v); }
 
-// ------------------------------------------------------------------ shared-memory tile ring
-
 __device__ __forceinline__ unsigned int smem_u32(const void* p) {
   return static_cast<unsigned int>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned int bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// One bulk copy global -> shared; src and dst 16-byte aligned, bytes a multiple of 16.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned int bytes,
-                                          unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
-}
-
-// Waits for the phase with the given parity; gives up after kWaitLimit polls.  With kSleepNs > 0
-// the thread sleeps that long between polls (the producer, which otherwise spins beside the
-// consumer warps of its scheduler).
-template <unsigned int kSleepNs = 0>
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned int parity) {
-  const unsigned int addr = smem_u32(bar);
-  for (unsigned int i = 0; i < kWaitLimit; ++i) {
-    unsigned int ok;
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (ok) return true;
-    if (kSleepNs > 0) __nanosleep(kSleepNs);
-  }
-  return false;
-}
-
-struct __align__(128) Ring {
-  unsigned char tile[kStages][kTileBytes];
-  unsigned long long full[kStages];    // producer -> consumers: the stage's bytes have landed
-  unsigned long long empty[kStages];   // consumers -> producer: every consumer has read the stage
-  int meta_tensor[kStages];            // tensor the stage's tile belongs to; -1 ends the sequence
-  unsigned int meta_tile[kStages];     // and which of its tiles
-  int fail;
-};
-
-// Producer: start the copies of tile `tile` of tensor `p` into stage `s` (one copy when rows
-// are contiguous, else one per row segment) and arm the stage's barrier with the byte count.
-__device__ __forceinline__ void ring_issue(Ring& ring, const Params& p, unsigned int tile, int s) {
-  const unsigned int b0 = tile * kTile;
-  unsigned int nb = min(static_cast<unsigned int>(kTile), p.nblk - b0);
-  mbar_expect_tx(&ring.full[s], nb * 32u);
-  unsigned char* dst = ring.tile[s];
-  if (p.contiguous) {
-    bulk_load(dst, p.W + static_cast<size_t>(b0) * 16, nb * 32u, &ring.full[s]);
-    return;
-  }
-  unsigned int row = b0 / p.nbc, cb = b0 - row * p.nbc;
-  while (nb > 0) {
-    const unsigned int seg = min(nb, p.nbc - cb);
-    bulk_load(dst, p.W + static_cast<long long>(row) * p.ld + static_cast<long long>(cb) * 16, seg * 32u,
-              &ring.full[s]);
-    dst += seg * 32u;
-    nb -= seg;
-    ++row;
-    cb = 0;
-  }
-}
-
-// Tensor and tile-within-tensor of position g of the batch's tile sequence.
-__device__ __forceinline__ int tensor_of(const Batch& bt, unsigned int g, unsigned int& tile) {
-  int ti = 0;
-  unsigned int base = 0;
-  while (g >= bt.tile_end[ti]) {
-    base = bt.tile_end[ti];
-    ++ti;
-  }
-  tile = g - base;
-  return ti;
-}
-
-// All threads: barriers ready before anyone uses them.
-__device__ __forceinline__ void ring_init(Ring& ring) {
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&ring.full[s], 1);
-      mbar_init(&ring.empty[s], kTile);
-    }
-    ring.fail = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-}
-
-__device__ __forceinline__ bool is_producer_warp() { return threadIdx.x >= kTile; }
-
 __device__ __forceinline__ void record_failure(const Batch& bt) {
   for (int i = 0; i < bt.n; ++i)
     if (bt.t[i].ws != nullptr) atomicOr(&bt.t[i].ws->error, kErrWait);
-}
-
-// Producer (one thread): walks the CTA's share of the tile sequence (positions blockIdx.x,
-// + gridDim.x, ..., from the front or, for `reverse`, from the back: consecutive passes
-// alternate so that a pass starts on what the previous one left in L2), skipping tensors
-// whose bit in `run_mask` is clear, and refills a stage as soon as every consumer has handed it
-// back.  After the last tile it posts an end marker.  A wait that gives up records the
-// failure, lets copies still in flight land (bounded) and ends the sequence; the consumers
-// then give up on their own.
-__device__ __forceinline__ void ring_produce(Ring& ring, const Batch& bt, int reverse, unsigned int run_mask) {
-  if (bt.idle_producer) return;   // test hook: nothing is fetched and nothing is in flight; the consumers give up
-  unsigned int n = 0;
-  bool ok = true;
-  for (unsigned int g0 = blockIdx.x; g0 < bt.total_tiles; g0 += gridDim.x) {
-    unsigned int tile;
-    const int ti = tensor_of(bt, reverse ? bt.total_tiles - 1 - g0 : g0, tile);
-    if (!((run_mask >> ti) & 1u)) continue;
-    const int s = static_cast<int>(n % kStages);
-    if (n >= static_cast<unsigned int>(kStages)) ok = mbar_wait<kProducerSleepNs>(&ring.empty[s], (n / kStages - 1) & 1u);
-    if (!ok || *static_cast<volatile int*>(&ring.fail)) { ok = false; break; }
-    ring.meta_tensor[s] = ti;
-    ring.meta_tile[s] = tile;
-    ring_issue(ring, bt.t[ti], tile, s);
-    ++n;
-  }
-  if (ok) {   // end marker: completes the stage's phase with no bytes
-    const int s = static_cast<int>(n % kStages);
-    if (n >= static_cast<unsigned int>(kStages)) ok = mbar_wait<kProducerSleepNs>(&ring.empty[s], (n / kStages - 1) & 1u);
-    if (ok) {
-      ring.meta_tensor[s] = -1;
-      mbar_arrive(&ring.full[s]);
-    }
-  }
-  if (!ok) {
-    *static_cast<volatile int*>(&ring.fail) = 1;
-    record_failure(bt);
-    for (unsigned int m = (n > static_cast<unsigned int>(kStages) ? n - kStages : 0); m < n; ++m)
-      (void)mbar_wait(&ring.full[m % kStages], (m / kStages) & 1u);
-  }
-}
-
-// Consumer: the CTA's n-th stage.  Returns 0 with this thread's 32 bytes, the
-// tile's tensor and its number, the stage handed back; 1 at the end marker; 2 when the wait
-// gave up.  On 1 and 2 the caller leaves its tile loop.
-__device__ __forceinline__ int ring_consume(Ring& ring, const Batch& bt, unsigned int n, uint4& v0, uint4& v1,
-                                            int& ti, unsigned int& tile) {
-  const int s = static_cast<int>(n % kStages);
-  // the outcome is made the same for the whole warp
-  if (!__all_sync(0xFFFFFFFFu, mbar_wait(&ring.full[s], (n / kStages) & 1u))) {
-    *static_cast<volatile int*>(&ring.fail) = 1;
-    record_failure(bt);
-    return 2;
-  }
-  ti = ring.meta_tensor[s];
-  if (ti < 0) return 1;
-  tile = ring.meta_tile[s];
-  const uint4* src = reinterpret_cast<const uint4*>(ring.tile[s] + threadIdx.x * 32);
-  v0 = src[0];
-  v1 = src[1];
-  mbar_arrive(&ring.empty[s]);
-  return 0;
 }
 
 // ------------------------------------------------------------------ block helpers
@@ -514,55 +341,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// The sixteen column weights of block column cb, widened to binary64 (exact).
-__device__ __forceinline__ void load_weights(const float* h, unsigned int cb, double (&hd)[16]) {
-  const float4* src = reinterpret_cast<const float4*>(h) + static_cast<size_t>(cb) * 4;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const float4 v = __ldg(src + q);
-    hd[4 * q] = static_cast<double>(v.x);
-    hd[4 * q + 1] = static_cast<double>(v.y);
-    hd[4 * q + 2] = static_cast<double>(v.z);
-    hd[4 * q + 3] = static_cast<double>(v.w);
-  }
-}
-
-// Per-tensor partial sums of a CTA, in shared memory.  Each consumer warp adds its sums for a
-// tensor once (when the CTA's tile sequence leaves the tensor, or ends); the warp that arrives
-// last forwards the CTA's total to the tensor's global accumulators, one atomicAdd each.  No
-// CTA-wide barrier is involved.
-template <int N>
-struct Slots {
-  double acc[kMaxBatch][N];
-  unsigned int count[kMaxBatch];
-};
-
-// All threads, before the tile loop (a __syncthreads follows in ring_init).
-template <int N>
-__device__ __forceinline__ void slots_clear(Slots<N>& sl) {
-  for (int i = threadIdx.x; i < kMaxBatch * N; i += blockDim.x) (&sl.acc[0][0])[i] = 0.0;
-  for (int i = threadIdx.x; i < kMaxBatch; i += blockDim.x) sl.count[i] = 0;
-}
-
-// Whole consumer warp: adds v[] for tensor `ti` and clears it.
-template <int N>
-__device__ __forceinline__ void slots_add(Slots<N>& sl, int ti, double (&v)[N], double* const (&dst)[N]) {
-#pragma unroll
-  for (int i = 0; i < N; ++i) v[i] = warp_sum(v[i]);
-  if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) atomicAdd(&sl.acc[ti][i], v[i]);
-    __threadfence_block();
-    if (atomicAdd(&sl.count[ti], 1u) == kTile / 32 - 1) {
-      __threadfence_block();
-#pragma unroll
-      for (int i = 0; i < N; ++i) atomicAdd(dst[i], atomicAdd(&sl.acc[ti][i], 0.0));
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < N; ++i) v[i] = 0.0;
-}
-
 // Deterministic mode, whole warp: the sum of the n per-CTA values at `parts` in a fixed order (lane l
 // adds entries l, l + 32, ... in turn, then a fixed exchange tree); every lane gets the same bits.
 __device__ __forceinline__ double ordered_sum(const double* parts, int n) {
@@ -589,14 +367,24 @@ __device__ __forceinline__ bool stops_after(double prev, double cur, float eps) 
 
 // ------------------------------------------------------------------ kernels
 
-// Sum of squares of a block's sixteen bf16 values in binary64 (every square is exact).  The
-// widening is the float-to-double conversion instruction, which issues beside the integer pipe
-// that carries the rest of the pass.
+// The two bf16 values of a word in binary64 (exact).  The conversion instruction takes the halves as they are, and issues
+// beside the integer pipe that carries the rest of a pass.
+__device__ __forceinline__ double widen_low(unsigned int u) {
+  double d;
+  asm("{\n.reg .b16 l, h;\nmov.b32 {l, h}, %1;\ncvt.f64.bf16 %0, l;\n}" : "=d"(d) : "r"(u));
+  return d;
+}
+__device__ __forceinline__ double widen_high(unsigned int u) {
+  double d;
+  asm("{\n.reg .b16 l, h;\nmov.b32 {l, h}, %1;\ncvt.f64.bf16 %0, h;\n}" : "=d"(d) : "r"(u));
+  return d;
+}
+
+// Sum of squares of a block's sixteen bf16 values in binary64 (every square is exact).
 __device__ __forceinline__ void sumsq_block(const unsigned int (&u)[8], double& s0, double& s1) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const double dl = static_cast<double>(__uint_as_float(u[i] << 16));
-    const double dh = static_cast<double>(__uint_as_float(u[i] & 0xFFFF0000u));
+    const double dl = widen_low(u[i]), dh = widen_high(u[i]);
     s0 = fma(dl, dl, s0);
     s1 = fma(dh, dh, s1);
   }
@@ -714,81 +502,7 @@ __device__ __forceinline__ size_t swizzled_offset(unsigned int row, unsigned int
 #include "solo_kernel.cuh"
 #include "weighted_kernel.cuh"
 #include "mx_kernel.cuh"
-
-// Eq. 3-4 on stored outputs: sum (w - q s)^2 and sum w^2, one binary64 fma per term, with the
-// bf16 values widened by the conversion instruction (which runs beside the integer and
-// binary64 pipes) and the signed E2M1 values read from a 16-entry table in shared memory.
-// A wait that gave up turns the results into NaN.  kWeighted multiplies every term by its
-// column's weight h_j.
-template <bool kWeighted>
-__global__ void __launch_bounds__(kThreads) dequant_error_kernel(const __grid_constant__ Batch bt,
-                                                                 const uint8_t* scales, int swizzled,
-                                                                 unsigned int col_tiles, const float* alpha_ptr,
-                                                                 const float* h, double* out_sse,
-                                                                 double* out_sumsq) {
-  __shared__ Ring ring;
-  __shared__ Slots<2> slots;
-  __shared__ double s_q[16];
-  const Params& p = bt.t[0];
-  slots_clear(slots);
-  if (threadIdx.x < 16) {
-    const double mag = static_cast<double>(e2m1_code_value(threadIdx.x & 7u));
-    s_q[threadIdx.x] = (threadIdx.x & 8u) ? -mag : mag;
-  }
-  ring_init(ring);
-  if (is_producer_warp()) {
-    if (threadIdx.x == kTile) ring_produce(ring, bt, 0, 1u);
-    return;
-  }
-  const double alpha_d = static_cast<double>(*alpha_ptr);
-  double acc[2] = {0.0, 0.0};
-  for (unsigned int n = 0;; ++n) {
-    uint4 v0, v1;
-    int ti;
-    unsigned int tile;
-    if (ring_consume(ring, bt, n, v0, v1, ti, tile) != 0) break;
-    const unsigned int b = tile * kTile + threadIdx.x;
-    if (b >= p.nblk) continue;
-    const uint2 cw = reinterpret_cast<const uint2*>(p.packed)[b];
-    int dc;
-    if (swizzled) {
-      const unsigned int row = b / p.nbc, cb = b - row * p.nbc;
-      dc = scales[swizzled_offset(row, cb, col_tiles)];
-    } else {
-      dc = scales[b];
-    }
-    const double s = alpha_d * static_cast<double>(e4m3_value(dc & 0x7F));
-    const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    double hd[16];
-    if (kWeighted) load_weights(h, b % p.nbc, hd);
-    double e0 = 0.0, e1 = 0.0, q0 = 0.0, q1 = 0.0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const double wl = static_cast<double>(__uint_as_float(u[i] << 16));
-      const double wh = static_cast<double>(__uint_as_float(u[i] & 0xFFFF0000u));
-      const unsigned int word = (i < 4) ? cw.x : cw.y;
-      const double ql = s_q[(word >> (8 * (i & 3))) & 0xFu], qh = s_q[(word >> (8 * (i & 3) + 4)) & 0xFu];
-      const double dl = fma(-ql, s, wl), dh = fma(-qh, s, wh);
-      if (kWeighted) {
-        e0 = fma(hd[2 * i], dl * dl, e0);
-        e1 = fma(hd[2 * i + 1], dh * dh, e1);
-        q0 = fma(hd[2 * i], wl * wl, q0);
-        q1 = fma(hd[2 * i + 1], wh * wh, q1);
-      } else {
-        e0 = fma(dl, dl, e0);
-        e1 = fma(dh, dh, e1);
-        q0 = fma(wl, wl, q0);
-        q1 = fma(wh, wh, q1);
-      }
-    }
-    acc[0] += e0 + e1;
-    acc[1] += q0 + q1;
-  }
-  const bool failed = *static_cast<volatile int*>(&ring.fail) != 0;
-  if (failed) acc[0] = acc[1] = __longlong_as_double(0x7FF8000000000000ll);
-  double* const dst[2] = {out_sse, out_sumsq};
-  slots_add(slots, 0, acc, dst);
-}
+#include "error_kernel.cuh"
 
 // Counts the binary32 inputs with biased exponent lo_exp..hi_exp (all 2^23 significands each)
 // on which recip_fast differs from rcp.rn.
@@ -860,18 +574,6 @@ int sm_count() {
     g_sm_count[dev] = n;
   }
   return g_sm_count[dev];
-}
-
-// Grid of a persistent kernel: every SM filled to the kernel's occupancy, never more CTAs
-// than tiles.
-template <typename K>
-unsigned int persistent_grid(K kernel, unsigned int tiles, int threads) {
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess || per_sm <= 0)
-    per_sm = 2;
-  unsigned int cap = static_cast<unsigned int>(sm_count() * per_sm);
-  if (cap > static_cast<unsigned int>(kMaxGrid)) cap = kMaxGrid;   // the deterministic mode keeps one slot per CTA
-  return tiles < cap ? (tiles ? tiles : 1u) : cap;
 }
 
 size_t round256(size_t n) { return (n + 255) / 256 * 256; }
@@ -1392,34 +1094,38 @@ int dequant_error_impl(const void* W_bf16, int64_t rows, int64_t cols, int64_t l
   if (scale_layout != SOAR_SCALES_LINEAR && scale_layout != SOAR_SCALES_SWIZZLED) return SOAR_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(fp4_packed) % 8 != 0) return SOAR_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  Params p;
-  memset(&p, 0, sizeof(p));
+  ErrorArgs a;
+  memset(&a, 0, sizeof(a));
+  Params& p = a.m.t[0];
   p.W = static_cast<const uint16_t*>(W_bf16);
   p.packed = const_cast<uint8_t*>(static_cast<const uint8_t*>(fp4_packed));
   p.ld = ld;
   p.nbc = static_cast<unsigned int>(cols / 16);
   p.nblk = static_cast<unsigned int>(rows * (cols / 16));
-  p.ntiles = (p.nblk + kTile - 1) / kTile;
+  p.ntiles = (p.nblk + 31) / 32;
+  set_division(p);
   p.contiguous = (ld == cols) ? 1 : 0;
-  if (cudaMemsetAsync(out_sse, 0, sizeof(double), st) != cudaSuccess) return SOAR_ERR_CUDA;
-  if (cudaMemsetAsync(out_sumsq, 0, sizeof(double), st) != cudaSuccess) return SOAR_ERR_CUDA;
-  {
-    ScopedLaunch sl(K_DEQUANT_ERROR, st);
-    Batch bt;
-    memset(&bt, 0, sizeof(bt));
-    bt.n = 1;
-    bt.idle_producer = g_idle_producer;
-    bt.t[0] = p;
-    bt.total_tiles = p.ntiles;
-    for (int j = 0; j < kMaxBatch; ++j) bt.tile_end[j] = j == 0 ? p.ntiles : 0xFFFFFFFFu;
-    const uint8_t* sc = static_cast<const uint8_t*>(e4m3_scales);
-    const int sw = scale_layout == SOAR_SCALES_SWIZZLED ? 1 : 0;
-    if (h == nullptr)
-      dequant_error_kernel<false><<<persistent_grid(dequant_error_kernel<false>, p.ntiles, kThreads), kThreads, 0,
-                                    st>>>(bt, sc, sw, (p.nbc + 3) / 4, global_fp32, nullptr, out_sse, out_sumsq);
-    else
-      dequant_error_kernel<true><<<persistent_grid(dequant_error_kernel<true>, p.ntiles, kThreads), kThreads, 0,
-                                   st>>>(bt, sc, sw, (p.nbc + 3) / 4, global_fp32, h, out_sse, out_sumsq);
+  a.scales = static_cast<const uint8_t*>(e4m3_scales);
+  a.alpha = global_fp32;
+  a.h = h;
+  a.sse = out_sse;
+  a.sumsq = out_sumsq;
+  a.tiled = scale_layout == SOAR_SCALES_SWIZZLED ? 1 : 0;
+  a.idle = g_idle_producer;
+  // the two sums start at zero; where they lie side by side one memset does
+  if (out_sumsq == out_sse + 1) {
+    if (cudaMemsetAsync(out_sse, 0, 2 * sizeof(double), st) != cudaSuccess) return SOAR_ERR_CUDA;
+  } else if (cudaMemsetAsync(out_sse, 0, sizeof(double), st) != cudaSuccess ||
+             cudaMemsetAsync(out_sumsq, 0, sizeof(double), st) != cudaSuccess) {
+    return SOAR_ERR_CUDA;
+  }
+  ScopedLaunch sl(K_DEQUANT_ERROR, st);
+  if (h == nullptr) {
+    static std::atomic<int> known[64];
+    dequant_error_kernel<false><<<stage_grid(dequant_error_kernel<false>, known, p.ntiles), kQThreads, 0, st>>>(a);
+  } else {
+    static std::atomic<int> known[64];
+    dequant_error_kernel<true><<<stage_grid(dequant_error_kernel<true>, known, p.ntiles), kQThreads, 0, st>>>(a);
   }
   return cudaGetLastError() == cudaSuccess ? SOAR_OK : SOAR_ERR_CUDA;
 }

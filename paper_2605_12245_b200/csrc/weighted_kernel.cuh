@@ -10,9 +10,8 @@
 // and 24 + 6 significant bits).
 //
 // What bounds it: the binary64 pipe, which issues one instruction in two cycles.  A candidate costs three operations per
-// element, p = h (2m), A += p |w|, B += p (2m), 192 for the four of a block.  So everything else stays off that pipe: the
-// code values 2m become binary64 by two byte permutes per four elements (their high words have two non-zero bytes), and
-// weights and magnitudes are widened once per block, not once per candidate, by the conversion instruction.
+// element, p = h (4m), A += p |w|, B += p (4m), 192 for the four of a block.  So everything else stays off that pipe: the
+// code values become binary64 by byte permutes (code_words), and weights and magnitudes are widened once per block, not once per candidate, by the conversion instruction.
 // Measured on a decoder layer of 193 million weights: see weighted_iterate_pass.
 
 #pragma once
@@ -46,31 +45,30 @@ __device__ __forceinline__ void wide_magnitudes(const PairBlock& b, double (&wd)
   }
 }
 
-// 2A and 4B of a code vector (sign bits ignored): sums in element order.
+// 4A and 16B of a code vector (sign bits ignored): sums in element order (the powers of two scale every term and every
+// partial sum exactly).
 struct WeightedSums {
-  double a2, b4;
+  double a4, b16;
 };
+// Error minus sum h W^2, over sd / 2, of a vector under the dequantization scale sd.
+__device__ __forceinline__ double weighted_rank(const WeightedSums& s, double sd) { return fma(0.125 * sd, s.b16, -s.a4); }
 __device__ __forceinline__ void weighted_sums(const double (&hd)[16], const double (&wd)[16], unsigned int c0, unsigned int c1,
                                               WeightedSums& s) {
-  const unsigned int m[2] = {c0 & 0x77777777u, c1 & 0x77777777u};
   double a = 0.0, b = 0.0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const unsigned int sel = m[q >> 1] >> (16 * (q & 1));
-    // bytes 3 and 2 of the binary64 high words of 0, 1, 2, 3, 4, 6, 8, 12; the lower bytes are zero
-    const unsigned int b3 = __byte_perm(0x40403F00u, 0x40404040u, sel), b2 = __byte_perm(0x0800F000u, 0x28201810u, sel);
-    const unsigned int p01 = __byte_perm(b2, b3, 0x5140), p23 = __byte_perm(b2, b3, 0x7362);
-    const unsigned int hi[4] = {p01 << 16, p01 & 0xFFFF0000u, p23 << 16, p23 & 0xFFFF0000u};
+    unsigned int hi[4];
+    code_words<false>((q < 2 ? c0 : c1) >> (16 * (q & 1)), hi);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const double dm = __hiloint2double(static_cast<int>(hi[i]), 0);   // 2 m_j
+      const double dm = __hiloint2double(static_cast<int>(hi[i]), 0);   // 4 m_j
       const double p = hd[4 * q + i] * dm;
       a = fma(p, wd[4 * q + i], a);
       b = fma(p, dm, b);
     }
   }
-  s.a2 = a;
-  s.b4 = b;
+  s.a4 = a;
+  s.b16 = b;
 }
 
 // What a search has found for a block.
@@ -112,7 +110,7 @@ __device__ __noinline__ WeightedFound weighted_search_general(const Params& p, c
   best.g = __longlong_as_double(0x7FF0000000000000ll);
   best.c0 = best.c1 = 0u;
   best.d = clip_code(d_lo);
-  best.s.a2 = best.s.b4 = 0.0;
+  best.s.a4 = best.s.b16 = 0.0;
   if (!coupled && p.beta_step_pct >= 1 && n_beta >= kBracketMinBeta && !zero_weight) {
     const float k_scale = 100.0f / static_cast<float>(p.beta_step_pct);
     const float k_off = static_cast<float>(n_beta / 2) - k_scale, per_center = __fdividef(k_scale, center);
@@ -133,7 +131,7 @@ __device__ __noinline__ WeightedFound weighted_search_general(const Params& p, c
         round_pairs(blk, recip_fast_ok(sk) ? recip_fast(sk) : __frcp_rn(sk), c0, c1);
         WeightedSums s;
         weighted_sums(hd, wd, c0, c1, s);
-        const double g = sd * fma(0.25 * sd, s.b4, -s.a2);
+        const double g = 0.5 * sd * weighted_rank(s, sd);
         // equal errors: the earlier multiplier, then the smaller code, as in grid order
         if (g < best.g || (g == best.g && k < best_k)) {
           best.g = g; best.s = s; best.c0 = c0; best.c1 = c1; best.d = dc; best_k = k;
@@ -146,7 +144,7 @@ __device__ __noinline__ WeightedFound weighted_search_general(const Params& p, c
   for (int k = 0; k < n_beta; ++k) {
     unsigned int c0 = 0, c1 = 0;
     WeightedSums s;
-    s.a2 = s.b4 = 0.0;
+    s.a4 = s.b16 = 0.0;
     if (!coupled) {
       round_pairs(blk, recip_scale(alpha, __fmul_rn(center, s_beta[k].x)), c0, c1);
       weighted_sums(hd, wd, c0, c1, s);
@@ -159,7 +157,7 @@ __device__ __noinline__ WeightedFound weighted_search_general(const Params& p, c
         weighted_sums(hd, wd, c0, c1, s);
       }
       const double sd = alpha_d * static_cast<double>(dv);
-      const double g = sd * fma(0.25 * sd, s.b4, -s.a2);
+      const double g = 0.5 * sd * weighted_rank(s, sd);
       if (g < best.g) { best.g = g; best.s = s; best.c0 = c0; best.c1 = c1; best.d = dc; }
     }
   }
@@ -208,8 +206,7 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
         for (int i = 0; i < 8; ++i) {
           // magnitude bit patterns order like the magnitudes; NaN patterns lie above infinity's
           mx = max(mx, max(u[i] & 0x7FFFu, (u[i] >> 16) & 0x7FFFu));
-          const double wl = static_cast<double>(__uint_as_float(u[i] << 16));
-          const double wh = static_cast<double>(__uint_as_float(u[i] & 0xFFFF0000u));
+          const double wl = widen_low(u[i]), wh = widen_high(u[i]);
           sq[0] = fma(static_cast<double>(hv[2 * i]) * wl, wl, sq[0]);
           sq[1] = fma(static_cast<double>(hv[2 * i + 1]) * wh, wh, sq[1]);
         }
@@ -225,7 +222,7 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
 // A block's carried state: {A, B} of the current codes as binary32, which is all Eq. 6 takes from them; where it takes the
 // stored scale instead (B = 0, or the arm that keeps it), {scale code, B}.  Both zero for an all-zero block.
 __device__ __forceinline__ uint2 weighted_state(const WeightedSums& s, int d, bool keep_scale) {
-  const float A = static_cast<float>(0.5 * s.a2), B = static_cast<float>(0.25 * s.b4);
+  const float A = static_cast<float>(0.25 * s.a4), B = static_cast<float>(0.0625 * s.b16);
   return make_uint2((B > 0.0f && !keep_scale) ? __float_as_uint(A) : static_cast<unsigned int>(d), __float_as_uint(B));
 }
 
@@ -306,8 +303,8 @@ __device__ __forceinline__ void weighted_init_pass(S& sh, const Batch& bt, const
           scales[b] = static_cast<uint8_t>(d);
         }
         const double vd = static_cast<double>(v), sd = alpha_d * vd;
-        acc[0] = fma(s.b4, vd * vd, acc[0]);
-        acc[1] += sd * fma(0.25 * sd, s.b4, -s.a2);
+        acc[0] = fma(s.b16, 0.25 * vd * vd, acc[0]);
+        acc[1] += 0.5 * sd * weighted_rank(s, sd);
       });
 }
 
@@ -354,7 +351,7 @@ __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, co
         WeightedFound f;
         f.c0 = f.c1 = 0u;
         f.d = 0;
-        f.s.a2 = f.s.b4 = f.g = 0.0;
+        f.s.a4 = f.s.b16 = f.g = 0.0;
         bool direct = false;
         if (kFast) {
           float hv[16];
@@ -401,24 +398,25 @@ __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, co
           WeightedSums s0, s1;
           weighted_sums(hd, wd, c[0][0], c[0][1], s0);
           weighted_sums(hd, wd, c[1][0], c[1][1], s1);
-          double e0 = fma(0.25 * sd0, s0.b4, -s0.a2), e1 = fma(0.25 * sd0, s1.b4, -s1.a2);
+          double e0 = weighted_rank(s0, sd0), e1 = weighted_rank(s1, sd0);
           f.c0 = c[0][0];
           f.c1 = c[0][1];
           f.s = s0;
           if (e1 < e0) { f.c0 = c[1][0]; f.c1 = c[1][1]; f.s = s1; e0 = e1; }
-          f.g = sd0 * e0;
+          f.g = 0.5 * sd0 * e0;
           f.d = static_cast<int>(dv0 >> 20) - 960;
           weighted_sums(hd, wd, c[2][0], c[2][1], s0);
           weighted_sums(hd, wd, c[3][0], c[3][1], s1);
-          e0 = fma(0.25 * sd1, s0.b4, -s0.a2);
-          e1 = fma(0.25 * sd1, s1.b4, -s1.a2);
+          e0 = weighted_rank(s0, sd1);
+          e1 = weighted_rank(s1, sd1);
           if (e1 < e0) { c[2][0] = c[3][0]; c[2][1] = c[3][1]; s0 = s1; e0 = e1; }
           // equal errors: the earlier multiplier, as in grid order (the second code's are never earlier)
-          if (sd1 * e0 < f.g) {
+          const double g1 = 0.5 * sd1 * e0;
+          if (g1 < f.g) {
             f.c0 = c[2][0];
             f.c1 = c[2][1];
             f.s = s0;
-            f.g = sd1 * e0;
+            f.g = g1;
             f.d = static_cast<int>(dv1 >> 20) - 960;
           }
         }
@@ -439,7 +437,7 @@ __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, co
           }
           if (keep) state[b] = weighted_state(f.s, f.d, keep_scale);
           const double vd = static_cast<double>(e4m3_value(f.d));
-          acc[0] = fma(f.s.b4, vd * vd, acc[0]);
+          acc[0] = fma(f.s.b16, 0.25 * vd * vd, acc[0]);
           acc[1] += f.g;
         }
       });
