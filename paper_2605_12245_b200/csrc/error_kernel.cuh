@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kQThreads, kWeighted ? 2 : 4) dequant_error_ke
       sc = __ldg(a.scales + at);
     }
   };
-  fetch(first_block<Shared>());
+  fetch(first_block());
   double e[2] = {0.0, 0.0}, q[2] = {0.0, 0.0};
   walk_tiles<kWeighted, false>(
       sh, a.m, false, [](int) {},

@@ -515,10 +515,13 @@ __device__ __forceinline__ unsigned int slots_of(S& sh, unsigned int warp) {
   else return smem_u32(sh.ring[warp]);
 }
 
+// A warp's number in the grid.  Neighbouring numbers lie in different CTAs, so that the last, partial turn over the tiles
+// gives every SM its part instead of some SMs a whole turn and the others none (2048 x 2048: 8192 tiles over 2368 warps are
+// 55 or 56 an SM instead of 48 or 64).
+__device__ __forceinline__ unsigned int warp_number(unsigned int warp) { return warp * gridDim.x + blockIdx.x; }
 // The first block of a lane's first tile of a forward pass over one tensor.
-template <typename S>
 __device__ __forceinline__ unsigned int first_block() {
-  return (blockIdx.x * cta_warps<S>() + (threadIdx.x >> 5)) * 32 + (threadIdx.x & 31u);
+  return warp_number(threadIdx.x >> 5) * 32 + (threadIdx.x & 31u);
 }
 
 // Waits until at most n of the lane's copy groups are in flight.
@@ -537,7 +540,7 @@ __device__ __forceinline__ void copies_wait_upto(unsigned int n) {
 template <bool kState, typename S, typename B, typename Enter, typename Leave, typename Body>
 __device__ __forceinline__ void walk_resident(S& sh, const B& bt, Enter enter, Leave leave, Body body) {
   const unsigned int lane = threadIdx.x & 31u, warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
-  const unsigned int warps = gridDim.x * cta_warps<S>(), me = blockIdx.x * cta_warps<S>() + warp, tiles = bt.t[0].ntiles;
+  const unsigned int warps = gridDim.x * cta_warps<S>(), me = warp_number(warp), tiles = bt.t[0].ntiles;
   if (me >= tiles) return;
   const unsigned int n = (tiles - 1 - me) / warps + 1;
   unsigned int at = slots_of(sh, warp);
@@ -567,7 +570,7 @@ __device__ __forceinline__ void load_resident(S& sh, const B& bt) {
   const unsigned int lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = gridDim.x * cta_warps<S>();
   unsigned int at = slots_of(sh, warp) + tile_chunk(lane) * 16;
   const unsigned char* const w = reinterpret_cast<const unsigned char*>(p.W);
-  for (unsigned int tile = blockIdx.x * cta_warps<S>() + warp; tile < p.ntiles; tile += warps) {
+  for (unsigned int tile = warp_number(warp); tile < p.ntiles; tile += warps) {
 #pragma unroll
     for (unsigned int h = 0; h < 2; ++h) {
       const unsigned int b = tile * 32 + h * 16 + (lane >> 1);
@@ -594,7 +597,7 @@ __device__ __forceinline__ void walk_tiles(S& sh, const B& bt, bool reverse, Ent
     return;
   } else {
   const unsigned int lane = threadIdx.x & 31u, warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
-  const unsigned int warps = gridDim.x * cta_warps<S>(), me = blockIdx.x * cta_warps<S>() + warp;
+  const unsigned int warps = gridDim.x * cta_warps<S>(), me = warp_number(warp);
   const unsigned int ring = slots_of(sh, warp);
   const unsigned int put = ring + tile_chunk(lane) * 16, get = ring + tile_chunk(2 * lane) * 16;
   const unsigned int put_state = ring + kQStages * kQTileBytes + lane * 16, get_state = ring + kQStages * kQTileBytes + lane * 8;

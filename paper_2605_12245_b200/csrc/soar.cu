@@ -789,30 +789,79 @@ unsigned long long call_nonce() {
   return z ^ (z >> 31);
 }
 
-// One matrix in one launch (see solo_grid); the tiles stay in shared memory when every warp's fit its slots.
-template <int kMode, bool kRes>
+// One matrix in one launch (see solo_grid, cluster_size); the tiles stay in shared memory when every warp's fit its slots.
+template <int kMode, int kPlace>
 cudaError_t launch_solo(const SoloArgs& a, unsigned int grid, unsigned int warps, cudaStream_t st) {
-  const unsigned int slots = warps * (kRes ? a.per_warp : static_cast<unsigned int>(kQStages));
+  const unsigned int slots = warps * (kPlace != kStreamed ? a.per_warp : static_cast<unsigned int>(kQStages));
   const size_t dynamic = static_cast<size_t>(slots) * (kQTileBytes + kQStateBytes);
+  const auto kernel = solo_kernel<kMode, kPlace>;
   {
     static std::atomic<bool> raised[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!raised[dev].load(std::memory_order_acquire)) {
-      const unsigned int most = kSoloWarps * (kRes ? kResidentTiles : static_cast<unsigned int>(kQStages));
-      const cudaError_t err = cudaFuncSetAttribute(solo_kernel<kMode, kRes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   static_cast<int>(most * (kQTileBytes + kQStateBytes)));
+      const unsigned int most = kSoloWarps * (kPlace != kStreamed ? kResidentTiles : static_cast<unsigned int>(kQStages));
+      cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             static_cast<int>(most * (kQTileBytes + kQStateBytes)));
+      if (err == cudaSuccess && kPlace == kKeptInCluster)
+        err = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (err != cudaSuccess) return err;
       raised[dev].store(true, std::memory_order_release);
     }
   }
   if (grid == 1) {
-    solo_kernel<kMode, kRes><<<1, warps * 32, dynamic, st>>>(a);
+    kernel<<<1, warps * 32, dynamic, st>>>(a);
     return cudaGetLastError();
   }
-  void* args[] = {const_cast<SoloArgs*>(&a)};
-  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&solo_kernel<kMode, kRes>), dim3(grid), dim3(warps * 32), args,
-                                     dynamic, st);
+  cudaLaunchAttribute how;
+  memset(&how, 0, sizeof(how));
+  if (kPlace == kKeptInCluster) {
+    how.id = cudaLaunchAttributeClusterDimension;
+    how.val.clusterDim.x = grid;
+    how.val.clusterDim.y = how.val.clusterDim.z = 1;
+  } else {
+    how.id = cudaLaunchAttributeCooperative;
+    how.val.cooperative = 1;
+  }
+  cudaLaunchConfig_t lc;
+  memset(&lc, 0, sizeof(lc));
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(warps * 32);
+  lc.dynamicSmemBytes = dynamic;
+  lc.stream = st;
+  lc.attrs = &how;
+  lc.numAttrs = 1;
+  return cudaLaunchKernelEx(&lc, kernel, a);
+}
+
+// Whether this device has a cluster of the largest size for us (asked once per device).
+bool clusters_fit() {
+  static std::atomic<int> known[64];   // 0: not asked, 1: yes, 2: no
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  int k = known[dev].load(std::memory_order_relaxed);
+  if (k == 0) {
+    const auto kernel = solo_kernel<4, kKeptInCluster>;
+    cudaLaunchAttribute how;
+    memset(&how, 0, sizeof(how));
+    how.id = cudaLaunchAttributeClusterDimension;
+    how.val.clusterDim.x = kClusterMost;
+    how.val.clusterDim.y = how.val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc;
+    memset(&lc, 0, sizeof(lc));
+    lc.gridDim = dim3(kClusterMost);
+    lc.blockDim = dim3(kSoloWarps * 32);
+    lc.dynamicSmemBytes = 0;
+    lc.attrs = &how;
+    lc.numAttrs = 1;
+    int n = 0;
+    const bool yes = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                     cudaOccupancyMaxActiveClusters(&n, kernel, &lc) == cudaSuccess && n > 0;
+    if (!yes) (void)cudaGetLastError();
+    k = yes ? 1 : 2;
+    known[dev].store(k, std::memory_order_relaxed);
+  }
+  return k == 1;
 }
 
 int run_solo(const soar_tensor_desc& d, const soar_cfg* cfg, uint8_t* workspace, int mode, cudaStream_t st) {
@@ -855,12 +904,18 @@ int run_solo(const soar_tensor_desc& d, const soar_cfg* cfg, uint8_t* workspace,
   a.rows = static_cast<unsigned int>(d.rows);
   a.tiled_only = want_lin ? 0 : 1;
   a.idle = g_idle_producer;
-  const unsigned int sms = static_cast<unsigned int>(sm_count()), warps = solo_warps(p.ntiles);
-  const unsigned int grid = solo_grid(p.ntiles, sms < kSoloMaxGrid ? sms : kSoloMaxGrid);
+  const unsigned int sms = static_cast<unsigned int>(sm_count());
+  // (the test hook makes the waits of the counter run out; a cluster's barrier is the hardware's)
+  const bool cluster = p.ntiles > kOneCtaTiles && p.ntiles <= kClusterTiles && !a.idle && clusters_fit();
+  const unsigned int warps = cluster ? cluster_warps(p.ntiles) : p.ntiles <= kOneCtaTiles ? kOneCtaTiles : kSoloWarps;
+  const unsigned int grid = cluster ? cluster_size(p.ntiles) : solo_grid(p.ntiles, sms < kSoloMaxGrid ? sms : kSoloMaxGrid);
   a.per_warp = (p.ntiles + grid * warps - 1) / (grid * warps);
-  const bool resident = a.per_warp <= kResidentTiles;
+  const bool kept = a.per_warp <= kResidentTiles;
   cudaError_t err;
-#define SOAR_SOLO(M) err = resident ? launch_solo<M, true>(a, grid, warps, st) : launch_solo<M, false>(a, grid, warps, st)
+#define SOAR_SOLO(M)                                              \
+  err = cluster ? launch_solo<M, kKeptInCluster>(a, grid, warps, st) \
+        : kept  ? launch_solo<M, kKept>(a, grid, warps, st)       \
+                : launch_solo<M, kStreamed>(a, grid, warps, st)
   switch (mode) {
     case 0: SOAR_SOLO(0); break;
     case 1: SOAR_SOLO(1); break;

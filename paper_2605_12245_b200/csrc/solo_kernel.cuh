@@ -9,6 +9,10 @@
 // when some wait for others, as they do.)  The grid is one CTA of 16 warps per SM rather than two of 8: 296 CTAs need
 // 0.7 us more.
 //
+// The smallest matrices (see kClusterTiles) run in one cluster of up to 16 CTAs: the sums travel through distributed shared
+// memory and the CTAs meet at the hardware's cluster barrier, with nothing in global memory and no cooperative launch.  256
+// tiles: an iteration with one candidate 2.2 us (3.2 through the counter), a max-based call 6.5 us (9.4).
+//
 // Matrices whose tiles fit the shared memory of the grid (12 million weights) are read from HBM once and stay
 // there, and so do their block states (kResident); larger ones stream through the passes like a batch.
 //
@@ -20,16 +24,27 @@
 
 #pragma once
 
-constexpr int kSoloWarps = 16;                     // most warps of a CTA (8 in small grids)
+constexpr int kSoloWarps = 16;                     // warps of a CTA: one CTA an SM
 constexpr unsigned int kSoloMaxGrid = 160;
 constexpr unsigned int kResidentTiles = 10;        // slots a warp can have: 200 KB a CTA
 constexpr size_t kSlotBytes = 24;                  // three numbers of one CTA and pass
 
-// One warp per tile while 32 CTAs of 8 warps suffice (fewer warps an SM make a tile's latency shorter), then CTAs of 16
-// warps, one an SM.
-constexpr unsigned int solo_warps(unsigned int tiles) { return tiles <= 256 ? 8 : kSoloWarps; }
+// Up to kOneCtaTiles tiles run in one CTA; up to kClusterTiles in a cluster, a warp to a tile while 256 warps suffice.  At
+// 768 tiles (three a warp) the cluster's shorter exchange and the grid's 48 warps more than weigh each other: max-based
+// calls 8.4 against 9.4 us, an iteration of the search 4.6 us either way; at 1024 the search is slower, 6.2 against 4.6.
+constexpr unsigned int kOneCtaTiles = 8, kClusterMost = 16, kClusterTiles = 768;
+constexpr unsigned int cluster_warps(unsigned int tiles) {
+  const unsigned int even = (tiles + kClusterMost - 1) / kClusterMost;
+  return even < 4 ? 4 : even > kSoloWarps ? kSoloWarps : even;
+}
+constexpr unsigned int cluster_size(unsigned int tiles) {   // a power of two
+  const unsigned int want = (tiles + cluster_warps(tiles) - 1) / cluster_warps(tiles);
+  unsigned int n = 1;
+  while (n < want && n < kClusterMost) n *= 2;
+  return n;
+}
 constexpr unsigned int solo_grid(unsigned int tiles, unsigned int most) {
-  const unsigned int want = (tiles + solo_warps(tiles) - 1) / solo_warps(tiles);
+  const unsigned int want = tiles <= kOneCtaTiles ? 1 : (tiles + kSoloWarps - 1) / kSoloWarps;
   return want < most ? want : most;
 }
 // Workspace of the exchange: epoch, flag and counter, then the slots of even and of odd passes; none for one CTA.
@@ -51,13 +66,17 @@ struct SoloArgs {
   int idle;                // test hook: nobody arrives, every wait runs out
 };
 
-template <bool kRes>
+// Where a matrix's tiles stay and how its CTAs meet.
+constexpr int kStreamed = 0, kKept = 1, kKeptInCluster = 2;
+
+template <int kPlace>
 struct __align__(128) SoloShared {
-  static constexpr bool kOrdered = true, kSolo = true, kResident = kRes;
+  static constexpr bool kOrdered = true, kSolo = true, kResident = kPlace != kStreamed, kCluster = kPlace == kKeptInCluster;
   View view[1];
   float2 beta[SOAR_MAX_BETA];
   double part[kSoloWarps][2];        // each warp's sums of the pass
-  unsigned long long red[2][kSoloMaxGrid / 32][3];   // the grid's numbers, by the warp that read them
+  // the grid's numbers, by the warp that read them; in a cluster by the CTA that sent them
+  unsigned long long red[2][kCluster ? kClusterMost : kSoloMaxGrid / 32][3];
   double trace_alpha[SOAR_MAX_ITERS + 1], trace_sse[SOAR_MAX_ITERS + 1];
   float alpha[1];
   unsigned int amax[1], zeros[1], wide[1];
@@ -91,10 +110,63 @@ __device__ __forceinline__ void open_counter(const SoloArgs& a, unsigned long lo
   }
 }
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// exchange() inside a cluster: every CTA writes its numbers into everybody's shared memory.
+template <bool kMax, typename S>
+__device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, Totals& out) {
+  __syncthreads();
+  const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
+  if (tid < 32) {
+    double x = 0.0, g = 0.0;
+    if (lane < blockDim.x / 32) {
+      x = sh.part[lane][0];
+      g = sh.part[lane][1];
+    }
+    x = warp_sum(x);
+    g = warp_sum(g);
+    const unsigned long long second = kMax ? sh.amax[0] : static_cast<unsigned long long>(__double_as_longlong(g));
+    const unsigned long long counts = sh.zeros[0] | (static_cast<unsigned long long>(sh.wide[0]) << 32);
+    __syncwarp();
+    if (lane == 0) sh.zeros[0] = sh.wide[0] = 0u;
+    if (lane < grid) {
+      unsigned int at;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(&sh.red[turn][blockIdx.x][0])), "r"(lane));
+      asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at), "l"(__double_as_longlong(x)) : "memory");
+      asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at + 8), "l"(second) : "memory");
+      asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at + 16), "l"(counts) : "memory");
+    }
+  }
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();
+  double x = 0.0, g = 0.0;
+  unsigned int mx = 0;
+  unsigned long long counts = 0;
+  if (lane < grid) {
+    const volatile unsigned long long* const r = sh.red[turn][lane];
+    x = __longlong_as_double(static_cast<long long>(r[0]));
+    if (kMax) mx = static_cast<unsigned int>(r[1]);
+    else g = __longlong_as_double(static_cast<long long>(r[1]));
+    counts = r[2];
+  }
+  out.a = warp_sum(x);
+  out.g = kMax ? 0.0 : warp_sum(g);
+  out.amax = kMax ? __reduce_max_sync(0xFFFFFFFFu, mx) : 0u;
+  if (blockIdx.x == 0) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) counts += __shfl_xor_sync(0xFFFFFFFFu, counts, o);
+  }
+  out.counts = counts;
+  return true;
+}
+
 // After a pass, all threads of all CTAs: exchanges the CTAs' sums.  `pass` counts from 1.  What the CTAs wrote to global
 // memory before is visible to all after.  With `last` only CTA 0 waits for the sums.  False when a wait ran out.
 template <bool kMax, typename S>
 __device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned int pass, bool last, Totals& out) {
+  if constexpr (S::kCluster) return exchange_in_cluster<kMax>(sh, pass, out);
   __syncthreads();
   const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
   unsigned long long* const slots = reinterpret_cast<unsigned long long*>(a.exchange + 256 + turn * (grid * kSlotBytes));
@@ -189,10 +261,12 @@ __device__ __forceinline__ void clear_tile_padding(const Params& p, unsigned int
       for (unsigned int c = nbc; c < ct * 4; ++c) tiled[swizzled_offset(r, c, ct)] = 0;
 }
 
-template <int kMode, bool kRes>
+template <int kMode, int kPlace>
 __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_constant__ SoloArgs a) {
   extern __shared__ __align__(128) unsigned char tile_slots[];
-  __shared__ SoloShared<kRes> sh;
+  __shared__ SoloShared<kPlace> sh;
+  constexpr bool kRes = kPlace != kStreamed, kCluster = kPlace == kKeptInCluster;
+  if (kCluster) cluster_arrive();   // (waited for before anything is written into another CTA)
   const int tid = threadIdx.x;
   const Params& p = a.m.t[0];
   const int T = p.max_iters, flags = p.flags;
@@ -211,7 +285,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   }
   if (tid < kSoloWarps) sh.part[tid][0] = sh.part[tid][1] = 0.0;
   unsigned long long epoch = 0;
-  if (gridDim.x > 1) epoch = __ldcg(reinterpret_cast<const unsigned long long*>(a.exchange));
+  if (!kCluster && gridDim.x > 1) epoch = __ldcg(reinterpret_cast<const unsigned long long*>(a.exchange));
   if (kMode == 0 || kMode >= 3) {
     const int n_beta = p.n_beta, step = p.beta_step_pct;
     for (int k = tid; k < n_beta; k += static_cast<int>(blockDim.x)) {
@@ -223,11 +297,15 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   __syncthreads();
   if (kRes) load_resident(sh, a.m);
   if (T == 0 && a.tiled != nullptr) clear_tile_padding(p, a.rows, a.tiled);
-  if (gridDim.x > 1 && tid == 0) open_counter(a, a.nonce + epoch, sh.failed);
+  if (!kCluster && gridDim.x > 1 && tid == 0) open_counter(a, a.nonce + epoch, sh.failed);
   unsigned int pass = 0;
   Totals tot;
   bool ok;
   amax_pass(sh, a.m);
+  if (kCluster) {
+    __syncwarp();
+    cluster_wait();
+  }
   ok = exchange<true>(sh, a, ++pass, false, tot);
   const double sumsq = tot.a;
   const unsigned int amax_bits = tot.amax;
@@ -277,7 +355,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   if (!ok) {
     // a wait ran out: say so in the report and leave
     if (tid == 0) {
-      if (gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange) = epoch + 1;
+      if (!kCluster && gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange) = epoch + 1;
       if (a.result != nullptr) {
         a.result->status = SOAR_STATUS_INTERNAL;
         a.result->iters_run = 0;
@@ -287,7 +365,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   }
   if (blockIdx.x != 0) return;
   if (tid == 0) {
-    if (gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange) = epoch + 1;
+    if (!kCluster && gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange) = epoch + 1;
     *a.alpha = alpha;
     if (a.result != nullptr) {
       soar_result* const res = a.result;
