@@ -1154,8 +1154,8 @@ __device__ __forceinline__ void iterate_pass(S& sh, const B& bt, bool reverse, u
           direct = false;
         }
         // A = afix / (2 S); error minus sum W^2 = alpha (h e) 4 / S^2
-        float v = __uint_as_float(dv_bits), A = __fmul_rn(__uint2float_rn(w.afix), __uint_as_float(s_exp - (11u << 23)));
-        int d = (kMode == 1 && n_dq > 2) ? e4m3_encode(v) : static_cast<int>(dv_bits >> 20) - 960;
+        const float v = __uint_as_float(dv_bits), A = __fmul_rn(__uint2float_rn(w.afix), __uint_as_float(s_exp - (11u << 23)));
+        const int d = (kMode == 1 && n_dq > 2) ? e4m3_encode(v) : static_cast<int>(dv_bits >> 20) - 960;
         const double g_scale = __hiloint2double(__double2hiint(alpha_d) + static_cast<int>(s_exp >> 2) - (272 << 20),
                                           __double2loint(alpha_d));
         if (active && !direct) {
@@ -1165,19 +1165,23 @@ __device__ __forceinline__ void iterate_pass(S& sh, const B& bt, bool reverse, u
                                                     (flags & SOAR_FLAG_COUPLED_SCALE) != 0, &wide)
                                      : search_general<kMode>(bt.t[tensor], b, alpha, center, sh.beta, n_beta, n_dq, k_scale,
                                                              k_off, &wide);
-          w.c0 = f.c0;
-          w.c1 = f.c1;
-          w.b4 = f.b4;
-          d = f.d;
-          v = e4m3_value(d);
-          A = f.A;
-          g_scaled = 0.0;
+          // (stored here: merging it into the common path costs that path a move per value)
+          uint8_t *packed, *scales;
+          uint2* states;
+          load_view(view, packed, scales, states);
+          if (emit) {
+            reinterpret_cast<uint2*>(packed)[b] = make_uint2(f.c0, f.c1);
+            scales[b] = static_cast<uint8_t>(f.d);
+          }
+          if (keep)
+            put_state<S>(states, b, state_at, make_uint2(__float_as_uint(f.A), pack_state(st.y & 0x7F800000u, f.d, f.b4)));
+          const float fv = e4m3_value(f.d);
+          acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(fv, fv), __uint2float_rn(f.b4)));
           acc[1] += f.g;
-        }
-        uint8_t *packed, *scales;
-        uint2* states;
-        load_view(view, packed, scales, states);
-        if (active) {
+        } else if (active) {
+          uint8_t *packed, *scales;
+          uint2* states;
+          load_view(view, packed, scales, states);
           if (emit) {
             reinterpret_cast<uint2*>(packed)[b] = make_uint2(w.c0, w.c1);
             scales[b] = static_cast<uint8_t>(d);
