@@ -9,10 +9,10 @@
 // the unweighted search do not apply: the sums are binary64, taken in element order, every product exact (24 + 8 + 3
 // and 24 + 6 significant bits).
 //
-// What bounds it: the binary64 pipe, which issues one instruction in two cycles.  A candidate costs three operations per
-// element, p = h (4m), A += p |w|, B += p (4m), 192 for the four of a block.  So everything else stays off that pipe: the
-// code values become binary64 by byte permutes (code_words), and weights and magnitudes are widened once per block, not once per candidate, by the conversion instruction.
-// Measured on a decoder layer of 193 million weights: see weighted_iterate_pass.
+// What bounds it: instruction issue, 760 a block with the binary64 pipe, which issues one in two cycles, at 36 %.  A
+// candidate costs three binary64 operations per element, p = h (4m), A += p |w|, B += p (4m); the code values become
+// binary64 by byte permutes (code_words; the integer conversion instruction instead, for half or all of one candidate,
+// was 0 to 4 % slower).  28672 x 8192, one iteration: 1084 -> 498 us; the whole call 4 iterations, 2.31 ms.
 
 #pragma once
 
@@ -69,6 +69,39 @@ __device__ __forceinline__ void weighted_sums(const double (&hd)[16], const doub
   }
   s.a4 = a;
   s.b16 = b;
+}
+
+// The sums of two code vectors at once, widening each weight and magnitude where it is used, by asm that the compiler does
+// not lift out: the 32 widened values kept over all candidates take 64 registers and spill (573 against 510 us an
+// iteration on 28672 x 8192).
+__device__ __forceinline__ void weighted_sums_of_two(const float (&hv)[16], const PairBlock& blk, const unsigned int (&ca)[2],
+                                                     const unsigned int (&cb)[2], WeightedSums& sa, WeightedSums& sb) {
+  double a0 = 0.0, b0 = 0.0, a1 = 0.0, b1 = 0.0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    unsigned int ha[4], hb[4];
+    code_words<false>(ca[q >> 1] >> (16 * (q & 1)), ha);
+    code_words<false>(cb[q >> 1] >> (16 * (q & 1)), hb);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int j = 4 * q + i;
+      float lo, hi;
+      halves(blk.w[j >> 1], lo, hi);
+      double w, h;
+      asm volatile("cvt.f64.f32 %0, %1;" : "=d"(w) : "f"(fabsf((j & 1) ? hi : lo)));
+      asm volatile("cvt.f64.f32 %0, %1;" : "=d"(h) : "f"(hv[j]));
+      const double da = __hiloint2double(static_cast<int>(ha[i]), 0), db = __hiloint2double(static_cast<int>(hb[i]), 0);
+      const double pa = h * da, pb = h * db;
+      a0 = fma(pa, w, a0);
+      b0 = fma(pa, da, b0);
+      a1 = fma(pb, w, a1);
+      b1 = fma(pb, db, b1);
+    }
+  }
+  sa.a4 = a0;
+  sa.b16 = b0;
+  sb.a4 = a1;
+  sb.b16 = b1;
 }
 
 // What a search has found for a block.
@@ -388,16 +421,9 @@ __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, co
           unsigned int c[4][2];
           round_pairs(blk, r00, c[0][0], c[0][1]);
           round_pairs(blk, r01, c[1][0], c[1][1]);
-          round_pairs(blk, r10, c[2][0], c[2][1]);
-          round_pairs(blk, r11, c[3][0], c[3][1]);
-          double hd[16], wd[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j) hd[j] = static_cast<double>(hv[j]);
-          wide_magnitudes(blk, wd);
           const double sd0 = alpha_d * scaled_value(dv0, 0), sd1 = alpha_d * scaled_value(dv1, 0);
           WeightedSums s0, s1;
-          weighted_sums(hd, wd, c[0][0], c[0][1], s0);
-          weighted_sums(hd, wd, c[1][0], c[1][1], s1);
+          weighted_sums_of_two(hv, blk, c[0], c[1], s0, s1);
           double e0 = weighted_rank(s0, sd0), e1 = weighted_rank(s1, sd0);
           f.c0 = c[0][0];
           f.c1 = c[0][1];
@@ -405,8 +431,9 @@ __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, co
           if (e1 < e0) { f.c0 = c[1][0]; f.c1 = c[1][1]; f.s = s1; e0 = e1; }
           f.g = 0.5 * sd0 * e0;
           f.d = static_cast<int>(dv0 >> 20) - 960;
-          weighted_sums(hd, wd, c[2][0], c[2][1], s0);
-          weighted_sums(hd, wd, c[3][0], c[3][1], s1);
+          round_pairs(blk, r10, c[2][0], c[2][1]);
+          round_pairs(blk, r11, c[3][0], c[3][1]);
+          weighted_sums_of_two(hv, blk, c[2], c[3], s0, s1);
           e0 = weighted_rank(s0, sd1);
           e1 = weighted_rank(s1, sd1);
           if (e1 < e0) { c[2][0] = c[3][0]; c[2][1] = c[3][1]; s0 = s1; e0 = e1; }
