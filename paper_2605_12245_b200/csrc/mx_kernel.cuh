@@ -16,6 +16,11 @@
 // equal.  They are common (bf16 inputs sit exactly on midpoints in a fifth of all blocks): inside the bracket the grid's
 // order decides, outside it every code change changes the error strictly (see winning_range).
 //
+// Two multipliers per code are enough, the last one below the code's band and its successor, also where that successor lies
+// in the band, which it does in one block in seventeen: a bf16 magnitude over a power of two has eight significant bits,
+// so it is a rounding midpoint exactly or misses it by 2^-8, far more than the band's 2^-21; the successor's codes are then
+// nearest ones, ties either way, its error is the least there is, and only an earlier multiplier can share the first place.
+//
 // Bound by instruction issue: see mx_kernel for what it measures.
 
 #pragma once
@@ -130,9 +135,8 @@ __device__ __forceinline__ int mx_score(const PairBlock& b, const FixedPairs& fx
 }
 
 // kSearch 0: the plain rule; 1: the search by the general rules; 2: the search with two codes on a grid that starts at
-// half the center or below and has steps of a quarter or less (the paper's: 0.50 .. 1.50 in hundredths), where a block
-// has two multipliers per code to try, or three when one falls on the code exactly, which with eight significant bits
-// in bmax is one block in seventeen.
+// half the center or below and has steps of a quarter or less (the paper's: 0.50 .. 1.50 in hundredths): two multipliers
+// per code in straight line.
 //
 // The result is also where the sums meet: CTA 0 clears it while the tiles are on their way and opens it by writing the
 // call's tag to `reserved`, the other CTAs add when they have seen the tag, and the one that comes last turns the sums
@@ -176,7 +180,8 @@ __global__ void __launch_bounds__(kQThreads, kSearch == 0 ? 3 : 2) mx_kernel(con
   const float sixth = __frcp_rn(6.0f);
   const int n_beta = a.n_beta;
   const float k_scale = 100.0f / static_cast<float>(max(a.step_pct, 1));
-  const float k_off = static_cast<float>(n_beta / 2) - k_scale;
+  // (a pair is chosen so that a multiplier in the code's band is its second: see below)
+  const float k_off = static_cast<float>(n_beta / 2) - k_scale - 5e-4f;
   const unsigned int pairs = smem_u32(sh.beta);
   double acc = 0.0, sq[2] = {0.0, 0.0};
   unsigned int zeros = 0, wide = 0, mx = 0;
@@ -244,11 +249,10 @@ __global__ void __launch_bounds__(kQThreads, kSearch == 0 ? 3 : 2) mx_kernel(con
           float a0, b0f, a1, b1;
           halves(n0, a0, b0f);
           halves(n1, a1, b1);
-          constexpr float kUnder = 1.0f - 0x1.8p-22f, kOver = 1.0f + 0x1.8p-22f;   // as in iterate_pass
-          const bool below0 = -a0 <= v0f * kUnder, above0 = -b0f >= v0f * kOver;
-          const bool below1 = -a1 <= v1f * kUnder, above1 = -b1 >= v1f * kOver;
+          constexpr float kUnder = 1.0f - 0x1.8p-22f;   // as in iterate_pass
           // even the last multiplier's divisor lies before the upper code: it alone can win
           const bool high1 = k1 == n_beta - 2 && -b1 <= v1f * kUnder;
+          direct = direct && -a0 <= v0f * kUnder && -b0f > v0f * kUnder && -a1 <= v1f * kUnder && (-b1 > v1f * kUnder || high1);
           if (high1) n1 = pair_of(b1, b1);
           FixedPairs fx;
           make_fixed_pairs(blk, __uint_as_float((265u << 23) - dv0), fx);   // S = 2^(11 - cf)
@@ -262,18 +266,6 @@ __global__ void __launch_bounds__(kQThreads, kSearch == 0 ? 3 : 2) mx_kernel(con
           int s2 = mx_score(blk, fx, r10, 10, 0xFFFFFFFFu, d0, d1);
           const int s3 = mx_score(blk, fx, r11, 10, 0xFFFFFFFFu, e0, e1);
           if (s3 < s2) { s2 = s3; d0 = e0; d1 = e1; }
-          if (!(below0 && above0 && below1 && (above1 || high1))) {
-            // a multiplier inside a code's band: its neighbour on the other side can win too (equal errors: the earlier)
-            const int t0k = !below0 ? k0 - 1 : !above0 ? k0 + 2 : -1, t1k = !below1 ? k1 - 1 : !above1 && !high1 ? k1 + 2 : -1;
-            if (t0k >= 0 && t0k < n_beta) {
-              const int s = mx_score(blk, fx, recip_fast(__fmul_rn(center, sh.beta[t0k].x)), 9, pair_mask, e0, e1);
-              if (s < s0 || (!below0 && s == s0)) { s0 = s; c0 = e0; c1 = e1; }
-            }
-            if (t1k >= 0 && t1k < n_beta) {
-              const int s = mx_score(blk, fx, recip_fast(__fmul_rn(center, sh.beta[t1k].x)), 10, pair_mask, e0, e1);
-              if (s < s2 || (!below1 && s == s2)) { s2 = s; d0 = e0; d1 = e1; }
-            }
-          }
           code = static_cast<int>(dv0 >> 23);
           if (2 * s2 < s0) { s0 = 2 * s2; c0 = d0; c1 = d1; ++code; }
           // error minus sum W^2 = 2^(2 cf - 11) s0
