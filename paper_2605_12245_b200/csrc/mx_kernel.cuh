@@ -21,7 +21,8 @@
 // so it is a rounding midpoint exactly or misses it by 2^-8, far more than the band's 2^-21; the successor's codes are then
 // nearest ones, ties either way, its error is the least there is, and only an earlier multiplier can share the first place.
 //
-// Bound by instruction issue: see mx_kernel for what it measures.
+// Bound by instruction issue, 380 a lane of sixteen elements: 28672 x 8192 with the search 665 -> 219 us (594 MB: 2.7 TB/s),
+// by the plain rule 200 -> 123 us.
 
 #pragma once
 
@@ -34,9 +35,11 @@ struct MxArgs {
   int idle;                 // test hook: the result is never opened, every wait runs out
 };
 
+// kRing: tiles come through the warps' slots (walk_tiles).
+template <bool kRing>
 struct __align__(128) MxShared {
   static constexpr bool kOrdered = true, kSolo = true, kResident = false;
-  unsigned char ring[kQWarps][kQStages * (kQTileBytes + kQStateBytes)];
+  unsigned char ring[kRing ? kQWarps : 1][kRing ? kQStages * (kQTileBytes + kQStateBytes) : 128];
   float2 beta[SOAR_MAX_BETA];
   double part[kQWarps][2];
   unsigned int count[1], start[1], total;
@@ -144,7 +147,8 @@ __device__ __forceinline__ int mx_score(const PairBlock& b, const FixedPairs& fx
 // No memset before, no kernel after.
 template <int kSearch>
 __global__ void __launch_bounds__(kQThreads, kSearch == 0 ? 3 : 2) mx_kernel(const __grid_constant__ MxArgs a) {
-  __shared__ MxShared sh;
+  constexpr bool kRing = kSearch != 2;   // the search is bound by instruction issue: 227 -> 219 us through registers
+  __shared__ MxShared<kRing> sh;
   const Params& p = a.m.t[0];
   const unsigned int tid = threadIdx.x, lane = tid & 31u;
   soar_mx_result* const res = a.res;
@@ -190,7 +194,7 @@ __global__ void __launch_bounds__(kQThreads, kSearch == 0 ? 3 : 2) mx_kernel(con
   unsigned int nblk = p.nblk;
   asm volatile("" : "+l"(packed), "+l"(scales), "+r"(nblk));
   __builtin_assume(__isGlobal(packed) && __isGlobal(scales));
-  walk_tiles<true, false>(
+  walk_tiles<kRing, false>(
       sh, a.m, false, [](int) {},
       [&](int) {
         double v[2] = {acc, sq[0] + sq[1]};
