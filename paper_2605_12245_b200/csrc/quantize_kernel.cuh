@@ -410,6 +410,7 @@ __device__ __forceinline__ void load_view(unsigned int at, uint8_t*& packed, uin
 template <bool kDet>
 struct __align__(128) QShared {
   static constexpr bool kOrdered = kDet, kSolo = false, kResident = false;
+  static constexpr bool kFinal = false;   // whether the start pass is known to be the last one
   unsigned char ring[kQWarps][kQStages * (kQTileBytes + kQStateBytes)];   // also write_report's scratch
   View view[kMaxBatch];
   float2 beta[SOAR_MAX_BETA];              // {multiplier k, multiplier k + 1}
@@ -904,7 +905,7 @@ __device__ __forceinline__ void init_pass(S& sh, const B& bt) {
           round_pairs(blk, 1.0f, c0, c1);
           reinterpret_cast<uint2*>(packed)[b] = make_uint2(c0, c1);
           put_scale(sh, bt.t[tensor], scales, b, 0);
-          if (keep) put_state<S>(state, b, state_at, make_uint2(0u, 0u));
+          if (!S::kFinal && keep) put_state<S>(state, b, state_at, make_uint2(0u, 0u));
           ++zeros;
           return;
         }
@@ -933,15 +934,15 @@ __device__ __forceinline__ void init_pass(S& sh, const B& bt) {
           f = start_general(bt.t[tensor], b, alpha, &wide);
           v = e4m3_value(f.d);
         }
-        if (!keep) {
+        if (S::kFinal || !keep) {
           reinterpret_cast<uint2*>(packed)[b] = make_uint2(f.c0, f.c1);
           put_scale(sh, bt.t[tensor], scales, b, f.d);
         } else {
           put_state<S>(state, b, state_at,
                        make_uint2(__float_as_uint(f.A), pack_state(__float_as_uint(bmax) & 0x7F800000u, f.d, f.b4)));
         }
-        // v^2 4B is exact in binary32: 8 + 12 significant bits
-        acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(v, v), __uint2float_rn(f.b4)));
+        // v^2 4B is exact in binary32: 8 + 12 significant bits (no Eq. 5 follows the last pass)
+        if (!S::kFinal) acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(v, v), __uint2float_rn(f.b4)));
         acc[1] += f.g;
       });
 }

@@ -802,7 +802,7 @@ cudaError_t launch_solo(const SoloArgs& a, unsigned int grid, unsigned int warps
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!raised[dev].load(std::memory_order_acquire)) {
-      const unsigned int most = kSoloWarps * (kPlace != kStreamed ? kResidentTiles : static_cast<unsigned int>(kQStages));
+      const unsigned int most = kPlace != kStreamed ? kResidentTiles : solo_most_warps(kMode) * kQStages;
       cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(most * (kQTileBytes + kQStateBytes)));
       if (err == cudaSuccess && kPlace == kKeptInCluster)
@@ -909,16 +909,21 @@ int run_solo(const soar_tensor_desc& d, const soar_cfg* cfg, uint8_t* workspace,
   const unsigned int sms = static_cast<unsigned int>(sm_count());
   // (the test hook makes the waits of the counter run out; a cluster's barrier is the hardware's)
   const bool cluster = p.ntiles > kOneCtaTiles && p.ntiles <= kClusterTiles && !a.idle && clusters_fit();
-  const unsigned int warps = cluster ? cluster_warps(p.ntiles) : p.ntiles <= kOneCtaTiles ? kOneCtaTiles : kSoloWarps;
+  if (cfg->max_iters == 0) mode = kNoIterations;
+  // (more than 16 warps an SM only once every SM has its 16)
+  const unsigned int warps = cluster ? cluster_warps(p.ntiles)
+                             : p.ntiles <= kOneCtaTiles ? kOneCtaTiles
+                             : p.ntiles > sms * kSoloWarps ? solo_most_warps(mode) : kSoloWarps;
   const unsigned int grid = cluster ? cluster_size(p.ntiles) : solo_grid(p.ntiles, sms < kSoloMaxGrid ? sms : kSoloMaxGrid);
   a.per_warp = (p.ntiles + grid * warps - 1) / (grid * warps);
-  const bool kept = a.per_warp <= kResidentTiles;
+  const bool kept = a.per_warp * warps <= kResidentTiles;
   cudaError_t err;
 #define SOAR_SOLO(M)                                              \
   err = cluster ? launch_solo<M, kKeptInCluster>(a, grid, warps, st) \
         : kept  ? launch_solo<M, kKept>(a, grid, warps, st)       \
                 : launch_solo<M, kStreamed>(a, grid, warps, st)
   switch (mode) {
+    case kNoIterations: SOAR_SOLO(kNoIterations); break;
     case 0: SOAR_SOLO(0); break;
     case 1: SOAR_SOLO(1); break;
     case 2: SOAR_SOLO(2); break;

@@ -25,8 +25,11 @@
 #pragma once
 
 constexpr int kSoloWarps = 16;                     // warps of a CTA: one CTA an SM
+// A call without iterations (kMode -1) has only the light passes and half the registers: 32 warps an SM.
+constexpr int kNoIterations = -1;
+constexpr unsigned int solo_most_warps(int mode) { return mode == kNoIterations ? 32 : kSoloWarps; }
 constexpr unsigned int kSoloMaxGrid = 160;
-constexpr unsigned int kResidentTiles = 10;        // slots a warp can have: 200 KB a CTA
+constexpr unsigned int kResidentTiles = 160;       // slots a CTA can have: 200 KB
 constexpr size_t kSlotBytes = 24;                  // three numbers of one CTA and pass
 
 // Up to kOneCtaTiles tiles run in one CTA; up to kClusterTiles in a cluster, a warp to a tile while 256 warps suffice.  At
@@ -69,12 +72,13 @@ struct SoloArgs {
 // Where a matrix's tiles stay and how its CTAs meet.
 constexpr int kStreamed = 0, kKept = 1, kKeptInCluster = 2;
 
-template <int kPlace>
+template <int kPlace, bool kNoIter>
 struct __align__(128) SoloShared {
+  static constexpr bool kFinal = kNoIter;
   static constexpr bool kOrdered = true, kSolo = true, kResident = kPlace != kStreamed, kCluster = kPlace == kKeptInCluster;
   View view[1];
   float2 beta[SOAR_MAX_BETA];
-  double part[kSoloWarps][2];        // each warp's sums of the pass
+  double part[32][2];                // each warp's sums of the pass
   // the grid's numbers, by the warp that read them; in a cluster by the CTA that sent them
   unsigned long long red[2][kCluster ? kClusterMost : kSoloMaxGrid / 32][3];
   double trace_alpha[SOAR_MAX_ITERS + 1], trace_sse[SOAR_MAX_ITERS + 1];
@@ -262,9 +266,9 @@ __device__ __forceinline__ void clear_tile_padding(const Params& p, unsigned int
 }
 
 template <int kMode, int kPlace>
-__global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_constant__ SoloArgs a) {
+__global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 : kMode) * 32, 1) solo_kernel(const __grid_constant__ SoloArgs a) {
   extern __shared__ __align__(128) unsigned char tile_slots[];
-  __shared__ SoloShared<kPlace> sh;
+  __shared__ SoloShared<kPlace, kMode == kNoIterations> sh;
   constexpr bool kRes = kPlace != kStreamed, kCluster = kPlace == kKeptInCluster;
   if (kCluster) cluster_arrive();   // (waited for before anything is written into another CTA)
   const int tid = threadIdx.x;
@@ -283,7 +287,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
     sh.tiled_only = a.tiled_only;
     sh.failed = 0;
   }
-  if (tid < kSoloWarps) sh.part[tid][0] = sh.part[tid][1] = 0.0;
+  if (tid < 32) sh.part[tid][0] = sh.part[tid][1] = 0.0;
   unsigned long long epoch = 0;
   if (!kCluster && gridDim.x > 1) epoch = __ldcg(reinterpret_cast<const unsigned long long*>(a.exchange));
   if (kMode == 0 || kMode >= 3) {
@@ -330,6 +334,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
       sh.trace_sse[0] = sse;
     }
     const bool may_stop = p.early_stop_rel > 0.0f;
+    if constexpr (kMode != kNoIterations)
     for (int t = 0; st == 0 && ok && t < T; ++t) {
       // Eq. 5; the numerator follows from the two sums carried (see file_sums)
       const double ad = static_cast<double>(alpha), den = 0.25 * tot.a;
