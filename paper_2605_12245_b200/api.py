@@ -201,10 +201,15 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+# The current device, and the handle of its current stream.  (torch.cuda.current_device() and current_stream() wrap these:
+# building a torch.cuda.Stream takes longer than the launch.)
+_device = torch.cuda.current_device
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda dev: torch.cuda.current_stream(dev).cuda_stream)
+
+
 def _stream_ptr(stream):
     if stream is None:
-        # the handle itself: building a torch.cuda.Stream around it takes longer than the launch
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        return _raw_stream(_device())
     if stream.device.index != torch.cuda.current_device():
         raise SoarError(f"stream belongs to cuda:{stream.device.index} but the current device is "
                         f"cuda:{torch.cuda.current_device()}")
@@ -283,10 +288,18 @@ def soar_quantize(W: torch.Tensor, cfg: SoarCfg, out: QuantBuffers | None = None
         out = alloc_buffers(rows, cols, cfg, W.device)
     packed, scales, scales_sw, alpha, result, ws = (out.packed, out.scales, out.scales_sw, out.alpha, out.result,
                                                     out.workspace)
-    _require_cuda(W, packed, scales, scales_sw, alpha, result, ws)
+    # (written out: this is the path of the smallest calls, which take a few microseconds on the device)
+    dev = _device()
+    if not (W.get_device() == dev and (packed is None or packed.get_device() == dev)
+            and (scales is None or scales.get_device() == dev) and (scales_sw is None or scales_sw.get_device() == dev)
+            and (alpha is None or alpha.get_device() == dev) and (result is None or result.get_device() == dev)
+            and (ws is None or ws.get_device() == dev)):
+        _require_cuda(W, packed, scales, scales_sw, alpha, result, ws)
     rc = (_lib or lib()).soar_quantize(
-        W.data_ptr(), rows, cols, W.stride(0) if ld is None else ld, C.byref(cfg), _ptr(packed), _ptr(scales),
-        _ptr(scales_sw), _ptr(alpha), _ptr(ws), ws.numel(), _ptr(result), _stream_ptr(stream))
+        W.data_ptr(), rows, cols, W.stride(0) if ld is None else ld, cfg, None if packed is None else packed.data_ptr(),
+        None if scales is None else scales.data_ptr(), None if scales_sw is None else scales_sw.data_ptr(),
+        None if alpha is None else alpha.data_ptr(), None if ws is None else ws.data_ptr(), ws.numel(),
+        None if result is None else result.data_ptr(), _raw_stream(dev) if stream is None else _stream_ptr(stream))
     if rc:
         _check(rc, "soar_quantize")
     return out

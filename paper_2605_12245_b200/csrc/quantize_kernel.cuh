@@ -564,12 +564,12 @@ __device__ __forceinline__ void walk_resident(S& sh, const B& bt, Enter enter, L
   leave(0);
 }
 
-// Starts the copies of every tile of the warp into its slots.
-template <typename S, typename B>
-__device__ __forceinline__ void load_resident(S& sh, const B& bt) {
+// Starts the copies of every tile of the warp into its slots, per_warp of them at `slots` for each warp.
+template <typename B>
+__device__ __forceinline__ void load_resident(const B& bt, unsigned int slots, unsigned int per_warp) {
   const Params& p = bt.t[0];
-  const unsigned int lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = gridDim.x * cta_warps<S>();
-  unsigned int at = slots_of(sh, warp) + tile_chunk(lane) * 16;
+  const unsigned int lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = gridDim.x * (blockDim.x >> 5);
+  unsigned int at = slots + warp * per_warp * (kQTileBytes + kQStateBytes) + tile_chunk(lane) * 16;
   const unsigned char* const w = reinterpret_cast<const unsigned char*>(p.W);
   for (unsigned int tile = warp_number(warp); tile < p.ntiles; tile += warps) {
 #pragma unroll

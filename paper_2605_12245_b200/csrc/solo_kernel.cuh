@@ -98,24 +98,35 @@ struct Totals {
   unsigned long long counts;         // zero blocks in the low half, wide candidates in the high one (CTA 0 only)
 };
 
-// Before the first exchange (one thread): CTA 0 clears the counter and opens the flag, the others wait for it.
-__device__ __forceinline__ void open_counter(const SoloArgs& a, unsigned long long tag, int& failed) {
-  unsigned long long* const flag = reinterpret_cast<unsigned long long*>(a.exchange + 8);
-  if (blockIdx.x == 0) {
-    *reinterpret_cast<volatile unsigned int*>(a.exchange + 64) = 0u;
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(flag), "l"(tag) : "memory");
-  } else {
-    unsigned long long seen = 0;
-    unsigned int polls = 0;
-    do {
-      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(flag) : "memory");
-    } while (seen != tag && ++polls < kGridWaitLimit);
-    if (seen != tag) failed = 1;
-  }
+// Where the exchange keeps its words: epoch, then flag and counter in one sixteen-byte unit.
+constexpr size_t kEpochAt = 0, kFlagAt = 16, kCounterAt = 24;
+
+// At the start of the call (one thread of CTA 0): clears the counter and opens the flag in one store, which nothing has to
+// be waited for.
+__device__ __forceinline__ void open_counter(const SoloArgs& a, unsigned long long tag) {
+  asm volatile("{\n.reg .b128 p;\nmov.b128 p, {%1, %2};\nst.relaxed.gpu.global.b128 [%0], p;\n}" ::"l"(a.exchange + kFlagAt), "l"(tag),
+               "l"(0ull)
+               : "memory");
+}
+// Before the first arrival (one thread of every CTA).
+__device__ __forceinline__ bool counter_open(const SoloArgs& a, unsigned long long tag) {
+  unsigned long long seen = 0;
+  unsigned int polls = 0;
+  do {
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(a.exchange + kFlagAt) : "memory");
+  } while (seen != tag && ++polls < kGridWaitLimit);
+  return seen == tag;
 }
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// Sum over lanes 0..15 of a warp whose upper lanes hold the same values again.
+__device__ __forceinline__ double half_warp_sum(double v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
 
 // exchange() inside a cluster: every CTA writes its numbers into everybody's shared memory.
 template <bool kMax, typename S>
@@ -124,12 +135,12 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, To
   const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
   if (tid < 32) {
     double x = 0.0, g = 0.0;
-    if (lane < blockDim.x / 32) {
-      x = sh.part[lane][0];
-      g = sh.part[lane][1];
+    if ((lane & 15u) < blockDim.x / 32) {   // (at most sixteen warps)
+      x = sh.part[lane & 15u][0];
+      g = sh.part[lane & 15u][1];
     }
-    x = warp_sum(x);
-    g = warp_sum(g);
+    x = half_warp_sum(x);
+    if (!kMax) g = half_warp_sum(g);
     const unsigned long long second = kMax ? sh.amax[0] : static_cast<unsigned long long>(__double_as_longlong(g));
     const unsigned long long counts = sh.zeros[0] | (static_cast<unsigned long long>(sh.wide[0]) << 32);
     __syncwarp();
@@ -147,29 +158,32 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, To
   cluster_wait();
   double x = 0.0, g = 0.0;
   unsigned int mx = 0;
-  unsigned long long counts = 0;
-  if (lane < grid) {
-    const volatile unsigned long long* const r = sh.red[turn][lane];
+  unsigned int zeros = 0, wide = 0;
+  if ((lane & 15u) < grid) {
+    const volatile unsigned long long* const r = sh.red[turn][lane & 15u];
     x = __longlong_as_double(static_cast<long long>(r[0]));
     if (kMax) mx = static_cast<unsigned int>(r[1]);
     else g = __longlong_as_double(static_cast<long long>(r[1]));
-    counts = r[2];
+    if (!kMax && lane < 16) {
+      zeros = static_cast<unsigned int>(r[2]);
+      wide = static_cast<unsigned int>(r[2] >> 32);
+    }
   }
-  out.a = warp_sum(x);
-  out.g = kMax ? 0.0 : warp_sum(g);
+  out.a = half_warp_sum(x);
+  out.g = kMax ? 0.0 : half_warp_sum(g);
   out.amax = kMax ? __reduce_max_sync(0xFFFFFFFFu, mx) : 0u;
-  if (blockIdx.x == 0) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) counts += __shfl_xor_sync(0xFFFFFFFFu, counts, o);
-  }
-  out.counts = counts;
+  out.counts = 0;
+  if (!kMax && blockIdx.x == 0)
+    out.counts = __reduce_add_sync(0xFFFFFFFFu, zeros) |
+                 (static_cast<unsigned long long>(__reduce_add_sync(0xFFFFFFFFu, wide)) << 32);
   return true;
 }
 
 // After a pass, all threads of all CTAs: exchanges the CTAs' sums.  `pass` counts from 1.  What the CTAs wrote to global
 // memory before is visible to all after.  With `last` only CTA 0 waits for the sums.  False when a wait ran out.
 template <bool kMax, typename S>
-__device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned int pass, bool last, Totals& out) {
+__device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned long long tag, unsigned int pass, bool last,
+                                         Totals& out) {
   if constexpr (S::kCluster) return exchange_in_cluster<kMax>(sh, pass, out);
   __syncthreads();
   const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
@@ -198,7 +212,8 @@ __device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned int 
                lane == 0 ? static_cast<unsigned long long>(__double_as_longlong(x)) : lane == 1 ? second : counts);
       __syncwarp();
       if (lane == 0) {
-        unsigned int* const arrived = reinterpret_cast<unsigned int*>(a.exchange + 64);
+        unsigned int* const arrived = reinterpret_cast<unsigned int*>(a.exchange + kCounterAt);
+        if (pass == 1 && !counter_open(a, tag)) sh.failed = 1;
         if (!a.idle) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
         if (!last || blockIdx.x == 0) {
           unsigned int seen = 0, polls = 0;
@@ -252,13 +267,17 @@ __device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned int 
   return sh.failed == 0;
 }
 
-// Zeroes of the tiled layout: rows up to a multiple of 128, scale columns up to a multiple of 4.
+// Zeroes of the tiled layout: rows up to a multiple of 128, scale columns up to a multiple of 4.  Four columns of a row are
+// four bytes side by side.
 __device__ __forceinline__ void clear_tile_padding(const Params& p, unsigned int rows, uint8_t* tiled) {
   const unsigned int nbc = p.nbc, ct = (nbc + 3) / 4, padded = (rows + 127) / 128 * 128;
   const unsigned int me = blockIdx.x * blockDim.x + threadIdx.x, all = gridDim.x * blockDim.x;
-  for (unsigned int i = me; i < (padded - rows) * ct * 4; i += all) {
-    const unsigned int r = i / (ct * 4), c = i - r * (ct * 4);
-    tiled[swizzled_offset(rows + r, c, ct)] = 0;
+  const bool words = reinterpret_cast<uintptr_t>(tiled) % 4 == 0;
+  for (unsigned int i = me; i < (padded - rows) * ct; i += all) {
+    const unsigned int r = i / ct, t = i - r * ct;
+    uint8_t* const at = tiled + swizzled_offset(rows + r, t * 4, ct);
+    if (words) *reinterpret_cast<unsigned int*>(at) = 0u;
+    else at[0] = at[1] = at[2] = at[3] = 0;
   }
   if (nbc % 4 != 0)
     for (unsigned int r = me; r < rows; r += all)
@@ -274,6 +293,10 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
   const int tid = threadIdx.x;
   const Params& p = a.m.t[0];
   const int T = p.max_iters, flags = p.flags;
+  unsigned long long epoch = 0;
+  if (!kCluster && gridDim.x > 1) epoch = __ldcg(reinterpret_cast<const unsigned long long*>(a.exchange + kEpochAt));
+  if (kRes) load_resident(a.m, smem_u32(tile_slots), a.per_warp);
+  if (!kCluster && gridDim.x > 1 && blockIdx.x == 0 && tid == 0) open_counter(a, a.nonce + epoch);
   if (tid == 0) {
     sh.view[0].packed = p.packed;
     sh.view[0].scales = p.scales;
@@ -288,8 +311,6 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
     sh.failed = 0;
   }
   if (tid < 32) sh.part[tid][0] = sh.part[tid][1] = 0.0;
-  unsigned long long epoch = 0;
-  if (!kCluster && gridDim.x > 1) epoch = __ldcg(reinterpret_cast<const unsigned long long*>(a.exchange));
   if (kMode == 0 || kMode >= 3) {
     const int n_beta = p.n_beta, step = p.beta_step_pct;
     for (int k = tid; k < n_beta; k += static_cast<int>(blockDim.x)) {
@@ -298,10 +319,11 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
       sh.beta[k] = make_float2(lo, hi);
     }
   }
+  // what of the report does not depend on the sums
+  if (blockIdx.x == 0 && a.result != nullptr)
+    for (int i = T + 1 + tid; i <= SOAR_MAX_ITERS; i += static_cast<int>(blockDim.x)) a.result->trace_alpha[i] = a.result->trace_sse[i] = 0.0;
   __syncthreads();
-  if (kRes) load_resident(sh, a.m);
   if (T == 0 && a.tiled != nullptr) clear_tile_padding(p, a.rows, a.tiled);
-  if (!kCluster && gridDim.x > 1 && tid == 0) open_counter(a, a.nonce + epoch, sh.failed);
   unsigned int pass = 0;
   Totals tot;
   bool ok;
@@ -310,7 +332,7 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
     __syncwarp();
     cluster_wait();
   }
-  ok = exchange<true>(sh, a, ++pass, false, tot);
+  ok = exchange<true>(sh, a, a.nonce + epoch, ++pass, false, tot);
   const double sumsq = tot.a;
   const unsigned int amax_bits = tot.amax;
   const int st = status_from_amax(amax_bits);
@@ -324,7 +346,7 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
   if (ok && !(st & (SOAR_STATUS_NONFINITE | SOAR_STATUS_RANGE))) {
     const bool tile_after = T > 0 && a.tiled != nullptr;
     init_pass(sh, a.m);
-    ok = exchange<false>(sh, a, ++pass, T == 0, tot);
+    ok = exchange<false>(sh, a, a.nonce + epoch, ++pass, T == 0, tot);
     if (T == 0 && blockIdx.x != 0) return;   // nothing left to do but CTA 0's report
     if (st == 0) sse = fmax(sumsq + tot.g, 0.0);
     zero_blocks = tot.counts & 0xFFFFFFFFull;
@@ -342,7 +364,7 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
       sh.alpha[0] = alpha;
       iterate_pass<kMode>(sh, a.m, (t & 1) != 0, may_stop || t == T - 1, t != T - 1);
       const bool last = t == T - 1 && !tile_after;
-      ok = exchange<false>(sh, a, ++pass, last, tot);
+      ok = exchange<false>(sh, a, a.nonce + epoch, ++pass, last, tot);
       if (last && blockIdx.x != 0) return;
       const double cur = fmax(sumsq + tot.g, 0.0);
       wide += tot.counts >> 32;
@@ -360,7 +382,7 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
   if (!ok) {
     // a wait ran out: say so in the report and leave
     if (tid == 0) {
-      if (!kCluster && gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange) = epoch + 1;
+      if (!kCluster && gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange + kEpochAt) = epoch + 1;
       if (a.result != nullptr) {
         a.result->status = SOAR_STATUS_INTERNAL;
         a.result->iters_run = 0;
@@ -370,7 +392,7 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
   }
   if (blockIdx.x != 0) return;
   if (tid == 0) {
-    if (!kCluster && gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange) = epoch + 1;
+    if (!kCluster && gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange + kEpochAt) = epoch + 1;
     *a.alpha = alpha;
     if (a.result != nullptr) {
       soar_result* const res = a.result;
@@ -387,7 +409,7 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
   }
   if (a.result != nullptr) {
     __syncthreads();
-    for (int i = tid; i <= SOAR_MAX_ITERS; i += static_cast<int>(blockDim.x)) {
+    for (int i = tid; i <= T; i += static_cast<int>(blockDim.x)) {
       a.result->trace_alpha[i] = i == 0 ? static_cast<double>(alpha0) : i <= iters ? sh.trace_alpha[i] : 0.0;
       a.result->trace_sse[i] = (i <= iters && st == 0) ? sh.trace_sse[i] : 0.0;
     }
