@@ -33,6 +33,12 @@ struct __align__(128) ErrorShared {
   unsigned int slots, per_warp;
 };
 
+__global__ void clear_sums_kernel(double* sse, double* sumsq) {
+  let_next_begin();   // (it waits for this kernel's end)
+  after_previous();
+  if (threadIdx.x == 0) *sse = *sumsq = 0.0;
+}
+
 template <bool kWeighted>
 __global__ void __launch_bounds__(kQThreads, kWeighted ? 2 : 4) dequant_error_kernel(const __grid_constant__ ErrorArgs a) {
   using Shared = ErrorShared<kWeighted>;
@@ -47,6 +53,7 @@ __global__ void __launch_bounds__(kQThreads, kWeighted ? 2 : 4) dequant_error_ke
   }
   if (tid < kQWarps) sh.part[tid][0] = sh.part[tid][1] = 0.0;
   __syncthreads();
+  after_previous();
   const double quarter_alpha = 0.25 * static_cast<double>(__ldg(a.alpha));
   const unsigned int nblk = p.nblk, step = gridDim.x * kQThreads;
   const uint2* const codes = reinterpret_cast<const uint2*>(p.packed);
@@ -103,6 +110,7 @@ __global__ void __launch_bounds__(kQThreads, kWeighted ? 2 : 4) dequant_error_ke
         }
         next();
       });
+  let_next_begin();
   __syncthreads();
   if (tid < 2) {
     double v = 0.0;

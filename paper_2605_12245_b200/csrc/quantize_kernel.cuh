@@ -38,6 +38,11 @@ __device__ __forceinline__ unsigned int pack_state(unsigned int eb_field, int d,
   return eb_field | (static_cast<unsigned int>(d) << 12) | b4;
 }
 
+// Head of a kernel launched by launch_chained: waits until everything before it in the stream is done and visible.
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// From here on the next such kernel may take its place on the SMs.
+__device__ __forceinline__ void let_next_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Position of 16-byte chunk j in a tile slot.
 __device__ __forceinline__ unsigned int tile_chunk(unsigned int j) { return j ^ ((j >> 3) & 1u); }
 

@@ -776,6 +776,31 @@ int search_mode(const soar_cfg* cfg) {
   return (cfg->flags & SOAR_FLAG_KEEP_BLOCK_SCALE) ? 3 : 4;
 }
 
+// Launches a kernel that may begin while the one before it in the stream ends (programmatic stream serialization): the
+// kernel waits at its head (after_previous) for everything before it, and the gap between two launches shrinks from 1 to 2
+// us, a multiple of about a microsecond from start to start, to half a microsecond.  Cooperative launches cannot.  cluster: CTAs of
+// a cluster, or 0.
+template <typename... Want, typename... Have>
+cudaError_t launch_chained(void (*kernel)(Want...), unsigned int grid, unsigned int threads, size_t dynamic, unsigned int cluster,
+                           cudaStream_t st, const Have&... args) {
+  cudaLaunchAttribute how[2];
+  memset(how, 0, sizeof(how));
+  how[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  how[0].val.programmaticStreamSerializationAllowed = 1;
+  how[1].id = cudaLaunchAttributeClusterDimension;
+  how[1].val.clusterDim.x = cluster;
+  how[1].val.clusterDim.y = how[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t lc;
+  memset(&lc, 0, sizeof(lc));
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(threads);
+  lc.dynamicSmemBytes = dynamic;
+  lc.stream = st;
+  lc.attrs = how;
+  lc.numAttrs = cluster > 0 ? 2 : 1;
+  return cudaLaunchKernelEx(&lc, kernel, args...);
+}
+
 // A number no earlier call of this process used, and that memory left by another is not likely to hold: a counter
 // from a random start through a 64-bit mixing function (the finalizer of SplitMix64; Steele, Lea and Flood, "Fast
 // splittable pseudorandom number generators", OOPSLA 2014).
@@ -811,29 +836,10 @@ cudaError_t launch_solo(const SoloArgs& a, unsigned int grid, unsigned int warps
       raised[dev].store(true, std::memory_order_release);
     }
   }
-  if (grid == 1) {
-    kernel<<<1, warps * 32, dynamic, st>>>(a);
-    return cudaGetLastError();
-  }
-  cudaLaunchAttribute how;
-  memset(&how, 0, sizeof(how));
-  if (kPlace == kKeptInCluster) {
-    how.id = cudaLaunchAttributeClusterDimension;
-    how.val.clusterDim.x = grid;
-    how.val.clusterDim.y = how.val.clusterDim.z = 1;
-  } else {
-    how.id = cudaLaunchAttributeCooperative;
-    how.val.cooperative = 1;
-  }
-  cudaLaunchConfig_t lc;
-  memset(&lc, 0, sizeof(lc));
-  lc.gridDim = dim3(grid);
-  lc.blockDim = dim3(warps * 32);
-  lc.dynamicSmemBytes = dynamic;
-  lc.stream = st;
-  lc.attrs = &how;
-  lc.numAttrs = 1;
-  return cudaLaunchKernelEx(&lc, kernel, a);
+  if (grid == 1 || kPlace == kKeptInCluster)
+    return launch_chained(kernel, grid, warps * 32, dynamic, grid == 1 ? 0 : grid, st, a);
+  void* args[] = {const_cast<SoloArgs*>(&a)};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3(grid), dim3(warps * 32), args, dynamic, st);
 }
 
 // Whether this device has a cluster of the largest size for us (asked once per device).
@@ -1174,22 +1180,18 @@ int dequant_error_impl(const void* W_bf16, int64_t rows, int64_t cols, int64_t l
   a.sumsq = out_sumsq;
   a.tiled = scale_layout == SOAR_SCALES_SWIZZLED ? 1 : 0;
   a.idle = g_idle_producer;
-  // the two sums start at zero; where they lie side by side one memset does
-  if (out_sumsq == out_sse + 1) {
-    if (cudaMemsetAsync(out_sse, 0, 2 * sizeof(double), st) != cudaSuccess) return SOAR_ERR_CUDA;
-  } else if (cudaMemsetAsync(out_sse, 0, sizeof(double), st) != cudaSuccess ||
-             cudaMemsetAsync(out_sumsq, 0, sizeof(double), st) != cudaSuccess) {
-    return SOAR_ERR_CUDA;
-  }
+  // the two sums start at zero (a kernel of ours rather than a memset, so that the next one can be chained to it)
   ScopedLaunch sl(K_DEQUANT_ERROR, st);
+  cudaError_t err = launch_chained(clear_sums_kernel, 1, 32, 0, 0, st, out_sse, out_sumsq);
+  if (err != cudaSuccess) return SOAR_ERR_CUDA;
   if (h == nullptr) {
     static std::atomic<int> known[64];
-    dequant_error_kernel<false><<<stage_grid(dequant_error_kernel<false>, known, p.ntiles), kQThreads, 0, st>>>(a);
+    err = launch_chained(dequant_error_kernel<false>, stage_grid(dequant_error_kernel<false>, known, p.ntiles), kQThreads, 0, 0, st, a);
   } else {
     static std::atomic<int> known[64];
-    dequant_error_kernel<true><<<stage_grid(dequant_error_kernel<true>, known, p.ntiles), kQThreads, 0, st>>>(a);
+    err = launch_chained(dequant_error_kernel<true>, stage_grid(dequant_error_kernel<true>, known, p.ntiles), kQThreads, 0, 0, st, a);
   }
-  return cudaGetLastError() == cudaSuccess ? SOAR_OK : SOAR_ERR_CUDA;
+  return err == cudaSuccess ? SOAR_OK : SOAR_ERR_CUDA;
 }
 }  // namespace
 

@@ -290,6 +290,7 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
   __shared__ SoloShared<kPlace, kMode == kNoIterations> sh;
   constexpr bool kRes = kPlace != kStreamed, kCluster = kPlace == kKeptInCluster;
   if (kCluster) cluster_arrive();   // (waited for before anything is written into another CTA)
+  after_previous();
   const int tid = threadIdx.x;
   const Params& p = a.m.t[0];
   const int T = p.max_iters, flags = p.flags;
@@ -379,6 +380,7 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
     }
     if (ok && tile_after) tile_scales(p, a.rows, a.tiled);
   }
+  let_next_begin();
   if (!ok) {
     // a wait ran out: say so in the report and leave
     if (tid == 0) {
