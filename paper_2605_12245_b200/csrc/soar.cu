@@ -827,7 +827,7 @@ cudaError_t launch_solo(const SoloArgs& a, unsigned int grid, unsigned int warps
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!raised[dev].load(std::memory_order_acquire)) {
-      const unsigned int most = kPlace != kStreamed ? kResidentTiles : solo_most_warps(kMode) * kQStages;
+      const unsigned int most = kPlace != kStreamed ? kResidentTiles : kSoloWarps * kQStages;
       cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(most * (kQTileBytes + kQStateBytes)));
       if (err == cudaSuccess && kPlace == kKeptInCluster)
@@ -840,6 +840,29 @@ cudaError_t launch_solo(const SoloArgs& a, unsigned int grid, unsigned int warps
     return launch_chained(kernel, grid, warps * 32, dynamic, grid == 1 ? 0 : grid, st, a);
   void* args[] = {const_cast<SoloArgs*>(&a)};
   return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3(grid), dim3(warps * 32), args, dynamic, st);
+}
+
+// A call without iterations on a matrix of more than kClusterTiles tiles.
+cudaError_t launch_max_based(const SoloArgs& a, cudaStream_t st) {
+  constexpr size_t dynamic = static_cast<size_t>(kMaxBasedThreads / 32) * kQStages * (kQTileBytes + kQStateBytes);
+  static std::atomic<bool> raised[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  cudaError_t err = cudaSuccess;
+  if (!raised[dev].load(std::memory_order_acquire)) {
+    err = cudaFuncSetAttribute(max_based_amax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dynamic));
+    if (err == cudaSuccess)
+      err = cudaFuncSetAttribute(max_based_codes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(dynamic));
+    if (err != cudaSuccess) return err;
+    raised[dev].store(true, std::memory_order_release);
+  }
+  // as many slots as exchange_bytes gave room for; a CTA for every sixteen tiles until every SM has one
+  const unsigned int sms = static_cast<unsigned int>(sm_count());
+  const unsigned int grid = solo_grid(a.m.t[0].ntiles, sms < kSoloMaxGrid ? sms : kSoloMaxGrid);
+  const unsigned int threads = a.m.t[0].ntiles > sms * kSoloWarps ? kMaxBasedThreads : kSoloWarps * 32;
+  err = launch_chained(max_based_amax_kernel, grid, threads, dynamic, 0, st, a);
+  if (err == cudaSuccess) err = launch_chained(max_based_codes_kernel, grid, threads, dynamic, 0, st, a);
+  return err;
 }
 
 // Whether this device has a cluster of the largest size for us (asked once per device).
@@ -916,10 +939,7 @@ int run_solo(const soar_tensor_desc& d, const soar_cfg* cfg, uint8_t* workspace,
   // (the test hook makes the waits of the counter run out; a cluster's barrier is the hardware's)
   const bool cluster = p.ntiles > kOneCtaTiles && p.ntiles <= kClusterTiles && !a.idle && clusters_fit();
   if (cfg->max_iters == 0) mode = kNoIterations;
-  // (more than 16 warps an SM only once every SM has its 16)
-  const unsigned int warps = cluster ? cluster_warps(p.ntiles)
-                             : p.ntiles <= kOneCtaTiles ? kOneCtaTiles
-                             : p.ntiles > sms * kSoloWarps ? solo_most_warps(mode) : kSoloWarps;
+  const unsigned int warps = cluster ? cluster_warps(p.ntiles) : p.ntiles <= kOneCtaTiles ? kOneCtaTiles : kSoloWarps;
   const unsigned int grid = cluster ? cluster_size(p.ntiles) : solo_grid(p.ntiles, sms < kSoloMaxGrid ? sms : kSoloMaxGrid);
   a.per_warp = (p.ntiles + grid * warps - 1) / (grid * warps);
   const bool kept = a.per_warp * warps <= kResidentTiles;
@@ -929,7 +949,11 @@ int run_solo(const soar_tensor_desc& d, const soar_cfg* cfg, uint8_t* workspace,
         : kept  ? launch_solo<M, kKept>(a, grid, warps, st)       \
                 : launch_solo<M, kStreamed>(a, grid, warps, st)
   switch (mode) {
-    case kNoIterations: SOAR_SOLO(kNoIterations); break;
+    case kNoIterations:
+      err = cluster     ? launch_solo<kNoIterations, kKeptInCluster>(a, grid, warps, st)
+            : grid == 1 ? launch_solo<kNoIterations, kKept>(a, grid, warps, st)
+                        : launch_max_based(a, st);
+      break;
     case 0: SOAR_SOLO(0); break;
     case 1: SOAR_SOLO(1); break;
     case 2: SOAR_SOLO(2); break;

@@ -25,9 +25,7 @@
 #pragma once
 
 constexpr int kSoloWarps = 16;                     // warps of a CTA: one CTA an SM
-// A call without iterations (kMode -1) has only the light passes and half the registers: 32 warps an SM.
-constexpr int kNoIterations = -1;
-constexpr unsigned int solo_most_warps(int mode) { return mode == kNoIterations ? 32 : kSoloWarps; }
+constexpr int kNoIterations = -1;                   // kMode of a call without iterations
 constexpr unsigned int kSoloMaxGrid = 160;
 constexpr unsigned int kResidentTiles = 160;       // slots a CTA can have: 200 KB
 constexpr size_t kSlotBytes = 24;                  // three numbers of one CTA and pass
@@ -285,7 +283,7 @@ __device__ __forceinline__ void clear_tile_padding(const Params& p, unsigned int
 }
 
 template <int kMode, int kPlace>
-__global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 : kMode) * 32, 1) solo_kernel(const __grid_constant__ SoloArgs a) {
+__global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_constant__ SoloArgs a) {
   extern __shared__ __align__(128) unsigned char tile_slots[];
   __shared__ SoloShared<kPlace, kMode == kNoIterations> sh;
   constexpr bool kRes = kPlace != kStreamed, kCluster = kPlace == kKeptInCluster;
@@ -415,5 +413,145 @@ __global__ void __launch_bounds__(solo_most_warps(kPlace == kKeptInCluster ? 0 :
       a.result->trace_alpha[i] = i == 0 ? static_cast<double>(alpha0) : i <= iters ? sh.trace_alpha[i] : 0.0;
       a.result->trace_sse[i] = (i <= iters && st == 0) ? sh.trace_sse[i] : 0.0;
     }
+  }
+}
+
+// ------------------------------------------------------------------ calls without iterations on larger matrices
+//
+// The max-based rule alone is two light passes with one meeting between them.  As two chained kernels (launch_chained) of
+// 32 warps an SM the boundary is the meeting: no cooperative launch and no arrival to wait for.  Every CTA leaves its
+// numbers in a slot; the second kernel reads all of them at its head, and the CTA that ends last adds up the second
+// pass's and writes the report.
+
+constexpr int kMaxBasedThreads = 1024;
+
+struct __align__(128) MaxBasedShared {
+  static constexpr bool kOrdered = true, kSolo = true, kResident = false, kFinal = true;
+  View view[1];
+  double part[kMaxBasedThreads / 32][2];
+  double red[kMaxBasedThreads / 32][2];
+  float alpha[1];
+  unsigned int amax[1], zeros[1], wide[1];
+  unsigned int start[1], count[1], total;
+  unsigned int slots, per_warp;
+  int tiled_only;
+  unsigned int most, zeros_all, wide_all, arrived;
+};
+
+// A CTA's numbers: sum W^2, error minus sum W^2; the maximum's bits, zero blocks, wide candidates.
+struct MaxBasedSlot {
+  double sumsq, gsum;
+  unsigned int amax, zeros, wide, pad;
+};
+static_assert(sizeof(MaxBasedSlot) <= 2 * kSlotBytes, "the exchange's workspace holds a slot per CTA");
+
+__device__ __forceinline__ MaxBasedSlot* max_based_slots(const SoloArgs& a) { return reinterpret_cast<MaxBasedSlot*>(a.exchange + 256); }
+
+__device__ __forceinline__ void max_based_head(MaxBasedShared& sh, const SoloArgs& a) {
+  extern __shared__ __align__(128) unsigned char tile_slots[];
+  const Params& p = a.m.t[0];
+  const unsigned int tid = threadIdx.x;
+  if (tid == 0) {
+    sh.view[0].packed = p.packed;
+    sh.view[0].scales = p.scales;
+    sh.view[0].state = nullptr;
+    sh.view[0].tiled = a.tiled;
+    sh.amax[0] = sh.zeros[0] = sh.wide[0] = 0u;
+    sh.start[0] = 0u;
+    sh.count[0] = sh.total = p.ntiles;
+    sh.slots = smem_u32(tile_slots);
+    sh.per_warp = kQStages;
+    sh.tiled_only = a.tiled_only;
+    sh.most = sh.zeros_all = sh.wide_all = 0u;
+  }
+  if (tid < kMaxBasedThreads / 32) sh.part[tid][0] = sh.part[tid][1] = 0.0;
+  __syncthreads();
+  after_previous();
+}
+
+// Sum of the CTAs' numbers `of(slot)`, the same bits in every thread: warp w adds slots 32 w .. 32 w + 31.
+template <typename Of>
+__device__ __forceinline__ double max_based_sum(MaxBasedShared& sh, int which, Of of) {
+  const unsigned int tid = threadIdx.x, grid = gridDim.x, warps = (grid + 31) / 32;
+  if (tid < warps * 32) {
+    const double v = warp_sum(tid < grid ? of(tid) : 0.0);
+    if ((tid & 31u) == 0) sh.red[tid >> 5][which] = v;
+  }
+  __syncthreads();
+  double v = 0.0;
+  for (unsigned int w = 0; w < warps; ++w) v += sh.red[w][which];
+  return v;
+}
+
+__global__ void __launch_bounds__(kMaxBasedThreads, 1) max_based_amax_kernel(const __grid_constant__ SoloArgs a) {
+  __shared__ MaxBasedShared sh;
+  max_based_head(sh, a);
+  let_next_begin();
+  if (a.tiled != nullptr) clear_tile_padding(a.m.t[0], a.rows, a.tiled);
+  amax_pass(sh, a.m);
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double v = warp_sum(sh.part[threadIdx.x][0]);
+    if (threadIdx.x == 0) {
+      MaxBasedSlot& s = max_based_slots(a)[blockIdx.x];
+      s.sumsq = v;
+      s.amax = sh.amax[0];
+      if (blockIdx.x == 0) *reinterpret_cast<unsigned int*>(a.exchange + kCounterAt) = 0u;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kMaxBasedThreads, 1) max_based_codes_kernel(const __grid_constant__ SoloArgs a) {
+  __shared__ MaxBasedShared sh;
+  max_based_head(sh, a);
+  const unsigned int tid = threadIdx.x, grid = gridDim.x;
+  MaxBasedSlot* const slots = max_based_slots(a);
+  unsigned int* const counter = reinterpret_cast<unsigned int*>(a.exchange + kCounterAt);
+  if (tid < grid) atomicMax(&sh.most, __ldcg(&slots[tid].amax));
+  const double sumsq = max_based_sum(sh, 0, [&](unsigned int j) { return __ldcg(&slots[j].sumsq); });
+  const unsigned int amax_bits = sh.most;
+  const int st = status_from_amax(amax_bits);
+  const float alpha = amax_bits == 0 ? 1.0f : __fdiv_rn(bits_to_mag(amax_bits), 2688.0f);
+  const bool go = !(st & (SOAR_STATUS_NONFINITE | SOAR_STATUS_RANGE));
+  sh.alpha[0] = alpha;
+  if (go) init_pass(sh, a.m);
+  let_next_begin();
+  __syncthreads();
+  if (tid < 32) {
+    const double v = warp_sum(sh.part[tid][1]);
+    if (tid == 0) {
+      slots[blockIdx.x].gsum = v;
+      slots[blockIdx.x].zeros = sh.zeros[0];
+      slots[blockIdx.x].wide = sh.wide[0];
+      __threadfence();
+      sh.arrived = atomicAdd(counter, 1u);
+    }
+  }
+  __syncthreads();
+  if (sh.arrived != grid - 1) return;
+  // the last CTA: the report
+  __threadfence();
+  if (tid < grid) {
+    atomicAdd(&sh.zeros_all, __ldcg(&slots[tid].zeros));
+    atomicAdd(&sh.wide_all, __ldcg(&slots[tid].wide));
+  }
+  const double gsum = max_based_sum(sh, 1, [&](unsigned int j) { return __ldcg(&slots[j].gsum); });
+  soar_result* const res = a.result;
+  if (tid == 0) *a.alpha = alpha;
+  if (res == nullptr) return;
+  const double sse = st == 0 ? fmax(sumsq + gsum, 0.0) : 0.0;
+  if (tid == 0) {
+    res->status = a.idle ? SOAR_STATUS_INTERNAL : st;
+    res->iters_run = 0;
+    res->alpha = alpha;
+    res->amax = bits_to_mag(amax_bits);
+    res->sse = res->sse_init = sse;
+    res->sumsq = (st & SOAR_STATUS_ZERO_TENSOR) ? 0.0 : sumsq;
+    res->zero_blocks = static_cast<int64_t>(sh.zeros_all);
+    res->wide_candidates = static_cast<int64_t>(sh.wide_all);
+  }
+  if (tid <= SOAR_MAX_ITERS) {
+    res->trace_alpha[tid] = tid == 0 ? static_cast<double>(alpha) : 0.0;
+    res->trace_sse[tid] = tid == 0 ? sse : 0.0;
   }
 }
