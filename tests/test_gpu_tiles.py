@@ -57,3 +57,50 @@ def test_a_cluster_call_replays_and_repeats(rows, cols):
         assert torch.equal(out.packed, want.packed) and torch.equal(out.scales, want.scales)
         assert torch.equal(out.alpha, want.alpha)
         assert out.read_result().sse == want.read_result().sse
+
+
+# one warp tile is 32 blocks of 16: a lone block, a ragged tile, a whole one, one block more, more tiles than warps of a device
+EDGES = [(1, 16), (1, 16 * 31), (2, 16 * 16), (3, 16 * 11), (1, 16 * 4097), (9, 16 * 8421)]
+
+
+@pytest.mark.parametrize("rows,cols", EDGES)
+@pytest.mark.parametrize("ld_extra", [0, 8])
+@pytest.mark.parametrize("cfgkw", [dict(max_iters=2), dict(max_iters=1, early_stop_rel=0.0, n_dq=2, n_beta=1)])
+def test_weighted_calls_at_the_edges_of_a_tile(rows, cols, ld_extra, cfgkw):
+    w = WL.small_case(rows, cols, cols, outlier_entry_frac=0.002, outlier_scale=30.0)
+    h = WL.column_weights(cols, rows)
+    cfg, ref_cfg = P.cfg_pair(**cfgkw)
+    out = api.soar_quantize_weighted(P.to_device(w, cols + ld_extra), torch.from_numpy(h).cuda(), cfg)
+    torch.cuda.synchronize()
+    gpu = P.GpuOut(out.packed.cpu().numpy(), out.scales.cpu().numpy(), float(out.alpha.cpu()[0]), out.read_result(), out)
+    P.assert_parity(gpu, R.quantize(w, ref_cfg, h=h), mismatch_cap=max(1, w.size // 160000))
+
+
+# one warp tile is 16 blocks of 32
+@pytest.mark.parametrize("rows,cols", [(1, 32), (1, 32 * 15), (2, 32 * 8), (1, 32 * 17), (1, 32 * 2049), (9, 32 * 4211)])
+@pytest.mark.parametrize("ld_extra", [0, 8])
+@pytest.mark.parametrize("cfgkw", [dict(n_beta=0), dict(), dict(n_dq=1, n_beta=5)])
+def test_mxfp4_calls_at_the_edges_of_a_tile(rows, cols, ld_extra, cfgkw):
+    w = WL.small_case(rows, cols, cols)
+    out = api.soar_mx_quantize(P.to_device(w, cols + ld_extra), **cfgkw)
+    torch.cuda.synchronize()
+    ref, res = R.mx_quantize(w, **cfgkw), out.read_result()
+    bad = (out.packed.cpu().numpy() != ref.packed).reshape(rows, cols // 32, 16).any(axis=2) | (out.scales.cpu().numpy() != ref.scales)
+    assert not (bad & ~ref.tie_flags.astype(bool)).any() and bad.sum() <= max(1, bad.size // 10000)
+    assert res.sse == pytest.approx(ref.sse, rel=P.SSE_RTOL) and res.sumsq == pytest.approx(ref.sumsq, rel=1e-12)
+
+
+@pytest.mark.parametrize("rows,cols", EDGES + [(127, 16 * 5), (129, 16 * 4)])
+@pytest.mark.parametrize("ld_extra", [0, 8])
+def test_error_check_at_the_edges_of_a_tile(rows, cols, ld_extra):
+    w = WL.small_case(rows, cols, cols)
+    h = WL.column_weights(cols, rows)
+    W, H = P.to_device(w, cols + ld_extra), torch.from_numpy(h).cuda()
+    cfg = api.soar_default_cfg(api.PRESET_SINGLE_PASS, scale_layout=api.SCALES_LINEAR | api.SCALES_SWIZZLED)
+    b = api.soar_quantize(W, cfg)
+    packed, scales, alpha = b.packed.cpu().numpy(), b.scales.cpu().numpy(), float(b.alpha.cpu()[0])
+    for layout, sc in ((api.SCALES_LINEAR, b.scales), (api.SCALES_SWIZZLED, b.scales_sw)):
+        for e, want in ((api.soar_dequant_error(W, b.packed, sc, b.alpha, layout), R.dequant_error(w, packed, scales, alpha)),
+                        (api.soar_dequant_error_weighted(W, H, b.packed, sc, b.alpha, layout),
+                         R.dequant_error(w, packed, scales, alpha, h=h))):
+            assert e.cpu().numpy() == pytest.approx(np.array(want), rel=1e-11)    # the oracle adds term after term
