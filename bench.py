@@ -130,18 +130,18 @@ def kernel_bytes_per_elem(name: str, cfg, t: int = 0) -> float:
     return 0.0
 
 
-# DRAM bytes per element (dram__bytes_read.sum + dram__bytes_write.sum of one launch, ncu, config 5:
+# DRAM bytes per element (dram__bytes_read.sum + dram__bytes_write.sum of one stage's launch, ncu, config 5:
 # profiles/single_pass_kernels_config5.md, profiles/iterate_kernel_paper_config5.md and
 # profiles/weighted_iterate_kernel_config5.md).  Traffic grows in
 # proportion to the elements, so a launch's traffic is this figure times its elements.  The figures
 # belong to one version of the kernels: they are dropped when the device part of the source (everything above
-# the host-side section of soar.cu) no longer matches.
+# the host-side section of soar.cu, and the kernel headers) no longer matches.
 NCU_TRAFFIC = {
-    "kernel_source_sha256_16": "01bec268fb069bbc",
-    "bytes_per_elem": {"amax_kernel": 2.02, "init_kernel": 2.44, "iterate_kernel/single": 3.01,
-                       "iterate_kernel/grid": 3.47, "weighted_iterate_kernel": 4.57},
-    "inst_per_block": {"amax_kernel": 125, "init_kernel": 218, "iterate_kernel/single": 258,
-                       "iterate_kernel/grid": 490, "weighted_iterate_kernel": 1204},
+    "kernel_source_sha256_16": "",
+    "bytes_per_elem": {"amax_kernel": 2.02, "init_kernel": 2.45, "iterate_kernel/single": 3.01,
+                       "iterate_kernel/grid": 3.45, "weighted_iterate_kernel": 3.48},
+    "inst_per_block": {"amax_kernel": 87, "init_kernel": 186, "iterate_kernel/single": 258,
+                       "iterate_kernel/grid": 361, "weighted_iterate_kernel": 760},
 }
 
 
@@ -149,17 +149,30 @@ HOST_MARKER = b"// -------------------------------------------------------------
 
 
 def kernel_source_hash() -> str | None:
-    """sha256 (16 hex digits) of the device part of soar.cu: everything above the host-side section."""
-    src = os.path.join(ROOT, "paper_2605_12245_b200", "csrc", "soar.cu")
+    """sha256 (16 hex digits) of the device code: soar.cu above the host-side section, then the kernel headers by name."""
+    import glob
     import hashlib
+    csrc = os.path.join(ROOT, "paper_2605_12245_b200", "csrc")
     try:
-        with open(src, "rb") as f:
+        with open(os.path.join(csrc, "soar.cu"), "rb") as f:
             text = f.read()
+        if HOST_MARKER not in text:
+            return None
+        digest = hashlib.sha256(text.split(HOST_MARKER)[0])
+        for name in sorted(glob.glob(os.path.join(csrc, "*.cuh"))):
+            with open(name, "rb") as f:
+                digest.update(f.read())
     except OSError:
         return None
-    if HOST_MARKER not in text:
-        return None
-    return hashlib.sha256(text.split(HOST_MARKER)[0]).hexdigest()[:16]
+    return digest.hexdigest()[:16]
+
+
+def kernel_launches_per_step(n_tensors: int, batched: bool, cfg, elements_each) -> int:
+    """Launches of an untraced step: one for a call over up to 16 tensors; a call on one tensor without iterations
+    takes two where the tensor has more than 768 tiles of 512 elements."""
+    if batched and n_tensors > 1:
+        return (n_tensors + 15) // 16
+    return sum(2 if cfg.max_iters == 0 and e > 768 * 512 else 1 for e in elements_each)
 
 
 def _profile_key(name: str, cfg) -> str:
@@ -385,15 +398,16 @@ def run_ours(args):
     host_ms = []
     sampler = ClockSampler(local)
     sampler.start()
-    # headline: K steps with nothing between the kernels; then the same K steps again with an
-    # event pair around every kernel (which costs a few microseconds per launch) for the shares
+    # headline: K steps as a user makes them, all passes of a call in one launch; then the same K steps again with
+    # every pass a launch of its own between two events (which costs a few microseconds each) for the shares
     ms, _ = timed(step, args.steps, args.warmup, trace=False)
     traced_ms, trace = timed(eager_step if args.graph else step, args.steps, 0, trace=True)
     clocks = sampler.stop()
     results = [o.read_result() for o in outs]
     iters = [r.iters_run for r in results]
     value = world * 2.0 * elements / (ms * 1e-3) / 1e9
-    launches = sum(v[0] for v in trace.values())
+    launches = args.steps * kernel_launches_per_step(len(wl.tensors), not args.no_batch, cfg,
+                                                     [t.rows * t.cols for t in wl.tensors])
 
     # ---- the timed batch's outputs against one soar_quantize call per tensor (same bytes expected)
     bad = []
@@ -580,7 +594,7 @@ def run_ours(args):
         dist.destroy_process_group()
 
 
-WEIGHTED_STATE_BYTES = 17.0 / 16    # {A, B} in binary64 and the scale code per 16-element block
+WEIGHTED_STATE_BYTES = 0.5          # 8 bytes per 16-element block
 
 
 def weighted_kernel_bytes_per_elem(name: str, cfg, t: int = 0) -> float:
@@ -672,7 +686,7 @@ def run_weighted(args):
     results = [o.read_result() for o in outs]
     iters = [r.iters_run for r in results]
     value = world * 2.0 * elements / (ms * 1e-3) / 1e9
-    launches = sum(v[0] for v in trace.values())
+    launches = args.steps * (len(wl.tensors) if args.no_batch else (len(wl.tensors) + 15) // 16)
     dom = max(trace, key=lambda k: trace[k][1])
     n_launch, tot_ms = trace[dom]
     it_bytes = sum(s.rows * s.cols * weighted_kernel_bytes_per_elem("weighted_iterate_kernel", cfg, t)

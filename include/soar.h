@@ -71,7 +71,7 @@ extern "C" {
                                           sums of Eq. 5 and of the error are binary64 additions in the order
                                           the thread blocks finish, so their last bits, and through alpha in
                                           rare cases a code, can differ between runs.  With this flag every
-                                          thread block stores its sums in a slot of its own and the next kernel
+                                          thread block stores its sums in a slot of its own and the next pass
                                           adds the slots in a fixed order.  Needs 56 KB more workspace per
                                           matrix (soar_workspace_bytes accounts for it).  soar_quantize,
                                           soar_quantize_batch, soar_quantize_host and the pipeline only:
@@ -99,7 +99,7 @@ typedef struct soar_cfg {
   int32_t flags;          /* SOAR_FLAG_* bits; 0 = Algorithm 1                              */
 } soar_cfg;
 
-/* Per-call report (device memory, written by the last kernel of soar_quantize). */
+/* Per-call report (device memory, written by the last pass of soar_quantize). */
 typedef struct soar_result {
   int32_t status;                           /* SOAR_STATUS_* bits                            */
   int32_t iters_run;                        /* iterations of Algorithm 1 executed            */
@@ -124,8 +124,9 @@ int soar_default_cfg(soar_cfg* cfg, int preset);
 
 /* Bytes of device scratch soar_quantize needs for this shape and cfg (0 on bad arguments).
  * It is a small fixed part for the tensor-wide sums of Eq. 5; 8 bytes per block of state
- * carried between iterations when cfg->max_iters > 0; and, when cfg->scale_layout lacks
- * SOAR_SCALES_LINEAR, rows*cols/16 bytes for the row-major scales the loop works on. */
+ * carried between iterations when cfg->max_iters > 0; when cfg->scale_layout lacks
+ * SOAR_SCALES_LINEAR, rows*cols/16 bytes for the row-major scales the loop works on; and at most
+ * 8 KB in which the thread blocks leave their sums for each other. */
 size_t soar_workspace_bytes(int64_t rows, int64_t cols, const soar_cfg* cfg);
 
 /* Bytes of the swizzled scale buffer: scales padded to multiples of 128 rows and 4 columns. */
@@ -176,10 +177,9 @@ size_t soar_batch_workspace_bytes(const soar_tensor_desc* tensors, int n, const 
 
 /*
  * Algorithm 1 on n independent matrices with shared settings; every matrix gets exactly the
- * outputs soar_quantize would give it.  The matrices' tiles are walked as one sequence by the
- * same kernels (up to 16 matrices per launch), so a model's many small matrices cost a few
- * launches per group instead of a few per matrix; matrices that stop early (Sec. 4.1) drop
- * out of later iterations on their own.  `tensors` is host memory (n descriptors, read before
+ * outputs soar_quantize would give it.  The matrices' tiles are walked as one sequence by one
+ * kernel (up to 16 matrices per launch), so a model's many small matrices share its passes;
+ * matrices that stop early (Sec. 4.1) drop out of later iterations on their own.  `tensors` is host memory (n descriptors, read before
  * the call returns); `workspace` is device scratch of soar_batch_workspace_bytes(), 256-byte
  * aligned.  Argument errors of any matrix are returned before anything is enqueued.
  */
@@ -337,15 +337,15 @@ int soar_dequant_error(const void* W_bf16, int64_t rows, int64_t cols, int64_t l
  *               SOAR_STATUS_BAD_WEIGHT in out_result->status and the outputs are unspecified.
  *               Only ratios between weights matter to the minimiser.
  *   workspace   device, 256-byte aligned, >= soar_weighted_workspace_bytes(rows, cols, cfg):
- *               2 KB of accumulators plus, when max_iters > 0, 17 bytes per block (A and B in
- *               binary64 and the stored scale code), plus rows*cols/16 bytes when the row-major
+ *               2 KB of accumulators plus, when max_iters > 0, 17 bytes per block (of which the
+ *               state carried between iterations uses 8), plus rows*cols/16 bytes when the row-major
  *               scale layout is not requested.
  * Every other argument, the stream semantics, ownership and the error codes are those of
  * soar_quantize.  The block sums are accumulated in binary64 in element order, so the pass is
  * bound by arithmetic, not by HBM, even with one candidate.
  *
  * soar_quantize_weighted_batch is the same on n independent matrices with shared settings, walked
- * by the same kernels (up to 16 matrices per launch) like soar_quantize_batch: `tensors` and
+ * by one kernel (up to 16 matrices per launch) like soar_quantize_batch: `tensors` and
  * `col_weights` are host arrays of n entries (col_weights[i]: the device vector of matrix i's
  * `cols` weights), `workspace` is device scratch of soar_weighted_batch_workspace_bytes() (the sum
  * of soar_weighted_workspace_bytes over the matrices), 256-byte aligned.  Every matrix gets exactly
@@ -398,7 +398,7 @@ typedef struct soar_mx_result {
   int32_t status;            /* SOAR_STATUS_* bits                                              */
   uint32_t amax_bits;        /* bf16 bit pattern of max |W|                                     */
   float amax;                /* max |W|                                                         */
-  int32_t pad_;
+  int32_t pad_;              /* internal                                                        */
   double sse;                /* sum (W - What)^2                                                */
   double sumsq;              /* sum W^2                                                         */
   double reserved;           /* internal: sse - sumsq before clamping                           */
@@ -424,8 +424,8 @@ int soar_mx_quantize(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld,
  *     soar_quantize.
  *   - The first call on each device looks up the array's device address (with that device
  *     current) before it enqueues anything; make that first call outside any stream capture.
- *   - There is one array per device, shared by every call and every stream.  The call
- *     clears the part that must start at zero, so leftovers of earlier calls do no harm,
+ *   - There is one array per device, shared by every call and every stream.  Leftovers of
+ *     earlier calls do no harm,
  *     but two calls that overlap on the GPU (different streams, no ordering) race on it
  *     and give unspecified results: order them, or use soar_quantize with separate
  *     workspaces.
@@ -437,13 +437,14 @@ int soar_quantize_static(const void* W_bf16, int64_t rows, int64_t cols, int64_t
                          void* out_e4m3_scales_sw, float* out_global_fp32,
                          soar_result* out_result, void* stream);
 
-/* Number of kernels soar_quantize enqueues for this cfg (host-side bookkeeping for callers
- * that count launches); 0 on bad arguments. */
+/* Number of stages of a soar_quantize call for this cfg: the launches of a call that runs them one by
+ * one (soar_quantize_stage, or while a trace is on), the tiled scale layout's included.  Any other call
+ * runs all of them in one launch (two for a large matrix without iterations).  0 on bad arguments. */
 int soar_quantize_launches(const soar_cfg* cfg);
 
 /* Launch tracing for benchmarks (no counterpart in the paper).  Between soar_trace_begin()
- * and soar_trace_end(), every kernel the library launches is bracketed by two CUDA events on
- * its stream.  soar_trace_end() waits for those events and writes, per kernel name, the
+ * and soar_trace_end(), a call enqueues each of its stages as a launch of its own, named after the
+ * stage and bracketed by two CUDA events on its stream; outputs are the same.  soar_trace_end() waits for those events and writes, per kernel name, the
  * number of launches and the summed device time in milliseconds into out[0..capacity)
  * (host); *count receives the number of distinct kernels seen.  Process-wide, not re-entrant. */
 typedef struct soar_trace_entry {
@@ -467,12 +468,13 @@ int soar_selftest_reciprocal(int lo_exp, int hi_exp, unsigned long long* out_mis
 
 /*
  * Test hook for the kernels' bounded waits (no counterpart in the paper).  Every wait inside a
- * kernel (a consumer warp waiting for the tile its producer fetches) counts its polls and gives
+ * kernel (thread blocks waiting for each other between two passes) counts its polls and gives
  * up at a limit; the call then reports SOAR_STATUS_INTERNAL instead of hanging.  While the hook
- * is on, kernels launched afterwards fetch no tiles at all, so their consumers' waits run to
- * the limit (a quarter of a million polls, about a second per kernel) with no copy in flight:
- * the pass kernels then return, the remaining kernels of the call return at once,
- * soar_result.status carries SOAR_STATUS_INTERNAL and the outputs are unspecified.  on = 0
+ * is on, the thread blocks of kernels launched afterwards do not arrive where they meet, so the
+ * waits run to the limit (two million polls, a second or two per kernel) with no copy in flight
+ * and the kernel returns: the status carries SOAR_STATUS_INTERNAL (the sums of
+ * soar_dequant_error are NaN) and the outputs are unspecified.  (A matrix of at most 256 blocks
+ * runs in one thread block, which has nobody to wait for.)  on = 0
  * restores normal operation.  Process-wide; not for production use.
  */
 int soar_debug_fail_waits(int on);

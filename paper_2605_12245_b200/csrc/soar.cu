@@ -1,25 +1,21 @@
 // SOAR NVFP4 weight quantizer for NVIDIA B200 (sm_100a): kernels and the C ABI of soar.h.
 //
-// What runs on the device, in launch order (Algorithm 1 of the SOAR paper):
-//   amax_kernel      tensor-wide max |W|, sum W^2 and a non-finite check        (Eq. 1)
-//   init_kernel      max-based scales, first codes, first tensor sums          (Eq. 1-2, Alg. 1 "Initialization")
-//   iterate_kernel   T times: global scale (Eq. 5) from the previous kernel's sums, block
-//                    scale (Eq. 6), candidate search (Eq. 8, App. B.3), winners stored,
-//                    next sums accumulated
-//   finalize_kernel  early-stop bookkeeping (Sec. 4.1), alpha and the report
-//   swizzle_kernel   optional 128x4-tiled copy of the block scales
+// What runs on the device, in order (Algorithm 1 of the SOAR paper), as passes over W:
+//   amax       tensor-wide max |W|, sum W^2 and a non-finite check               (Eq. 1)
+//   init       max-based scales, first codes, first tensor sums                  (Eq. 1-2, Alg. 1 "Initialization")
+//   iterate    T times: global scale (Eq. 5) from the previous pass's sums, block scale (Eq. 6), candidate search
+//              (Eq. 8, App. B.3), winners stored, next sums accumulated
+//   report     early-stop bookkeeping (Sec. 4.1), alpha and the report; a 128x4-tiled copy of the scales if asked for
 //
-// Batches.  Every kernel works on up to 16 matrices at once: their tiles form one sequence
-// walked by one persistent grid, so a model's many small matrices share launches; a single
-// matrix is a batch of one.  Matrices that have stopped early drop out of later iterations.
+// Launches.  A pass cannot begin before the sums of the one before are known to every CTA, so the passes of a call run in
+// one persistent cooperative kernel whose CTAs meet between them: solo_kernel for one matrix, quantize_kernel for up to
+// 16 matrices at once, whose tiles form one sequence walked by the whole grid, so that a model's many small matrices
+// share passes; matrices that have stopped early drop out of later ones.  Small matrices run in one cluster, calls
+// without iterations on large ones in two chained kernels (see solo_kernel.cuh).  A staged or traced call enqueues each
+// stage as a launch of its own (the names in a trace are the stages').
 //
-// Data movement.  The three passes over W are persistent, warp-specialised kernels: each CTA
-// walks tiles of 256 blocks (8 KB of bf16).  One thread of a producer warp fetches them with
-// bulk asynchronous copies (cp.async.bulk, completion on a "full" mbarrier) into a
-// four-stage shared-memory ring; 256 consumer threads, one per 16-element block, pull their
-// 32 bytes into registers, hand the stage back through an "empty" mbarrier and work from
-// registers, so no CTA-wide barrier sits in the tile loop and the copies of the next tiles
-// are always in flight.
+// Data movement.  Every warp feeds itself with tiles of 32 blocks (1 KB of bf16), in registers or through its own slots
+// of shared memory (see quantize_kernel.cuh).
 //
 // State between iterations is 8 bytes per block in the workspace: the winner's
 // A = sum |W| m (binary32, exact), 4B = sum (2m)^2 and its E4M3 scale code.  That is all
@@ -33,12 +29,8 @@
 // the block maximum times the reciprocal scale is at most 32; otherwise a binary64 path is
 // taken.  Tensor sums and candidate comparisons are binary64.
 //
-// Column-weighted objective (Sec. 5 in diagonal form; soar_quantize_weighted): the same passes as
-// weighted_amax_kernel, weighted_init_kernel and weighted_iterate_kernel (batched like the others).
-// Block sums carry a binary32 weight per column, so they are binary64 sums in element order
-// (17 bytes of state per block); the candidate loop ranks on exact integer sums over
-// fixed-point images of the weighted magnitudes and falls back to binary64 sums only for
-// blocks where the images' rounding could change the winner.
+// Column-weighted objective (Sec. 5 in diagonal form; soar_quantize_weighted): the same stages with passes of their own,
+// whose block sums are binary64 (see weighted_kernel.cuh).
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -87,7 +79,7 @@ constexpr unsigned int kErrWeight = 2u;   // a column weight outside the accepte
 
 // Deterministic reduce mode (SOAR_FLAG_DETERMINISTIC): instead of adding its sums to the tensor's
 // accumulators with atomics (in arrival order), every CTA of a pass stores them in a slot of its
-// own, and the head of the next kernel adds the slots in index order.  Two stage buffers alternate
+// own, and the head of the next stage adds the slots in index order.  Two stage buffers alternate
 // so that a pass can fill one while late CTAs of it still read the other.
 constexpr int kMaxGrid = 1024;   // no pass has more CTAs (SM count x occupancy, at most 6 per SM)
 struct DetParts {
@@ -121,7 +113,7 @@ struct Params {
 constexpr int kMaxBatch = 16;
 struct Batch {
   int n;
-  int idle_producer;          // test hook: no CTA arrives anywhere, so every wait runs out
+  int idle;                   // test hook: no CTA arrives anywhere, so every wait runs out
   Params t[kMaxBatch];
 };
 // The same for one tensor (a smaller parameter block makes a cheaper launch).
@@ -564,8 +556,8 @@ struct ScopedLaunch {
 
 int g_sm_count[64];
 
-// Test hook (soar_debug_fail_waits): what the launches put into Batch::idle_producer.
-int g_idle_producer = 0;
+// Test hook (soar_debug_fail_waits): what the launches put into Batch::idle and its like.
+int g_idle = 0;
 
 int sm_count() {
   int dev = 0;
@@ -934,7 +926,7 @@ int run_solo(const soar_tensor_desc& d, const soar_cfg* cfg, uint8_t* workspace,
   a.nonce = call_nonce();
   a.rows = static_cast<unsigned int>(d.rows);
   a.tiled_only = want_lin ? 0 : 1;
-  a.idle = g_idle_producer;
+  a.idle = g_idle;
   const unsigned int sms = static_cast<unsigned int>(sm_count());
   // (the test hook makes the waits of the counter run out; a cluster's barrier is the hardware's)
   const bool cluster = p.ntiles > kOneCtaTiles && p.ntiles <= kClusterTiles && !a.idle && clusters_fit();
@@ -1021,7 +1013,7 @@ int run_batch(const soar_tensor_desc* tensors, int n, const soar_cfg* cfg, void*
     memset(&bt, 0, sizeof(bt));
     memset(&rp, 0, sizeof(rp));
     bt.n = (n - first < kMaxBatch) ? n - first : kMaxBatch;
-    bt.idle_producer = g_idle_producer;
+    bt.idle = g_idle;
     unsigned int tiles = 0;
     for (int j = 0; j < bt.n; ++j) {
       const soar_tensor_desc& d = tensors[first + j];
@@ -1203,7 +1195,7 @@ int dequant_error_impl(const void* W_bf16, int64_t rows, int64_t cols, int64_t l
   a.sse = out_sse;
   a.sumsq = out_sumsq;
   a.tiled = scale_layout == SOAR_SCALES_SWIZZLED ? 1 : 0;
-  a.idle = g_idle_producer;
+  a.idle = g_idle;
   // the two sums start at zero (a kernel of ours rather than a memset, so that the next one can be chained to it)
   ScopedLaunch sl(K_DEQUANT_ERROR, st);
   cudaError_t err = launch_chained(clear_sums_kernel, 1, 32, 0, 0, st, out_sse, out_sumsq);
@@ -1293,7 +1285,7 @@ int soar_quantize_weighted_batch(const soar_tensor_desc* tensors, const float* c
     memset(&wt, 0, sizeof(wt));
     memset(&rp, 0, sizeof(rp));
     bt.n = (n - first < kMaxBatch) ? n - first : kMaxBatch;
-    bt.idle_producer = g_idle_producer;
+    bt.idle = g_idle;
     unsigned int tiles = 0;
     for (int j = 0; j < bt.n; ++j) {
       const soar_tensor_desc& d = tensors[first + j];
@@ -1608,7 +1600,7 @@ int soar_mx_quantize(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld,
   a.n_dq = n_dq;
   a.n_beta = n_beta;
   a.step_pct = beta_step_pct;
-  a.idle = g_idle_producer;
+  a.idle = g_idle;
   ScopedLaunch sl(K_MX, st);
   cudaError_t err;
   if (n_beta == 0) err = launch_mx<0>(a, st);
@@ -1620,7 +1612,7 @@ int soar_mx_quantize(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld,
 }
 
 int soar_debug_fail_waits(int on) {
-  g_idle_producer = on ? 1 : 0;
+  g_idle = on ? 1 : 0;
   return SOAR_OK;
 }
 
