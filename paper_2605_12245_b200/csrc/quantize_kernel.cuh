@@ -599,9 +599,13 @@ __device__ __forceinline__ void load_resident(const B& bt, unsigned int slots, u
 // looks), its 32 bytes and, with kState, its block state, and calls next() once it is done with these registers;
 // state_at is where a resident block keeps its state in shared memory.  kRing: tiles
 // come through the warp's slots in shared memory, three ahead; else through registers, one ahead.  The warp
-// number is broadcast so that the compiler sees the bookkeeping as uniform.
-template <bool kRing, bool kState, typename S, typename B, typename Enter, typename Leave, typename Body>
-__device__ __forceinline__ void walk_tiles(S& sh, const B& bt, bool reverse, Enter enter, Leave leave, Body body) {
+// number is broadcast so that the compiler sees the bookkeeping as uniform.  `fed()` is called once by every warp when
+// the copies of its first tiles are on their way; the walk ends there if it returns false.
+struct Go {
+  __device__ __forceinline__ bool operator()() const { return true; }
+};
+template <bool kRing, bool kState, typename S, typename B, typename Enter, typename Leave, typename Body, typename Fed = Go>
+__device__ __forceinline__ void walk_tiles(S& sh, const B& bt, bool reverse, Enter enter, Leave leave, Body body, Fed fed = Fed()) {
   if constexpr (S::kResident) {
     walk_resident<kState>(sh, bt, enter, leave, body);
     return;
@@ -692,6 +696,10 @@ __device__ __forceinline__ void walk_tiles(S& sh, const B& bt, bool reverse, Ent
     }
   } else {
     feed_registers(v0, v1, st);
+  }
+  if (!fed()) {
+    copies_wait<0>();
+    return;
   }
   Run r;
   r.ti = -1;
@@ -866,8 +874,8 @@ __device__ __forceinline__ void amax_pass(S& sh, const B& bt) {
 // Algorithm 1 "Initialization" (Eq. 1): dd0 = E4M3(bmax/(6 alpha0)), dq0 = dd0; first codes (Eq. 2); stage-0 sums for
 // Eq. 5 and the starting error.  Codes and scales are written here only when no iteration follows, the block states only when
 // one does.
-template <typename S, typename B>
-__device__ __forceinline__ void init_pass(S& sh, const B& bt) {
+template <typename S, typename B, typename Fed = Go>
+__device__ __forceinline__ void init_pass(S& sh, const B& bt, Fed fed = Fed()) {
   float alpha = 1.0f, six_alpha = 6.0f, six_inv = 0.0f;
   double alpha_d = 1.0;
   bool tame = false;
@@ -953,7 +961,8 @@ __device__ __forceinline__ void init_pass(S& sh, const B& bt) {
         // v^2 4B is exact in binary32: 8 + 12 significant bits (no Eq. 5 follows the last pass)
         if (!S::kFinal) acc[0] += static_cast<double>(__fmul_rn(__fmul_rn(v, v), __uint2float_rn(f.b4)));
         acc[1] += f.g;
-      });
+      },
+      fed);
 }
 
 // One iteration of Algorithm 1 for every block: Eq. 6 with the new alpha, App. B.3 candidate sets, Eq. 8 search,
