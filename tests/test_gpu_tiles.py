@@ -77,7 +77,7 @@ def test_weighted_calls_at_the_edges_of_a_tile(rows, cols, ld_extra, cfgkw):
 
 
 # one warp tile is 16 blocks of 32
-@pytest.mark.parametrize("rows,cols", [(1, 32), (1, 32 * 15), (2, 32 * 8), (1, 32 * 17), (1, 32 * 2049), (9, 32 * 4211)])
+@pytest.mark.parametrize("rows,cols", [(1, 32), (1, 32 * 15), (2, 32 * 8), (1, 32 * 17), (1, 32 * 2049), (9, 32 * 4211), (3, 32 * 18945)])
 @pytest.mark.parametrize("ld_extra", [0, 8])
 @pytest.mark.parametrize("cfgkw", [dict(n_beta=0), dict(), dict(n_dq=1, n_beta=5)])
 def test_mxfp4_calls_at_the_edges_of_a_tile(rows, cols, ld_extra, cfgkw):
