@@ -21,8 +21,8 @@
 // so it is a rounding midpoint exactly or misses it by 2^-8, far more than the band's 2^-21; the successor's codes are then
 // nearest ones, ties either way, its error is the least there is, and only an earlier multiplier can share the first place.
 //
-// Bound by instruction issue, 380 a lane of sixteen elements: 28672 x 8192 with the search 665 -> 219 us (594 MB: 2.7 TB/s),
-// by the plain rule 200 -> 123 us.
+// Bound by instruction issue, 373 a lane of sixteen elements in 70 % of the cycles: 28672 x 8192 with the search 665 -> 216 us
+// (594 MB: 2.7 TB/s), by the plain rule (211 instructions) 200 -> 123 us.
 
 #pragma once
 
