@@ -1064,25 +1064,26 @@ cudaError_t run_solo(const soar_tensor_desc& d, const soar_cfg* cfg, uint8_t* wo
 // The MXFP4 pass.  Up to a tile a warp the call is bound by the host's launches (7.1 us in one, 8.7 in two) and the pass
 // clears its result itself; cooperative, because its CTAs then wait for CTA 0.  From there on two chained launches are
 // shorter on the device.
-template <int kSearch>
+template <int kSearch, bool kPlain>
 cudaError_t launch_mx(MxArgs& a, cudaStream_t st) {
   static std::atomic<int> known[64];
   unsigned int per_sm = 1;
-  const unsigned int grid = stage_grid(mx_kernel<kSearch>, known, a.m.t[0].ntiles, &per_sm);
+  const unsigned int tiles = (a.m.t[0].nblk / 2 + 31) / 32;   // a block of 32 a lane
+  const unsigned int grid = stage_grid(mx_kernel<kSearch, kPlain>, known, tiles, &per_sm);
   auto chained = [&]() {
     a.chained = 1;
     const cudaError_t err = launch_chained(clear_mx_kernel, 1, 32, 0, 0, st, a.res);
-    return err != cudaSuccess ? err : launch_chained(mx_kernel<kSearch>, grid, kQThreads, 0, 0, st, a);
+    return err != cudaSuccess ? err : launch_chained(mx_kernel<kSearch, kPlain>, grid, kQThreads, 0, 0, st, a);
   };
-  if (a.m.t[0].ntiles > grid * kQWarps) return chained();
+  if (tiles > grid * kQWarps) return chained();
   a.tag = call_nonce();
   if (grid == 1) {
-    mx_kernel<kSearch><<<1, kQThreads, 0, st>>>(a);
+    mx_kernel<kSearch, kPlain><<<1, kQThreads, 0, st>>>(a);
     return cudaGetLastError();
   }
   void* args[] = {&a};
   const cudaError_t err =
-      launch_cooperative(reinterpret_cast<const void*>(&mx_kernel<kSearch>), grid, per_sm, kQThreads, args, 0, st);
+      launch_cooperative(reinterpret_cast<const void*>(&mx_kernel<kSearch, kPlain>), grid, per_sm, kQThreads, args, 0, st);
   return grid_refused(err) ? chained() : err;
 }
 
@@ -1731,11 +1732,13 @@ int soar_mx_quantize(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld,
   a.idle = g_idle;
   ScopedLaunch sl(K_MX, st);
   cudaError_t err;
-  if (n_beta == 0) err = launch_mx<0>(a, st);
+  // every block of 32 is 64 bytes at a multiple of 32: two 256-bit loads
+  const bool plain = p.contiguous && reinterpret_cast<uintptr_t>(W_bf16) % 32 == 0;
+  if (n_beta == 0) err = plain ? launch_mx<0, true>(a, st) : launch_mx<0, false>(a, st);
   else if (n_dq == 2 && n_beta >= kBracketMinBeta && beta_step_pct >= 1 && beta_step_pct <= 25 &&
            100 - (n_beta / 2) * beta_step_pct <= 50 && (n_beta - 1 - n_beta / 2) >= 1)
-    err = launch_mx<2>(a, st);
-  else err = launch_mx<1>(a, st);
+    err = plain ? launch_mx<2, true>(a, st) : launch_mx<2, false>(a, st);
+  else err = launch_mx<1, false>(a, st);
   return err == cudaSuccess ? SOAR_OK : SOAR_ERR_CUDA;
 }
 

@@ -192,6 +192,35 @@ def test_mxfp4_calls_at_the_edges_of_a_tile(rows, cols, ld_extra, cfgkw):
     assert res.sse == pytest.approx(ref.sse, rel=P.SSE_RTOL) and res.sumsq == pytest.approx(ref.sumsq, rel=1e-12)
 
 
+# a lane has a block of 32: the edges of a warp's 32 blocks, and of a turn of a device's warps over them
+@pytest.mark.parametrize("rows,cols", [(1, 32 * 31), (1, 32 * 32), (3, 32 * 11), (1, 32 * 65), (37, 32 * 2048), (41, 32 * 1849)])
+@pytest.mark.parametrize("offset,ld_extra", [(0, 0), (8, 0), (0, 8)])    # 32-byte aligned, 16-byte aligned, rows apart
+@pytest.mark.parametrize("cfgkw", [dict(n_beta=0), dict()])
+def test_mxfp4_irregular_blocks_between_regular_ones(rows, cols, offset, ld_extra, cfgkw):
+    """Zero, vanishing and very small or large blocks anywhere in a lane's share, the first and the last ones among them."""
+    w = WL.small_case(rows, cols, cols + rows)
+    rng = np.random.default_rng(cols)
+    blocks = w.reshape(-1, 32)
+    n = len(blocks)
+    pick = np.unique(np.concatenate([[0, 30, n - 1], rng.integers(0, n, max(4, n // 50))]))
+    for i, b in enumerate(pick):
+        v = WL.bf16_bits_to_f32(blocks[b]).astype(np.float64)
+        v = v * (0.0, 2.0 ** -118, 2.0 ** -70, 2.0 ** 75)[i % 4]
+        blocks[b] = WL.f32_to_bf16_bits(v.astype(np.float32))
+    ld = cols + ld_extra
+    buf = torch.zeros(rows * ld + offset, dtype=torch.bfloat16, device="cuda")
+    W = buf[offset:offset + rows * ld].view(rows, ld)[:, :cols]
+    W.copy_(P.to_device(w))
+    out = api.soar_mx_quantize(W, **cfgkw)
+    torch.cuda.synchronize()
+    ref, res = R.mx_quantize(w, **cfgkw), out.read_result()
+    bad = (out.packed.cpu().numpy() != ref.packed).reshape(rows, cols // 32, 16).any(axis=2) | (out.scales.cpu().numpy() != ref.scales)
+    assert not (bad & ~ref.tie_flags.astype(bool)).any() and bad.sum() <= max(1, bad.size // 10000)
+    # (the large blocks' terms differ by 2^75 squared from the others': both sides add in binary64)
+    assert res.sse == pytest.approx(ref.sse, rel=P.SSE_RTOL) and res.sumsq == pytest.approx(ref.sumsq, rel=1e-12)
+    assert res.zero_blocks == int((ref.scales == 0).sum())
+
+
 @pytest.mark.parametrize("rows,cols", EDGES + [(127, 16 * 5), (129, 16 * 4)])
 @pytest.mark.parametrize("ld_extra", [0, 8])
 def test_error_check_at_the_edges_of_a_tile(rows, cols, ld_extra):
