@@ -681,20 +681,29 @@ __device__ __forceinline__ void walk_tiles(S& sh, const B& bt, bool reverse, Ent
     }
     if (--f.left == 0) enter_feed();
   };
+  // (registers) Plain tiles left of the feeding run: one check a tile, everything else is out of the loop's way.
+  unsigned int f_quick = 0;
   auto feed_registers = [&](uint4& v0, uint4& v1, uint2& st) {
-    if (f.left == 0) return;
-    if (f_plain) {
-      load_block32(f_w + static_cast<size_t>(f_b) * 32, v0, v1);
-      if (kState) st = load_state(f_state + static_cast<size_t>(f_b) * 8);
-    } else {
-      const Params& p = bt.t[f.ti];
-      if (f_b < p.nblk) {
-        load_block(p, f_b, v0, v1);
-        if (kState) st = load_state(f_state + static_cast<size_t>(f_b) * 8);
+    if (f_quick == 0) {
+      if (f.left == 0) enter_feed();
+      if (f.left == 0) return;
+      if (!f_plain) {
+        const Params& p = bt.t[f.ti];
+        if (f_b < p.nblk) {
+          load_block(p, f_b, v0, v1);
+          if (kState) st = load_state(f_state + static_cast<size_t>(f_b) * 8);
+        }
+        f_b += f_step;
+        --f.left;
+        return;
       }
+      f_quick = f.left;
+      f.left = 0;
     }
+    load_block32(f_w + static_cast<size_t>(f_b) * 32, v0, v1);
+    if (kState) st = load_state(f_state + static_cast<size_t>(f_b) * 8);
     f_b += f_step;
-    if (--f.left == 0) enter_feed();
+    --f_quick;
   };
 
   uint4 v0 = make_uint4(0u, 0u, 0u, 0u), v1 = v0;
@@ -1083,8 +1092,16 @@ __device__ __forceinline__ void iterate_pass(S& sh, const B& bt, bool reverse, u
           // from here to the scaled value (2^-24 each; see winning_range): 6 * 2^-24 does.  Where one of the two lies
           // inside the band, in one block of seven thousand, its neighbour on the other side can win too.
           constexpr float kUnder = 1.0f - 0x1.8p-22f, kOver = 1.0f + 0x1.8p-22f;
-          const bool below0 = a0 <= v0f * kUnder, above0 = b0f >= v0f * kOver;
-          const bool below1 = a1 <= v1f * kUnder, above1 = b1 >= v1f * kOver;
+          // a (1 + margin) - v and b (1 - margin) - v of either code: enclosed when the first is negative and the second is
+          // not (a first one of zero counts as not enclosed: the third multiplier is then looked at without need)
+          const pair_t margins = pair_of(kOver, kUnder);
+          float lo0, hi0, lo1, hi1;
+          halves(pair_fma(pair_of(a0, b0f), margins, pair_of(-v0f, -v0f)), lo0, hi0);
+          halves(pair_fma(pair_of(a1, b1), margins, pair_of(-v1f, -v1f)), lo1, hi1);
+          const bool below0 = __float_as_int(lo0) < 0, above0 = __float_as_int(hi0) >= 0;
+          const bool below1 = __float_as_int(lo1) < 0, above1 = __float_as_int(hi1) >= 0;
+          const bool enclosed =
+              (__float_as_int(lo0) & __float_as_int(lo1) & ~(__float_as_int(hi0) | __float_as_int(hi1))) < 0;
           // Mode 5, where the grid ends before the band does: one multiplier is all that can win, the first one when
           // even its divisor lies beyond the band, the last one when even its divisor lies before it.  The pair then
           // holds that multiplier twice.
@@ -1108,7 +1125,6 @@ __device__ __forceinline__ void iterate_pass(S& sh, const B& bt, bool reverse, u
           halves(n0, s00, s01);
           s_exp = __float_as_uint(s00) & 0x7F800000u;
           // the largest magnitude of the block below 32 times the smallest scale, from the exponents
-          const bool enclosed = below0 && above0 && below1 && above1;
           direct = direct && st.y < s_exp + (5u << 23);
           if (kMode == 5) direct = direct && ((below0 && above0) || low0 || high0) && ((below1 && above1) || low1 || high1);
           if (kMode == 3) direct = direct && enclosed;
@@ -1118,15 +1134,15 @@ __device__ __forceinline__ void iterate_pass(S& sh, const B& bt, bool reverse, u
           const int k_field = static_cast<int>(135u << 20) - static_cast<int>(s_exp >> 3);
           const double h0 = scaled_value(dv0, k_field), h1 = scaled_value(dv1, k_field);
           const double rho0 = alpha_d * h0, rho1 = alpha_d * h1;
-          Candidate x, y2;
+          Candidate x, w2, y2;   // (four scored before any is dropped: independent work for the scheduler)
           float r00, r01, r10, r11;
           pair_recip(n0, r00, r01);
           pair_recip(n1, r10, r11);
           score_pairs(blk, fx, r00, rho0, w);
-          score_pairs(blk, fx, r01, rho0, x);
-          if (x.e < w.e) w = x;
+          score_pairs(blk, fx, r01, rho0, w2);
           score_pairs(blk, fx, r10, rho1, x);
           score_pairs(blk, fx, r11, rho1, y2);
+          if (w2.e < w.e) w = w2;
           if (y2.e < x.e) x = y2;
           if (kMode == 3) {
             float r02, r12;
