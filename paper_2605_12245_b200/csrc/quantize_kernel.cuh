@@ -500,6 +500,10 @@ struct Run {
   int tile, step;
 };
 
+// Warps that share tensor ti's tiles.
+template <typename S>
+__device__ __forceinline__ unsigned int span_of(const S&, int, unsigned int warps) { return warps; }
+
 // The run after `r` (r.ti = -1: the first one); left == 0 when the warp's share of the pass is over.
 template <typename S>
 __device__ __forceinline__ void next_run(const S& sh, int n, bool reverse, unsigned int warp, unsigned int warps, Run& r) {
@@ -508,17 +512,17 @@ __device__ __forceinline__ void next_run(const S& sh, int n, bool reverse, unsig
   if (r.ti < 0) at = -1;
   while (++at < n) {
     const int ti = reverse ? n - 1 - at : at;
-    const unsigned int count = sh.count[ti];
+    const unsigned int count = sh.count[ti], span = span_of(sh, ti, warps);
     unsigned int first = warp;
     if constexpr (!S::kSolo) {
       const unsigned int past = sh.start[ti] % warps;
       first = warp >= past ? warp - past : warp + warps - past;
     }
-    if (first < count) {
+    if (first < count && first < span) {
       r.ti = ti;
-      r.left = (count - 1 - first) / warps + 1;
-      r.tile = static_cast<int>(reverse ? first + (r.left - 1) * warps : first);
-      r.step = reverse ? -static_cast<int>(warps) : static_cast<int>(warps);
+      r.left = (count - 1 - first) / span + 1;
+      r.tile = static_cast<int>(reverse ? first + (r.left - 1) * span : first);
+      r.step = reverse ? -static_cast<int>(span) : static_cast<int>(span);
       return;
     }
   }

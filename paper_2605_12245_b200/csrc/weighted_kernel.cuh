@@ -33,6 +33,22 @@ __device__ __forceinline__ void weights_of(const float* h, unsigned int cb, floa
     hv[4 * q + 3] = v.w;
   }
 }
+// What a CTA shares, and by how many warps each tensor is walked.
+struct __align__(128) WeightedShared : QShared<false> {
+  unsigned int span[kMaxBatch];
+};
+__device__ __forceinline__ unsigned int span_of(const WeightedShared& sh, int ti, unsigned int) { return sh.span[ti]; }
+
+// A lane whose blocks all lie in one block column reads that column's weights once and widens them once (see
+// `column` in the passes), so a tensor is walked by as many warps as make a step a whole number of rows: a multiple of
+// nbc / gcd(nbc, 32) tiles.  4096 and 8192 columns divide the warps of the device's grid as it is (2368 = 64 * 37); 12288 and
+// 28672 columns leave 16 of them out.  Where more than a thirtieth would be left out, or where a tensor has only a few turns, all warps
+// walk it and the weights are read again when the column changes.
+__device__ __forceinline__ unsigned int column_span(const Params& p, unsigned int warps) {
+  const unsigned int unit = p.nbc / min(p.nbc & (0u - p.nbc), 32u), span = warps / unit * unit;
+  return span * 30 >= warps * 29 && p.ntiles >= 8 * warps ? span : warps;
+}
+
 __device__ __forceinline__ bool weight_ok(float h) { return h == 0.0f || (h >= 0x1p-20f && h <= 0x1p20f); }
 
 // Magnitudes of a block in binary64.
@@ -204,10 +220,21 @@ __device__ __noinline__ WeightedFound weighted_search_general(const Params& p, c
 template <typename S>
 __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const Weighted& wt) {
   const unsigned int lane = threadIdx.x & 31u;
-  unsigned int mx = 0, nblk = 0, nbc = 1, magic = 0, shift = 0;
+  unsigned int mx = 0, nblk = 0, nbc = 1, magic = 0, shift = 0, column = 0;
   const float* h = nullptr;
   bool bad = false;
-  double sq[2] = {0.0, 0.0};
+  double sq[2] = {0.0, 0.0}, squares[16];   // sum W^2 of each of the column's sixteen weights since it began
+#pragma unroll
+  for (int j = 0; j < 16; ++j) squares[j] = 0.0;
+  auto end_column = [&]() {
+    float hv[16];
+    weights_of(h, column, hv);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      sq[j & 1] = fma(static_cast<double>(hv[j]), squares[j], sq[j & 1]);
+      squares[j] = 0.0;
+    }
+  };
   walk_tiles<true, false>(
       sh, bt, false,
       [&](int ti) {
@@ -217,8 +244,11 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
         magic = p.nbc_magic;
         shift = p.nbc_shift;
         h = wt.h[ti];
+        column = 0;
       },
       [&](int ti) {
+        end_column();
+        mx = max(mx & 0xFFFFu, mx >> 16);
         mx = __reduce_max_sync(0xFFFFFFFFu, mx);
         const bool any_bad = __any_sync(0xFFFFFFFFu, bad);
         if (lane == 0) {
@@ -233,19 +263,28 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
       },
       [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next, unsigned int) {
         if (b >= nblk) return;
-        float hv[16];
-        weights_of(h, b - (__umulhi(2u * b, magic) >> shift) * nbc, hv);
+        const unsigned int here = b - (__umulhi(2u * b, magic) >> shift) * nbc;
+        if (here != column) {
+          end_column();
+          column = here;
+        }
         const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+        unsigned int bmx = 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          // magnitude bit patterns order like the magnitudes; NaN patterns lie above infinity's
-          mx = max(mx, max(u[i] & 0x7FFFu, (u[i] >> 16) & 0x7FFFu));
+          // (a NaN input comes out of the maximum as NaN, whose bits are above the infinity pattern)
+          unsigned int m;
+          asm("abs.bf16x2 %0, %1;" : "=r"(m) : "r"(u[i]));
+          asm("max.NaN.bf16x2 %0, %0, %1;" : "+r"(bmx) : "r"(m));
           const double wl = widen_low(u[i]), wh = widen_high(u[i]);
-          sq[0] = fma(static_cast<double>(hv[2 * i]) * wl, wl, sq[0]);
-          sq[1] = fma(static_cast<double>(hv[2 * i + 1]) * wh, wh, sq[1]);
+          squares[2 * i] = fma(wl, wl, squares[2 * i]);
+          squares[2 * i + 1] = fma(wh, wh, squares[2 * i + 1]);
         }
+        mx = __vmaxu2(mx, bmx & 0x7FFF7FFFu);
         // the blocks of the first row meet every weight once
         if (b < nbc) {
+          float hv[16];
+          weights_of(h, here, hv);
 #pragma unroll
           for (int j = 0; j < 16; ++j) bad = bad || !weight_ok(hv[j]);
         }
@@ -271,7 +310,10 @@ __device__ __forceinline__ void weighted_init_pass(S& sh, const Batch& bt, const
   unsigned int zeros = 0, wide = 0, nblk = 0, nbc = 1, magic = 0, shift = 0, view = 0;
   const float* h = nullptr;
   const bool keep_scale = (bt.t[0].flags & SOAR_FLAG_KEEP_BLOCK_SCALE) != 0;
-  unsigned int keep = bt.t[0].max_iters > 0;
+  unsigned int keep = bt.t[0].max_iters > 0, column = 0xFFFFFFFFu;
+  double hd[16];   // the column's weights
+#pragma unroll
+  for (int j = 0; j < 16; ++j) hd[j] = 0.0;
   asm volatile("" : "+r"(keep));
   walk_tiles<true, false>(
       sh, bt, true,
@@ -288,6 +330,7 @@ __device__ __forceinline__ void weighted_init_pass(S& sh, const Batch& bt, const
         shift = p.nbc_shift;
         view = smem_u32(&sh.view[ti]);
         h = wt.h[ti];
+        column = 0xFFFFFFFFu;
       },
       [&](int ti) {
         hand_over(sh, ti, acc);
@@ -320,13 +363,15 @@ __device__ __forceinline__ void weighted_init_pass(S& sh, const Batch& bt, const
         const int d = max(e4m3_encode(tame ? quotient(bmax, six_alpha, six_inv) : __fdiv_rn(bmax, six_alpha)), 1);
         const float v = e4m3_value(d);
         round_pairs(blk, recip_scale(alpha, v), c0, c1);
-        double hd[16], wd[16];
-        {
+        const unsigned int here = b - (__umulhi(2u * b, magic) >> shift) * nbc;
+        if (here != column) {
+          column = here;
           float hv[16];
-          weights_of(h, b - (__umulhi(2u * b, magic) >> shift) * nbc, hv);
+          weights_of(h, here, hv);
 #pragma unroll
           for (int j = 0; j < 16; ++j) hd[j] = static_cast<double>(hv[j]);
         }
+        double wd[16];
         wide_magnitudes(blk, wd);
         WeightedSums s;
         weighted_sums(hd, wd, c0, c1, s);
@@ -489,6 +534,7 @@ template <bool kFast>
 __global__ void __launch_bounds__(kQThreads, 2)
 weighted_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Weighted wt, const __grid_constant__ Reports rp,
                 int stage_lo, int stage_hi) {
-  __shared__ QShared<false> sh;
+  __shared__ WeightedShared sh;
+  if (threadIdx.x < static_cast<unsigned int>(bt.n)) sh.span[threadIdx.x] = column_span(bt.t[threadIdx.x], gridDim.x * kQWarps);
   run_stages<false>(sh, static_cast<double (*)[3]>(nullptr), bt, rp, stage_lo, stage_hi, WeightedPasses<kFast>{wt});
 }
