@@ -67,6 +67,12 @@ struct SoloArgs {
   int idle;                // test hook: nobody arrives at the counter, its waits run out
 };
 
+// Words that CTAs add to when they meet by sums (meet_by_sums): kSumWords that are waited for, one set on a line for the meetings
+// of even and one for those of odd number, and two counts that are read at the end.  They lie in the header that only the
+// stages of other calls use.  (The words of a set on lines of their own arrive up to a microsecond apart.)
+constexpr unsigned int kSumWords = 5, kSetWords = 16, kWords = 3 * kSetWords;
+static_assert(kWords * 8 <= kWsFixedBytes, "no room for the words of the meetings");
+
 // Where a matrix's tiles stay and how its CTAs meet.
 constexpr int kStreamed = 0, kKept = 1, kKeptInCluster = 2;
 
@@ -79,6 +85,7 @@ struct __align__(128) SoloShared {
   double part[32][2];                // each warp's sums of the pass
   // the grid's numbers, by the warp that read them; in a cluster by the CTA that sent them
   unsigned long long red[2][kCluster ? kClusterMost : kSoloMaxGrid / 32][3];
+  unsigned long long before[2][kSumWords];   // the words of either set when its last meeting was over
   double trace_alpha[SOAR_MAX_ITERS + 1], trace_sse[SOAR_MAX_ITERS + 1];
   float alpha[1];
   unsigned int amax[1], zeros[1], wide[1], wide_high[1];
@@ -89,9 +96,6 @@ struct __align__(128) SoloShared {
   int failed;
 };
 
-// The kind of pass whose numbers are exchanged.
-constexpr int kAmaxPass = 0, kStartPass = 1, kIteration = 2;
-
 // Sums of the grid, the same bits in every thread.
 struct Totals {
   double a, g;                       // sum W^2 and nothing (kMax), else 4 den and gsum
@@ -99,12 +103,12 @@ struct Totals {
   unsigned long long counts;         // see counts_word (CTA 0 only)
 };
 
-// A CTA's counts of a pass in one word: after the start pass (the second) zero blocks in the low half and wide candidates,
-// at most one a block, in the high one; after an iteration, where no zero block is counted, the wide candidates of up to
-// 8,192 a block, which pass 32 bits.  (A matrix has fewer than 2^31 blocks; sums of these words do not carry over.)
-template <int kPass, typename S>
-__device__ __forceinline__ unsigned long long counts_word(const S& sh) {
-  return kPass == kAmaxPass ? 0ull : kPass == kStartPass ? count_of(sh.zeros[0], sh.wide[0]) : count_of(sh.wide[0], sh.wide_high[0]);
+// A CTA's counts of a pass in one word: after the start pass (`first`) zero blocks in the low half and wide candidates, at most
+// one a block, in the high one; after an iteration, where no zero block is counted, the wide candidates of up to 8,192 a
+// block, which pass 32 bits.  (A matrix has fewer than 2^31 blocks; sums of these words do not carry over.)
+template <typename S>
+__device__ __forceinline__ unsigned long long counts_word(const S& sh, bool first) {
+  return count_of(first ? sh.zeros[0] : sh.wide[0], first ? sh.wide[0] : sh.wide_high[0]);
 }
 
 // Where the exchange keeps its words: epoch, then flag and counter in one sixteen-byte unit.
@@ -117,6 +121,7 @@ __device__ __forceinline__ void open_counter(const SoloArgs& a, unsigned long lo
                "l"(0ull)
                : "memory");
 }
+__device__ __forceinline__ unsigned long long* sum_words(const SoloArgs& a) { return reinterpret_cast<unsigned long long*>(a.m.t[0].ws); }
 // Before the first arrival (one thread of every CTA).
 __device__ __forceinline__ bool counter_open(const SoloArgs& a, unsigned long long tag) {
   unsigned long long seen = 0;
@@ -138,9 +143,8 @@ __device__ __forceinline__ double half_warp_sum(double v) {
 }
 
 // exchange() inside a cluster: every CTA writes its numbers into everybody's shared memory.
-template <int kPass, typename S>
-__device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, Totals& out) {
-  constexpr bool kMax = kPass == kAmaxPass;
+template <bool kMax, typename S>
+__device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, bool first, Totals& out) {
   __syncthreads();
   const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
   if (tid < 32) {
@@ -152,7 +156,7 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, To
     x = half_warp_sum(x);
     if (!kMax) g = half_warp_sum(g);
     const unsigned long long second = kMax ? sh.amax[0] : static_cast<unsigned long long>(__double_as_longlong(g));
-    const unsigned long long counts = counts_word<kPass>(sh);
+    const unsigned long long counts = kMax ? 0ull : counts_word(sh, first);
     __syncwarp();
     if (lane == 0) sh.zeros[0] = sh.wide[0] = sh.wide_high[0] = 0u;
     if (lane < grid) {
@@ -191,11 +195,11 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, To
 
 // After a pass, all threads of all CTAs: exchanges the CTAs' sums.  `pass` counts from 1.  What the CTAs wrote to global
 // memory before is visible to all after.  With `last` only CTA 0 waits for the sums.  False when a wait ran out.
-template <int kPass, typename S>
-__device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned long long tag, unsigned int pass, bool last,
+// kMax: after the pass for the maximum; first: after the start pass.
+template <bool kMax, typename S>
+__device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned long long tag, unsigned int pass, bool first, bool last,
                                          Totals& out) {
-  if constexpr (S::kCluster) return exchange_in_cluster<kPass>(sh, pass, out);
-  constexpr bool kMax = kPass == kAmaxPass;
+  if constexpr (S::kCluster) return exchange_in_cluster<kMax>(sh, pass, first, out);
   __syncthreads();
   const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
   unsigned long long* const slots = reinterpret_cast<unsigned long long*>(a.exchange + 256 + turn * (grid * kSlotBytes));
@@ -208,7 +212,7 @@ __device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned long
     x = warp_sum(x);
     g = warp_sum(g);
     const unsigned long long second = kMax ? sh.amax[0] : static_cast<unsigned long long>(__double_as_longlong(g));
-    const unsigned long long counts = counts_word<kPass>(sh);
+    const unsigned long long counts = kMax ? 0ull : counts_word(sh, first);
     __syncwarp();
     if (lane == 0) sh.zeros[0] = sh.wide[0] = sh.wide_high[0] = 0u;
     if (grid == 1) {
@@ -278,6 +282,106 @@ __device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned long
   return sh.failed == 0;
 }
 
+// A sum's share as a fixed-point number of 80 bits under 2^e, in two parts of which a word holds one beside a 16-bit count of
+// arrivals: sixteen bits up, so that the parts of 160 CTAs add up without reaching the count or the word's end.
+__device__ __forceinline__ double power_of_two(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+__device__ __forceinline__ void split_fixed(double x, int e, unsigned long long& hi, unsigned long long& lo) {
+  const double s = x * power_of_two(39 - e), f = floor(s);
+  hi = static_cast<unsigned long long>(__double2ll_rn(f)) << 16;
+  lo = static_cast<unsigned long long>(__double2ll_rn((s - f) * 0x1p40)) << 16;
+}
+__device__ __forceinline__ double join_fixed(unsigned long long hi, unsigned long long lo, int e) {
+  return fma(static_cast<double>(lo >> 16), 0x1p-40, static_cast<double>(static_cast<long long>(hi) >> 16)) * power_of_two(e - 39);
+}
+
+// After the start pass and the iterations of a resident matrix, all threads of all CTAs of a grid: the sums of exchange() in
+// one trip.  A CTA adds its parts to the words of the meeting and polls them until everybody's are in: the data is its own
+// arrival, so that nothing has to be made visible before it or read after it, where exchange()'s release waits for the
+// codes written in the pass (1.0 us) and its slots are another trip (0.8 us).  2048 x 2048, from the last arrival until
+// all go on: 3.0 -> 1.8 us.  (A matrix that streams meets by exchange(): its passes are long, and the words cost its
+// search registers, 760 -> 806 us a call of 28672 x 8192.)
+// 4 den is a multiple of 2^-18 below 2^29 a block, its sum exact.  gsum is taken under 64 amax^2 a block (a block's error is
+// at most 16 amax^2 unless its scale is out of all proportion); a share beyond that is announced in the fifth word, and
+// everybody sees so and goes through exchange() instead.  Nothing that the CTAs wrote before is visible after.
+template <typename S>
+__device__ __forceinline__ bool meet_by_sums(S& sh, const SoloArgs& a, unsigned int pass, unsigned int amax_bits, bool& beyond, Totals& out) {
+  __syncthreads();
+  const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
+  if (tid < 32) {
+    double x = 0.0, g = 0.0;
+    if (lane < blockDim.x / 32) {
+      x = sh.part[lane][0];
+      g = sh.part[lane][1];
+    }
+    x = warp_sum(x);
+    g = warp_sum(g);
+    const int blocks = 32 - __clz(a.m.t[0].nblk);   // nblk < 2^blocks
+    const int e_a = 29 + blocks, e_g = 2 * (static_cast<int>(amax_bits >> 7) - 127) + 8 + blocks;
+    const bool fits = fabs(g) < power_of_two(e_g);
+    unsigned long long word[4];
+    split_fixed(x, e_a, word[0], word[1]);
+    split_fixed(fits ? g : 0.0, e_g, word[2], word[3]);
+    unsigned long long mine = fits ? 0ull : 1ull << 16;
+#pragma unroll
+    for (unsigned int i = 0; i < 4; ++i) mine = lane == i ? word[i] : mine;
+    const unsigned int zeros = sh.zeros[0];
+    const unsigned long long wide = count_of(sh.wide[0], sh.wide_high[0]);
+    __syncwarp();
+    if (lane == 0) {
+      sh.zeros[0] = sh.wide[0] = sh.wide_high[0] = 0u;
+      if (zeros != 0u) atomicAdd(sum_words(a) + 2 * kSetWords, static_cast<unsigned long long>(zeros));
+      if (wide != 0ull) atomicAdd(sum_words(a) + 2 * kSetWords + 1, wide);
+    }
+    __syncwarp();
+    if (zeros != 0u || wide != 0ull) __threadfence();
+    unsigned long long* const at = sum_words(a) + turn * kSetWords + lane;
+    unsigned long long before = 0, seen = 0;
+    if (lane < kSumWords) {
+      if (pass > 2) before = sh.before[turn][lane];
+      if (!a.idle) atomicAdd(at, mine + 1);
+    }
+    // (what is done with the words is done on every poll: after a pass its code comes from L2, a microsecond better spent while
+    // others are late)
+    unsigned int polls = 0;
+    bool all;
+    do {
+      if (lane < kSumWords) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(at) : "memory");
+      const unsigned long long sum = seen - before - grid;
+      all = __all_sync(0xFFFFFFFFu, lane >= kSumWords || (sum & 0xFFFFull) == 0ull);
+#pragma unroll
+      for (unsigned int i = 0; i < 4; ++i) word[i] = __shfl_sync(0xFFFFFFFFu, sum, i);
+      const unsigned long long over = __shfl_sync(0xFFFFFFFFu, sum, 4);
+      if (lane == 0) {
+        sh.red[turn][0][0] = static_cast<unsigned long long>(__double_as_longlong(join_fixed(word[0], word[1], e_a)));
+        sh.red[turn][0][1] = static_cast<unsigned long long>(__double_as_longlong(join_fixed(word[2], word[3], e_g)));
+        sh.red[turn][0][2] = over;
+      }
+    } while (!all && ++polls < kGridWaitLimit);
+    if (lane < kSumWords) sh.before[turn][lane] = seen;
+    if (!all && lane == 0) sh.failed = 1;
+  }
+  __syncthreads();
+  out.a = __longlong_as_double(static_cast<long long>(sh.red[turn][0][0]));
+  out.g = __longlong_as_double(static_cast<long long>(sh.red[turn][0][1]));
+  out.counts = 0;
+  beyond = sh.red[turn][0][2] != 0ull;
+  return sh.failed == 0;
+}
+
+// The meeting after the start pass (`first`) or an iteration: by sums where a grid goes on from it, else by exchange().
+template <typename S>
+__device__ __forceinline__ bool combine(S& sh, const SoloArgs& a, unsigned long long tag, unsigned int& exchanged, unsigned int& met,
+                                        bool first, bool last, unsigned int amax_bits, Totals& out) {
+  if constexpr (S::kResident && !S::kCluster && !S::kFinal) {
+    if (gridDim.x > 1 && !last) {
+      bool beyond;
+      if (!meet_by_sums(sh, a, ++met, amax_bits, beyond, out)) return false;
+      if (!beyond) return true;
+    }
+  }
+  return exchange<false>(sh, a, tag, ++exchanged, first, last, out);
+}
+
 // Zeroes of the tiled layout: rows up to a multiple of 128, scale columns up to a multiple of 4.  A warp clears the rows of
 // one tile of the last tile row, a lane the words of rows lane, lane + 32, lane + 64 and lane + 96, which lie side by side.
 // (Counted in tiles: the number of padding words can pass 2^32, at one row of 2.2e9 weights.)
@@ -313,7 +417,10 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   unsigned long long epoch = 0;
   if (!kCluster && gridDim.x > 1) epoch = __ldcg(reinterpret_cast<const unsigned long long*>(a.exchange + kEpochAt));
   if (kRes) load_resident(a.m, smem_u32(tile_slots), a.per_warp);
-  if (!kCluster && gridDim.x > 1 && blockIdx.x == 0 && tid == 0) open_counter(a, a.nonce + epoch);
+  if (!kCluster && gridDim.x > 1 && blockIdx.x == 0) {
+    if (tid == 0) open_counter(a, a.nonce + epoch);
+    if (!kNoIter && tid < static_cast<int>(kWords)) __stcg(sum_words(a) + tid, 0ull);   // (seen by all after the first exchange)
+  }
   if (tid == 0) {
     sh.view[0].packed = p.packed;
     sh.view[0].scales = p.scales;
@@ -341,7 +448,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
     for (int i = T + 1 + tid; i <= SOAR_MAX_ITERS; i += static_cast<int>(blockDim.x)) a.result->trace_alpha[i] = a.result->trace_sse[i] = 0.0;
   __syncthreads();
   if (kNoIter && a.tiled != nullptr) clear_tile_padding(p, a.rows, a.tiled);
-  unsigned int pass = 0;
+  unsigned int exchanged = 0, met = 0;   // meetings through slots and by sums
   Totals tot;
   bool ok;
   amax_pass(sh, a.m);
@@ -349,7 +456,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
     __syncwarp();
     cluster_wait();
   }
-  ok = exchange<kAmaxPass>(sh, a, a.nonce + epoch, ++pass, false, tot);
+  ok = exchange<true>(sh, a, a.nonce + epoch, ++exchanged, false, false, tot);
   const double sumsq = tot.a;
   const unsigned int amax_bits = tot.amax;
   const int st = status_from_amax(amax_bits);
@@ -363,7 +470,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   if (ok && !(st & (SOAR_STATUS_NONFINITE | SOAR_STATUS_RANGE))) {
     const bool tile_after = !kNoIter && a.tiled != nullptr;
     init_pass(sh, a.m);
-    ok = exchange<kStartPass>(sh, a, a.nonce + epoch, ++pass, kNoIter, tot);
+    ok = combine(sh, a, a.nonce + epoch, exchanged, met, true, kNoIter, amax_bits, tot);
     if (kNoIter && blockIdx.x != 0) return;   // nothing left to do but CTA 0's report
     if (st == 0) sse = fmax(sumsq + tot.g, 0.0);
     zero_blocks = tot.counts & 0xFFFFFFFFull;
@@ -381,7 +488,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
       sh.alpha[0] = alpha;
       iterate_pass<kMode>(sh, a.m, (t & 1) != 0, may_stop || t == T - 1, t != T - 1);
       const bool last = t == T - 1 && !tile_after;
-      ok = exchange<kIteration>(sh, a, a.nonce + epoch, ++pass, last, tot);
+      ok = combine(sh, a, a.nonce + epoch, exchanged, met, false, last, amax_bits, tot);
       if (last && blockIdx.x != 0) return;
       const double cur = fmax(sumsq + tot.g, 0.0);
       wide += tot.counts;
@@ -394,7 +501,10 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
       sse = cur;
       if (stop) break;
     }
-    if (ok && tile_after) tile_scales(p, a.rows, a.tiled);
+    if (tile_after) {
+      if (!kCluster && met > 0 && ok) ok = exchange<false>(sh, a, a.nonce + epoch, ++exchanged, false, false, tot);   // the scales of all
+      if (ok) tile_scales(p, a.rows, a.tiled);
+    }
   }
   let_next_begin();
   if (!ok) {
@@ -411,6 +521,11 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   if (blockIdx.x != 0) return;
   if (tid == 0) {
     if (!kCluster && gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange + kEpochAt) = epoch + 1;
+    if (!kCluster && !kNoIter && gridDim.x > 1 && met > 0) {   // (the last meeting's arrivals came after the counts)
+      __threadfence();
+      zero_blocks += __ldcg(sum_words(a) + 2 * kSetWords);
+      wide += __ldcg(sum_words(a) + 2 * kSetWords + 1);
+    }
     *a.alpha = alpha;
     if (a.result != nullptr) {
       soar_result* const res = a.result;
