@@ -10,7 +10,7 @@
 // 0.7 us more.
 //
 // The smallest matrices (see kClusterTiles) run in one cluster of up to 16 CTAs: the sums travel through distributed shared
-// memory and the CTAs meet at the hardware's cluster barrier, with nothing in global memory and no cooperative launch.  256
+// memory (exchange_in_cluster), with nothing in global memory and no cooperative launch.  256
 // tiles: an iteration with one candidate 2.2 us (3.2 through the counter), a max-based call 6.5 us (9.4).
 //
 // Matrices whose tiles fit the shared memory of the grid (12 million weights) are read from HBM once and stay
@@ -85,6 +85,7 @@ struct __align__(128) SoloShared {
   double part[32][2];                // each warp's sums of the pass
   // the grid's numbers, by the warp that read them; in a cluster by the CTA that sent them
   unsigned long long red[2][kCluster ? kClusterMost : kSoloMaxGrid / 32][3];
+  unsigned long long landed[2];              // (cluster) mbarriers of the meetings of even and of odd number
   unsigned long long before[2][kSumWords];   // the words of either set when its last meeting was over
   double trace_alpha[SOAR_MAX_ITERS + 1], trace_sse[SOAR_MAX_ITERS + 1];
   float alpha[1];
@@ -142,7 +143,10 @@ __device__ __forceinline__ double half_warp_sum(double v) {
   return v;
 }
 
-// exchange() inside a cluster: every CTA writes its numbers into everybody's shared memory.
+// exchange() inside a cluster: every CTA sends its numbers into everybody's shared memory with stores that count themselves
+// off at the receiver's mbarrier, so that nothing is released and nobody waits for the codes written in the pass (at the
+// hardware's cluster barrier instead: 1.7 us after an iteration that wrote codes, 0.9 after
+// the other passes; now 1.4 and 0.5).
 template <bool kMax, typename S>
 __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, bool first, Totals& out) {
   __syncthreads();
@@ -158,18 +162,31 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, bo
     const unsigned long long second = kMax ? sh.amax[0] : static_cast<unsigned long long>(__double_as_longlong(g));
     const unsigned long long counts = kMax ? 0ull : counts_word(sh, first);
     __syncwarp();
-    if (lane == 0) sh.zeros[0] = sh.wide[0] = sh.wide_high[0] = 0u;
-    if (lane < grid) {
-      unsigned int at;
-      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(&sh.red[turn][blockIdx.x][0])), "r"(lane));
-      asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at), "l"(__double_as_longlong(x)) : "memory");
-      asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at + 8), "l"(second) : "memory");
-      asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at + 16), "l"(counts) : "memory");
+    const unsigned int landed = smem_u32(&sh.landed[turn]);
+    if (lane == 0) {
+      sh.zeros[0] = sh.wide[0] = sh.wide_high[0] = 0u;
+      asm volatile("{\n.reg .b64 t;\nmbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1;\n}" ::"r"(landed), "r"(grid * 24u) : "memory");
     }
+    if (lane < grid) {
+      unsigned int at, bar;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(&sh.red[turn][blockIdx.x][0])), "r"(lane));
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(landed), "r"(lane));
+      const unsigned long long v[3] = {static_cast<unsigned long long>(__double_as_longlong(x)), second, counts};
+#pragma unroll
+      for (unsigned int i = 0; i < 3; ++i)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.u64 [%0], %1, [%2];" ::"r"(at + 8 * i), "l"(v[i]), "r"(bar) : "memory");
+    }
+    // (the mbarrier's phase: this is its (pass - 1) / 2 th meeting)
+    unsigned int done = 0, polls = 0;
+    do {
+      asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                   : "=r"(done)
+                   : "r"(landed), "r"(((pass - 1) >> 1) & 1u)
+                   : "memory");
+    } while (!done && ++polls < kGridWaitLimit);
+    if (!done) sh.failed = 1;
   }
-  __syncwarp();
-  cluster_arrive();
-  cluster_wait();
+  __syncthreads();
   double x = 0.0, g = 0.0;
   unsigned int mx = 0;
   unsigned int counts[2] = {0, 0};   // (a cluster's 24,576 blocks have fewer than 2^32 candidates)
@@ -190,7 +207,7 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, bo
   if (!kMax && blockIdx.x == 0)
     out.counts = __reduce_add_sync(0xFFFFFFFFu, counts[0]) |
                  (static_cast<unsigned long long>(__reduce_add_sync(0xFFFFFFFFu, counts[1])) << 32);
-  return true;
+  return sh.failed == 0;
 }
 
 // After a pass, all threads of all CTAs: exchanges the CTAs' sums.  `pass` counts from 1.  What the CTAs wrote to global
@@ -404,12 +421,33 @@ __device__ __forceinline__ void clear_tile_padding(const Params& p, unsigned int
       for (unsigned int c = nbc; c < ct * 4; ++c) tiled[swizzled_offset(r, c, ct)] = 0;
 }
 
+// The tiled copy of a resident matrix's scales: every warp its own blocks', from their states.  (No CTA waits for another's
+// scales; 5003 x 2352: the meeting before tile_scales and that pass itself took 5 us, this 1.6.)
+template <typename S>
+__device__ __forceinline__ void tile_resident(S& sh, const Params& p, uint8_t* tiled) {
+  const unsigned int lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = gridDim.x * cta_warps<S>(), ct = (p.nbc + 3) / 4;
+  unsigned int at = slots_of(sh, warp) + kQTileBytes + lane * 8;
+  for (unsigned int tile = warp_number(warp); tile < p.ntiles; tile += warps) {
+    const unsigned int b = tile * 32 + lane, row = __umulhi(2u * b, p.nbc_magic) >> p.nbc_shift;
+    if (b < p.nblk) tiled[swizzled_offset(row, b - row * p.nbc, ct)] = static_cast<uint8_t>((lds64(at).y >> 12) & 0x7Fu);
+    at += kQTileBytes + kQStateBytes;
+  }
+}
+
 template <int kMode, int kPlace>
 __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_constant__ SoloArgs a) {
   extern __shared__ __align__(128) unsigned char tile_slots[];
   constexpr bool kRes = kPlace != kStreamed, kCluster = kPlace == kKeptInCluster, kNoIter = kMode == kNoIterations;
   __shared__ SoloShared<kPlace, kNoIter> sh;
-  if (kCluster) cluster_arrive();   // (waited for before anything is written into another CTA)
+  if (kCluster) {   // (waited for before anything is sent to another CTA)
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&sh.landed[i])) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    cluster_arrive();
+  }
   after_previous();
   const int tid = threadIdx.x;
   const Params& p = a.m.t[0];
@@ -447,7 +485,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   if (blockIdx.x == 0 && a.result != nullptr)
     for (int i = T + 1 + tid; i <= SOAR_MAX_ITERS; i += static_cast<int>(blockDim.x)) a.result->trace_alpha[i] = a.result->trace_sse[i] = 0.0;
   __syncthreads();
-  if (kNoIter && a.tiled != nullptr) clear_tile_padding(p, a.rows, a.tiled);
+  if ((kNoIter || kRes) && a.tiled != nullptr) clear_tile_padding(p, a.rows, a.tiled);
   unsigned int exchanged = 0, met = 0;   // meetings through slots and by sums
   Totals tot;
   bool ok;
@@ -486,7 +524,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
       const double ad = static_cast<double>(alpha), den = 0.25 * tot.a;
       if (den > 0.0 && !(flags & SOAR_FLAG_KEEP_ALPHA)) alpha = static_cast<float>((ad * ad * den - tot.g) / (2.0 * ad * den));
       sh.alpha[0] = alpha;
-      iterate_pass<kMode>(sh, a.m, (t & 1) != 0, may_stop || t == T - 1, t != T - 1);
+      iterate_pass<kMode>(sh, a.m, (t & 1) != 0, may_stop || t == T - 1, t != T - 1 || (kRes && tile_after));
       const bool last = t == T - 1 && !tile_after;
       ok = combine(sh, a, a.nonce + epoch, exchanged, met, false, last, amax_bits, tot);
       if (last && blockIdx.x != 0) return;
@@ -501,9 +539,9 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
       sse = cur;
       if (stop) break;
     }
-    if (tile_after) {
-      if (!kCluster && met > 0 && ok) ok = exchange<false>(sh, a, a.nonce + epoch, ++exchanged, false, false, tot);   // the scales of all
-      if (ok) tile_scales(p, a.rows, a.tiled);
+    if (ok && tile_after) {
+      if constexpr (kRes) tile_resident(sh, p, a.tiled);
+      else tile_scales(p, a.rows, a.tiled);
     }
   }
   let_next_begin();
