@@ -49,11 +49,6 @@ __device__ __forceinline__ unsigned int column_span(const Params& p, unsigned in
   return span * 30 >= warps * 29 && p.ntiles >= 8 * warps ? span : warps;
 }
 
-// Whether some weight of a matrix is zero: a word of its header beside the arrival counter's, set by the maximum's pass.
-__device__ __forceinline__ unsigned int* zero_weights(const Params& p) {
-  return reinterpret_cast<unsigned int*>(reinterpret_cast<unsigned char*>(p.ws) + kWsFixedBytes - 60);
-}
-
 __device__ __forceinline__ bool weight_ok(float h) { return h == 0.0f || (h >= 0x1p-20f && h <= 0x1p20f); }
 
 // Magnitudes of a block in binary64.
@@ -134,54 +129,10 @@ struct WeightedFound {
   double g;
 };
 
-// The first multiplier whose codes equal those of multiplier k wherever the weight is not zero (m0, m1: a nibble each), and its
-// codes.  A column of zero weight costs nothing whatever its code, so that the winner's error is shared by every multiplier
-// that differs from it in such columns alone; grid order takes the first of them.  Codes never rise with the multiplier, so
-// these lie side by side, and the first is found by bisection: seven roundings.  8192 x 8192 with 1 % zero weights: every
-// multiplier of the grid scored in turn, as such blocks once were, 15.1 ms; by bisection 1.04 ms (0.70 without zero weights).
-__device__ __forceinline__ void first_alike(const PairBlock& blk, unsigned int m0, unsigned int m1, float alpha, float center,
-                                            const float2* s_beta, int& k, unsigned int& c0, unsigned int& c1) {
-  int lo = 0;
-  while (lo < k) {
-    const int mid = (lo + k) >> 1;
-    const float s = grid_divisor(alpha, center, s_beta[mid].x);
-    unsigned int d0, d1;
-    round_pairs(blk, recip_fast_ok(s) ? recip_fast(s) : __frcp_rn(s), d0, d1);
-    if ((((c0 ^ d0) & m0) | ((c1 ^ d1) & m1)) == 0u) {
-      k = mid;
-      c0 = d0;
-      c1 = d1;
-    } else {
-      lo = mid + 1;
-    }
-  }
-}
-__device__ __forceinline__ void weighted_nibbles(const float (&hv)[16], unsigned int& m0, unsigned int& m1) {
-  m0 = m1 = 0u;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    m0 |= hv[j] != 0.0f ? 0xFu << (4 * j) : 0u;
-    m1 |= hv[8 + j] != 0.0f ? 0xFu << (4 * j) : 0u;
-  }
-}
-// The same for a block of the straight line, out of line and fed from memory.
-__device__ __noinline__ uint2 first_alike_of(const Params& p, const float* h, unsigned int b, float alpha, float center,
-                                             const float2* s_beta, int k, unsigned int c0, unsigned int c1) {
-  uint4 v0, v1;
-  load_block(p, b, v0, v1);
-  PairBlock blk;
-  unpack_pairs(v0, v1, blk);
-  float hv[16];
-  weights_of(h, b - (__umulhi(2u * b, p.nbc_magic) >> p.nbc_shift) * p.nbc, hv);
-  unsigned int m0, m1;
-  weighted_nibbles(hv, m0, m1);
-  first_alike(blk, m0, m1, alpha, center, s_beta, k, c0, c1);
-  return make_uint2(c0, c1);
-}
-
 // The search by the general rules, out of line and fed from memory: any number of codes, short grids, and, where the
-// coupled arm or a grid of one multiplier rules the bracket out, every multiplier in turn.  First minimum in (beta, code)
-// order.
+// coupled arm, a grid of one multiplier or a zero weight (whose column costs nothing whatever its code, so that equal
+// errors of different codes occur all along the grid) rules the bracket out, every multiplier in turn.  First minimum
+// in (beta, code) order.
 __device__ __noinline__ WeightedFound weighted_search_general(const Params& p, const float* h, unsigned int b, float alpha,
                                                               float center, const float2* s_beta, unsigned int* whole_grid) {
   uint4 v0, v1;
@@ -189,15 +140,16 @@ __device__ __noinline__ WeightedFound weighted_search_general(const Params& p, c
   PairBlock blk;
   unpack_pairs(v0, v1, blk);
   double hd[16], wd[16];
-  unsigned int m0, m1;
+  bool zero_weight = false;
   {
     float hv[16];
     weights_of(h, b - (__umulhi(2u * b, p.nbc_magic) >> p.nbc_shift) * p.nbc, hv);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) hd[j] = static_cast<double>(hv[j]);
-    weighted_nibbles(hv, m0, m1);
+    for (int j = 0; j < 16; ++j) {
+      hd[j] = static_cast<double>(hv[j]);
+      zero_weight = zero_weight || hv[j] == 0.0f;
+    }
   }
-  const bool zero_weight = (m0 & m1) != 0xFFFFFFFFu;
   wide_magnitudes(blk, wd);
   const int n_beta = p.n_beta, n_dq = p.n_dq;
   const bool coupled = (p.flags & SOAR_FLAG_COUPLED_SCALE) != 0;
@@ -209,8 +161,7 @@ __device__ __noinline__ WeightedFound weighted_search_general(const Params& p, c
   best.c0 = best.c1 = 0u;
   best.d = clip_code(d_lo);
   best.s.a4 = best.s.b16 = 0.0;
-  if (!coupled && p.beta_step_pct >= 1 && n_beta >= kBracketMinBeta) {
-    if (zero_weight) ++*whole_grid;   // (counted in the report as blocks that tie along the grid)
+  if (!coupled && p.beta_step_pct >= 1 && n_beta >= kBracketMinBeta && !zero_weight) {
     const float k_scale = 100.0f / static_cast<float>(p.beta_step_pct);
     const float k_off = static_cast<float>(n_beta / 2) - k_scale, per_center = __fdividef(k_scale, center);
     int best_k = 0, prev = -1;
@@ -231,11 +182,9 @@ __device__ __noinline__ WeightedFound weighted_search_general(const Params& p, c
         WeightedSums s;
         weighted_sums(hd, wd, c0, c1, s);
         const double g = 0.5 * sd * weighted_rank(s, sd);
-        int at = k;
-        if (zero_weight && g <= best.g) first_alike(blk, m0, m1, alpha, center, s_beta, at, c0, c1);
         // equal errors: the earlier multiplier, then the smaller code, as in grid order
-        if (g < best.g || (g == best.g && at < best_k)) {
-          best.g = g; best.s = s; best.c0 = c0; best.c1 = c1; best.d = dc; best_k = at;
+        if (g < best.g || (g == best.g && k < best_k)) {
+          best.g = g; best.s = s; best.c0 = c0; best.c1 = c1; best.d = dc; best_k = k;
         }
       }
     }
@@ -273,7 +222,7 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
   const unsigned int lane = threadIdx.x & 31u;
   unsigned int mx = 0, nblk = 0, nbc = 1, magic = 0, shift = 0, column = 0;
   const float* h = nullptr;
-  bool bad = false, zero = false;
+  bool bad = false;
   double sq[2] = {0.0, 0.0}, squares[16];   // sum W^2 of each of the column's sixteen weights since it began
 #pragma unroll
   for (int j = 0; j < 16; ++j) squares[j] = 0.0;
@@ -301,16 +250,15 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
         end_column();
         mx = max(mx & 0xFFFFu, mx >> 16);
         mx = __reduce_max_sync(0xFFFFFFFFu, mx);
-        const bool any_bad = __any_sync(0xFFFFFFFFu, bad), any_zero = __any_sync(0xFFFFFFFFu, zero);
+        const bool any_bad = __any_sync(0xFFFFFFFFu, bad);
         if (lane == 0) {
           if (mx) atomicMax(&sh.amax[ti], mx);
           if (any_bad) atomicOr(&bt.t[ti].ws->error, kErrWeight);
-          if (any_zero) *zero_weights(bt.t[ti]) = 1u;
         }
         double v[2] = {sq[0] + sq[1], 0.0};
         hand_over(sh, ti, v);
         mx = 0;
-        bad = zero = false;
+        bad = false;
         sq[0] = sq[1] = 0.0;
       },
       [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next, unsigned int) {
@@ -338,10 +286,7 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
           float hv[16];
           weights_of(h, here, hv);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            bad = bad || !weight_ok(hv[j]);
-            zero = zero || hv[j] == 0.0f;
-          }
+          for (int j = 0; j < 16; ++j) bad = bad || !weight_ok(hv[j]);
         }
         next();
       });
@@ -445,9 +390,8 @@ __device__ __forceinline__ void weighted_init_pass(S& sh, const Batch& bt, const
 // One iteration of Algorithm 1 under the weighted objective: Eq. 6 per block from its stored {A, B}, App. B.3's candidates,
 // Eq. 8 with the weighted error written as sum h w^2 + sd^2 B - 2 sd A, first minimum in (beta, code) order.  kFast: the
 // paper's two E4M3 codes on a grid that holds their brackets; the weighted error of an element is convex in its code
-// value like the unweighted one, so per code only the multipliers of winning_range can win.  kZeros: some weight is zero (what
-// such a block needs beyond that costs the others 2 % in registers).
-template <bool kFast, bool kZeros, typename S>
+// value like the unweighted one, so per code only the multipliers of winning_range can win.
+template <bool kFast, typename S>
 __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, const Weighted& wt, bool reverse, unsigned int emit,
                                                       unsigned int keep) {
   asm volatile("" : "+r"(emit), "+r"(keep));
@@ -503,8 +447,8 @@ __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, co
           const float per_center = y * k_scale;
           const float t0 = __fadd_rd(__fmaf_rn(v0f, per_center, k_off), 12582912.0f);
           const float t1 = __fadd_rd(__fmaf_rn(v1f, per_center, k_off), 12582912.0f);
-          const unsigned int k0 = __float_as_uint(t0) & (SOAR_MAX_BETA - 1), k1 = __float_as_uint(t1) & (SOAR_MAX_BETA - 1);
-          const uint2 q0 = lds64(pairs + 8u * k0), q1 = lds64(pairs + 8u * k1);
+          const uint2 q0 = lds64(pairs + 8u * (__float_as_uint(t0) & (SOAR_MAX_BETA - 1)));
+          const uint2 q1 = lds64(pairs + 8u * (__float_as_uint(t1) & (SOAR_MAX_BETA - 1)));
           const pair_t cc = pair_of(center, center), aa = pair_of(-alpha, -alpha);
           const pair_t m0 = pair_mul(cc, pair_of(__uint_as_float(q0.x), __uint_as_float(q0.y)));
           const pair_t m1 = pair_mul(cc, pair_of(__uint_as_float(q1.x), __uint_as_float(q1.y)));
@@ -513,12 +457,10 @@ __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, co
           halves(m1, a1, b1);
           constexpr float kUnder = 1.0f - 0x1.8p-22f, kOver = 1.0f + 0x1.8p-22f;   // as in iterate_pass
           unsigned int least = 0x7F800000u;   // smallest weight (bit patterns of non-negative floats order like them)
-          if (kZeros) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) least = min(least, __float_as_uint(hv[j]));
-          }
+          for (int j = 0; j < 16; ++j) least = min(least, __float_as_uint(hv[j]));
           direct = __float_as_uint(center) - 0x3C800000u < 0x43E00000u - 0x3C800000u && a0 <= v0f * kUnder &&
-                   b0f >= v0f * kOver && a1 <= v1f * kUnder && b1 >= v1f * kOver;
+                   b0f >= v0f * kOver && a1 <= v1f * kUnder && b1 >= v1f * kOver && least != 0u;
           float r00, r01, r10, r11;
           pair_recip(pair_mul(aa, m0), r00, r01);
           pair_recip(pair_mul(aa, m1), r10, r11);
@@ -532,8 +474,7 @@ __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, co
           f.c0 = c[0][0];
           f.c1 = c[0][1];
           f.s = s0;
-          bool later = e1 < e0;   // than the first multiplier of its pair
-          if (later) { f.c0 = c[1][0]; f.c1 = c[1][1]; f.s = s1; e0 = e1; }
+          if (e1 < e0) { f.c0 = c[1][0]; f.c1 = c[1][1]; f.s = s1; e0 = e1; }
           f.g = 0.5 * sd0 * e0;
           f.d = static_cast<int>(dv0 >> 20) - 960;
           round_pairs(blk, r10, c[2][0], c[2][1]);
@@ -541,27 +482,15 @@ __device__ __forceinline__ void weighted_iterate_pass(S& sh, const Batch& bt, co
           weighted_sums_of_two(hv, blk, c[2], c[3], s0, s1);
           e0 = weighted_rank(s0, sd1);
           e1 = weighted_rank(s1, sd1);
-          const bool later1 = e1 < e0;
-          if (later1) { c[2][0] = c[3][0]; c[2][1] = c[3][1]; s0 = s1; e0 = e1; }
-          // equal errors: the earlier multiplier, as in grid order (the second code's are never earlier, unless a weight is zero)
+          if (e1 < e0) { c[2][0] = c[3][0]; c[2][1] = c[3][1]; s0 = s1; e0 = e1; }
+          // equal errors: the earlier multiplier, as in grid order (the second code's are never earlier)
           const double g1 = 0.5 * sd1 * e0;
-          const bool second = g1 < f.g;
-          if (kZeros && least == 0u) direct = direct && g1 != f.g;
-          if (second) {
-            later = later1;
+          if (g1 < f.g) {
             f.c0 = c[2][0];
             f.c1 = c[2][1];
             f.s = s0;
             f.g = g1;
             f.d = static_cast<int>(dv1 >> 20) - 960;
-          }
-          if (kZeros && least == 0u && active && direct) {
-            ++whole;
-            if (!later) {
-              const uint2 e = first_alike_of(bt.t[tensor], h, b, alpha, center, sh.beta, static_cast<int>(second ? k1 : k0), f.c0, f.c1);
-              f.c0 = e.x;
-              f.c1 = e.y;
-            }
           }
         }
         next();
@@ -597,11 +526,7 @@ struct WeightedPasses {
   __device__ __forceinline__ void init(S& sh, const Batch& bt) const { weighted_init_pass(sh, bt, wt); }
   template <typename S>
   __device__ __forceinline__ void iterate(S& sh, const Batch& bt, bool reverse, bool emit, bool keep) const {
-    bool zeros = false;
-    if (kFast)
-      for (int i = 0; i < bt.n; ++i) zeros = zeros || __ldcg(zero_weights(bt.t[i])) != 0u;
-    if (kFast && zeros) weighted_iterate_pass<kFast, kFast>(sh, bt, wt, reverse, emit, keep);
-    else weighted_iterate_pass<kFast, false>(sh, bt, wt, reverse, emit, keep);
+    weighted_iterate_pass<kFast>(sh, bt, wt, reverse, emit, keep);
   }
 };
 

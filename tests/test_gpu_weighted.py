@@ -49,30 +49,6 @@ def test_weighted_parity(rows, cols, ld, seed, kw, cfgkw):
     assert gpu.result.sumsq == pytest.approx(ref.sumsq, rel=1e-12)
 
 
-@pytest.mark.parametrize("zero_frac", [0.01, 0.3, 0.9])
-@pytest.mark.parametrize("cfgkw", [
-    dict(max_iters=3, early_stop_rel=0.0),                                                        # two codes, the paper's grid
-    dict(max_iters=2, early_stop_rel=0.0, n_dq=1, n_beta=2, beta_step_pct=1),
-    dict(max_iters=2, early_stop_rel=0.0, n_dq=4, n_beta=7, beta_step_pct=5),                     # brackets past both ends
-    dict(max_iters=2, early_stop_rel=0.0, n_dq=2, n_beta=101, flags=R.FLAG_KEEP_BLOCK_SCALE),    # a multiplier on the code
-])
-def test_zero_weights_take_the_first_of_the_multipliers_that_tie(zero_frac, cfgkw):
-    # a column's code is free where its weight is zero: the winner's error is shared along the grid.  One block column has no
-    # other weights; the second matrix has coarse values (rounding midpoints, equal errors), zero blocks and zero columns.
-    for rows, cols, seed in ((65, 336, 31), (16, 1024, 32)):
-        w = WL.small_case(rows, cols, seed, outlier_entry_frac=0.01, outlier_scale=20.0)
-        if seed == 32:
-            w = ((w.astype(np.uint32) & 0xFFE0).astype(np.uint16)).reshape(rows, cols)
-            w[3, :48] = 0
-            w[:, 128:160] = 0
-        h = WL.column_weights(cols, seed, zero_frac=zero_frac)
-        h[64:80] = 0.0
-        cfg, ref_cfg = P.cfg_pair(**cfgkw)
-        gpu, _, _ = run_weighted(w, h, cfg)
-        ref = R.quantize(w, ref_cfg, h=h)
-        P.assert_parity(gpu, ref, mismatch_cap=0)   # (blocks that tie included)
-
-
 def test_unit_weights_give_exactly_what_the_unweighted_entry_gives():
     w = WL.small_case(200, 2048, 11, outlier_entry_frac=0.001, outlier_scale=30.0)
     for cfgkw in (dict(), dict(max_iters=1, early_stop_rel=0.0, n_dq=2, n_beta=1)):
