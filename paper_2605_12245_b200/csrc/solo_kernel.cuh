@@ -6,7 +6,8 @@
 // iteration at any size.  Here every CTA stores its sums in a slot of its own, arrives at a counter and, when all
 // have, reads everybody's slots and adds them in the same order on every run: 1.6 us from the last arrival on, for 2 to
 // 148 CTAs.  (Polling tagged slots instead, with no counter, is 0.7 us when all CTAs come at the same moment but 3 us
-// when some wait for others, as they do.)  The grid is one CTA of 16 warps per SM rather than two of 8: 296 CTAs need
+// when some wait for others, as they do.)  A matrix that stays in shared memory has a shorter way after the start pass and the
+// iterations (meet_by_sums).  The grid is one CTA of 16 warps per SM rather than two of 8: 296 CTAs need
 // 0.7 us more.
 //
 // The smallest matrices (see kClusterTiles) run in one cluster of up to 16 CTAs: the sums travel through distributed shared
