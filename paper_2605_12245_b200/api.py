@@ -616,9 +616,9 @@ def soar_selftest_reciprocal(lo_exp: int = 2, hi_exp: int = 252, stream=None) ->
     return int(out.cpu()[0])
 
 
-def soar_debug_fail_waits(on: bool) -> None:
+def soar_debug_fail_waits(on: bool | int) -> None:
     """Test hook: while on, the kernels' polled waits run out (see ``soar_debug_fail_waits`` in soar.h)."""
-    _check(lib().soar_debug_fail_waits(1 if on else 0), "soar_debug_fail_waits")
+    _check(lib().soar_debug_fail_waits(int(on) if isinstance(on, int) else int(bool(on))), "soar_debug_fail_waits")
 
 
 def soar_trace_begin() -> None:

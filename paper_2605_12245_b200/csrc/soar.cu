@@ -54,6 +54,9 @@ namespace {
 
 constexpr size_t kWsFixedBytes = 2048;
 constexpr unsigned int kGridWaitLimit = 1u << 21;  // polls of the grid's arrival counter before a CTA gives up (each most of a microsecond)
+constexpr unsigned int kClusterWaitLimit = 1u << 24;  // polls of an mbarrier of its own shared memory (each some tens of nanoseconds)
+// What soar_debug_fail_waits makes the CTAs of a launch withhold: their arrivals, or what a cluster's CTAs send each other.
+enum WaitHook : int { kNobodyArrives = 1, kNobodySends = 2 };
 constexpr int kBracketMinBeta = 2;             // the bracket needs two multipliers; a single one is modes 1-3
 
 struct Ws {
@@ -558,7 +561,7 @@ struct ScopedLaunch {
 
 int g_sm_count[64];
 
-// Test hook (soar_debug_fail_waits): what the launches put into Batch::idle and its like, read only where a kernel waits.
+// Test hook (soar_debug_fail_waits): what the launches put into Batch::idle and its like, read only where CTAs meet.
 int g_idle = 0;
 
 int sm_count() {
@@ -1135,7 +1138,7 @@ int run_batch(const soar_tensor_desc* tensors, int n, const soar_cfg* cfg, void*
     memset(&bt, 0, sizeof(bt));
     memset(&rp, 0, sizeof(rp));
     bt.n = (n - first < kMaxBatch) ? n - first : kMaxBatch;
-    bt.idle = g_idle;
+    bt.idle = g_idle == kNobodyArrives;
     unsigned int tiles = 0;
     for (int j = 0; j < bt.n; ++j) {
       const soar_tensor_desc& d = tensors[first + j];
@@ -1412,7 +1415,7 @@ int soar_quantize_weighted_batch(const soar_tensor_desc* tensors, const float* c
     memset(&wt, 0, sizeof(wt));
     memset(&rp, 0, sizeof(rp));
     bt.n = (n - first < kMaxBatch) ? n - first : kMaxBatch;
-    bt.idle = g_idle;
+    bt.idle = g_idle == kNobodyArrives;
     unsigned int tiles = 0;
     for (int j = 0; j < bt.n; ++j) {
       const soar_tensor_desc& d = tensors[first + j];
@@ -1729,7 +1732,7 @@ int soar_mx_quantize(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld,
   a.n_dq = n_dq;
   a.n_beta = n_beta;
   a.step_pct = beta_step_pct;
-  a.idle = g_idle;
+  a.idle = g_idle == kNobodyArrives;
   ScopedLaunch sl(K_MX, st);
   cudaError_t err;
   // every block of 32 is 64 bytes at a multiple of 32: two 256-bit loads
@@ -1743,7 +1746,7 @@ int soar_mx_quantize(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld,
 }
 
 int soar_debug_fail_waits(int on) {
-  g_idle = on ? 1 : 0;
+  g_idle = on == kNobodySends ? on : on ? kNobodyArrives : 0;
   return SOAR_OK;
 }
 

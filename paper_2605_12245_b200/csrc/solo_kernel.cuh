@@ -65,7 +65,7 @@ struct SoloArgs {
   unsigned int rows;
   unsigned int per_warp;   // resident: slots of a warp
   int tiled_only;          // the caller wants no row-major scales
-  int idle;                // test hook: nobody arrives at the counter, its waits run out
+  int idle;                // test hook, see WaitHook
 };
 
 // Words that CTAs add to when they meet by sums (meet_by_sums): kSumWords that are waited for, one set on a line for the meetings
@@ -148,8 +148,12 @@ __device__ __forceinline__ double half_warp_sum(double v) {
 // off at the receiver's mbarrier, so that nothing is released and nobody waits for the codes written in the pass (at the
 // hardware's cluster barrier instead: 1.7 us after an iteration that wrote codes, 0.9 after
 // the other passes; now 1.4 and 0.5).
+// One try_wait, which sleeps until the numbers are there (test_wait alone: 0.1 us more a call), then polls with test_wait,
+// which returns at once: how long a try_wait may stay suspended is the hardware's choice, so that a count of them bounds
+// nothing.  The polls cannot run out in earnest, since a cluster's CTAs run together and a pass waits for nobody; a CTA that gives
+// up all the same stays until no other can send to it (see the end of solo_kernel).
 template <bool kMax, typename S>
-__device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, bool first, Totals& out) {
+__device__ __forceinline__ bool exchange_in_cluster(S& sh, int idle, unsigned int pass, bool first, Totals& out) {
   __syncthreads();
   const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
   if (tid < 32) {
@@ -168,7 +172,7 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, bo
       sh.zeros[0] = sh.wide[0] = sh.wide_high[0] = 0u;
       asm volatile("{\n.reg .b64 t;\nmbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1;\n}" ::"r"(landed), "r"(grid * 24u) : "memory");
     }
-    if (lane < grid) {
+    if (lane < grid && idle != kNobodySends) {
       unsigned int at, bar;
       asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(&sh.red[turn][blockIdx.x][0])), "r"(lane));
       asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(landed), "r"(lane));
@@ -179,12 +183,15 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, bo
     }
     // (the mbarrier's phase: this is its (pass - 1) / 2 th meeting)
     unsigned int done = 0, polls = 0;
-    do {
-      asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(done)
+                 : "r"(landed), "r"(((pass - 1) >> 1) & 1u)
+                 : "memory");
+    while (!done && polls++ < kClusterWaitLimit)
+      asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
                    : "=r"(done)
                    : "r"(landed), "r"(((pass - 1) >> 1) & 1u)
                    : "memory");
-    } while (!done && ++polls < kGridWaitLimit);
     if (!done) sh.failed = 1;
   }
   __syncthreads();
@@ -217,7 +224,7 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, unsigned int pass, bo
 template <bool kMax, typename S>
 __device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned long long tag, unsigned int pass, bool first, bool last,
                                          Totals& out) {
-  if constexpr (S::kCluster) return exchange_in_cluster<kMax>(sh, pass, first, out);
+  if constexpr (S::kCluster) return exchange_in_cluster<kMax>(sh, a.idle, pass, first, out);
   __syncthreads();
   const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
   unsigned long long* const slots = reinterpret_cast<unsigned long long*>(a.exchange + 256 + turn * (grid * kSlotBytes));
@@ -247,7 +254,7 @@ __device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned long
       if (lane == 0) {
         unsigned int* const arrived = reinterpret_cast<unsigned int*>(a.exchange + kCounterAt);
         if (pass == 1 && !counter_open(a, tag)) sh.failed = 1;
-        if (!a.idle) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
+        if (a.idle != kNobodyArrives) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
         if (!last || blockIdx.x == 0) {
           unsigned int seen = 0, polls = 0;
           do {
@@ -356,7 +363,7 @@ __device__ __forceinline__ bool meet_by_sums(S& sh, const SoloArgs& a, unsigned 
     unsigned long long before = 0, seen = 0;
     if (lane < kSumWords) {
       if (pass > 2) before = sh.before[turn][lane];
-      if (!a.idle) atomicAdd(at, mine + 1);
+      if (a.idle != kNobodyArrives) atomicAdd(at, mine + 1);
     }
     // (what is done with the words is done on every poll: after a pass its code comes from L2, a microsecond better spent while
     // others are late)
@@ -547,7 +554,12 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   }
   let_next_begin();
   if (!ok) {
-    // a wait ran out: say so in the report and leave
+    // a wait ran out: say so in the report and leave, a CTA of a cluster not before everybody there has given up or ended
+    if (kCluster) {
+      __syncwarp();
+      cluster_arrive();
+      cluster_wait();
+    }
     if (tid == 0) {
       if (!kCluster && gridDim.x > 1) *reinterpret_cast<volatile unsigned long long*>(a.exchange + kEpochAt) = epoch + 1;
       if (a.result != nullptr) {
