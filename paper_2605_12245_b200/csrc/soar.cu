@@ -811,22 +811,24 @@ cudaError_t launch_stages(int mode, bool det, const Batch& bt, const Reports& rp
 }
 
 // The same for the weighted kernel.
-template <bool kFast>
+template <bool kFast, bool kColumns>
 cudaError_t launch_weighted(const Batch& bt, const Weighted& wt, const Reports& rp, unsigned int tiles, int lo, int hi,
                             cudaStream_t st) {
   static std::atomic<int> known[64];
   unsigned int per_sm = 1;
-  const unsigned int grid = stage_grid(weighted_kernel<kFast>, known, tiles, &per_sm);
+  const unsigned int grid = stage_grid(weighted_kernel<kFast, kColumns>, known, tiles, &per_sm);
+  if constexpr (kColumns)
+    if (!has_steady_columns(bt, grid * kQWarps)) return launch_weighted<kFast, false>(bt, wt, rp, tiles, lo, hi, st);
   if (hi - lo == 1) {
-    weighted_kernel<kFast><<<grid, kQThreads, 0, st>>>(bt, wt, rp, lo, hi);
+    weighted_kernel<kFast, kColumns><<<grid, kQThreads, 0, st>>>(bt, wt, rp, lo, hi);
     return cudaGetLastError();
   }
   void* args[] = {const_cast<Batch*>(&bt), const_cast<Weighted*>(&wt), const_cast<Reports*>(&rp), &lo, &hi};
-  return launch_cooperative(reinterpret_cast<const void*>(&weighted_kernel<kFast>), grid, per_sm, kQThreads, args, 0, st);
+  return launch_cooperative(reinterpret_cast<const void*>(&weighted_kernel<kFast, kColumns>), grid, per_sm, kQThreads, args, 0, st);
 }
 cudaError_t launch_weighted(bool fast, const Batch& bt, const Weighted& wt, const Reports& rp, unsigned int tiles, int lo, int hi,
                             cudaStream_t st) {
-  return fast ? launch_weighted<true>(bt, wt, rp, tiles, lo, hi, st) : launch_weighted<false>(bt, wt, rp, tiles, lo, hi, st);
+  return fast ? launch_weighted<true, true>(bt, wt, rp, tiles, lo, hi, st) : launch_weighted<false, true>(bt, wt, rp, tiles, lo, hi, st);
 }
 
 // kMode of quantize_kernel for a call's settings (see iterate_pass).

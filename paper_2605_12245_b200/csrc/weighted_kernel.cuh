@@ -33,21 +33,34 @@ __device__ __forceinline__ void weights_of(const float* h, unsigned int cb, floa
     hv[4 * q + 3] = v.w;
   }
 }
-// What a CTA shares, and by how many warps each tensor is walked.
-struct __align__(128) WeightedShared : QShared<false> {
-  unsigned int span[kMaxBatch];
-};
-__device__ __forceinline__ unsigned int span_of(const WeightedShared& sh, int ti, unsigned int) { return sh.span[ti]; }
-
-// A lane whose blocks all lie in one block column reads that column's weights once and widens them once (see
-// `column` in the passes), so a tensor is walked by as many warps as make a step a whole number of rows: a multiple of
+// A lane whose blocks all lie in one block column reads that column's weights once and widens them once (see `steady` in the
+// passes), so a tensor is walked by as many warps as make a step a whole number of rows: a multiple of
 // nbc / gcd(nbc, 32) tiles.  4096 and 8192 columns divide the warps of the device's grid as it is (2368 = 64 * 37); 12288 and
-// 28672 columns leave 16 of them out.  Where more than a thirtieth would be left out, or where a tensor has only a few turns, all warps
-// walk it and the weights are read again when the column changes.
-__device__ __forceinline__ unsigned int column_span(const Params& p, unsigned int warps) {
-  const unsigned int unit = p.nbc / min(p.nbc & (0u - p.nbc), 32u), span = warps / unit * unit;
-  return span * 30 >= warps * 29 && p.ntiles >= 8 * warps ? span : warps;
+// 28672 columns leave 16 of them out.  Where more than a thirtieth would be left out, or where a tensor has fewer than eight turns, all
+// warps walk it and the weights are read again when the column changes.
+constexpr unsigned int kColumnTurns = 8;
+__host__ __device__ __forceinline__ unsigned int column_span(const Params& p, unsigned int warps) {
+  const unsigned int low = p.nbc & (0u - p.nbc), unit = p.nbc / (low < 32u ? low : 32u), span = warps / unit * unit;
+  return span * 30 >= warps * 29 && p.ntiles >= kColumnTurns * warps ? span : warps;
 }
+__host__ __device__ __forceinline__ bool whole_rows(const Params& p, unsigned int span) { return span * 32 % p.nbc == 0; }
+// Whether a launch takes the kernel whose lanes stay in their columns: where a matrix of eight turns or more has lanes that do.  The
+// code for it costs calls of smaller ones up to 3 % (a layer of 896, 128 and 2688 columns 163 -> 168 us, of 1600, 320 and 4800
+// 355 -> 365, in the kernel without it 163 and 356; of 2048, 512 and 6144 it takes 547 -> 536, of 3072, 1024 and 8192 1050 -> 1023).
+inline bool has_steady_columns(const Batch& bt, unsigned int warps) {
+  for (int i = 0; i < bt.n; ++i)
+    if (bt.t[i].ntiles >= kColumnTurns * warps && whole_rows(bt.t[i], column_span(bt.t[i], warps))) return true;
+  return false;
+}
+
+// What a CTA shares; with columns also by how many warps each tensor is walked, and whether a lane's blocks of it then all
+// lie in one block column.
+template <bool kWithColumns>
+struct __align__(128) WeightedShared : QShared<false> {
+  static constexpr bool kColumns = kWithColumns;
+  unsigned int span[kWithColumns ? kMaxBatch : 1], steady[kWithColumns ? kMaxBatch : 1];
+};
+__device__ __forceinline__ unsigned int span_of(const WeightedShared<true>& sh, int ti, unsigned int) { return sh.span[ti]; }
 
 __device__ __forceinline__ bool weight_ok(float h) { return h == 0.0f || (h >= 0x1p-20f && h <= 0x1p20f); }
 
@@ -222,19 +235,10 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
   const unsigned int lane = threadIdx.x & 31u;
   unsigned int mx = 0, nblk = 0, nbc = 1, magic = 0, shift = 0, column = 0;
   const float* h = nullptr;
-  bool bad = false;
-  double sq[2] = {0.0, 0.0}, squares[16];   // sum W^2 of each of the column's sixteen weights since it began
+  bool bad = false, steady = false;
+  double sq[2] = {0.0, 0.0}, squares[16];   // (steady) sum W^2 of each of the column's sixteen weights
 #pragma unroll
   for (int j = 0; j < 16; ++j) squares[j] = 0.0;
-  auto end_column = [&]() {
-    float hv[16];
-    weights_of(h, column, hv);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      sq[j & 1] = fma(static_cast<double>(hv[j]), squares[j], sq[j & 1]);
-      squares[j] = 0.0;
-    }
-  };
   walk_tiles<true, false>(
       sh, bt, false,
       [&](int ti) {
@@ -244,10 +248,21 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
         magic = p.nbc_magic;
         shift = p.nbc_shift;
         h = wt.h[ti];
-        column = 0;
+        if constexpr (S::kColumns) {
+          steady = sh.steady[ti] != 0u;
+          column = 0;   // (a lane that meets no block of this tensor)
+        }
       },
       [&](int ti) {
-        end_column();
+        if (S::kColumns && steady) {
+          float hv[16];
+          weights_of(h, column, hv);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            sq[j & 1] = fma(static_cast<double>(hv[j]), squares[j], sq[j & 1]);
+            squares[j] = 0.0;
+          }
+        }
         mx = max(mx & 0xFFFFu, mx >> 16);
         mx = __reduce_max_sync(0xFFFFFFFFu, mx);
         const bool any_bad = __any_sync(0xFFFFFFFFu, bad);
@@ -263,11 +278,7 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
       },
       [&](unsigned int b, const uint4& v0, const uint4& v1, const uint2&, auto next, unsigned int) {
         if (b >= nblk) return;
-        const unsigned int here = b - (__umulhi(2u * b, magic) >> shift) * nbc;
-        if (here != column) {
-          end_column();
-          column = here;
-        }
+        column = b - (__umulhi(2u * b, magic) >> shift) * nbc;
         const unsigned int u[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
         unsigned int bmx = 0;
 #pragma unroll
@@ -276,15 +287,29 @@ __device__ __forceinline__ void weighted_amax_pass(S& sh, const Batch& bt, const
           unsigned int m;
           asm("abs.bf16x2 %0, %1;" : "=r"(m) : "r"(u[i]));
           asm("max.NaN.bf16x2 %0, %0, %1;" : "+r"(bmx) : "r"(m));
-          const double wl = widen_low(u[i]), wh = widen_high(u[i]);
-          squares[2 * i] = fma(wl, wl, squares[2 * i]);
-          squares[2 * i + 1] = fma(wh, wh, squares[2 * i + 1]);
         }
         mx = __vmaxu2(mx, bmx & 0x7FFF7FFFu);
+        if (S::kColumns && steady) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const double wl = widen_low(u[i]), wh = widen_high(u[i]);
+            squares[2 * i] = fma(wl, wl, squares[2 * i]);
+            squares[2 * i + 1] = fma(wh, wh, squares[2 * i + 1]);
+          }
+        } else {
+          float hv[16];
+          weights_of(h, column, hv);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const double wl = widen_low(u[i]), wh = widen_high(u[i]);
+            sq[0] = fma(static_cast<double>(hv[2 * i]) * wl, wl, sq[0]);
+            sq[1] = fma(static_cast<double>(hv[2 * i + 1]) * wh, wh, sq[1]);
+          }
+        }
         // the blocks of the first row meet every weight once
         if (b < nbc) {
           float hv[16];
-          weights_of(h, here, hv);
+          weights_of(h, column, hv);
 #pragma unroll
           for (int j = 0; j < 16; ++j) bad = bad || !weight_ok(hv[j]);
         }
@@ -364,7 +389,7 @@ __device__ __forceinline__ void weighted_init_pass(S& sh, const Batch& bt, const
         const float v = e4m3_value(d);
         round_pairs(blk, recip_scale(alpha, v), c0, c1);
         const unsigned int here = b - (__umulhi(2u * b, magic) >> shift) * nbc;
-        if (here != column) {
+        if (!S::kColumns || here != column) {
           column = here;
           float hv[16];
           weights_of(h, here, hv);
@@ -530,11 +555,18 @@ struct WeightedPasses {
   }
 };
 
-template <bool kFast>
+template <bool kFast, bool kColumns>
 __global__ void __launch_bounds__(kQThreads, 2)
 weighted_kernel(const __grid_constant__ Batch bt, const __grid_constant__ Weighted wt, const __grid_constant__ Reports rp,
                 int stage_lo, int stage_hi) {
-  __shared__ WeightedShared sh;
-  if (threadIdx.x < static_cast<unsigned int>(bt.n)) sh.span[threadIdx.x] = column_span(bt.t[threadIdx.x], gridDim.x * kQWarps);
+  __shared__ WeightedShared<kColumns> sh;
+  if constexpr (kColumns) {
+    if (threadIdx.x < static_cast<unsigned int>(bt.n)) {
+      const Params& p = bt.t[threadIdx.x];
+      const unsigned int span = column_span(p, gridDim.x * kQWarps);
+      sh.span[threadIdx.x] = span;
+      sh.steady[threadIdx.x] = whole_rows(p, span);
+    }
+  }
   run_stages<false>(sh, static_cast<double (*)[3]>(nullptr), bt, rp, stage_lo, stage_hi, WeightedPasses<kFast>{wt});
 }

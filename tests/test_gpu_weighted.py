@@ -250,3 +250,35 @@ def test_weighted_batch_gives_each_matrix_what_a_single_call_gives():
         if rb.status == 0 and i % 3 == 0:
             g = P.GpuOut(o.packed.cpu().numpy(), o.scales.cpu().numpy(), float(o.alpha.cpu()[0]), rb, o)
             P.assert_parity(g, R.quantize(w, ref_cfg, h=h), mismatch_cap=(0 if w.size < 16 * 20000 else None))
+
+
+@pytest.mark.parametrize("cfgkw", [dict(max_iters=2, early_stop_rel=0.0),
+                                   dict(max_iters=1, early_stop_rel=0.0, n_dq=4, n_beta=5, beta_step_pct=3)])
+def test_lanes_that_stay_in_a_block_column_and_lanes_that_do_not(cfgkw):
+    """Warps walk a matrix of 12288 or 2352 columns in steps of whole rows from eight turns of a device on (2368 warps, 18,944
+    tiles) and leave some out, one of 4096 columns in such steps anyway, one of 528 never; in one call behind each other,
+    forwards and backwards, each with the oracle's bytes.  Without the tall ones the call takes the kernel that keeps no
+    columns, and gives the same."""
+    shapes = [(37, 528, 528), (791, 12288, 12288), (4127, 2352, 2368), (593, 4096, 4104), (77, 12288, 12288)]
+    ws = [WL.small_case(r, c, 700 + i, outlier_entry_frac=0.001, outlier_scale=20.0) for i, (r, c, _) in enumerate(shapes)]
+    hs = [WL.column_weights(c, 800 + i) for i, (_, c, _) in enumerate(shapes)]
+    cfg, ref_cfg = P.cfg_pair(**cfgkw)
+    dev = [P.to_device(w, ld) for w, (_, _, ld) in zip(ws, shapes)]
+    hd = [torch.from_numpy(h).cuda() for h in hs]
+    outs = [api.alloc_buffers(r, c, cfg) for r, c, _ in shapes]
+    for o in outs:
+        o.packed.fill_(0x77), o.scales.fill_(0x7F)        # no block's scale: a tile left out shows
+    api.soar_quantize_weighted_batch(dev, hd, cfg, outs)
+    low = [i for i, (r, _, _) in enumerate(shapes) if r < 700]
+    again = [api.alloc_buffers(*shapes[i][:2], cfg) for i in low]
+    api.soar_quantize_weighted_batch([dev[i] for i in low], [hd[i] for i in low], cfg, again)
+    torch.cuda.synchronize()
+    for i, o in zip(low, again):
+        assert torch.equal(o.packed, outs[i].packed) and torch.equal(o.scales, outs[i].scales) and torch.equal(o.alpha, outs[i].alpha)
+        assert o.read_result().sumsq == pytest.approx(outs[i].read_result().sumsq, rel=1e-12)
+    for w, h, o in zip(ws, hs, outs):
+        gpu = P.GpuOut(o.packed.cpu().numpy(), o.scales.cpu().numpy(), float(o.alpha.cpu()[0]), o.read_result(), o)
+        ref = R.quantize(w, ref_cfg, h=h)
+        P.assert_parity(gpu, ref, mismatch_cap=max(1, w.size // 160000))
+        # (the oracle adds n terms one after the other: n 2^-53 of the sum at most)
+        assert gpu.result.sumsq == pytest.approx(ref.sumsq, rel=max(1e-12, w.size * 2.0 ** -53))
