@@ -95,6 +95,7 @@ struct __align__(128) SoloShared {
   unsigned int slots;                // shared address of the warps' tile slots
   unsigned int per_warp;
   int tiled_only;
+  int error_exp;                     // exponent under which meet_by_sums takes a share of the error
   int failed;
 };
 
@@ -325,11 +326,13 @@ __device__ __forceinline__ double join_fixed(unsigned long long hi, unsigned lon
 // codes written in the pass (1.0 us) and its slots are another trip (0.8 us).  2048 x 2048, from the last arrival until
 // all go on: 3.0 -> 1.8 us.  (A matrix that streams meets by exchange(): its passes are long, and the words cost its
 // search registers, 760 -> 806 us a call of 28672 x 8192.)
-// 4 den is a multiple of 2^-18 below 2^29 a block, its sum exact.  gsum is taken under 64 amax^2 a block (a block's error is
-// at most 16 amax^2 unless its scale is out of all proportion); a share beyond that is announced in the fifth word, and
-// everybody sees so and goes through exchange() instead.  Nothing that the CTAs wrote before is visible after.
+// 4 den is a multiple of 2^-18 below 2^29 a block, its sum exact.  gsum, the error minus sum W^2, is rounded to multiples of at
+// most 2^-77 of sum W^2, which everybody has from the first meeting: 160 CTAs are off by 2^-70 of it together, where the
+// binary64 sums that the error is made of round by 2^-53, and a share above 2^-25 of it keeps every bit.  (Nearest codes
+// leave hardly more error than zeros would; a share beyond twice sum W^2 is announced in the fifth word, and everybody
+// sees so and goes through exchange() instead.)  Nothing that the CTAs wrote before is visible after.
 template <typename S>
-__device__ __forceinline__ bool meet_by_sums(S& sh, const SoloArgs& a, unsigned int pass, unsigned int amax_bits, bool& beyond, Totals& out) {
+__device__ __forceinline__ bool meet_by_sums(S& sh, const SoloArgs& a, unsigned int pass, bool& beyond, Totals& out) {
   __syncthreads();
   const unsigned int tid = threadIdx.x, lane = tid & 31u, grid = gridDim.x, turn = pass & 1u;
   if (tid < 32) {
@@ -341,7 +344,7 @@ __device__ __forceinline__ bool meet_by_sums(S& sh, const SoloArgs& a, unsigned 
     x = warp_sum(x);
     g = warp_sum(g);
     const int blocks = 32 - __clz(a.m.t[0].nblk);   // nblk < 2^blocks
-    const int e_a = 29 + blocks, e_g = 2 * (static_cast<int>(amax_bits >> 7) - 127) + 8 + blocks;
+    const int e_a = 29 + blocks, e_g = sh.error_exp;
     const bool fits = fabs(g) < power_of_two(e_g);
     unsigned long long word[4];
     split_fixed(x, e_a, word[0], word[1]);
@@ -396,11 +399,11 @@ __device__ __forceinline__ bool meet_by_sums(S& sh, const SoloArgs& a, unsigned 
 // The meeting after the start pass (`first`) or an iteration: by sums where a grid goes on from it, else by exchange().
 template <typename S>
 __device__ __forceinline__ bool combine(S& sh, const SoloArgs& a, unsigned long long tag, unsigned int& exchanged, unsigned int& met,
-                                        bool first, bool last, unsigned int amax_bits, Totals& out) {
+                                        bool first, bool last, Totals& out) {
   if constexpr (S::kResident && !S::kCluster && !S::kFinal) {
     if (gridDim.x > 1 && !last) {
       bool beyond;
-      if (!meet_by_sums(sh, a, ++met, amax_bits, beyond, out)) return false;
+      if (!meet_by_sums(sh, a, ++met, beyond, out)) return false;
       if (!beyond) return true;
     }
   }
@@ -513,10 +516,12 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
   double sse = 0.0;
   // every thread keeps the call's scalars itself, and writes the same alpha for the passes to read
   sh.alpha[0] = alpha;
+  // 2^error_exp: more than twice sum W^2, at most four times (a matrix of zeros has no error, any will do)
+  sh.error_exp = max((__double2hiint(sumsq) >> 20) - 1023, -300) + 2;
   if (ok && !(st & (SOAR_STATUS_NONFINITE | SOAR_STATUS_RANGE))) {
     const bool tile_after = !kNoIter && a.tiled != nullptr;
     init_pass(sh, a.m);
-    ok = combine(sh, a, a.nonce + epoch, exchanged, met, true, kNoIter, amax_bits, tot);
+    ok = combine(sh, a, a.nonce + epoch, exchanged, met, true, kNoIter, tot);
     if (kNoIter && blockIdx.x != 0) return;   // nothing left to do but CTA 0's report
     if (st == 0) sse = fmax(sumsq + tot.g, 0.0);
     zero_blocks = tot.counts & 0xFFFFFFFFull;
@@ -534,7 +539,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
       sh.alpha[0] = alpha;
       iterate_pass<kMode>(sh, a.m, (t & 1) != 0, may_stop || t == T - 1, t != T - 1 || (kRes && tile_after));
       const bool last = t == T - 1 && !tile_after;
-      ok = combine(sh, a, a.nonce + epoch, exchanged, met, false, last, amax_bits, tot);
+      ok = combine(sh, a, a.nonce + epoch, exchanged, met, false, last, tot);
       if (last && blockIdx.x != 0) return;
       const double cur = fmax(sumsq + tot.g, 0.0);
       wide += tot.counts;

@@ -35,6 +35,29 @@ def test_the_last_matrix_that_stays_in_shared_memory_and_the_first_that_does_not
     assert one.result.sse == pytest.approx(batched.result.sse, rel=1e-12)
 
 
+@pytest.mark.parametrize("seed", range(6))
+def test_the_error_of_a_resident_matrix_keeps_its_bits_beside_one_large_weight(seed):
+    """One weight stands a hundred thousand times above the others (4096 and some hundredths), so that a CTA's share of the error is a small part of what
+    bounds it.  All rows but one are alike and every warp has nine of them, so that what the CTAs round off their shares adds
+    up.  (Both layouts: the last meeting is then one by sums too.)"""
+    rows = 9 * 16 * torch.cuda.get_device_properties(0).multi_processor_count    # a tile a row
+    row = WL.small_case(1, 512, seed)[0]
+    odd = row.copy()
+    odd[511] = WL.f32_to_bf16_bits(np.float32([4096.0]))[0]       # the maximum: 2^12, the others about 2^-5
+    w = np.tile(row, (rows, 1))
+    w[-1] = odd                                    # few additions follow in its lane
+    cfg = api.soar_default_cfg(api.PRESET_PAPER, max_iters=2, early_stop_rel=0.0,
+                               scale_layout=api.SCALES_LINEAR | api.SCALES_SWIZZLED)
+    gpu = P.run_gpu(w, cfg)
+    for r in (1, rows // 2, rows - 2):             # equal blocks have equal codes
+        assert np.array_equal(gpu.packed[r], gpu.packed[0]) and np.array_equal(gpu.scales[r], gpu.scales[0])
+    each = [R.dequant_error(w[r:r + 1], gpu.packed[r:r + 1], gpu.scales[r:r + 1], gpu.alpha) for r in (0, rows - 1)]
+    sse, sumsq = ((rows - 1) * each[0][i] + each[1][i] for i in (0, 1))
+    # The report is sum W^2 plus (error minus sum W^2), either off by some twenty roundings of 2^-53: nine additions in the lane
+    # with the large weight, ten over its CTA's warps, a few over the CTAs.
+    assert abs(gpu.result.sse - sse) <= 2.0 ** -47 * sumsq
+
+
 @pytest.mark.parametrize("rows,cols", [(2, 128), (16, 8192), (16, 8224), (200, 2064)])
 def test_a_cluster_call_replays_and_repeats(rows, cols):
     """The replay of a captured call, and calls on a workspace that held anything, give what a first call gives."""
