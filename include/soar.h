@@ -492,6 +492,9 @@ int soar_selftest_reciprocal(int lo_exp, int hi_exp, unsigned long long* out_mis
  * fits one thread block or gives some lane more than one block of 32, and single stages.
  * on = 2 does the same to the thread blocks of a cluster alone (one unweighted matrix of 257 to
  * 24,576 blocks): they do not send each other their sums, and give up after sixteen million polls.
+ * on = 3 does it from the second meeting of an unweighted matrix of more than 256 blocks on, in a cluster or on the grid.
+ * on = 4 lets every wait end, but has one thread block of a grid announce at each meeting that its share of the error
+ * is too large for the sums (see meet_by_sums in solo_kernel.cuh): the results are the normal ones.
  * on = 0 restores normal operation.  Process-wide; not for production use.
  */
 int soar_debug_fail_waits(int on);

@@ -55,8 +55,9 @@ namespace {
 constexpr size_t kWsFixedBytes = 2048;
 constexpr unsigned int kGridWaitLimit = 1u << 21;  // polls of the grid's arrival counter before a CTA gives up (each most of a microsecond)
 constexpr unsigned int kClusterWaitLimit = 1u << 24;  // polls of an mbarrier of its own shared memory (each some tens of nanoseconds)
-// What soar_debug_fail_waits makes the CTAs of a launch withhold: their arrivals, or what a cluster's CTAs send each other.
-enum WaitHook : int { kNobodyArrives = 1, kNobodySends = 2 };
+// What soar_debug_fail_waits makes the CTAs of a launch withhold: their arrivals, what a cluster's CTAs send each other, either
+// from the second meeting of a call on one matrix on; or it has one CTA say that its share of the error does not fit.
+enum WaitHook : int { kNobodyArrives = 1, kNobodySends = 2, kNobodyMeetsAgain = 3, kShareBeyond = 4 };
 constexpr int kBracketMinBeta = 2;             // the bracket needs two multipliers; a single one is modes 1-3
 
 struct Ws {
@@ -1748,7 +1749,7 @@ int soar_mx_quantize(const void* W_bf16, int64_t rows, int64_t cols, int64_t ld,
 }
 
 int soar_debug_fail_waits(int on) {
-  g_idle = on == kNobodySends ? on : on ? kNobodyArrives : 0;
+  g_idle = on >= 0 && on <= kShareBeyond ? on : kNobodyArrives;
   return SOAR_OK;
 }
 

@@ -173,7 +173,7 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, int idle, unsigned in
       sh.zeros[0] = sh.wide[0] = sh.wide_high[0] = 0u;
       asm volatile("{\n.reg .b64 t;\nmbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1;\n}" ::"r"(landed), "r"(grid * 24u) : "memory");
     }
-    if (lane < grid && idle != kNobodySends) {
+    if (lane < grid && idle != kNobodySends && (kMax || idle != kNobodyMeetsAgain)) {
       unsigned int at, bar;
       asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(&sh.red[turn][blockIdx.x][0])), "r"(lane));
       asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(landed), "r"(lane));
@@ -255,7 +255,8 @@ __device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned long
       if (lane == 0) {
         unsigned int* const arrived = reinterpret_cast<unsigned int*>(a.exchange + kCounterAt);
         if (pass == 1 && !counter_open(a, tag)) sh.failed = 1;
-        if (a.idle != kNobodyArrives) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
+        if (a.idle != kNobodyArrives && (kMax || a.idle != kNobodyMeetsAgain))
+          asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
         if (!last || blockIdx.x == 0) {
           unsigned int seen = 0, polls = 0;
           do {
@@ -345,7 +346,7 @@ __device__ __forceinline__ bool meet_by_sums(S& sh, const SoloArgs& a, unsigned 
     g = warp_sum(g);
     const int blocks = 32 - __clz(a.m.t[0].nblk);   // nblk < 2^blocks
     const int e_a = 29 + blocks, e_g = sh.error_exp;
-    const bool fits = fabs(g) < power_of_two(e_g);
+    const bool fits = fabs(g) < power_of_two(e_g) && !(a.idle == kShareBeyond && blockIdx.x == 1);
     unsigned long long word[4];
     split_fixed(x, e_a, word[0], word[1]);
     split_fixed(fits ? g : 0.0, e_g, word[2], word[3]);
@@ -366,7 +367,7 @@ __device__ __forceinline__ bool meet_by_sums(S& sh, const SoloArgs& a, unsigned 
     unsigned long long before = 0, seen = 0;
     if (lane < kSumWords) {
       if (pass > 2) before = sh.before[turn][lane];
-      if (a.idle != kNobodyArrives) atomicAdd(at, mine + 1);
+      if (a.idle != kNobodyMeetsAgain) atomicAdd(at, mine + 1);
     }
     // (what is done with the words is done on every poll: after a pass its code comes from L2, a microsecond better spent while
     // others are late)
@@ -522,7 +523,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
     const bool tile_after = !kNoIter && a.tiled != nullptr;
     init_pass(sh, a.m);
     ok = combine(sh, a, a.nonce + epoch, exchanged, met, true, kNoIter, tot);
-    if (kNoIter && blockIdx.x != 0) return;   // nothing left to do but CTA 0's report
+    if (kNoIter && blockIdx.x != 0 && (ok || !kCluster)) return;   // nothing left to do but CTA 0's report
     if (st == 0) sse = fmax(sumsq + tot.g, 0.0);
     zero_blocks = tot.counts & 0xFFFFFFFFull;
     wide = tot.counts >> 32;
@@ -540,7 +541,7 @@ __global__ void __launch_bounds__(kSoloWarps * 32, 1) solo_kernel(const __grid_c
       iterate_pass<kMode>(sh, a.m, (t & 1) != 0, may_stop || t == T - 1, t != T - 1 || (kRes && tile_after));
       const bool last = t == T - 1 && !tile_after;
       ok = combine(sh, a, a.nonce + epoch, exchanged, met, false, last, tot);
-      if (last && blockIdx.x != 0) return;
+      if (last && blockIdx.x != 0 && (ok || !kCluster)) return;
       const double cur = fmax(sumsq + tot.g, 0.0);
       wide += tot.counts;
       iters = t + 1;

@@ -37,9 +37,9 @@ def test_the_last_matrix_that_stays_in_shared_memory_and_the_first_that_does_not
 
 @pytest.mark.parametrize("seed", range(6))
 def test_the_error_of_a_resident_matrix_keeps_its_bits_beside_one_large_weight(seed):
-    """One weight stands a hundred thousand times above the others (4096 and some hundredths), so that a CTA's share of the error is a small part of what
-    bounds it.  All rows but one are alike and every warp has nine of them, so that what the CTAs round off their shares adds
-    up.  (Both layouts: the last meeting is then one by sums too.)"""
+    """One weight stands a hundred thousand times above the others (4096 and some hundredths), so that a CTA's share of the
+    error is a small part of what bounds it.  All rows but one are alike and every warp has nine of them, so that what the CTAs
+    round off their shares adds up.  (Both layouts: the last meeting is then one by sums too.)"""
     rows = 9 * 16 * torch.cuda.get_device_properties(0).multi_processor_count    # a tile a row
     row = WL.small_case(1, 512, seed)[0]
     odd = row.copy()
