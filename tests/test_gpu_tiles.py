@@ -58,6 +58,34 @@ def test_the_error_of_a_resident_matrix_keeps_its_bits_beside_one_large_weight(s
     assert abs(gpu.result.sse - sse) <= 2.0 ** -47 * sumsq
 
 
+@pytest.mark.parametrize("rows,cols,ld_extra", [(5003, 2352, 0), (1025, 1040, 8), (127, 6416, 0)])
+@pytest.mark.parametrize("cfgkw", [dict(), dict(max_iters=1, early_stop_rel=0.0, n_dq=2, n_beta=1)])
+def test_tiled_scales_of_a_resident_matrix_with_ragged_edges(rows, cols, ld_extra, cfgkw):
+    """Grids whose CTAs lay their own scales out: rows that end within a tile of 128, block columns that end within four, a last
+    warp tile that is not full; the bytes of the row-major layout, and zeroes in the padding."""
+    w = WL.small_case(rows, cols, rows)
+    w[5, :16] = 0
+    lin, _ = P.cfg_pair(**cfgkw)
+    both, _ = P.cfg_pair(**cfgkw)
+    both.scale_layout = api.SCALES_LINEAR | api.SCALES_SWIZZLED
+    tiled, _ = P.cfg_pair(**cfgkw)
+    tiled.scale_layout = api.SCALES_SWIZZLED
+    W = P.to_device(w, cols + ld_extra)
+    want = api.soar_quantize(W, lin)
+    r, c = np.meshgrid(np.arange(rows), np.arange(cols // 16), indexing="ij")
+    at = (r // 128 * ((cols // 16 + 3) // 4) + c // 4) * 512 + r % 32 * 16 + r % 128 // 32 * 4 + c % 4
+    for cfg in (both, tiled):
+        out = api.alloc_buffers(rows, cols, cfg)
+        out.scales_sw.fill_(255)
+        api.soar_quantize(W, cfg, out)
+        torch.cuda.synchronize()
+        expect = np.zeros(out.scales_sw.numel(), np.uint8)
+        expect[at] = want.scales.cpu().numpy()
+        assert np.array_equal(out.scales_sw.cpu().numpy(), expect)
+        assert torch.equal(out.packed, want.packed) and torch.equal(out.alpha, want.alpha)
+        assert out.scales is None or torch.equal(out.scales, want.scales)
+
+
 @pytest.mark.parametrize("rows,cols", [(2, 128), (16, 8192), (16, 8224), (200, 2064)])
 def test_a_cluster_call_replays_and_repeats(rows, cols):
     """The replay of a captured call, and calls on a workspace that held anything, give what a first call gives."""
@@ -201,12 +229,18 @@ def test_weighted_calls_at_the_edges_of_a_tile(rows, cols, ld_extra, cfgkw):
     P.assert_parity(gpu, R.quantize(w, ref_cfg, h=h), mismatch_cap=max(1, w.size // 160000))
 
 
-# one warp tile is 16 blocks of 32
-@pytest.mark.parametrize("rows,cols", [(1, 32), (1, 32 * 15), (2, 32 * 8), (1, 32 * 17), (1, 32 * 2049), (9, 32 * 4211), (3, 32 * 18945)])
+# A lane has a block of 32: a lone block, a warp's ragged, whole and overfull turn, one CTA's and one more, and two matrices that
+# give the lanes of a device (two CTAs of 256 an SM, 75,776; three would be 113,664) a second turn, the last one partly filled.
+@pytest.mark.parametrize("rows,cols", [(1, 32), (1, 32 * 15), (2, 32 * 16), (1, 32 * 33), (1, 32 * 257), (1, 32 * 2049), (9, 32 * 4211),
+                                       (3, 32 * 18945), (1021, 32 * 149), (3, 32 * 50527)])
 @pytest.mark.parametrize("ld_extra", [0, 8])
-@pytest.mark.parametrize("cfgkw", [dict(n_beta=0), dict(), dict(n_dq=1, n_beta=5)])
+@pytest.mark.parametrize("cfgkw", [dict(n_beta=0), dict(), dict(n_dq=1, n_beta=5), dict(n_dq=4)])
 def test_mxfp4_calls_at_the_edges_of_a_tile(rows, cols, ld_extra, cfgkw):
     w = WL.small_case(rows, cols, cols)
+    n = rows * cols // 32
+    for i, b in enumerate({0, n // 2, n - 1} if n > 100_000 else ()):      # irregular blocks in the first turn and the last
+        part = w.reshape(-1, 32)[b]
+        part[:] = 0 if i == 0 else WL.f32_to_bf16_bits(WL.bf16_bits_to_f32(part) * np.float32(2.0 ** (-70 if i == 1 else 75)))
     out = api.soar_mx_quantize(P.to_device(w, cols + ld_extra), **cfgkw)
     torch.cuda.synchronize()
     ref, res = R.mx_quantize(w, **cfgkw), out.read_result()
