@@ -137,11 +137,11 @@ def kernel_bytes_per_elem(name: str, cfg, t: int = 0) -> float:
 # belong to one version of the kernels: they are dropped when the device part of the source (everything above
 # the host-side section of soar.cu, and the kernel headers) no longer matches.
 NCU_TRAFFIC = {
-    "kernel_source_sha256_16": "cd229a9d13c4c622",
-    "bytes_per_elem": {"amax_kernel": 2.01, "init_kernel": 2.43, "iterate_kernel/single": 3.01,
+    "kernel_source_sha256_16": "0d55839b97b7ccbb",
+    "bytes_per_elem": {"amax_kernel": 2.01, "init_kernel": 2.43, "iterate_kernel/single": 3.00,
                        "iterate_kernel/grid": 3.45, "weighted_iterate_kernel": 3.48},
-    "inst_per_block": {"amax_kernel": 88, "init_kernel": 181, "iterate_kernel/single": 223,
-                       "iterate_kernel/grid": 360, "weighted_iterate_kernel": 760},
+    "inst_per_block": {"amax_kernel": 88, "init_kernel": 180, "iterate_kernel/single": 223,
+                       "iterate_kernel/grid": 352, "weighted_iterate_kernel": 761},
 }
 
 

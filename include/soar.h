@@ -486,8 +486,8 @@ int soar_selftest_reciprocal(int lo_exp, int hi_exp, unsigned long long* out_mis
  * hook is on, the thread blocks of kernels launched afterwards do not arrive where they meet, so
  * the waits run to the limit (two million polls, a second or two per kernel) with no copy in
  * flight and the kernel returns: the status carries SOAR_STATUS_INTERNAL and the outputs are
- * unspecified.  Calls whose kernels hold no polled wait, or one that on = 2 is for, are not affected and
- * give their normal results: soar_dequant_error, one unweighted matrix of at most 24,576 blocks (one
+ * unspecified.  on = 1: calls whose kernels hold no polled wait, or one that on = 2 is for, are not
+ * affected and give their normal results: soar_dequant_error, one unweighted matrix of at most 24,576 blocks (one
  * thread block, or a cluster) or without iterations, an MXFP4 matrix that
  * fits one thread block or gives some lane more than one block of 32, and single stages.
  * on = 2 does the same to the thread blocks of a cluster alone (one unweighted matrix of 257 to

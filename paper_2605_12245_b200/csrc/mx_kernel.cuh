@@ -22,10 +22,13 @@
 // so it is a rounding midpoint exactly or misses it by 2^-8, far more than the band's 2^-21; the successor's codes are then
 // nearest ones, ties either way, its error is the least there is, and only an earlier multiplier can share the first place.
 //
-// Bound by instruction issue, 300 per sixteen elements in 72 % of the cycles: 28672 x 8192 with the search 171 us (594 MB:
-// 3.5 TB/s), by the plain rule 115 us.  Two lanes to a block, which each did the whole of the block's own work (centre, brackets,
-// reciprocals) and exchanged their sums, took 373 instructions, 216 us and 122 us.  The two halves of a block go through the
-// four candidates one after the other; both at once spill (238 us).
+// The search is bound by instruction issue, 300 per sixteen elements in 71 % of the cycles: 28672 x 8192 171 us (594 MB:
+// 3.5 TB/s).  The plain rule, 146 instructions in 55 % of the cycles, waits for its loads: 115 us, 5.1 TB/s.  Two lanes to
+// a block, which each did the whole of the block's own work (centre, brackets, reciprocals) and exchanged their sums, took 373
+// instructions and 216 us, 211 and 122 us.  The two halves of a block go through the four candidates one after the other; both
+// at once spill (238 us).  Other forms on that shape, with two lanes and now: a base aligned to 16 bytes only 229 -> 183 us (plain
+// rule 122.5 -> 121), a row stride 8 above the columns 230 -> 184 (151 -> 123), one code on five multipliers 426 -> 322, four codes
+// on 101 1010 -> 642, where the general rules read the matrix a second time.
 
 #pragma once
 

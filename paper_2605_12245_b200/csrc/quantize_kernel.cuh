@@ -10,10 +10,11 @@
 //   The search is bound by instruction issue: a lane loads its next block, 32 bytes with one 256-bit load, into
 //   registers one tile ahead, which costs 20 instructions a block less.
 // 28672 x 8192, one pass as a launch of its own: maximum 82 -> 77 us (2.01 bytes an element, 6.1 TB/s), start 127 -> 111 us
-// (2.43 bytes, 181 instructions a block), iteration of the search 307 -> 215 us (3.45 bytes, 360 instructions a block, since then 352, issued in
-// 71 % of the cycles); within a call an iteration takes 191 us.
+// (2.43 bytes, 180 instructions a block), iteration of the search 307 -> 210 us (3.45 bytes, 352 instructions a block issued
+// in 71 % of the cycles).
 // Two CTAs of 256 threads per SM leave 128 registers a thread, which holds a block, the next one, the four candidates
-// of the search and their sums without spills (the deterministic forms spill up to 26 bytes).
+// of the search and their sums without spills (the deterministic forms spill up to 34 bytes, one of a single matrix that
+// streams 8).
 //
 // Bytes 16 apart in a slot are exchanged between its two 128-byte halves (tile_chunk) so that the 32-byte reads
 // of neighbouring lanes meet no bank conflict.

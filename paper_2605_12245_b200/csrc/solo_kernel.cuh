@@ -4,15 +4,16 @@
 // Small matrices are bound by latency: what counts is the chain from the last block of one pass to the first of the
 // next.  With the sums added by atomics in memory zeroed by a memset, that chain took 3.5 of the 5 microseconds of an
 // iteration at any size.  Here every CTA stores its sums in a slot of its own, arrives at a counter and, when all
-// have, reads everybody's slots and adds them in the same order on every run: 1.6 us from the last arrival on, for 2 to
-// 148 CTAs.  (Polling tagged slots instead, with no counter, is 0.7 us when all CTAs come at the same moment but 3 us
-// when some wait for others, as they do.)  A matrix that stays in shared memory has a shorter way after the start pass and the
+// have, reads everybody's slots and adds them in the same order on every run: 1.6 us when all come at the same moment;
+// within a call, from the last CTA's arrival until all go on, 2.3 to 3.1 us, on 28672 x 8192 3.3 and 4.1.  (Polling tagged
+// slots instead, with no counter, is 0.7 us when all CTAs come at the same moment but 3 us when some wait for others,
+// as they do.)  A matrix that stays in shared memory has a shorter way after the start pass and the
 // iterations (meet_by_sums).  The grid is one CTA of 16 warps per SM rather than two of 8: 296 CTAs need
 // 0.7 us more.
 //
 // The smallest matrices (see kClusterTiles) run in one cluster of up to 16 CTAs: the sums travel through distributed shared
-// memory (exchange_in_cluster), with nothing in global memory and no cooperative launch.  256
-// tiles: an iteration with one candidate 2.2 us (3.2 through the counter), a max-based call 6.5 us (9.4).
+// memory (exchange_in_cluster), with nothing in global memory and no cooperative launch.  256 tiles: an iteration with one
+// candidate 1.8 us (2.3 on a grid that meets by sums), of the search 2.3 (2.8), a max-based call 6.1 us (8.0 as two kernels).
 //
 // Matrices whose tiles fit the shared memory of the grid (12 million weights) are read from HBM once and stay
 // there, and so do their block states (kResident); larger ones stream through the passes like a batch.
@@ -31,9 +32,11 @@ constexpr unsigned int kSoloMaxGrid = 160;
 constexpr unsigned int kResidentTiles = 160;       // slots a CTA can have: 200 KB
 constexpr size_t kSlotBytes = 24;                  // three numbers of one CTA and pass
 
-// Up to kOneCtaTiles tiles run in one CTA; up to kClusterTiles in a cluster, a warp to a tile while 256 warps suffice.  At
-// 768 tiles (three a warp) the cluster's shorter exchange and the grid's 48 warps more than weigh each other: max-based
-// calls 8.4 against 9.4 us, an iteration of the search 4.6 us either way; at 1024 the search is slower, 6.2 against 4.6.
+// Up to kOneCtaTiles tiles run in one CTA; up to kClusterTiles in a cluster, a warp to a tile while 256 warps suffice.  The
+// cluster saves the cooperative launch and the first meetings' trips, the grid has three times the warps at 768 tiles: a search of
+// one iteration 11.6 us against 16.1 there, each further one 4.8 against 3.6, so that at the usual three the cluster is
+// ahead (21 against 23) and at 1024 tiles behind (24.5 against 22); with one candidate 9.7 against 14.4 and 3.1 against
+// 2.7; max-based calls 9.5 against 12.0, 7.2 against 8.0 at 1024.
 constexpr unsigned int kOneCtaTiles = 8, kClusterMost = 16, kClusterTiles = 768;
 constexpr unsigned int cluster_warps(unsigned int tiles) {
   const unsigned int even = (tiles + kClusterMost - 1) / kClusterMost;
@@ -146,9 +149,9 @@ __device__ __forceinline__ double half_warp_sum(double v) {
 }
 
 // exchange() inside a cluster: every CTA sends its numbers into everybody's shared memory with stores that count themselves
-// off at the receiver's mbarrier, so that nothing is released and nobody waits for the codes written in the pass (at the
-// hardware's cluster barrier instead: 1.7 us after an iteration that wrote codes, 0.9 after
-// the other passes; now 1.4 and 0.5).
+// off at the receiver's mbarrier, so that nothing is released and nobody waits for the codes written in the pass.  From the
+// last CTA's arrival until all go on 0.45 us after the maximum, 0.55 to 0.6 after the other passes (the hardware's
+// cluster barrier took 0.3 to 0.4 us more a meeting).
 // One try_wait, which sleeps until the numbers are there (test_wait alone: 0.1 us more a call), then polls with test_wait,
 // which returns at once: how long a try_wait may stay suspended is the hardware's choice, so that a count of them bounds
 // nothing.  The polls cannot run out in earnest, since a cluster's CTAs run together and a pass waits for nobody; a CTA that gives
@@ -219,8 +222,9 @@ __device__ __forceinline__ bool exchange_in_cluster(S& sh, int idle, unsigned in
   return sh.failed == 0;
 }
 
-// After a pass, all threads of all CTAs: exchanges the CTAs' sums.  `pass` counts from 1.  What the CTAs wrote to global
-// memory before is visible to all after.  With `last` only CTA 0 waits for the sums.  False when a wait ran out.
+// After a pass, all threads of all CTAs: exchanges the CTAs' sums.  `pass` counts from 1.  On a grid what the CTAs wrote to
+// global memory before is visible to all after (in a cluster it is not), and with `last` only CTA 0 waits for the sums.  False
+// when a wait ran out.
 // kMax: after the pass for the maximum; first: after the start pass.
 template <bool kMax, typename S>
 __device__ __forceinline__ bool exchange(S& sh, const SoloArgs& a, unsigned long long tag, unsigned int pass, bool first, bool last,
@@ -324,8 +328,8 @@ __device__ __forceinline__ double join_fixed(unsigned long long hi, unsigned lon
 // After the start pass and the iterations of a resident matrix, all threads of all CTAs of a grid: the sums of exchange() in
 // one trip.  A CTA adds its parts to the words of the meeting and polls them until everybody's are in: the data is its own
 // arrival, so that nothing has to be made visible before it or read after it, where exchange()'s release waits for the
-// codes written in the pass (1.0 us) and its slots are another trip (0.8 us).  2048 x 2048, from the last arrival until
-// all go on: 3.0 -> 1.8 us.  (A matrix that streams meets by exchange(): its passes are long, and the words cost its
+// codes written in the pass and its slots are another trip.  From the last arrival until all go on 1.5 to 2.1 us on 2048 x
+// 2048 and 1.3 to 1.6 on 5003 x 2352, by exchange() 2.5 to 2.9.  (A matrix that streams meets by exchange(): its passes are long, and the words cost its
 // search registers, 760 -> 806 us a call of 28672 x 8192.)
 // 4 den is a multiple of 2^-18 below 2^29 a block, its sum exact.  gsum, the error minus sum W^2, is rounded to multiples of at
 // most 2^-77 of sum W^2, which everybody has from the first meeting: 160 CTAs are off by 2^-70 of it together, where the

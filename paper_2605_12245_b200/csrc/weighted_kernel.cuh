@@ -12,8 +12,8 @@
 // What bounds it: instruction issue, 760 a block with the binary64 pipe, which issues one in two cycles, at 36 %.  A
 // candidate costs three binary64 operations per element, p = h (4m), A += p |w|, B += p (4m); the code values become
 // binary64 by byte permutes (code_words; the integer conversion instruction instead, for half or all of one candidate,
-// was 0 to 4 % slower).  28672 x 8192, one iteration within a call: 980 -> 474 us (as a launch of its own 1084 -> 520); the
-// whole call of 4 iterations 4.61 -> 2.32 ms.
+// was 0 to 4 % slower).  28672 x 8192, a launch a pass: iteration 1084 -> 508 us, the maximum 80 us, the start 181; one iteration
+// within a call 980 -> 474 us.
 
 #pragma once
 
